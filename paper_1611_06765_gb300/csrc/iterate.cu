@@ -807,47 +807,93 @@ void pnm_split_f2(const double* a, f2* b, long n, cudaStream_t s) {
 // End of one update: energy (Eq. ccdcorr, sum of v t over restricted amplitudes) and
 // residual norm per system from the block partials in a fixed order, the |dE| test, the
 // energy history, and the loop condition of the device-side loop.
+// It runs alone on one SM after the last block of the update, so its time adds to every update:
+// a chain of dependent round trips, not bandwidth.  Batches of at least FIN_WARP_SYSTEMS systems
+// take one warp per system (no block barrier between systems); fewer take the whole block per
+// system, which reads the several thousand partials of a large system with four times the loads
+// in flight.  FIN_UNROLL partial pairs are requested before the first is added.  120 systems of
+// 27 partials each, mixed solve of 20 updates read back whole: 21.0 -> 16.4 ms against the block
+// taking the systems one after the other (two reductions and three barriers each); a single
+// system of 66 states, 39 updates: 1.143 -> 1.122 ms from the earlier loads.
+constexpr int FIN_WARP_SYSTEMS = 4, FIN_UNROLL = 8;
+
+__device__ __forceinline__ void sum_partials(const FinArgs& f, int s, int first, int step, double& e, double& r) {
+  const int hi = f.hi[s];
+  e = 0.0;
+  r = 0.0;
+  int k = f.lo[s] + first;
+  for (; k + (FIN_UNROLL - 1) * step < hi; k += FIN_UNROLL * step) {
+    double a[FIN_UNROLL], b[FIN_UNROLL];
+#pragma unroll
+    for (int j = 0; j < FIN_UNROLL; j++) {
+      a[j] = __ldcg(f.eparts + k + j * step);
+      b[j] = __ldcg(f.rparts + k + j * step);
+    }
+#pragma unroll
+    for (int j = 0; j < FIN_UNROLL; j++) {
+      e += a[j];
+      r += b[j];
+    }
+  }
+  for (; k < hi; k += step) {
+    e += __ldcg(f.eparts + k);
+    r += __ldcg(f.rparts + k);
+  }
+}
+
+// One system's control block from its energy and squared residual (one thread).  S and the loop
+// control c are copies read before the sums, so that their loads overlap the partials'.
+__device__ __forceinline__ void finalize_one(const FinArgs& f, SysCtl S, const LoopCtl& c, int s, double e, double r,
+                                             bool& all_done, bool& bad) {
+  if (!S.done) {
+    S.iters += 1;
+    S.e_new = e;
+    S.resid = sqrt(r);
+    if (S.iters < f.hist_cap) f.hist[(long)s * f.hist_cap + S.iters] = e;
+    const double diff = fabs(e - S.e_old);
+    S.e_old = e;
+    S.grow = (diff > 2.0 * S.d_old && diff > S.tol) ? S.grow + 1 : 0;
+    S.d_old = diff;
+    bad = bad || !isfinite(e) || !isfinite(r) || S.grow >= PNM_DIVERGE_STEPS;
+    if (diff < S.tol && c.iter + 1 >= c.min_iter) {
+      S.done = 1;
+      S.frozen_at = c.iter;
+    }
+    f.sc[s] = S;
+  }
+  all_done = all_done && S.done;
+}
+
 __device__ void finalize_systems(const FinArgs& f, LoopCtl* ctl) {
   __shared__ double sh32f[32];
-  __shared__ int all_done, bad;
-  if (threadIdx.x == 0) {
-    all_done = 1;
-    bad = 0;
-  }
-  __syncthreads();
-  for (int s = 0; s < f.nsys; s++) {
-    double e = 0.0, r = 0.0;
-    for (int k = f.lo[s] + threadIdx.x; k < f.hi[s]; k += blockDim.x) {
-      e += __ldcg(f.eparts + k);
-      r += __ldcg(f.rparts + k);
+  const LoopCtl c = *ctl;
+  bool all_done = true, bad = false;  // of the systems this thread closes
+  double e, r;
+  if (f.nsys >= FIN_WARP_SYSTEMS) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int s = warp; s < f.nsys; s += nw) {
+      SysCtl S;
+      if (lane == 0) S = f.sc[s];
+      sum_partials(f, s, lane, 32, e, r);
+      e = warp_sum(e);
+      r = warp_sum(r);
+      if (lane == 0) finalize_one(f, S, c, s, e, r, all_done, bad);
     }
-    e = block_sum(e, sh32f);
-    r = block_sum(r, sh32f);
-    if (threadIdx.x == 0) {
-      SysCtl& S = f.sc[s];
-      if (!S.done) {
-        S.iters += 1;
-        S.e_new = e;
-        S.resid = sqrt(r);
-        if (S.iters < f.hist_cap) f.hist[(long)s * f.hist_cap + S.iters] = e;
-        double diff = fabs(e - S.e_old);
-        S.e_old = e;
-        S.grow = (diff > 2.0 * S.d_old && diff > S.tol) ? S.grow + 1 : 0;
-        S.d_old = diff;
-        if (!isfinite(e) || !isfinite(r) || S.grow >= PNM_DIVERGE_STEPS) bad = 1;
-        if (diff < S.tol && ctl->iter + 1 >= ctl->min_iter) {
-          S.done = 1;
-          S.frozen_at = ctl->iter;
-        }
-      }
-      if (!S.done) all_done = 0;
+    all_done = __syncthreads_and(all_done);
+    bad = __syncthreads_or(bad);
+  } else {
+    for (int s = 0; s < f.nsys; s++) {
+      SysCtl S;
+      if (threadIdx.x == 0) S = f.sc[s];
+      sum_partials(f, s, threadIdx.x, blockDim.x, e, r);
+      block_sum2(e, r, sh32f);
+      if (threadIdx.x == 0) finalize_one(f, S, c, s, e, r, all_done, bad);
     }
-    __syncthreads();
   }
   if (threadIdx.x == 0) {
-    ctl->iter += 1;
+    ctl->iter = c.iter + 1;
     int cont = 1;
-    if (ctl->dev_error) {
+    if (c.dev_error) {
       ctl->status = PNM_ETIMEOUT;
       cont = 0;
     } else if (bad) {
@@ -856,7 +902,7 @@ __device__ void finalize_systems(const FinArgs& f, LoopCtl* ctl) {
     } else if (all_done) {
       ctl->status = 1;
       cont = 0;
-    } else if (ctl->iter >= ctl->max_iter) {
+    } else if (c.iter + 1 >= c.max_iter) {
       ctl->status = PNM_ENOTCONV;
       cont = 0;
     }
@@ -1385,12 +1431,16 @@ __global__ void k_reduce_rows(const double* __restrict__ parts, const int* __res
 __global__ void k_start(const double* __restrict__ parts, const int* __restrict__ row_lo,
                         const int* __restrict__ row_hi, int nsys, SysCtl* __restrict__ sc,
                         LoopCtl* __restrict__ ctl, double* __restrict__ hist, int hist_cap) {
+  // one warp per system in batches (as in finalize_systems), else the whole block
   __shared__ double sh32[32];
-  for (int s = 0; s < nsys; s++) {
+  const bool by_warp = nsys >= FIN_WARP_SYSTEMS;
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int s = by_warp ? threadIdx.x >> 5 : 0; s < nsys; s += by_warp ? nw : 1) {
     double acc = 0.0;
-    for (int r = row_lo[s] + threadIdx.x; r < row_hi[s]; r += blockDim.x) acc += parts[r];
-    acc = block_sum(acc, sh32);
-    if (threadIdx.x == 0) {
+    for (int r = row_lo[s] + (by_warp ? lane : threadIdx.x); r < row_hi[s]; r += by_warp ? 32 : blockDim.x)
+      acc += parts[r];
+    acc = by_warp ? warp_sum(acc) : block_sum(acc, sh32);
+    if (by_warp ? lane == 0 : threadIdx.x == 0) {
       sc[s].e_old = acc;
       sc[s].e_new = acc;
       sc[s].resid = 0.0;
