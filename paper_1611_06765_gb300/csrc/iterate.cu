@@ -10,7 +10,8 @@
 //              <kl|chi|ij> = <kl|v|ij> + 1/2 <kl|v|cd> t_ij^cd per direct channel
 //   k_dchi     chi_p - eps_p per state, gathered over the pairs holding p
 //   k_ph       T_x = remap(t); C_x = V1_x + 1/2 W_x T_x; Q_x = T_x C_x per cross channel
-//   k_pp64     1/2 sum_cd <ab|v|cd> t_cd^ij, grouped over all channels with a V_pppp block (FP64)
+//   k_pp       1/2 sum_cd <ab|v|cd> t_cd^ij, grouped over all channels with a V_pppp block (FP64
+//              accuracy from digit products on the tensor cores)
 //   k_update   Jacobi step t_new = (v + rest) / eps_ij^ab, mixing, energy/residual partials
 //   finalize   (last block of k_update) Eq. (ccdcorr) energy per system, |dE| test,
 //              device-side loop condition
@@ -22,6 +23,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "dig.cuh"
 #include "pnm_context.cuh"
 
 #ifndef PNM_UPD_HH_UNROLL
@@ -161,13 +163,6 @@ __global__ void k_dchi(DevState D, int nsp_total) {
 template <typename T_, int TS>
 struct VecT;
 template <>
-struct VecT<double, 2> {
-  __device__ __forceinline__ static void ld(const double* p, double (&v)[2]) {
-    double2 a = *reinterpret_cast<const double2*>(p);
-    v[0] = a.x; v[1] = a.y;
-  }
-};
-template <>
 struct VecT<float, 2> {
   __device__ __forceinline__ static void ld(const float* p, float (&v)[2]) {
     float2 a = *reinterpret_cast<const float2*>(p);
@@ -181,28 +176,6 @@ struct VecT<float, 4> {
     v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
   }
 };
-template <>
-struct VecT<f2, 2> {
-  __device__ __forceinline__ static void ld(const f2* p, f2 (&v)[2]) {
-    float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = f2{q.x, q.y}; v[1] = f2{q.z, q.w};
-  }
-};
-
-// Element e of a cross channel's T: read from the FP32 copy in the cross-channel layout that
-// the mixed update scatters (xt), or gathered through the signed index map from the current
-// amplitudes (tcur): FP64, or their FP32-pair copy for the FP32-pair kernels.
-template <typename T_>
-__device__ __forceinline__ T_ ph_t(const DevState& D, const T_* __restrict__ tcur,
-                                   const T_* __restrict__ xt, long e) {
-  using A = Arith<T_>;
-  if (xt) return xt[e];
-  int cd = D.xmap[e];
-  if (cd == 0) return A::zero();
-  T_ g = tcur[cd > 0 ? cd - 1 : -cd - 1];
-  return cd < 0 ? A::neg(g) : g;
-}
-
 // Bytes reserved for the index tables at the start of a k_ph CTA's shared memory (R4 + 2 H4
 // ints are used; 2 (R4 + H4) with R4, H4 even keeps the reservation a multiple of 16 bytes).
 __host__ __device__ __forceinline__ size_t ph_index_bytes(int R4, int H4) { return sizeof(int) * 2 * (size_t)(R4 + H4); }
@@ -211,15 +184,14 @@ __host__ __device__ __forceinline__ size_t ph_index_bytes(int R4, int H4) { retu
 // channel as the pair (sum, difference) of half-size problems, Q written on its spin-up rows.
 // Per problem, in shared memory zero-padded to multiples of TS (R rows (a,i), H columns (k,c)):
 //   Ts = T (R x H), Xt = W^T staged as W (R x H), then T^T (H x R), Cs = C (H x H);
-//   C[(k,c)][(j,b)] = <kb|v|cj> + 1/2 sum_(e,l) <kl|v|ce> t_lj^eb   (xw == nullptr: <kb|v|cj>)
+//   C[(k,c)][(j,b)] = <kb|v|cj> + 1/2 sum_(e,l) <kl|v|ce> t_lj^eb
 //   Q[(a,i)][(j,b)] = sum_(k,c) t_ik^ac C[(k,c)][(j,b)]
 // Each thread accumulates TS x TS outputs of every problem per tile.  Element arithmetic is
 // that of Arith<T_> (FP64, FP32, or FP32 pairs with FP64 results).
 template <typename T_, int NT, int TS, int NM>
 __device__ __forceinline__ void ph_block(const DevState& D, int x, unsigned char* smraw,
-                                         const T_* __restrict__ tcur, const T_* __restrict__ xt,
-                                         const T_* __restrict__ xw, const T_* __restrict__ xv1,
-                                         typename Arith<T_>::Out* __restrict__ xq) {
+                                         const T_* __restrict__ xt, const T_* __restrict__ xw,
+                                         const T_* __restrict__ xv1, typename Arith<T_>::Out* __restrict__ xq) {
   using A = Arith<T_>;
   const int nph = D.x_nph[x], nhp = D.x_nhp[x];
   const int R = NM == 2 ? nph >> 1 : nph, H = NM == 2 ? nhp >> 1 : nhp;
@@ -247,7 +219,6 @@ __device__ __forceinline__ void ph_block(const DevState& D, int x, unsigned char
     }
     __syncthreads();
   }
-  const bool quad = xw != nullptr;
   // element e = u H4 + s of the staging loops: (u, s) advanced by NT per step without a division
   const int du = NT / H4, ds = NT % H4;
   int u = threadIdx.x / H4, s = threadIdx.x % H4;
@@ -257,19 +228,17 @@ __device__ __forceinline__ void ph_block(const DevState& D, int x, unsigned char
     if (u < R && s < H) {
       if constexpr (NM == 1) {
         long o = (long)u * nhp + s;
-        t0 = ph_t<T_>(D, tcur, xt, to + o);
-        if (quad) w0 = xw[wo + o];
+        t0 = xt[to + o];
+        w0 = xw[wo + o];
       } else {
         int row = sra[u], ca = sca[s], cb = scb[s];
         long oa = (long)row * nhp + ca, ob = (long)row * nhp + cb;
-        T_ ta = ph_t<T_>(D, tcur, xt, to + oa), tb = ph_t<T_>(D, tcur, xt, to + ob);
+        T_ ta = xt[to + oa], tb = xt[to + ob];
         t0 = A::add(ta, tb);
         t1 = A::sub(ta, tb);
-        if (quad) {
-          T_ wa = xw[wo + oa], wb = xw[wo + ob];
-          w0 = A::add(wa, wb);
-          w1 = A::sub(wa, wb);
-        }
+        T_ wa = xw[wo + oa], wb = xw[wo + ob];
+        w0 = A::add(wa, wb);
+        w1 = A::sub(wa, wb);
       }
     }
     Ts[e] = t0;
@@ -310,7 +279,7 @@ __device__ __forceinline__ void ph_block(const DevState& D, int x, unsigned char
   }
   __syncthreads();
   const int th = H4 / TS;
-  if (quad) {
+  {
     // C += 1/2 W^T T (padded rows and columns stay zero)
     for (int tile = threadIdx.x; tile < NM * th * th; tile += NT) {
       const int mtx = tile / (th * th), tt = tile % (th * th);
@@ -401,9 +370,8 @@ __device__ __forceinline__ void ph_block(const DevState& D, int x, unsigned char
 constexpr int PH_WARPS = PH_THREADS / 32;
 template <typename T_>
 __device__ __forceinline__ void ph_warp_body(const DevState& D, int x, int w, int lane, unsigned char* smraw,
-                                             const T_* __restrict__ tcur, const T_* __restrict__ xt,
-                                             const T_* __restrict__ xw, const T_* __restrict__ xv1,
-                                             typename Arith<T_>::Out* __restrict__ xq) {
+                                             const T_* __restrict__ xt, const T_* __restrict__ xw,
+                                             const T_* __restrict__ xv1, typename Arith<T_>::Out* __restrict__ xq) {
   using A = Arith<T_>;
   constexpr int S = PH_WARP_DIM;
   const int nph = D.x_nph[x], nhp = D.x_nhp[x];
@@ -429,21 +397,20 @@ __device__ __forceinline__ void ph_warp_body(const DevState& D, int x, int w, in
     }
   }
   __syncwarp();
-  const bool quad = xw != nullptr;
   for (int e = lane; e < R * H; e += 32) {
     int u = e / H, c = e % H;
     if (two) {
       long oa = (long)sra[u] * nhp + sca[c], ob = (long)sra[u] * nhp + scb[c];
-      T_ ta = ph_t<T_>(D, tcur, xt, to + oa), tb = ph_t<T_>(D, tcur, xt, to + ob);
+      T_ ta = xt[to + oa], tb = xt[to + ob];
       Ts[u * S + c] = A::add(ta, tb);
       Ts[S * S + u * S + c] = A::sub(ta, tb);
-      T_ wa = quad ? xw[wo + oa] : A::zero(), wb = quad ? xw[wo + ob] : A::zero();
+      T_ wa = xw[wo + oa], wb = xw[wo + ob];
       Ws[u * S + c] = A::add(wa, wb);
       Ws[S * S + u * S + c] = A::sub(wa, wb);
     } else {
       long o = (long)u * nhp + c;
-      Ts[u * S + c] = ph_t<T_>(D, tcur, xt, to + o);
-      Ws[u * S + c] = quad ? xw[wo + o] : A::zero();
+      Ts[u * S + c] = xt[to + o];
+      Ws[u * S + c] = xw[wo + o];
     }
   }
   __syncwarp();
@@ -459,7 +426,7 @@ __device__ __forceinline__ void ph_warp_body(const DevState& D, int x, int w, in
         v = xv1[co + (long)r * nhp + c];
       }
       T_ acc = A::zero();
-      for (int u = 0; u < R && quad; u++) A::mac(acc, Ws[m * S * S + u * S + r], Ts[m * S * S + u * S + c]);
+      for (int u = 0; u < R; u++) A::mac(acc, Ws[m * S * S + u * S + r], Ts[m * S * S + u * S + c]);
       Cs[m * S * S + r * S + c] = A::add(v, A::half(acc));
     }
   }
@@ -479,34 +446,23 @@ __device__ __forceinline__ void ph_warp_body(const DevState& D, int x, int w, in
   }
 }
 
-// The current amplitudes the ph kernels gather T from (not used when T is read from the
-// scattered FP32 copy): FP64, or the FP32-pair copy made at the start of the sweep.
-template <typename T_>
-__device__ __forceinline__ const T_* ph_tcur(const DevState& D, const LoopCtl* ctl, const T_* tpair) {
-  if constexpr (std::is_same<T_, double>::value) return cur_t(D, ctl);
-  else return tpair;
-}
-
 // The ph term over the S_z >= 0 cross channels (xlist): the first nblk CTAs take one channel
 // each (the costliest first), with the S_z > 0 or the S_z = 0 body chosen per channel; the
-// remaining CTAs take PH_WARPS small channels each, one per warp.  Channels are launched in two
-// size classes with their own shared memory (the larger ones by k_ph_big).
+// remaining CTAs take PH_WARPS small channels each, one per warp.  (FP32, the mixed iteration.)
 template <typename T_, int NT, int TS>
 __global__ void __launch_bounds__(NT) k_ph(DevState D, const LoopCtl* __restrict__ ctl,
                                            const int* __restrict__ xlist, int nblk, int nwarp,
-                                           const T_* __restrict__ tpair, const T_* __restrict__ xt,
-                                           const T_* __restrict__ xw, const T_* __restrict__ xv1,
-                                           typename Arith<T_>::Out* __restrict__ xq) {
+                                           const T_* __restrict__ xt, const T_* __restrict__ xw,
+                                           const T_* __restrict__ xv1, typename Arith<T_>::Out* __restrict__ xq) {
   static_assert(NT == PH_WARPS * 32, "one warp per small channel");
   extern __shared__ __align__(16) unsigned char smraw[];
-  const T_* tcur = xt ? nullptr : ph_tcur<T_>(D, ctl, tpair);
   if ((int)blockIdx.x < nblk) {
     const int x = xlist[blockIdx.x];
     if (sys_done(D, ctl, D.x_sys[x])) return;  // CTA-uniform
     if (D.x_cls[x] == 0)
-      ph_block<T_, NT, TS, 2>(D, x, smraw, tcur, xt, xw, xv1, xq);
+      ph_block<T_, NT, TS, 2>(D, x, smraw, xt, xw, xv1, xq);
     else
-      ph_block<T_, NT, TS, 1>(D, x, smraw, tcur, xt, xw, xv1, xq);
+      ph_block<T_, NT, TS, 1>(D, x, smraw, xt, xw, xv1, xq);
     return;
   }
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -514,25 +470,7 @@ __global__ void __launch_bounds__(NT) k_ph(DevState D, const LoopCtl* __restrict
   if (idx >= nwarp) return;  // whole warps leave; the warp path never synchronises the block
   const int x = xlist[nblk + idx];
   if (sys_done(D, ctl, D.x_sys[x])) return;  // warp-uniform
-  ph_warp_body<T_>(D, x, w, lane, smraw, tcur, xt, xw, xv1, xq);
-}
-
-// The channels of the larger size class: one CTA of PH_BIG_THREADS per channel.
-constexpr int PH_BIG_THREADS = 256;
-template <typename T_, int TS>
-__global__ void __launch_bounds__(PH_BIG_THREADS) k_ph_big(DevState D, const LoopCtl* __restrict__ ctl,
-                                                           const int* __restrict__ xlist,
-                                                           const T_* __restrict__ tpair, const T_* __restrict__ xt,
-                                                           const T_* __restrict__ xw, const T_* __restrict__ xv1,
-                                                           typename Arith<T_>::Out* __restrict__ xq) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int x = xlist[blockIdx.x];
-  if (sys_done(D, ctl, D.x_sys[x])) return;  // CTA-uniform
-  const T_* tcur = xt ? nullptr : ph_tcur<T_>(D, ctl, tpair);
-  if (D.x_cls[x] == 0)
-    ph_block<T_, PH_BIG_THREADS, TS, 2>(D, x, smraw, tcur, xt, xw, xv1, xq);
-  else
-    ph_block<T_, PH_BIG_THREADS, TS, 1>(D, x, smraw, tcur, xt, xw, xv1, xq);
+  ph_warp_body<T_>(D, x, w, lane, smraw, xt, xw, xv1, xq);
 }
 
 static size_t ph_warp_smem(size_t elem) {
@@ -546,131 +484,740 @@ size_t ph_smem_bytes(int max_dim, int nm, size_t elem) {
   return ph_index_bytes(m4, m4) + elem * 3 * (size_t)nm * m4 * m4;
 }
 
-// Shared memory of the launches: the larger size class alone (k_ph_big); for the 8-byte types
-// the middle and the small class each alone and the warp path alone (PNM_PH_CLASSES = 4), or
-// the smaller classes with the warp path in one launch (2, the default: the tails of the extra
-// launches cost more than their higher occupancy gains); FP32 in one launch.
-#ifndef PNM_PH_CLASSES
-#define PNM_PH_CLASSES 2
-#endif
-template <typename T_>
-static size_t ph_smem_of(const pnm_ctx* ctx) {
-  size_t b = sizeof(T_) == 8 ? std::max(ctx->ph_smem64, ctx->ph_mid_smem64)
-                             : std::max(std::max(ctx->ph_smem32, ctx->ph_mid_smem32), ctx->ph_big_smem32);
-  return ctx->n_ph_warp > 0 ? std::max(b, ph_warp_smem(sizeof(T_))) : b;
-}
-template <typename T_>
-static size_t ph_big_smem_of(const pnm_ctx* ctx) {
-  return sizeof(T_) == 8 ? ctx->ph_big_smem64 : ctx->ph_big_smem32;
+static size_t ph32_smem(const pnm_ctx* ctx) {
+  const size_t b = std::max(std::max(ctx->ph_smem32, ctx->ph_mid_smem32), ctx->ph_big_smem32);
+  return ctx->n_ph_warp > 0 ? std::max(b, ph_warp_smem(sizeof(float))) : b;
 }
 
-// Register tile of the ph kernels: 2 x 2 for FP64 (little padding; the FP64 pipe bounds the
-// kernel) and FP32 pairs, 4 x 4 for FP32 (fewer shared-memory loads per FMA).
+// Register tile of the FP32 ph kernel (4 x 4: few shared-memory loads per FMA).
 #ifndef PNM_PH32_TILE
 #define PNM_PH32_TILE 4
 #endif
-template <typename T_>
-constexpr int ph_tile() { return std::is_same<T_, float>::value ? PNM_PH32_TILE : 2; }
-
-// The ph term: one launch over the S_z >= 0 cross channels (ph_list, costliest first).
-// The 8-byte element types (FP64, FP32 pairs) are limited by shared memory: the larger channels
-// go to k_ph_big with their own allocation so that the others fit more CTAs per SM.  FP32 is
-// limited by registers: one launch, the larger channels first.
-template <typename T_>
-static void launch_ph_list(pnm_ctx* ctx, const T_* tpair, const T_* xt, const T_* xw, const T_* xv1,
-                           typename Arith<T_>::Out* xq, cudaStream_t s) {
-  constexpr int TS = ph_tile<T_>();
-  constexpr bool split = sizeof(T_) == 8;
-  const int nwb = (ctx->n_ph_warp + PH_WARPS - 1) / PH_WARPS;
-  if (!split) {
-    // FP32: every channel in one launch, the larger first
-    const int nblk = ctx->n_ph_big + ctx->n_ph_mid + ctx->n_ph;
-    if (nblk + nwb > 0)
-      k_ph<T_, PH_THREADS, TS><<<nblk + nwb, PH_THREADS, ph_smem_of<T_>(ctx), s>>>(
-          ctx->d, ctx->ctl, ctx->ph_list, nblk, ctx->n_ph_warp, tpair, xt, xw, xv1, xq);
-    return;
-  }
-  if (ctx->n_ph_big > 0)
-    k_ph_big<T_, TS><<<ctx->n_ph_big, PH_BIG_THREADS, ph_big_smem_of<T_>(ctx), s>>>(
-        ctx->d, ctx->ctl, ctx->ph_list, tpair, xt, xw, xv1, xq);
-  const int* mid = ctx->ph_list + ctx->n_ph_big;
-  if (PNM_PH_CLASSES == 4) {
-    const int* small = mid + ctx->n_ph_mid;
-    const int* warp = small + ctx->n_ph;
-    if (ctx->n_ph_mid > 0)
-      k_ph<T_, PH_THREADS, TS><<<ctx->n_ph_mid, PH_THREADS, ctx->ph_mid_smem64, s>>>(
-          ctx->d, ctx->ctl, mid, ctx->n_ph_mid, 0, tpair, xt, xw, xv1, xq);
-    if (ctx->n_ph > 0)
-      k_ph<T_, PH_THREADS, TS><<<ctx->n_ph, PH_THREADS, ctx->ph_smem64, s>>>(
-          ctx->d, ctx->ctl, small, ctx->n_ph, 0, tpair, xt, xw, xv1, xq);
-    if (nwb > 0)
-      k_ph<T_, PH_THREADS, TS><<<nwb, PH_THREADS, ph_warp_smem(sizeof(T_)), s>>>(
-          ctx->d, ctx->ctl, warp, 0, ctx->n_ph_warp, tpair, xt, xw, xv1, xq);
-  } else {
-    const int nblk = ctx->n_ph_mid + ctx->n_ph;
-    if (nblk + nwb > 0)
-      k_ph<T_, PH_THREADS, TS><<<nblk + nwb, PH_THREADS, ph_smem_of<T_>(ctx), s>>>(
-          ctx->d, ctx->ctl, mid, nblk, ctx->n_ph_warp, tpair, xt, xw, xv1, xq);
-  }
-}
-
-template <typename T_>
-static void ph_attributes(const pnm_ctx* ctx) {
-  smem_at_least(k_ph<T_, PH_THREADS, ph_tile<T_>()>, ph_smem_of<T_>(ctx));
-  smem_at_least(k_ph_big<T_, ph_tile<T_>()>, ph_big_smem_of<T_>(ctx));
-}
-
-// FP64 ph: T gathered from the current FP64 amplitudes (linear: without the quadratic part).
-void launch_ph64(pnm_ctx* ctx, cudaStream_t s, bool linear) {
-  launch_ph_list<double>(ctx, nullptr, nullptr, linear ? nullptr : ctx->d.x_w, ctx->d.x_v1, ctx->d.xq, s);
-}
-
-// The same term with FP32-pair arithmetic (T gathered from the FP32-pair copy of the current
-// amplitudes, W and <kb|v|cj> split into FP32 pairs once per context, Q stored as FP32 pairs in
-// the 8-byte slots of the FP64 Q): the contractions of the refinement sweeps.
-void launch_ph_f2(pnm_ctx* ctx, const f2* tpair, const f2* xw, const f2* xv1, cudaStream_t s) {
-  launch_ph_list<f2>(ctx, tpair, nullptr, xw, xv1, reinterpret_cast<f2*>(ctx->d.xq), s);
-}
 
 // Mixed ph: T read from the FP32 cross-channel copy the update scatters, Q in FP32 at its
 // cross-channel positions (the update gathers the four terms of each amplitude).
 void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* xv1, float* xq, cudaStream_t s) {
-  launch_ph_list<float>(ctx, nullptr, xt, xw, xv1, xq, s);
+  // one launch over the S_z >= 0 cross channels, the costliest first (limited by registers)
+  const int nwb = (ctx->n_ph_warp + PH_WARPS - 1) / PH_WARPS;
+  const int nblk = ctx->n_ph_big + ctx->n_ph_mid + ctx->n_ph;
+  if (nblk + nwb > 0)
+    k_ph<float, PH_THREADS, PNM_PH32_TILE><<<nblk + nwb, PH_THREADS, ph32_smem(ctx), s>>>(
+        ctx->d, ctx->ctl, ctx->ph_list, nblk, ctx->n_ph_warp, xt, xw, xv1, xq);
 }
 
-void pnm_ph_attributes(const pnm_ctx* ctx) {
-  ph_attributes<double>(ctx);
-  ph_attributes<float>(ctx);
-  ph_attributes<f2>(ctx);
+// ------------------------------------------------------------- ph term, FP64 accuracy (digits)
+// The FP64 and FP32-pair ph term as digit products on the tensor cores (dig.cuh), mma.sync because
+// the matrices are small (N = 66: 17 to 33 rows and columns): per problem (a S_z > 0 channel, or
+// the sum and the difference problem of an S_z = 0 channel)
+//   C[(k,c)][(j,b)] = <kb|v|cj> + 1/2 sum_(e,l) <kl|v|ce> t_lj^eb,   Q[(a,i)][(j,b)] = T C.
+// Operands are integers and their digits from end to end:
+//   - the amplitudes as digit words of one exponent per system (k_tmax, k_twords: two passes over
+//     them per update, where converting at the gather repeated the work for each of the three or
+//     four places of an amplitude and cost two more passes over shared memory);
+//   - W as digits in fragment order, <kb|v|cj> as integers, and the signed amplitude index of every
+//     staged element, fixed per context (k_ph_pack; sums and differences of S_z = 0 formed there);
+//   - T staged as words (sums and differences of S_z = 0 as exact integer sums), two neighbouring
+//     columns interleaved: the k index of the second product; the first reads its k pairs across
+//     rows;
+//   - C as integers, the two terms aligned to the coarser of their units (2^-60 of their bounds or
+//     finer), its digits stored interleaved by row pairs straight from the first product's registers.
+// Only the results leave as floating point.  A group of 32 threads (channels of at most PH_WARP_DIM
+// rows and columns) or of 128 (the others) takes a channel; a warp forms 16 x 8 blocks.
+// What bounds it: instruction issue and its latencies around the products (operand expansion,
+// drains, staging) at twelve warps per SM; without the MMAs it takes 6% less time.  Per launch with
+// the two passes over the amplitudes: N = 66, n^2 <= 42, FP64 149 us against 405 us on the FP64
+// pipe; three densities of N = 66, n^2 <= 36, pairs, 290 against 356 us on the FP32 pipe; symmetric
+// matter, 28 nucleons, n^2 <= 20, FP64 50 against 52 us launched one by one, and shorter beside the
+// ladder in a captured update (no FP64 pipe work to share).
+struct __align__(16) PhItem {
+  int x, sys;                    // cross channel, its system
+  unsigned short R, H, nm, nhp;  // rows, columns of a problem; problems (1: S_z > 0, 2: S_z = 0); channel columns
+  int po, ho;                    // pair offsets
+  // offsets: Q, source indices, W fragments (uint4), <kb|v|cj>, and of the smallest channels W and
+  // <kb|v|cj> as element values
+  unsigned to, src, wf, v1, fx, pad;
+};
+
+__host__ __device__ __forceinline__ int ph_h8(int H) { return (H + 7) & ~7; }
+// Row strides in 16-byte pairs: T's odd, C's 2 modulo 8, so that the fragment loads of the first
+// product (two rows per thread) and of the second spread over the banks.
+__host__ __device__ __forceinline__ int ph_ts(int H) { return ph_h8(H) / 2 + 1; }
+__host__ __device__ __forceinline__ int ph_cs(int H) { return ph_h8(H) + 2; }
+__host__ __device__ __forceinline__ size_t ph_dig_smem(int R, int H, int nm) {
+  return sizeof(uint4) * nm * ((size_t)ph_h8(R) * ph_ts(H) + (size_t)(ph_h8(H) / 2) * ph_cs(H)) +
+         sizeof(int) * ((size_t)ph_h8(R) + 2 * ph_h8(H));
 }
+
+template <int GT>
+__device__ __forceinline__ void group_sync() {
+  if constexpr (GT == 32) __syncwarp();
+  else __syncthreads();
+}
+
+// The term of one channel in FP64 arithmetic (infinities, NaN, or values so large that intermediate
+// results might overflow): the sums of the same expressions in order.
+template <typename Out, int GT>
+__device__ __noinline__ void ph_values(const DevState& D, const PhItem& it, int tid, uint4* Ts, uint4* Cs,
+                                       const int* sra, const int* sca, const int* scb, const double* __restrict__ t,
+                                       const int* __restrict__ src, bool quad, Out* __restrict__ xq) {
+  const int R = it.R, H = it.H, nm = it.nm, H8 = ph_h8(H), TS = ph_ts(H), CS = ph_cs(H);
+  const long TP = (long)ph_h8(R) * TS, CP = (long)(H8 / 2) * CS;
+  auto T = [&](int m, int u, int s) -> double& { return reinterpret_cast<double*>(Ts + m * TP + u * TS + (s >> 1))[s & 1]; };
+  auto C = [&](int m, int r, int c) -> double& { return reinterpret_cast<double*>(Cs + m * CP + (r >> 1) * CS + c)[r & 1]; };
+  auto amp = [&](int c) { return c == 0 ? 0.0 : (c > 0 ? t[c - 1] : -t[-c - 1]); };
+  const double* __restrict__ W = D.x_w + D.x_w_off[it.x];
+  const double* __restrict__ V = D.x_v1 + D.x_c_off[it.x];
+  for (int e = tid; e < R * H; e += GT) {
+    const int u = e / H, s = e % H;
+    if (nm == 1) T(0, u, s) = amp(src[it.src + u * H8 + s]);
+    else {
+      const int2 k = reinterpret_cast<const int2*>(src + it.src)[u * H8 + s];
+      const double a = amp(k.x), b = amp(k.y);
+      T(0, u, s) = a + b;
+      T(1, u, s) = a - b;
+    }
+  }
+  group_sync<GT>();
+  for (int e = tid; e < nm * H * H; e += GT) {
+    const int m = e / (H * H), r = (e % (H * H)) / H, c = e % H;
+    auto pick = [&](const double* __restrict__ M, long row, int col) {  // element of problem m
+      if (nm == 1) return M[row + col];
+      const double a = M[row + sca[col]], b = M[row + scb[col]];
+      return m == 0 ? a + b : a - b;
+    };
+    double acc = 0.0;
+    for (int u = 0; u < R && quad; u++) acc += pick(W, (long)(nm == 1 ? u : sra[u]) * it.nhp, r) * T(m, u, c);
+    C(m, r, c) = pick(V, (long)(nm == 1 ? r : sca[r]) * it.nhp, c) + 0.5 * acc;
+  }
+  group_sync<GT>();
+  for (int e = tid; e < R * H; e += GT) {
+    const int r = e / H, c = e % H;
+    double acc[2] = {0.0, 0.0};
+    for (int m = 0; m < nm; m++)
+      for (int u = 0; u < H; u++) acc[m] += T(m, r, u) * C(m, u, c);
+    if (nm == 1) xq[it.to + (long)r * it.nhp + c] = Arith<Out>::from_double(acc[0]);
+    else {
+      const long q = it.to + (long)sra[r] * it.nhp;
+      xq[q + sca[c]] = Arith<Out>::from_double(0.5 * (acc[0] + acc[1]));
+      xq[q + scb[c]] = Arith<Out>::from_double(0.5 * (acc[0] - acc[1]));
+    }
+  }
+}
+
+// Largest exponent of the amplitudes plus that of W beyond which ph_values is used: C and Q stay
+// finite below.
+constexpr int PH_MAX_EXP = 2900;
+
+// ex: exponents of W and of <kb|v|cj>.
+template <typename Out, int GT, int NM>
+__device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2 ex, unsigned char* smraw,
+                                       const double* __restrict__ t, const int* __restrict__ src,
+                                       const uint4* __restrict__ wf, const long long* __restrict__ v1, bool quad,
+                                       Out* __restrict__ xq) {
+  const int tid = GT == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, wid = tid >> 5;
+  constexpr int NW = GT / 32;
+  const int R = it.R, H = it.H, R8 = ph_h8(R), H8 = ph_h8(H), TS = ph_ts(H), CS = ph_cs(H);
+  const int TP = R8 * TS, CP = (H8 / 2) * CS;
+  uint4* Ts = reinterpret_cast<uint4*>(smraw);  // [problem][row][column pair]
+  uint4* Cs = Ts + NM * TP;                     // [problem][row pair][column]
+  int* sra = reinterpret_cast<int*>(Cs + NM * CP);
+  int* sca = sra + R8;
+  int* scb = sca + H8;
+  const int et = D.sys_texp[it.sys];
+  if constexpr (NM == 2) {
+    for (int k = tid; k < R; k += GT) sra[k] = D.x_rrow[it.po + k];
+    for (int k = tid; k < H; k += GT) {
+      const int a = D.x_rcol[it.ho + k];
+      sca[k] = a;
+      scb[k] = D.x_fcol[it.ho + a];
+    }
+  }
+  if (et >= DIG_NONFINITE || ex.x >= DIG_NONFINITE || ex.y >= DIG_NONFINITE || et + ex.x > PH_MAX_EXP) {
+    group_sync<GT>();  // the tables; group-uniform branch
+    ph_values<Out, GT>(D, it, tid, Ts, Cs, sra, sca, scb, t, src, quad, xq);
+    return;
+  }
+  // T: two neighbouring columns per step (index rows are padded to H8, rows past R read none)
+  {
+    const dig_t* __restrict__ tw = D.twords;
+    auto word = [&](int c) {
+      if (c == 0) return DIG_BIAS;
+      const dig_t w = tw[c > 0 ? c - 1 : -c - 1];
+      return c < 0 ? dig_neg(w) : w;
+    };
+    const int half = H8 / 2, total = R8 * half, live = R * half, du = GT / half, ds = GT % half;
+    int u = tid / half, s = tid % half;
+#pragma unroll 4
+    for (int f = tid; f < total; f += GT) {
+      uint4* pa = Ts + u * TS + s;
+      if constexpr (NM == 1) {
+        const int2 c = f < live ? reinterpret_cast<const int2*>(src + it.src)[f] : make_int2(0, 0);
+        *pa = dig_interleave(word(c.x), word(c.y));
+      } else {
+        const int4 c = f < live ? reinterpret_cast<const int4*>(src + it.src)[f] : make_int4(0, 0, 0, 0);
+        const dig_t a0 = word(c.x), b0 = word(c.y), a1 = word(c.z), b1 = word(c.w);
+        *pa = dig_interleave(dig_sum(a0, b0), dig_sum(a1, b1));
+        pa[TP] = dig_interleave(dig_diff(a0, b0), dig_diff(a1, b1));
+      }
+      u += du;
+      s += ds;
+      if (s >= half) {
+        s -= half;
+        u++;
+      }
+    }
+  }
+  group_sync<GT>();
+  // C: 16 x 8 blocks of every problem; the fragments of W are requested one step ahead, across
+  // blocks too
+  const int nt = H8 / 8, sc = (H + 15) >> 4, kr = (R + 15) >> 4, blocks = NM * sc * nt;
+  const int p1 = dig_power(ex.x, et) + 14 - 1, pv = ex.y - 1022 - 61;  // units of the two terms (factor 1/2)
+  const int pc = quad ? max(p1, pv) : pv, sx = min(pc - p1, 63), sv = min(pc - pv, 63);
+  const bool small_r = R <= DIG_SMALL_K, small_h = H <= DIG_SMALL_K;
+  uint4 w[4];
+  auto load_w = [&](int b, int ks) {  // block b is strip b / nt of the problems' strips in turn
+    const uint4* __restrict__ wp = wf + it.wf + ((long)(b / nt) * kr + ks) * 128 + lane;
+#pragma unroll
+    for (int r = 0; r < 4; r++) w[r] = __ldg(wp + r * 32);
+  };
+  if (quad && wid < blocks) load_w(wid, 0);
+  for (int b = wid; b < blocks; b += NW) {
+    const int ms = b / nt, m = ms / sc, strip = ms - m * sc, n0 = (b - ms * nt) * 8;
+    const longlong2* __restrict__ vp =
+        reinterpret_cast<const longlong2*>(v1 + it.v1) + (((long)ms * 16 + g) * H8 + n0) / 2 + q;
+    const longlong2 va = __ldg(vp), vb = __ldg(vp + 4 * H8);
+    dig_t c[4] = {(dig_t)(va.x >> sv), (dig_t)(va.y >> sv), (dig_t)(vb.x >> sv), (dig_t)(vb.y >> sv)};
+    if (quad) {
+      float acc[DIG_LEVELS][4] = {};
+      const uint4* tb = Ts + m * TP + (2 * q) * TS + ((n0 + g) >> 1);
+      for (int ks = 0; ks < kr; ks++) {
+        uint32_t a[4][DIG_LEVELS], bb[2][DIG_LEVELS];
+        const bool half = R - ks * 16 <= 8;
+#pragma unroll
+        for (int r = 0; r < 4; r++) dig_expand<DIG_LEVELS>(w[r], a[r]);
+        if (ks + 1 < kr) load_w(b, ks + 1);
+        else if (b + NW < blocks) load_w(b + NW, 0);
+        const uint4* tk = tb + ks * 16 * TS;
+        dig_expand_across(tk[0], tk[TS], g & 1, bb[0]);
+        if (!half) dig_expand_across(tk[8 * TS], tk[9 * TS], g & 1, bb[1]);
+        dig_block(acc, a, bb, half);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const DigSum x = small_r ? dig_drain_small(acc, k) : dig_drain(acc, k);
+        c[k] += (dig_t)(((x.hi << 18) + (x.lo >> 14)) >> sx);  // 2^-54 of the maxima's product or finer
+      }
+    }
+    // digits of the row pairs (g, g ^ 1): the lanes of even g take the block's even columns
+    const bool odd = g & 1;
+    const dig_t r0 = __shfl_xor_sync(0xffffffffu, odd ? c[0] : c[1], 4);
+    const dig_t r1 = __shfl_xor_sync(0xffffffffu, odd ? c[2] : c[3], 4);
+    const dig_t o0 = odd ? c[1] : c[0], o1 = odd ? c[3] : c[2];
+    uint4* pc0 = Cs + m * CP + ((strip * 16 + g) >> 1) * CS + n0 + 2 * q + (odd ? 1 : 0);
+    if (strip * 16 + g < H8)
+      *pc0 = dig_interleave(DIG_BIAS + (odd ? r0 : o0), DIG_BIAS + (odd ? o0 : r0));
+    if (strip * 16 + g + 8 < H8)
+      pc0[4 * CS] = dig_interleave(DIG_BIAS + (odd ? r1 : o1), DIG_BIAS + (odd ? o1 : r1));
+  }
+  group_sync<GT>();
+  // Q
+  const int sr = (R + 15) >> 4, kh = (H + 15) >> 4;
+  const int p2 = 56 + (et - 1022 - 61) + pc - (NM == 2 ? 1 : 0);  // the half of sum and difference
+  for (int b = wid; b < sr * nt; b += NW) {
+    const int m0 = (b / nt) * 16, n0 = (b % nt) * 8;
+    const bool low = m0 + 8 < R;  // rows m0 + 8 ... are stored
+    DigSum x[4] = {}, x0[4];  // the last problem's sums, and those of the one before
+#pragma unroll 1
+    for (int m = 0; m < NM; m++) {
+      float acc[DIG_LEVELS][4] = {};
+      for (int ks = 0; ks < kh; ks++) {
+        uint32_t a[4][DIG_LEVELS], bb[2][DIG_LEVELS];
+        const bool half = H - ks * 16 <= 8;
+        const uint4* ta = Ts + m * TP + (m0 + g) * TS + ks * 8 + q;
+        const uint4* cb = Cs + m * CP + (ks * 8 + q) * CS + n0 + g;
+        const uint4 zero = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
+        dig_expand<DIG_LEVELS>(ta[0], a[0]);
+        dig_expand<DIG_LEVELS>(low ? ta[8 * TS] : zero, a[1]);
+        dig_expand<DIG_LEVELS>(cb[0], bb[0]);
+        if (!half) {
+          dig_expand<DIG_LEVELS>(ta[4], a[2]);
+          dig_expand<DIG_LEVELS>(low ? ta[8 * TS + 4] : zero, a[3]);
+          dig_expand<DIG_LEVELS>(cb[4 * CS], bb[1]);
+        }
+        dig_block(acc, a, bb, half);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        x0[k] = x[k];
+        x[k] = small_h ? dig_drain_small(acc, k) : dig_drain(acc, k);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      const int r = m0 + g + 8 * (k >> 1), c = n0 + 2 * q + (k & 1);
+      if (r >= R || c >= H) continue;
+      if constexpr (NM == 1) {
+        xq[it.to + (long)r * it.nhp + c] = dig_result<Out>(x[k], p2);
+      } else {
+        // the spin-up row's two blocks; the flipped rows are never read (see qpos)
+        const long o = it.to + (long)sra[r] * it.nhp;
+        xq[o + sca[c]] = dig_result<Out>(DigSum{x0[k].hi + x[k].hi, x0[k].lo + x[k].lo}, p2);
+        xq[o + scb[c]] = dig_result<Out>(DigSum{x0[k].hi - x[k].hi, x0[k].lo - x[k].lo}, p2);
+      }
+    }
+  }
+}
+
+// Digit words of the current amplitudes of every system, of one exponent per system.  TW_PARTS CTAs
+// per system find the largest exponents of their parts (k_tmax); k_twords reduces them (again in
+// every CTA) and converts; part 0 publishes the system's exponent.
+constexpr int TW_THREADS = 256, TW_PARTS = 512;
+__global__ void __launch_bounds__(TW_THREADS) k_tmax(DevState D, const LoopCtl* __restrict__ ctl,
+                                                     const long* __restrict__ t_lo, int* __restrict__ parts) {
+  const int sys = blockIdx.y;
+  if (sys_done(D, ctl, sys)) return;
+  const double* __restrict__ t = cur_t(D, ctl);
+  const long hi = t_lo[sys + 1];
+  int e = 1;
+#pragma unroll 4
+  for (long z = t_lo[sys] + blockIdx.x * TW_THREADS + threadIdx.x; z < hi; z += gridDim.x * TW_THREADS)
+    e = max(e, dig_exp(t[z]));
+  e = __reduce_max_sync(0xffffffffu, e);
+  __shared__ int top;
+  if (threadIdx.x == 0) top = 1;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) atomicMax(&top, e);
+  __syncthreads();
+  if (threadIdx.x == 0) parts[sys * TW_PARTS + blockIdx.x] = top;
+}
+
+__global__ void __launch_bounds__(TW_THREADS) k_twords(DevState D, const LoopCtl* __restrict__ ctl,
+                                                       const long* __restrict__ t_lo, const int* __restrict__ parts,
+                                                       int nparts) {
+  const int sys = blockIdx.y;
+  if (sys_done(D, ctl, sys)) return;
+  int e = 1;
+  for (int k = threadIdx.x & 31; k < nparts; k += 32) e = max(e, parts[sys * TW_PARTS + k]);
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (blockIdx.x == 0 && threadIdx.x == 0) D.sys_texp[sys] = e;
+  if (e >= DIG_NONFINITE) return;  // the term is then formed from the FP64 values
+  const double* __restrict__ t = cur_t(D, ctl);
+  const long hi = t_lo[sys + 1];
+#pragma unroll 4
+  for (long z = t_lo[sys] + blockIdx.x * TW_THREADS + threadIdx.x; z < hi; z += gridDim.x * TW_THREADS)
+    D.twords[z] = dig_word(dig_fixed(t[z], e));
+}
+
+// Channels of at most PH_TINY_DIM (FP32-pair results) or PH_TINY_FP64 (FP64 results) rows and
+// columns per problem, one warp each, in the element arithmetic of the results, the pairs from the
+// pair copy of the amplitudes: a 7 x 7 problem would fill a fifth of a 16 x 8 x 8 block.  120 systems
+// of N = 14, all of whose channels are of this size: 695 us per launch in digits, 145 here (355 with
+// one gather loop per channel in the kernel of the larger channels, at its registers).  In FP64 the
+// line lies lower, the products then share the slow pipe: 28 nucleons, n^2 <= 20, take 94 us per
+// update with a line at 5 and 99 with one at 8; N = 14, n^2 <= 20, whose channels have up to 7 rows,
+// 34.8 and 36.0; n^2 <= 4 (up to 5 rows) 28.5, and in digits 30.
+// fixed: W [problem][row][column] then <kb|v|cj> [problem][row][column] of the channel.
+constexpr int PH_TINY_DIM = 8, PH_TINY_FP64 = 5;
+template <typename T_>
+__device__ __forceinline__ void ph_tiny(const DevState& D, const PhItem& it, T_* Ts,
+                                        const T_* __restrict__ t, const int* __restrict__ src,
+                                        const T_* __restrict__ fixed, bool quad, T_* __restrict__ xq) {
+  using A = Arith<T_>;
+  constexpr int S = PH_TINY_DIM;
+  const int lane = threadIdx.x & 31, R = it.R, H = it.H, nm = it.nm;
+  T_* Ws = Ts + 2 * S * S;  // [problem][row][column], as Ts
+  T_* Cs = Ws + 2 * S * S;
+  const T_* __restrict__ W = fixed + it.fx;
+  const T_* __restrict__ V1 = W + nm * R * H;
+  const int* __restrict__ sp = src + it.src;
+  auto read = [&](int c) {
+    if (c == 0) return A::zero();
+    const T_ v = t[c > 0 ? c - 1 : -c - 1];
+    return c < 0 ? A::neg(v) : v;
+  };
+  for (int e = lane; e < R * H; e += 32) {
+    const int u = e / H, c = e - u * H, k8 = u * ph_h8(H) + c;
+    if (nm == 2) {
+      const int2 k = reinterpret_cast<const int2*>(sp)[k8];
+      const T_ x = read(k.x), y = read(k.y);
+      Ts[u * S + c] = A::add(x, y);
+      Ts[S * S + u * S + c] = A::sub(x, y);
+      if (quad) Ws[S * S + u * S + c] = W[R * H + e];
+    } else {
+      Ts[u * S + c] = read(sp[k8]);
+    }
+    if (quad) Ws[u * S + c] = W[e];
+  }
+  __syncwarp();
+  for (int e = lane; e < nm * H * H; e += 32) {
+    const int m = e >= H * H, f = e - m * H * H, r = f / H, c = f - r * H;
+    T_ acc = A::zero();
+    for (int u = 0; u < R && quad; u++) A::mac(acc, Ws[m * S * S + u * S + r], Ts[m * S * S + u * S + c]);
+    Cs[m * S * S + r * S + c] = A::add(V1[e], A::half(acc));
+  }
+  __syncwarp();
+  for (int e = lane; e < R * H; e += 32) {
+    const int r = e / H, c = e - r * H;
+    T_ acc[2] = {A::zero(), A::zero()};
+    for (int m = 0; m < nm; m++)
+      for (int u = 0; u < H; u++) A::mac(acc[m], Ts[m * S * S + r * S + u], Cs[m * S * S + u * S + c]);
+    if (nm == 2) {
+      const long q = it.to + (long)D.x_rrow[it.po + r] * it.nhp;
+      const int ca = D.x_rcol[it.ho + c], cb = D.x_fcol[it.ho + ca];
+      xq[q + ca] = A::half(A::add(acc[0], acc[1]));
+      xq[q + cb] = A::half(A::sub(acc[0], acc[1]));
+    } else {
+      xq[it.to + (long)r * it.nhp + c] = acc[0];
+    }
+  }
+}
+
+// The first nblk CTAs take one channel each (the costliest first), the others PH_WARPS small
+// channels each, one per warp (stride warp_smem bytes of shared memory).
+template <typename Out>
+__global__ void __launch_bounds__(PH_THREADS, 3) k_ph_dig(DevState D, const LoopCtl* __restrict__ ctl,
+                                                          const PhItem* __restrict__ items, const int2* __restrict__ exps,
+                                                          int nblk, int nwarp, int warp_smem, const int* __restrict__ src,
+                                                          const uint4* __restrict__ wf, const long long* __restrict__ v1,
+                                                          int quad, Out* __restrict__ xq) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const double* __restrict__ t = cur_t(D, ctl);
+  if ((int)blockIdx.x < nblk) {
+    const PhItem it = items[blockIdx.x];
+    if (sys_done(D, ctl, it.sys)) return;  // CTA-uniform
+    const int2 ex = exps[blockIdx.x];
+    if (it.nm == 2) ph_dig<Out, PH_THREADS, 2>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq);
+    else ph_dig<Out, PH_THREADS, 1>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq);
+    return;
+  }
+  const int w = threadIdx.x >> 5, idx = ((int)blockIdx.x - nblk) * PH_WARPS + w;
+  if (idx >= nwarp) return;  // whole warps; the warp path never synchronises the block
+  const PhItem it = items[nblk + idx];
+  if (sys_done(D, ctl, it.sys)) return;
+  const int2 ex = exps[nblk + idx];
+  unsigned char* sm = smraw + (size_t)w * warp_smem;
+  if (it.nm == 2) ph_dig<Out, 32, 2>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq);
+  else ph_dig<Out, 32, 1>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq);
+}
+
+// The smallest channels, one warp each, in a kernel of their own: it needs a third of the registers.
+template <typename T_>
+__global__ void __launch_bounds__(PH_THREADS) k_ph_tiny(DevState D, const LoopCtl* __restrict__ ctl,
+                                                        const PhItem* __restrict__ items, int n,
+                                                        const int* __restrict__ src, const T_* __restrict__ fixed,
+                                                        const f2* __restrict__ tpair, int quad, T_* __restrict__ xq) {
+  __shared__ __align__(16) T_ sm[PH_WARPS][6 * PH_TINY_DIM * PH_TINY_DIM];
+  const int w = threadIdx.x >> 5, idx = blockIdx.x * PH_WARPS + w;
+  if (idx >= n) return;  // whole warps; no block barrier
+  const PhItem it = items[idx];
+  if (sys_done(D, ctl, it.sys)) return;
+  const T_* __restrict__ t;
+  if constexpr (std::is_same<T_, f2>::value) t = tpair;
+  else t = cur_t(D, ctl);
+  ph_tiny<T_>(D, it, sm[w], t, src, fixed, quad != 0, xq);
+}
+
+// The fixed operands of the items (one CTA each): source indices (rows padded to H8), <kb|v|cj> of
+// the problems as integers (padded to whole blocks) and the digits of W, with their exponents.
+__global__ void __launch_bounds__(128) k_ph_pack(DevState D, const PhItem* __restrict__ items, int2* __restrict__ exps,
+                                                 int* __restrict__ src, uint4* __restrict__ wf, long long* __restrict__ v1,
+                                                 double* __restrict__ fixed64, f2* __restrict__ fixed_f2) {
+  __shared__ int top[2];
+  const PhItem it = items[blockIdx.x];
+  const int R = it.R, H = it.H, H8 = ph_h8(H);
+  const int* __restrict__ rr = D.x_rrow + it.po;
+  const int* __restrict__ rc = D.x_rcol + it.ho;
+  const int* __restrict__ fc = D.x_fcol + it.ho;
+  const double* __restrict__ W = D.x_w + D.x_w_off[it.x];
+  const double* __restrict__ V = D.x_v1 + D.x_c_off[it.x];
+  const bool two = it.nm == 2;
+  const bool tiny = max(R, H) <= PH_TINY_DIM;  // element values too
+  auto put = [&](long o, double v) {
+    fixed64[it.fx + o] = v;
+    fixed_f2[it.fx + o] = Arith<f2>::from_double(v);
+  };
+  if (threadIdx.x < 2) top[threadIdx.x] = 1;
+  __syncthreads();
+  int e = 1;
+  for (int f = threadIdx.x; f < R * H8; f += blockDim.x) {
+    const int u = f / H8, s = f % H8, o = u * H + s;
+    if (two) {
+      int2 c = make_int2(0, 0);
+      if (s < H) {
+        const long oa = (long)rr[u] * it.nhp + rc[s], ob = (long)rr[u] * it.nhp + fc[rc[s]];
+        c = make_int2(D.xmap[it.to + oa], D.xmap[it.to + ob]);
+        e = max(e, max(dig_exp(W[oa]), dig_exp(W[ob])));
+        if (tiny) {
+          put(o, W[oa] + W[ob]);
+          put(R * H + o, W[oa] - W[ob]);
+        }
+      }
+      reinterpret_cast<int2*>(src + it.src)[f] = c;
+    } else {
+      src[it.src + f] = s < H ? D.xmap[it.to + o] : 0;
+      if (s < H) {
+        e = max(e, dig_exp(W[o]));
+        if (tiny) put(o, W[o]);
+      }
+    }
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) atomicMax(&top[0], e);
+  e = 1;
+  for (int f = threadIdx.x; f < H * H; f += blockDim.x) {
+    const int r = f / H, c = f % H;
+    if (two) {
+      const double a = V[(long)rc[r] * it.nhp + rc[c]], b = V[(long)rc[r] * it.nhp + fc[rc[c]]];
+      e = max(e, max(dig_exp(a), dig_exp(b)));
+      if (tiny) {
+        put(2 * R * H + f, a + b);
+        put(2 * R * H + H * H + f, a - b);
+      }
+    } else {
+      const double a = V[(long)r * it.nhp + c];
+      e = max(e, dig_exp(a));
+      if (tiny) put(R * H + f, a);
+    }
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) atomicMax(&top[1], e);
+  __syncthreads();
+  const int ew = top[0], ev = top[1];
+  if (threadIdx.x == 0) exps[blockIdx.x] = make_int2(ew, ev);
+  if (ew >= DIG_NONFINITE || ev >= DIG_NONFINITE) return;
+  const int sc = (H + 15) >> 4, kr = (R + 15) >> 4;
+  for (int f = threadIdx.x; f < sc * 16 * H8; f += blockDim.x) {
+    const int r = f / H8, c = f % H8;
+    long long sum = 0, dif = 0;
+    if (r < H && c < H) {
+      if (two) {
+        const long long a = dig_fixed(V[(long)rc[r] * it.nhp + rc[c]], ev);
+        const long long b = dig_fixed(V[(long)rc[r] * it.nhp + fc[rc[c]]], ev);
+        sum = a + b;
+        dif = a - b;
+      } else {
+        sum = dig_fixed(V[(long)r * it.nhp + c], ev);
+      }
+    }
+    v1[it.v1 + f] = sum;
+    if (two) v1[it.v1 + (long)sc * 16 * H8 + f] = dif;
+  }
+  // fragment order of W as the first operand: rows (k,c), columns (e,l); stored transposed in x_w
+  for (int f = threadIdx.x; f < sc * kr * 128; f += blockDim.x) {
+    const int lane = f & 31, grp = (f >> 5) & 3, ks = (f >> 7) % kr, strip = (f >> 7) / kr;
+    const int r = strip * 16 + (lane >> 2) + (grp & 1) * 8, u0 = ks * 16 + (lane & 3) * 2 + (grp >> 1) * 8;
+    long long sum[2] = {0, 0}, dif[2] = {0, 0};
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const int u = u0 + k;
+      if (r >= H || u >= R) continue;
+      if (two) {
+        const long o = (long)rr[u] * it.nhp;
+        const long long a = dig_fixed(W[o + rc[r]], ew), b = dig_fixed(W[o + fc[rc[r]]], ew);
+        sum[k] = a + b;
+        dif[k] = a - b;
+      } else {
+        sum[k] = dig_fixed(W[(long)u * it.nhp + r], ew);
+      }
+    }
+    wf[it.wf + f] = dig_interleave(dig_word(sum[0]), dig_word(sum[1]));
+    if (two) wf[it.wf + (long)sc * kr * 128 + f] = dig_interleave(dig_word(dif[0]), dig_word(dif[1]));
+  }
+}
+
+// Items and fixed operands of the digit ph term (once per context, on first use): the costliest
+// channels first, in ph_list's order; channels whose tiles need more than PH_DIG_SMEM bytes get a
+// launch of their own so that the others keep three CTAs per SM.
+constexpr size_t PH_DIG_SMEM = 72 * 1024;
+void pnm_need_phdig(pnm_ctx* ctx) {
+  if (ctx->ph_items) return;
+  cudaStream_t s = ctx->stream;
+  const int n = ctx->n_ph_big + ctx->n_ph_mid + ctx->n_ph, nw = ctx->n_ph_warp;
+  std::vector<PhItem> items;
+  items.reserve(n + nw);
+  long wf = 0, v1 = 0, src = 0, fixed = 0;
+  ctx->ph_warp_smem = 0;
+  ctx->n_ph_large = 0;
+  ctx->ph_large_smem = ctx->ph_dig_smem = 0;
+  auto add = [&](int x) {
+    PhItem it{};
+    it.x = x;
+    it.sys = ctx->h_x_sys[x];
+    it.nm = ctx->h_x_cls[x] == 0 ? 2 : 1;
+    it.R = ctx->h_x_nph[x] / it.nm;
+    it.H = ctx->h_x_nhp[x] / it.nm;
+    it.nhp = ctx->h_x_nhp[x];
+    it.po = ctx->h_x_ph_off[x];
+    it.ho = ctx->h_x_hp_off[x];
+    it.to = (unsigned)ctx->h_x_t_off[x];
+    it.src = (unsigned)src;
+    src += (long)it.nm * it.R * ph_h8(it.H);
+    it.wf = (unsigned)wf;
+    it.v1 = (unsigned)v1;
+    it.fx = (unsigned)fixed;
+    wf += (long)it.nm * ((it.H + 15) / 16) * ((it.R + 15) / 16) * 128;
+    v1 += (long)it.nm * ((it.H + 15) / 16) * 16 * ph_h8(it.H);
+    const bool tiny = std::max(it.R, it.H) <= PH_TINY_DIM;
+    if (tiny) fixed += (long)it.nm * it.H * (it.R + it.H);
+    items.push_back(it);
+    return ph_dig_smem(it.R, it.H, it.nm);
+  };
+  for (int part = 0; part < 2; part++)
+    for (int k = 0; k < n; k++) {
+      const int x = ctx->h_ph_list[k], nm = ctx->h_x_cls[x] == 0 ? 2 : 1;
+      if ((ph_dig_smem(ctx->h_x_nph[x] / nm, ctx->h_x_nhp[x] / nm, nm) > PH_DIG_SMEM) != (part == 0)) continue;
+      const size_t b = add(x);
+      size_t& most = part == 0 ? ctx->ph_large_smem : ctx->ph_dig_smem;
+      most = std::max(most, b);
+      if (part == 0) ctx->n_ph_large++;
+    }
+  // the warp path by decreasing dimension: the tiny channels of either result type are its end
+  std::vector<int> by_dim[PH_WARP_DIM + 1];
+  for (int k = 0; k < nw; k++) {
+    const int x = ctx->h_ph_list[n + k];
+    by_dim[std::max(ctx->h_x_nph[x], ctx->h_x_nhp[x]) / (ctx->h_x_cls[x] == 0 ? 2 : 1)].push_back(x);
+  }
+  ctx->n_ph_tiny64 = ctx->n_ph_tiny_f2 = 0;
+  for (int d = PH_WARP_DIM; d >= 0; d--) {
+    for (int x : by_dim[d]) ctx->ph_warp_smem = std::max(ctx->ph_warp_smem, (add(x) + 15) / 16 * 16);
+    if (d <= PH_TINY_FP64) ctx->n_ph_tiny64 += (int)by_dim[d].size();
+    if (d <= PH_TINY_DIM) ctx->n_ph_tiny_f2 += (int)by_dim[d].size();
+  }
+  if (std::max(std::max(wf, v1), std::max(src, fixed)) >= (1L << 32))
+    throw PnmError{PNM_EINVAL, "problem too large for 32-bit element maps"};
+  ctx->ph_dig_smem = std::max(ctx->ph_dig_smem, PH_WARPS * ctx->ph_warp_smem);
+  PhItem* d = ctx_alloc<PhItem>(ctx, items.size());
+  ctx->ph_exps = ctx_alloc<int2>(ctx, items.size());
+  ctx->ph_src = ctx_alloc<int>(ctx, src);
+  ctx->ph_wf = ctx_alloc<uint4>(ctx, wf);
+  ctx->ph_v1 = ctx_alloc<long long>(ctx, v1);
+  ctx->ph_fixed64 = ctx_alloc<double>(ctx, fixed);
+  ctx->ph_fixed_f2 = ctx_alloc<f2>(ctx, fixed);
+  if (!items.empty()) {
+    CUDA_TRY(cudaMemcpyAsync(d, items.data(), sizeof(PhItem) * items.size(), cudaMemcpyHostToDevice, s));
+    k_ph_pack<<<(unsigned)items.size(), 128, 0, s>>>(ctx->d, d, ctx->ph_exps, ctx->ph_src, ctx->ph_wf, ctx->ph_v1,
+                                                        ctx->ph_fixed64, ctx->ph_fixed_f2);
+    CUDA_TRY(cudaGetLastError());
+  }
+  const int nsys = (int)ctx->sys.size();
+  std::vector<long> lo(nsys + 1, ctx->nt);
+  long longest = 0;
+  for (int k = 0; k < nsys; k++) {
+    lo[k] = ctx->sys[k].t_begin;
+    longest = std::max(longest, ctx->sys[k].t_end - ctx->sys[k].t_begin);
+  }
+  // parts of about a thousand amplitudes
+  ctx->n_tw_parts = (int)std::max<long>(1, std::min<long>(TW_PARTS, longest / (4 * TW_THREADS)));
+  ctx->tw_lo = ctx_alloc<long>(ctx, nsys + 1);
+  ctx->tw_parts = ctx_alloc<int>(ctx, (size_t)nsys * TW_PARTS);
+  ctx->d.sys_texp = ctx_alloc<int>(ctx, nsys);
+  ctx->d.twords = ctx_alloc<unsigned long long>(ctx, ctx->nt);
+  CUDA_TRY(cudaMemcpyAsync(ctx->tw_lo, lo.data(), sizeof(long) * (nsys + 1), cudaMemcpyHostToDevice, s));
+  const size_t most = std::max(ctx->ph_large_smem, ctx->ph_dig_smem);
+  smem_at_least(k_ph_dig<double>, most);
+  smem_at_least(k_ph_dig<f2>, most);
+  ctx->ph_items = d;
+}
+
+template <typename Out>
+static void launch_ph_dig(pnm_ctx* ctx, bool linear, cudaStream_t s, cudaStream_t s_tiny) {
+  // made before any capture by the host-side callers
+  if (!ctx->ph_items) throw PnmError{PNM_EINVAL, "the ph term's operands have not been built"};
+  constexpr bool pair = std::is_same<Out, f2>::value;
+  const int nl = ctx->n_ph_large, n = ctx->n_ph_big + ctx->n_ph_mid + ctx->n_ph - nl;
+  const int ntiny = pair ? ctx->n_ph_tiny_f2 : ctx->n_ph_tiny64, nw = ctx->n_ph_warp - ntiny;
+  const int nwb = (nw + PH_WARPS - 1) / PH_WARPS, quad = linear ? 0 : 1;
+  Out* xq = reinterpret_cast<Out*>(ctx->d.xq);
+  const PhItem* items = ctx->ph_items;
+  if (nl + n + nw == 0) s_tiny = s;
+  if (nl + n + nw > 0) {
+    const dim3 grid(ctx->n_tw_parts, (unsigned)ctx->sys.size());
+    k_tmax<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts);
+    k_twords<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts, ctx->n_tw_parts);
+  }
+  if (nl > 0)
+    k_ph_dig<Out><<<nl, PH_THREADS, ctx->ph_large_smem, s>>>(ctx->d, ctx->ctl, items, ctx->ph_exps, nl, 0, 0, ctx->ph_src,
+                                                             ctx->ph_wf, ctx->ph_v1, quad, xq);
+  if (n + nwb > 0)
+    k_ph_dig<Out><<<n + nwb, PH_THREADS, ctx->ph_dig_smem, s>>>(ctx->d, ctx->ctl, items + nl, ctx->ph_exps + nl, n, nw,
+                                                                (int)ctx->ph_warp_smem, ctx->ph_src, ctx->ph_wf,
+                                                                ctx->ph_v1, quad, xq);
+  if (ntiny > 0) {
+    const Out* fixed;
+    if constexpr (pair) fixed = ctx->ph_fixed_f2;
+    else fixed = ctx->ph_fixed64;
+    k_ph_tiny<Out><<<(ntiny + PH_WARPS - 1) / PH_WARPS, PH_THREADS, 0, s_tiny>>>(
+        ctx->d, ctx->ctl, items + nl + n + nw, ntiny, ctx->ph_src, fixed, ctx->t_pair, quad, xq);
+  }
+}
+
+// FP64 ph term (linear: without the quadratic part), and the same with its results as FP32 pairs
+// in the 8-byte slots of the FP64 Q (the refinement sweeps with FP32-pair contractions).
+// s_tiny: the stream of the smallest channels, which wait for no digits (a captured update runs them
+// beside the two passes over the amplitudes; in a context without larger channels they keep s).
+void launch_ph64(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny, bool linear) {
+  launch_ph_dig<double>(ctx, linear, s, s_tiny);
+}
+void launch_ph_f2(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny) { launch_ph_dig<f2>(ctx, false, s, s_tiny); }
 
 // ------------------------------------------------------------------------ ladder basis
-// s(ij, q) = sum over the (one or two) pairs of vector q of sign * t(ij, pair), from the current
-// amplitudes (FP64, tsrc == nullptr) or their FP32-pair copy (tsrc); one CTA per (channel, ij)
-// row of a channel with V_pppp.
-template <typename T_>
-__global__ void __launch_bounds__(128) k_lad_gather(DevState D, const LoopCtl* __restrict__ ctl,
-                                                    const int2* __restrict__ rows, const T_* __restrict__ tsrc,
-                                                    T_* __restrict__ out) {
-  using A = Arith<T_>;
-  int2 it = rows[blockIdx.x];
-  int c = it.x, ij = it.y;
+// s(ij, q) = sum over the (one or two) pairs of vector q of sign * t(ij, pair) from the current
+// FP64 amplitudes, as digit words of the row's common exponent (dig.cuh), zero words in the
+// padding.  One CTA per (channel, ij) row of a channel with V_pppp.  A row that holds an infinity
+// or a NaN keeps its FP64 values instead of digits (exponent DIG_NONFINITE; the ladder kernel
+// then sums it in FP64).
+constexpr int TDIG_THREADS = 128;
+__global__ void __launch_bounds__(TDIG_THREADS) k_tdig(DevState D, const LoopCtl* __restrict__ ctl,
+                                                       const int2* __restrict__ rows) {
+  extern __shared__ double ssum[];
+  __shared__ int warp_max[TDIG_THREADS / 32];
+  const int2 it = rows[blockIdx.x];
+  const int c = it.x, ij = it.y;
   if (sys_done(D, ctl, D.ch_sys[c])) return;
-  const T_* __restrict__ t;
-  if constexpr (std::is_same<T_, double>::value) t = cur_t(D, ctl);
-  else t = tsrc;
-  int npp = D.ch_npp[c], nl = D.ch_nlad[c], off = D.ch_pp_off[c];
-  const T_* tr = t + D.ch_t_off[c] + (long)ij * npp;
-  T_* o = out + D.ch_s_off[c] + (long)ij * nl;
-  for (int q = threadIdx.x; q < nl; q += blockDim.x) {
-    int2 m = D.lad_mem[off + q];
-    T_ a = tr[(m.x > 0 ? m.x : -m.x) - 1];
-    T_ v = m.x > 0 ? a : A::neg(a);
+  const int npp = D.ch_npp[c], nl = D.ch_nlad[c], off = D.ch_pp_off[c];
+  const double* __restrict__ tr = cur_t(D, ctl) + D.ch_t_off[c] + (long)ij * npp;
+  int e = 1;
+  for (int q = threadIdx.x; q < nl; q += TDIG_THREADS) {
+    const int2 m = D.lad_mem[off + q];
+    const double a = tr[(m.x > 0 ? m.x : -m.x) - 1];
+    double v = m.x > 0 ? a : -a;
     if (m.y != 0) {
-      T_ b = tr[(m.y > 0 ? m.y : -m.y) - 1];
-      v = A::add(v, m.y > 0 ? b : A::neg(b));
+      const double b = tr[(m.y > 0 ? m.y : -m.y) - 1];
+      v += m.y > 0 ? b : -b;
     }
-    o[q] = v;
+    ssum[q] = v;
+    e = max(e, dig_exp(v));
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = e;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < TDIG_THREADS / 32; w++) e = max(e, warp_max[w]);
+  const int steps = (nl + 15) >> 4;
+  uint4* o = reinterpret_cast<uint4*>(D.tdig + D.ch_td_off[c]) + (long)ij * steps * 16;
+  if (threadIdx.x == 0) D.texp[D.ch_hh_off[c] + ij] = e;
+  // per 16-element step and quarter t the elements 2t, 2t + 1, 2t + 8, 2t + 9: the two registers
+  // of the product's column operand for every digit, 64 bytes
+  for (int f = threadIdx.x; f < steps * 4; f += TDIG_THREADS) {
+    const int k0 = (f >> 2) * 16 + (f & 3) * 2;
+    double v[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const int q = k0 + (u & 1) + (u >> 1) * 8;
+      v[u] = q < nl ? ssum[q] : 0.0;
+    }
+    if (e < DIG_NONFINITE) {
+      uint32_t b0[8], b1[8];
+      dig_expand<8>(dig_interleave(dig_word(dig_fixed(v[0], e)), dig_word(dig_fixed(v[1], e))), b0);
+      dig_expand<8>(dig_interleave(dig_word(dig_fixed(v[2], e)), dig_word(dig_fixed(v[3], e))), b1);
+#pragma unroll
+      for (int u = 0; u < 4; u++) o[f * 4 + u] = make_uint4(b0[2 * u], b1[2 * u], b0[2 * u + 1], b1[2 * u + 1]);
+    } else {
+      double* raw = reinterpret_cast<double*>(o + f * 4);
+#pragma unroll
+      for (int u = 0; u < 4; u++) raw[u] = v[u];
+    }
   }
 }
 
@@ -709,91 +1256,194 @@ __global__ void __launch_bounds__(128) k_lad_expand(DevState D, const T_* __rest
   }
 }
 
-// ---------------------------------------------------------------------- pp ladder FP64
+// ------------------------------------------------------------------- pp ladder, FP64 accuracy
 // R^T(ij, ab) = sum_cd t(ij, cd) <cd|v|ab>, restricted pairs (1/2 sum over ordered cd of a
-// pair-antisymmetric product = sum over c<d).  One CTA per work item (channel, 32 pp
-// columns); its 8 warps split the cd range, lane = column, so each warp streams coalesced
-// rows of the symmetric V block.  hh rows go in groups of 8 staged in shared memory; the 8
-// partial sums per output are added in a fixed order (deterministic).  Element arithmetic is
-// that of Arith<T_>: FP64, or FP32 pairs (V split once per context, the staged amplitudes
-// split on the way into shared memory, FP64 result).
-constexpr int PP64_COLS = 32, PP64_WARPS = 8, PP64_ROWS = 8;
-static size_t pp64_smem(int npp) {
-  return sizeof(double) * ((size_t)PP64_ROWS * npp + PP64_WARPS * PP64_ROWS * 32);
+// pair-antisymmetric product = sum over c<d), in the ladder basis, as digit products on the
+// tensor cores (dig.cuh), with FP64 results or FP32-pair ones (the refinement sweeps).
+// An item (PPItem) is a strip of 16 rows ab with up to 8 rows ij; wk warps share its columns cd (a
+// step of 16 each in turn) and add their integer sums, exactly, through shared memory: strips of
+// large channels would otherwise leave most SMs idle at the end (63% of the time busy with one warp
+// per strip), and a small system has too few strips to fill the GPU.  V streams in fragment order
+// (8 bytes per element); the amplitudes of the rows ij are the eight columns of the product, read
+// as FP16 digits.  Every lane copies the operands it reads itself asynchronously into its own part
+// of a PP_DEPTH-step ring in shared memory, so that a warp has PP_DEPTH - 1 steps (6 to 12 KB) in
+// flight without a barrier (one step ahead in registers held the stream to 2.8 TB/s).
+// Most channels have fewer than eight rows to compute (N = 66: 58% of V in channels of at most
+// four, symmetric matter 96%), so the columns hold SLOTS digits of 8 / SLOTS rows: slot s of a
+// column holds the digits from 8 / SLOTS * s on, and one MMA forms SLOTS levels; 36, 26 and 15
+// MMAs per 16 x 16 block of V for up to 8, 4 and 2 rows.
+// What bounds it: the V stream for few rows, the tensor pipe (1024 multiply-adds per clock and SM
+// through mma.sync) for many.  Per launch with k_tdig (N = 66, n^2 <= 42, FP64): 80 us (V 250 MB in
+// 60 us, 4.2 TB/s) against 291 us on the FP64 pipe; symmetric matter, 28 nucleons, n^2 <= 20: 43
+// against 119 us; three densities of N = 66, n^2 <= 36, pairs: 126 against 190 us on the FP32 pipe.
+constexpr int PP_WARPS = 4, PP_CTAS = 3, PP_DEPTH = 4;  // warps per CTA, CTAs per SM, ring steps
+constexpr size_t PP_SMEM = sizeof(uint4) * 256 * PP_DEPTH * PP_WARPS;  // 64 KB: three CTAs per SM
+constexpr int PP_MAX_NLAD = 3376;  // ladder basis of a channel (the amplitudes of a row in shared memory)
+
+// sum_cd t(ij, cd) V(cd, ab) in FP64 for a row ij kept as FP64 values (infinities, NaN).
+__device__ __noinline__ double pp_nonfinite(const uint4* __restrict__ vstrip, const double* __restrict__ trow, int row,
+                                            int nl, int vexp) {
+  double s = 0.0;
+  for (int k = 0; k < nl; k++) {
+    const int q = (k & 7) >> 1, half = (k >> 3) & 1;
+    const dig_t w = dig_pick(vstrip[((long)(k >> 4) * 4 + (row >> 3) + 2 * half) * 32 + (row & 7) * 4 + q], k & 1);
+    s += trow[((k >> 4) * 4 + q) * 8 + half * 2 + (k & 1)] * dig_to_double((long long)(w - DIG_BIAS), vexp - 1022 - 61);
+  }
+  return s;
 }
 
-template <typename T_>
-__global__ void __launch_bounds__(PP64_WARPS * 32) k_pp(DevState D, const LoopCtl* __restrict__ ctl,
-                                                        const int2* __restrict__ items, int rep_only,
-                                                        const T_* __restrict__ vpp) {
-  using A = Arith<T_>;
-  extern __shared__ __align__(16) unsigned char smpp[];  // ts[PP64_ROWS][npp], red[PP64_WARPS][PP64_ROWS][32]
-  int2 it = items[blockIdx.x];
-  int c = it.x, ab0 = it.y;
-  if (sys_done(D, ctl, D.ch_sys[c])) return;
-  // rep_only: the rows the updates compute (the list upd_row), else every hole pair
-  const int* __restrict__ rows = rep_only ? D.upd_row + D.ch_uoff[c] : nullptr;
-  int npp = D.ch_npp[c], nh = rep_only ? D.ch_uoff[c + 1] - D.ch_uoff[c] : D.ch_nhh[c];
-  long tb = D.ch_t_off[c];
-  // the ladder-basis amplitudes (FP64, or FP32 pairs in the same 8-byte slots)
-  const T_* __restrict__ t = reinterpret_cast<const T_*>(cur_t(D, ctl));
-  T_* ts = reinterpret_cast<T_*>(smpp);
-  T_* red = ts + PP64_ROWS * npp;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int ab = ab0 + lane;
-  bool col = ab < npp;
-  int chunk = (npp + PP64_WARPS - 1) / PP64_WARPS;
-  int lo = warp * chunk, hi = min(npp, lo + chunk);
-  const T_* __restrict__ V = vpp + D.ch_vpp_off[c] + (col ? ab : 0);
-  for (int g0 = 0; g0 < nh; g0 += PP64_ROWS) {
-    int nr = min(PP64_ROWS, nh - g0);
-    __syncthreads();
-    for (int e = threadIdx.x; e < nr * npp; e += blockDim.x) {
-      int g = g0 + e / npp;
-      ts[e] = t[tb + (long)(rows ? rows[g] : g) * npp + e % npp];
+// One step of an item's operands into this lane's ring slots: V's four 16-byte groups and the
+// Q / 2 groups of FP16 digits.
+template <int Q>
+__device__ __forceinline__ void pp_copy(uint4* __restrict__ slot, const uint4* __restrict__ vp,
+                                        const uint4* __restrict__ tp, int ks) {
+  auto cp = [](uint4* dst, const uint4* src) {  // V is read once: L2 only
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+  };
+#pragma unroll
+  for (int r = 0; r < 4; r++) cp(slot + r * 32, vp + (long)ks * 128 + r * 32);
+#pragma unroll
+  for (int r = 0; r < Q / 2; r++)  // the amplitudes are shared by the warps of an SM: L1 too
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(slot + (4 + r) * 32)),
+                 "l"(tp + (long)ks * 16 + r)
+                 : "memory");
+}
+
+// part: this warp's place among the wk warps of the item; ring: this warp's steps; red: the sums
+// of the item's warps (4 per lane and warp).
+template <int SLOTS, typename Out>
+__device__ __forceinline__ void pp_pass(const DevState& D, const PPItem& it, const int* __restrict__ rows, int part,
+                                        int wk, uint4* __restrict__ ring, DigSum* __restrict__ red) {
+  constexpr int Q = 8 / SLOTS;  // rows ij of this pass, and digits per slot
+  const int c = it.c, strip = it.strip, nl = it.nl, n0 = it.n0, nr = it.nr;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int steps = (nl + 15) >> 4;
+  const uint4* __restrict__ vstrip = reinterpret_cast<const uint4*>(D.vdig + it.voff);
+  const uint4* __restrict__ vp = vstrip + lane;
+  const int rg = min(n0 + g % Q, nr - 1), ijg = rows ? rows[rg] : rg;
+  const uint4* __restrict__ tch = reinterpret_cast<const uint4*>(D.tdig + D.ch_td_off[c]);
+  const uint4* __restrict__ tp = tch + ((long)ijg * steps * 4 + t) * 4 + (g / Q) * (Q / 2);
+  ring += lane;
+  const int mine = part < steps ? (steps - 1 - part) / wk + 1 : 0;  // this warp's steps
+#pragma unroll
+  for (int d = 0; d < PP_DEPTH - 1; d++) {
+    if (d < mine) pp_copy<Q>(ring + d * 256, vp, tp, part + d * wk);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float acc[DIG_LEVELS][4];
+#pragma unroll
+  for (int l = 0; l < DIG_LEVELS; l++)
+#pragma unroll
+    for (int e = 0; e < 4; e++) acc[l][e] = 0.0f;
+  DigSum sum[4] = {};
+  for (int k = 0; k < mine; k++) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PP_DEPTH - 2) : "memory");
+    const uint4* cur = ring + (k % PP_DEPTH) * 256;
+    uint32_t a[4][DIG_LEVELS], b[2][Q];
+#pragma unroll
+    for (int r = 0; r < 4; r++) dig_expand<DIG_LEVELS>(cur[r * 32], a[r]);
+#pragma unroll
+    for (int r = 0; r < Q / 2; r++) {
+      const uint4 v = cur[(4 + r) * 32];
+      b[0][2 * r] = v.x; b[1][2 * r] = v.y;
+      b[0][2 * r + 1] = v.z; b[1][2 * r + 1] = v.w;
     }
-    __syncthreads();
-    T_ acc[PP64_ROWS];
+    // the slot of the step before, read in full, takes the step PP_DEPTH - 1 ahead
+    if (k + PP_DEPTH - 1 < mine)
+      pp_copy<Q>(ring + ((k + PP_DEPTH - 1) % PP_DEPTH) * 256, vp, tp, part + (k + PP_DEPTH - 1) * wk);
+    asm volatile("cp.async.commit_group;" ::: "memory");
 #pragma unroll
-    for (int r = 0; r < PP64_ROWS; r++) acc[r] = A::zero();
-    if (col) {
-      int cd = lo;
-      for (; cd + 4 <= hi; cd += 4) {
-        T_ v0 = V[(long)cd * npp], v1 = V[(long)(cd + 1) * npp];
-        T_ v2 = V[(long)(cd + 2) * npp], v3 = V[(long)(cd + 3) * npp];
+    for (int i = 0; i < DIG_LEVELS; i++)
 #pragma unroll
-        for (int r = 0; r < PP64_ROWS; r++) {
-          if (r < nr) {
-            const T_* tr = ts + r * npp + cd;
-            A::mac(acc[r], tr[0], v0);
-            A::mac(acc[r], tr[1], v1);
-            A::mac(acc[r], tr[2], v2);
-            A::mac(acc[r], tr[3], v3);
-          }
-        }
-      }
-      for (; cd < hi; cd++) {
-        T_ v0 = V[(long)cd * npp];
+      for (int j = 0; j < Q; j++)
+        if (i + j < DIG_LEVELS) dig_mma16(acc[i + j], a[0][i], a[1][i], a[2][i], a[3][i], b[0][j], b[1][j]);
+    if ((k & (DIG_FLUSH / 16 - 1)) == DIG_FLUSH / 16 - 1 || k + 1 == mine) {
 #pragma unroll
-        for (int r = 0; r < PP64_ROWS; r++)
-          if (r < nr) A::mac(acc[r], ts[r * npp + cd], v0);
+      for (int e = 0; e < 4; e++) {
+        const DigSum x = dig_drain(acc, e);
+        sum[e].hi += x.hi;
+        sum[e].lo += x.lo;
+#pragma unroll
+        for (int l = 0; l < DIG_LEVELS; l++) acc[l][e] = 0.0f;
       }
     }
+  }
+  if (part != 0) {
 #pragma unroll
-    for (int r = 0; r < PP64_ROWS; r++) red[(warp * PP64_ROWS + r) * 32 + lane] = acc[r];
-    __syncthreads();
-    if ((int)threadIdx.x < nr * 32) {
-      int r = threadIdx.x >> 5, l = threadIdx.x & 31;
-      T_ s = A::zero();
+    for (int e = 0; e < 4; e++) red[(part * 4 + e) * 32 + lane] = sum[e];
+  }
+  __syncthreads();
+  if (part != 0) return;
+  for (int p = 1; p < wk; p++)
 #pragma unroll
-      for (int w = 0; w < PP64_WARPS; w++) s = A::add(s, red[(w * PP64_ROWS + r) * 32 + l]);
-      if (ab0 + l < npp)
-        reinterpret_cast<typename A::Out*>(D.rpp)[tb + (long)(rows ? rows[g0 + r] : g0 + r) * npp + ab0 + l] = A::out(s);
+    for (int e = 0; e < 4; e++) {
+      sum[e].hi += red[(p * 4 + e) * 32 + lane].hi;
+      sum[e].lo += red[(p * 4 + e) * 32 + lane].lo;
+    }
+  // accumulator columns 2t, 2t + 1: slot s counts 256^(-Q s); the slots of a row added up
+  const int vexp = D.ch_vexp[c];
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    const int s = (2 * t + (e & 1)) / Q;
+    DigSum x = sum[e];
+    if (s) {  // 16 s, 32 or 48 bits down
+      const int down = 8 * Q * s;
+      x = dig_add_low(DigSum{0, 0}, down < 32 ? (x.hi << (32 - down)) + (x.lo >> down) : (x.hi + (x.lo >> 32)) >> (down - 32));
+    }
+    if constexpr (SLOTS >= 2) {
+      x.hi += __shfl_xor_sync(0xffffffffu, x.hi, 2);
+      x.lo += __shfl_xor_sync(0xffffffffu, x.lo, 2);
+    }
+    if constexpr (SLOTS >= 4) {
+      x.hi += __shfl_xor_sync(0xffffffffu, x.hi, 1);
+      x.lo += __shfl_xor_sync(0xffffffffu, x.lo, 1);
+    }
+    const int col = 2 * t + (e & 1), row = g + 8 * (e >> 1), ab = strip * 16 + row;
+    if (col < Q && n0 + col < nr && ab < nl) {
+      const int ij = rows ? rows[n0 + col] : n0 + col;
+      const int te = D.texp[D.ch_hh_off[c] + ij];
+      Out v;
+      if (te < DIG_NONFINITE && vexp < DIG_NONFINITE) v = dig_result<Out>(x, dig_power(vexp, te));
+      else
+        v = Arith<Out>::from_double(
+            vexp < DIG_NONFINITE
+                ? pp_nonfinite(vstrip, reinterpret_cast<const double*>(tch + (long)ij * steps * 16), row, nl, vexp)
+                : __longlong_as_double(0x7ff8000000000000ll));
+      reinterpret_cast<Out*>(D.rpp)[D.ch_s_off[c] + (long)ij * nl + ab] = v;
     }
   }
 }
 
-// W in the ladder basis split into FP32 pairs (the refinement sweeps' copy of v_pppp).
+// rep_only: the rows ij of the items count the list upd_row of the channel, else every hole pair.
+// wk (2 or 4) divides PP_WARPS: PP_WARPS / wk items per CTA.  slots: ring steps per warp, PP_DEPTH or
+// as many as a warp has.
+template <typename Out>
+__global__ void __launch_bounds__(PP_WARPS * 32, PP_CTAS) k_pp(DevState D, const LoopCtl* __restrict__ ctl,
+                                                               const PPItem* __restrict__ items, int nitems, int rep_only,
+                                                               int wk, int slots) {
+  extern __shared__ __align__(16) uint4 pp_ring[];
+  __shared__ DigSum red[PP_WARPS * 128];
+  const int warp = threadIdx.x >> 5, part = warp % wk;
+  const int item = blockIdx.x * (PP_WARPS / wk) + warp / wk;
+  PPItem it;
+  if (item < nitems) it = items[item];
+  // the barrier of pp_pass is the block's only one: warps without work join it here
+  if (item >= nitems || sys_done(D, ctl, it.sys)) {
+    __syncthreads();
+    return;
+  }
+  const int* __restrict__ rows = rep_only ? D.upd_row + D.ch_uoff[it.c] : nullptr;
+  DigSum* mine = red + (warp / wk) * wk * 128;
+  uint4* ring = pp_ring + warp * slots * 256;
+  const int n = it.nr - it.n0;
+  if (n > 4) pp_pass<1, Out>(D, it, rows, part, wk, ring, mine);
+  else if (n > 2) pp_pass<2, Out>(D, it, rows, part, wk, ring, mine);
+  else pp_pass<4, Out>(D, it, rows, part, wk, ring, mine);
+}
+
+// FP32-pair copy of an FP64 array.
 __global__ void k_split_f2(const double* __restrict__ a, f2* __restrict__ b, long n) {
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) b[i] = Arith<f2>::from_double(a[i]);
@@ -1479,6 +2129,53 @@ __global__ void k_rowinfo(DevState D, const int4* __restrict__ items, UpdRow* __
   out[(long)blockIdx.x * UPD_ROWS + g] = r;
 }
 
+// pp items of nr[c] rows per channel in the order of decreasing work, so that the last CTAs are
+// short ones; the list goes to *dst.  Returns its length.
+static int pp_work_list(pnm_ctx* ctx, const std::vector<int>& nr, PPItem** dst) {
+  struct Pass {
+    long work;
+    int c, n0;
+  };
+  std::vector<Pass> passes;
+  size_t n = 0;
+  for (int c = 0; c < ctx->nch; c++) {
+    if (!ctx->h_vpp[c]) continue;
+    for (int n0 = 0; n0 < nr[c]; n0 += 8) {
+      passes.push_back({(long)ctx->h_nlad[c] * (nr[c] - n0 > 4 ? 36 : (nr[c] - n0 > 2 ? 26 : 15)), c, n0});
+      n += (ctx->h_nlad[c] + 15) / 16;
+    }
+  }
+  std::stable_sort(passes.begin(), passes.end(), [](const Pass& a, const Pass& b) { return a.work > b.work; });
+  std::vector<PPItem> items;
+  items.reserve(n);
+  for (const Pass& p : passes) {
+    const int nl = ctx->h_nlad[p.c], steps = (nl + 15) / 16;
+    for (int q = 0; q < steps; q++)
+      items.push_back(PPItem{p.c, q, p.n0, nr[p.c], nl, ctx->h_ch_sys[p.c], ctx->h_vd_off[p.c] + (long)q * steps * 256});
+  }
+  *dst = (PPItem*)dmalloc(ctx, sizeof(PPItem) * std::max<size_t>(1, n));
+  if (n) CUDA_TRY(cudaMemcpyAsync(*dst, items.data(), sizeof(PPItem) * n, cudaMemcpyHostToDevice, ctx->stream));
+  return (int)n;
+}
+
+// Work lists of the pp ladder (on first use): ladder rows (channel, ij), those the updates compute
+// first, and the items of the computed rows.
+void pnm_need_pp_lists(pnm_ctx* ctx) {
+  if (ctx->pp_items) return;
+  std::vector<int2> rows;
+  rows.reserve(ctx->nrows);
+  for (int part = 0; part < 2; part++) {
+    for (int r = 0; r < ctx->nrows; r++)
+      if (ctx->h_vpp[ctx->h_rows[r].x] && (ctx->h_row_mode[r] == 0) == (part == 1)) rows.push_back(ctx->h_rows[r]);
+    if (part == 0) ctx->n_lad_rep = (int)rows.size();
+  }
+  ctx->n_lad_rows = (int)rows.size();
+  ctx->lad_rows = (int2*)dmalloc(ctx, sizeof(int2) * std::max<size_t>(1, rows.size()));
+  if (!rows.empty())
+    CUDA_TRY(cudaMemcpyAsync(ctx->lad_rows, rows.data(), sizeof(int2) * rows.size(), cudaMemcpyHostToDevice, ctx->stream));
+  ctx->n_pp_items = pp_work_list(ctx, ctx->h_n_urow, &ctx->pp_items);
+}
+
 void pnm_prepare_iteration(pnm_ctx* ctx) {
   cudaStream_t s = ctx->stream;
   int nsys = (int)ctx->sys.size();
@@ -1496,9 +2193,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->row_lo_d = d;
   ctx->row_hi_d = d + nsys;
   ctx->lut_off_d = d + 2 * nsys;
-  // pp work list (channels with a V_pppp block): one item per 32 columns of the ladder basis;
-  // ladder rows (channel, ij) for the gather of the ladder-basis amplitudes
-  std::vector<int2> items, abit, lrows;
+  std::vector<int2> abit;
   std::vector<int4> upd;
   std::vector<int> ulo(nsys), uhi(nsys);
   int max_npp = 0, max_nlad = 0;
@@ -1509,8 +2204,6 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
     if (!ctx->h_vpp[c]) continue;
     int nl = ctx->h_nlad[c];
     max_nlad = std::max(max_nlad, nl);
-    for (int q0 = 0; q0 < nl; q0 += PP64_COLS) items.push_back(make_int2(c, q0));
-    for (int ij = 0; ij < ctx->h_nhh[c]; ij++) lrows.push_back(make_int2(c, ij));
   }
   // per-row items (channel, ij, first column), 128 columns each, grouped by system (the
   // learned-start kernels); update items (channel, first ij, first column, rows) with up to
@@ -1548,6 +2241,9 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
       int c = ctx->h_rows[r].x;
       urow[uoff[c] + ucnt[c]++] = ctx->h_rows[r].y;
     }
+  ctx->h_n_urow.resize(ctx->nch);
+  for (int c = 0; c < ctx->nch; c++) ctx->h_n_urow[c] = uoff[c + 1] - uoff[c];
+  ctx->nsm = nsm;
   ctx->d.upd_row = (int*)dmalloc(ctx, sizeof(int) * std::max<size_t>(1, urow.size()));
   if (!urow.empty())
     CUDA_TRY(cudaMemcpyAsync(ctx->d.upd_row, urow.data(), sizeof(int) * urow.size(), cudaMemcpyHostToDevice, s));
@@ -1579,15 +2275,6 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->upd_rows = G;
   ctx->max_npp = max_npp;
   ctx->max_nlad = max_nlad;
-  ctx->n_lad_rows = (int)lrows.size();
-  ctx->lad_rows = (int2*)dmalloc(ctx, sizeof(int2) * std::max<size_t>(1, lrows.size()));
-  if (!lrows.empty())
-    CUDA_TRY(cudaMemcpyAsync(ctx->lad_rows, lrows.data(), sizeof(int2) * lrows.size(), cudaMemcpyHostToDevice, s));
-  ctx->n_pp_items = (int)items.size();
-  ctx->pp_items = (int2*)dmalloc(ctx, sizeof(int2) * std::max<size_t>(1, items.size()));
-  if (!items.empty())
-    CUDA_TRY(cudaMemcpyAsync(ctx->pp_items, items.data(), sizeof(int2) * items.size(),
-                             cudaMemcpyHostToDevice, s));
   std::vector<int> alo(nsys), ahi(nsys);
   int max_nhh = 1;
   for (size_t k = 0; k < abit.size(); k++) max_nhh = std::max(max_nhh, ctx->h_nhh[abit[k].x]);
@@ -1655,6 +2342,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   // CTA per channel in three size classes (larger than PH_SMALL_DIM: k_ph_big; larger than
   // PH_MID_DIM; the rest), warp per channel (at most PH_WARP_DIM)
   std::vector<int> xb, xm, xl, xw;
+  size_t ph_staged = 0;  // three 8-byte matrices of the largest channel: the size limit of a context
   std::vector<long> xcost(ctx->nx, 0);
   for (int x = 0; x < ctx->nx; x++) {
     int c = ctx->h_x_cls[x];
@@ -1672,16 +2360,14 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
       continue;
     }
     int nm = c == 0 ? 2 : 1;
+    ph_staged = std::max(ph_staged, ph_smem_bytes(d, nm, sizeof(double)));
     if (d > PH_SMALL_DIM) {
-      ctx->ph_big_smem64 = std::max(ctx->ph_big_smem64, ph_smem_bytes(d, nm, sizeof(double)));
       ctx->ph_big_smem32 = std::max(ctx->ph_big_smem32, ph_smem_bytes(d, nm, sizeof(float)));
       xb.push_back(x);
     } else if (d > PH_MID_DIM) {
-      ctx->ph_mid_smem64 = std::max(ctx->ph_mid_smem64, ph_smem_bytes(d, nm, sizeof(double)));
       ctx->ph_mid_smem32 = std::max(ctx->ph_mid_smem32, ph_smem_bytes(d, nm, sizeof(float)));
       xm.push_back(x);
     } else {
-      ctx->ph_smem64 = std::max(ctx->ph_smem64, ph_smem_bytes(d, nm, sizeof(double)));
       ctx->ph_smem32 = std::max(ctx->ph_smem32, ph_smem_bytes(d, nm, sizeof(float)));
       xl.push_back(x);
     }
@@ -1699,21 +2385,21 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   xl.insert(xl.end(), xw.begin(), xw.end());
   xl.insert(xl.begin(), xm.begin(), xm.end());
   xl.insert(xl.begin(), xb.begin(), xb.end());
-  size_t ph_smem = std::max(std::max(ctx->ph_smem64, ctx->ph_mid_smem64), ctx->ph_big_smem64);
+  ctx->h_ph_list = xl;
   ctx->ph_list = (int*)dmalloc(ctx, sizeof(int) * std::max<size_t>(1, xl.size()));
   if (!xl.empty())
     CUDA_TRY(cudaMemcpyAsync(ctx->ph_list, xl.data(), sizeof(int) * xl.size(), cudaMemcpyHostToDevice, s));
-  size_t pp_smem = pp64_smem(max_nlad);
-  if (ph_smem > 227 * 1024 || pp_smem > 227 * 1024)
+  if (ph_staged > 227 * 1024 || max_nlad > PP_MAX_NLAD)
     throw PnmError{PNM_EINVAL, "channel too large for the shared-memory tiles"};
-  pnm_ph_attributes(ctx);
+  smem_at_least(k_ph<float, PH_THREADS, PNM_PH32_TILE>, ph32_smem(ctx));
   for (int k = 0; k < 2; k++) {
     CUDA_TRY(cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking));
     CUDA_TRY(cudaEventCreateWithFlags(&ctx->ev_join[k], cudaEventDisableTiming));
   }
   CUDA_TRY(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
-  smem_at_least(k_pp<double>, pp_smem);
-  smem_at_least(k_pp<f2>, pp_smem);
+  smem_at_least(k_tdig, sizeof(double) * max_nlad);
+  smem_at_least(k_pp<double>, PP_SMEM);
+  smem_at_least(k_pp<f2>, PP_SMEM);
   CUDA_TRY(cudaStreamSynchronize(s));
 }
 
@@ -1807,7 +2493,7 @@ __global__ void __launch_bounds__(128) k_mbpt3_rows(DevState D, double* __restri
 // amplitudes by the MBPT2 guess.
 void pnm_mbpt3_all(pnm_ctx* ctx, double* out) {
   cudaStream_t s = ctx->stream;
-  pnm_need_vpp64(ctx);
+  pnm_need_digits(ctx);
   int nsys = (int)ctx->sys.size();
   if (!ctx->mbpt3_buf) ctx->mbpt3_buf = (double*)dmalloc(ctx, sizeof(double) * (3 * (size_t)ctx->nrows + 3 * nsys));
   double* parts = ctx->mbpt3_buf;
@@ -1818,8 +2504,8 @@ void pnm_mbpt3_all(pnm_ctx* ctx, double* out) {
   CUDA_TRY(cudaMemsetAsync(&ctx->ctl->iter, 0, sizeof(int), s));
   CUDA_TRY(cudaMemsetAsync(&ctx->ctl->skip_done, 0, sizeof(int), s));
   k_init<<<ctx->nrows, 128, 0, s>>>(ctx->d, PNM_INIT_MBPT2);
-  pnm_launch_pp64(ctx, s);
-  if (ctx->nx > 0) launch_ph64(ctx, s, true);  // without cross channels no Q is read
+  pnm_launch_pp(ctx, s, true, false);
+  if (ctx->nx > 0) launch_ph64(ctx, s, s, true);  // without cross channels no Q is read
   k_mbpt3_rows<<<ctx->nrows, 128, 0, s>>>(ctx->d, parts, ctx->nrows);
   for (int k = 0; k < 3; k++)
     k_reduce_rows<<<nsys, 256, 0, s>>>(parts + (size_t)k * ctx->nrows, ctx->row_lo_d, ctx->row_hi_d,
@@ -1863,10 +2549,6 @@ FinArgs fin_args(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, bool 
   return f;
 }
 
-// The FP64 pp ladder in the ladder basis: the amplitudes gathered into it (s = sum of the
-// signed members of each vector), then k_pp64 on a view of the state whose channel width is
-// the basis size, whose amplitudes are s and whose V blocks are the ladder V; the result stays
-// in the ladder layout (consumers read it through lad_index).
 template <typename T_>
 static void lad_expand(pnm_ctx* ctx, const T_* rs, int planes, long pstride, double* host_out) {
   cudaStream_t s = ctx->stream;
@@ -1890,27 +2572,29 @@ void pnm_lad_expand(pnm_ctx* ctx, const f2* rs, int planes, long pstride, double
   lad_expand(ctx, rs, planes, pstride, host_out);
 }
 
-// rep_only: only the rows the updates compute (one of each spin-flip pair of rows); the ladder
-// operator of pnm_apply_pp_ladder takes every row.
-void pnm_launch_pp64(pnm_ctx* ctx, cudaStream_t s, bool rep_only, const f2* vpp_f2) {
-  // the FP64 ladder V is built before any capture by the host-side callers (pnm_need_vpp64)
-  if (!vpp_f2 && !ctx->d.v_pppp) throw PnmError{PNM_EINVAL, "the FP64 ladder V has not been built"};
-  if (ctx->n_pp_items == 0) return;
-  if (vpp_f2)
-    k_lad_gather<f2><<<ctx->n_lad_rows, 128, 0, s>>>(ctx->d, ctx->ctl, ctx->lad_rows, ctx->t_pair,
-                                                      reinterpret_cast<f2*>(ctx->d.s64));
-  else
-    k_lad_gather<double><<<ctx->n_lad_rows, 128, 0, s>>>(ctx->d, ctx->ctl, ctx->lad_rows, nullptr, ctx->d.s64);
-  DevState L = ctx->d;
-  L.ch_npp = ctx->d.ch_nlad;
-  L.ch_t_off = ctx->d.ch_s_off;
-  L.t0 = L.t1 = ctx->d.s64;
-  if (vpp_f2)
-    k_pp<f2><<<ctx->n_pp_items, PP64_WARPS * 32, pp64_smem(ctx->max_nlad), s>>>(L, ctx->ctl, ctx->pp_items,
-                                                                                rep_only ? 1 : 0, vpp_f2);
-  else
-    k_pp<double><<<ctx->n_pp_items, PP64_WARPS * 32, pp64_smem(ctx->max_nlad), s>>>(L, ctx->ctl, ctx->pp_items,
-                                                                                    rep_only ? 1 : 0, ctx->d.v_pppp);
+// The pp ladder in the ladder basis: the digits of the amplitudes, then the digit products
+// (pair: results stored as FP32 pairs); the result stays in the ladder layout
+// (consumers read it through lad_index).  rep_only: only the rows the updates compute (one of
+// each spin-flip pair of rows); the ladder operator of pnm_apply_pp_ladder takes every row.
+void pnm_launch_pp(pnm_ctx* ctx, cudaStream_t s, bool rep_only, bool pair) {
+  // the digits of V are built before any capture by the host-side callers (pnm_need_vdig)
+  if (!ctx->d.vdig) throw PnmError{PNM_EINVAL, "the ladder V has not been built"};
+  if (ctx->n_lad_rows == 0) return;
+  const int nrow = rep_only ? ctx->n_lad_rep : ctx->n_lad_rows;
+  k_tdig<<<nrow, TDIG_THREADS, sizeof(double) * ctx->max_nlad, s>>>(ctx->d, ctx->ctl, ctx->lad_rows);
+  if (!rep_only && !ctx->pp_items_all) ctx->n_pp_all = pp_work_list(ctx, ctx->h_nhh, &ctx->pp_items_all);
+  const PPItem* items = rep_only ? ctx->pp_items : ctx->pp_items_all;
+  const int n = rep_only ? ctx->n_pp_items : ctx->n_pp_all;
+  // four warps per item where two would not fill the GPU twice over
+  const int wk = (long)n * 2 < 2L * PP_WARPS * PP_CTAS * ctx->nsm ? 4 : 2;
+  const unsigned nb = (unsigned)((n + PP_WARPS / wk - 1) / (PP_WARPS / wk));
+  // no more ring than a warp has steps: a small system's CTAs then leave the SMs' split between L1
+  // and shared memory as the neighbouring kernels need it
+  const int steps = (ctx->max_nlad + 15) / 16;
+  const int slots = std::min(PP_DEPTH, std::max(1, (steps + wk - 1) / wk));
+  const size_t smem = PP_SMEM / PP_DEPTH * slots;
+  if (pair) k_pp<f2><<<nb, PP_WARPS * 32, smem, s>>>(ctx->d, ctx->ctl, items, n, rep_only ? 1 : 0, wk, slots);
+  else k_pp<double><<<nb, PP_WARPS * 32, smem, s>>>(ctx->d, ctx->ctl, items, n, rep_only ? 1 : 0, wk, slots);
 }
 
 // The ph term and the pp ladder do not depend on each other nor on the one-body sums: in a
@@ -1967,13 +2651,13 @@ static void enqueue_body_fp64(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHa
   pnm_fork(ctx);
   if (ctx->nx > 0 && ph_on) {
     prof_begin(ctx, pair ? KID_PH_F2 : KID_PH64);
-    if (pair) launch_ph_f2(ctx, ctx->t_pair, ctx->xw_f2, ctx->xv1_f2, s_ph);
-    else launch_ph64(ctx, s_ph, terms == PNM_TERMS_LINEAR);
+    if (pair) launch_ph_f2(ctx, s_ph, ctx->stream);
+    else launch_ph64(ctx, s_ph, ctx->stream, terms == PNM_TERMS_LINEAR);
     prof_end(ctx);
   }
-  if (ctx->n_pp_items > 0) {
+  if (ctx->n_lad_rows > 0) {
     prof_begin(ctx, pair ? KID_PP_F2 : KID_PP64);
-    pnm_launch_pp64(ctx, s_pp, true, pair ? ctx->vpp_f2 : nullptr);
+    pnm_launch_pp(ctx, s_pp, true, pair);
     prof_end(ctx);
   }
   if (terms == PNM_TERMS_FULL) pnm_enqueue_stats(ctx, false, pair);
@@ -2026,18 +2710,20 @@ void pnm_enqueue_body(pnm_ctx* ctx, int mode, int use_cond, cudaGraphConditional
   else pnm_enqueue_body_mixed(ctx, use_cond, h);
 }
 
-// FP32-pair copies of the ladder-basis V_pppp, V_pphh, W and <kb|v|cj> (once per context).
+// The digits of both contractions: V_pppp and the ph term's fixed operands (once per context).
+void pnm_need_digits(pnm_ctx* ctx) {
+  pnm_need_vdig(ctx);
+  pnm_need_phdig(ctx);
+}
+
+// What the sweeps with FP32-pair contractions add (once per context): the pair copy of V_pphh.
 void pnm_prepare_f2(pnm_ctx* ctx) {
   if (ctx->t_pair) return;
   cudaStream_t s = ctx->stream;
-  pnm_need_vpp_f2(ctx);
+  pnm_need_digits(ctx);
   ctx->t_pair = ctx_alloc<f2>(ctx, ctx->nt);
-  ctx->xw_f2 = ctx_alloc<f2>(ctx, ctx->nxt);
-  ctx->xv1_f2 = ctx_alloc<f2>(ctx, ctx->nxc);
   ctx->vpphh_f2 = ctx_alloc<f2>(ctx, ctx->nt);
   pnm_split_f2(ctx->d.v_pphh, ctx->vpphh_f2, ctx->nt, s);
-  pnm_split_f2(ctx->d.x_w, ctx->xw_f2, ctx->nxt, s);
-  pnm_split_f2(ctx->d.x_v1, ctx->xv1_f2, ctx->nxc, s);
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(s));
 }
@@ -2060,9 +2746,8 @@ void pnm_prepare_terms(pnm_ctx* ctx, int terms) {
 // the highest, so that the shorter branches (pp ladder, one-body sums) are dispatched ahead of
 // the many ph CTAs and run beside them instead of after them.
 static bool is_ph_kernel(const void* f) {
-  return f == (const void*)k_ph<double, PH_THREADS, 2> || f == (const void*)k_ph<float, PH_THREADS, ph_tile<float>()> ||
-         f == (const void*)k_ph<f2, PH_THREADS, 2> || f == (const void*)k_ph_big<double, 2> ||
-         f == (const void*)k_ph_big<float, ph_tile<float>()> || f == (const void*)k_ph_big<f2, 2>;
+  return f == (const void*)k_ph<float, PH_THREADS, PNM_PH32_TILE> || f == (const void*)k_ph_dig<double> ||
+         f == (const void*)k_ph_dig<f2> || f == (const void*)k_ph_tiny<double> || f == (const void*)k_ph_tiny<f2>;
 }
 
 void pnm_set_node_priorities(cudaGraph_t body) {
@@ -2324,7 +3009,7 @@ void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
   const bool pair = ((mode >> 8) & 1) != 0;
   int m = (mode & 15) == PNM_PREC_FP64 ? (pair ? 2 : 0) : 1;
   if (ctx->sched_tuned[m]) return;
-  if (m == 0) pnm_need_vpp64(ctx);
+  if (m == 0) pnm_need_digits(ctx);
   const std::string key = pnm_shape_key(ctx) + (m == 1 ? "|mixed" : m == 2 ? "|pair" : "|fp64");
   {
     std::lock_guard<std::mutex> lock(g_sched_mu);

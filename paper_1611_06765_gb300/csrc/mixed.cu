@@ -27,6 +27,7 @@
 #include <cuda.h>  // CUtensorMap and its enums (the encoder is fetched through the runtime)
 #include <cudaTypedefs.h>
 
+#include "dig.cuh"
 #include "pnm_context.cuh"
 #include "tc_ptx.cuh"
 
@@ -55,28 +56,61 @@ static_assert(TC_BK == 64, "tile_core_off assumes 64-element k-blocks");
 __device__ __forceinline__ int core_off(int r, int k) { return tile_core_off(r, k); }
 
 // ------------------------------------------------------------------------ kernels
-// V tiles of the channels with a V_pppp block (setup): one CTA per (item, k-block).
-// Read from the FP32-pair copy of V: its high part is the FP32 rounding of the FP64 element,
-// the value the BF16 split starts from.
-__global__ void k_pack_v(const TCItem* __restrict__ items, const f2* __restrict__ v_pppp,
-                         const long* __restrict__ ch_vpp_off, __nv_bfloat16* __restrict__ vt) {
+// V tiles of the channels with a V_pppp block (setup): one CTA per (item, k-block), the elements
+// straight from the interaction table as integers (dig.cuh), rounded to FP32 and split into BF16
+// hi + lo: neither an FP64 operation nor a stored V (forming them from a stored FP32-pair copy
+// took a write and a read of 8 bytes per element and four FP64-pipe instructions).
+__global__ void __launch_bounds__(256) k_pack_v(const TCItem* __restrict__ items, DevState D,
+                                                const int* __restrict__ lut_off, const int2* __restrict__ lut_info,
+                                                __nv_bfloat16* __restrict__ vt) {
+  extern __shared__ __align__(16) unsigned char psm[];
+  __shared__ int sh_max;
+  __shared__ char4 ra[TC_M], rb[TC_M], ca[TC_BK], cb[TC_BK];
+  __shared__ int rs[TC_M], cs[TC_BK];  // signs of the representatives, 0 past the matrix
   TCItem it = items[blockIdx.x];  // an unsplit item: kb0 = 0, nkb = all k-blocks
   int kb = blockIdx.y;
   if (kb >= it.nkb) return;
-  const f2* V = v_pppp + ch_vpp_off[it.ch];
+  const int2 li = lut_info[it.sys];  // table entries, 1 with protons
+  long long* xlut = reinterpret_cast<long long*>(psm);
+  const int e = stage_fixed_lut(D.lut + lut_off[it.sys], li.x, li.y != 0, xlut, &sh_max);
+  const int off = D.ch_pp_off[it.ch];
+  for (int r = threadIdx.x; r < TC_M + TC_BK; r += blockDim.x) {
+    const bool row = r < TC_M;
+    const int u = row ? r : r - TC_M, q = row ? it.mt * TC_M + u : kb * TC_BK + u;
+    char4 a = make_char4(0, 0, 0, 0), b = a;
+    int sg = 0;
+    if (q < it.npp) {
+      const int m = D.lad_mem[off + q].x;
+      const int2 pr = D.pp_pair[off + (m > 0 ? m : -m) - 1];
+      a = D.nvec[pr.x];
+      b = D.nvec[pr.y];
+      sg = m > 0 ? 1 : -1;
+    }
+    (row ? ra : ca)[u] = a;
+    (row ? rb : cb)[u] = b;
+    (row ? rs : cs)[u] = sg;
+  }
+  __syncthreads();
   __nv_bfloat16* hi = vt + it.voff + (long)kb * 2 * (TC_M * TC_BK);
   __nv_bfloat16* lo = hi + TC_M * TC_BK;
-  // V is symmetric (bit for bit: <ab|v|cd> and <cd|v|ab> are evaluated by the same
-  // arithmetic), so the element (cd, ab) is read as (ab, cd): consecutive threads then read
-  // consecutive doubles of one row.
-  for (int e = threadIdx.x; e < TC_M * TC_BK; e += blockDim.x) {
-    int r = e / TC_BK, k = e % TC_BK;
-    int ab = it.mt * TC_M + r, cd = kb * TC_BK + k;
-    double x = (ab < it.npp && cd < it.npp) ? (double)V[(long)ab * it.npp + cd].hi : 0.0;
-    __nv_bfloat16 h, l;
-    split_bf16(x, h, l);
-    hi[core_off(r, k)] = h;
-    lo[core_off(r, k)] = l;
+  // in the order of the tile (8 x 8 core matrices): eight neighbouring elements of a row per step
+  for (int f = threadIdx.x; f < TC_M * TC_BK / 8; f += blockDim.x) {
+    const int r = (f >> 6) * 8 + (f & 7), k0 = ((f >> 3) & 7) * 8;
+    __align__(16) __nv_bfloat16 h[8], l[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      const int sg = rs[r] * cs[k0 + j];
+      float x = 0.0f;
+      if (sg != 0) {
+        const long long v = v_minnesota_fixed(ca[k0 + j], cb[k0 + j], ra[r], rb[r], xlut);
+        x = e < DIG_NONFINITE ? scalbnf(__ll2float_rn(sg > 0 ? v : -v), e - 1022 - 61) : __int_as_float(0x7fc00000);
+      }
+      h[j] = __float2bfloat16_rn(x);
+      l[j] = __float2bfloat16_rn(x - __bfloat162float(h[j]));
+    }
+    const int o = core_off(r, k0);
+    *reinterpret_cast<uint4*>(hi + o) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(lo + o) = *reinterpret_cast<const uint4*>(l);
   }
 }
 
@@ -143,10 +177,10 @@ __global__ void __launch_bounds__(PP_THREADS, 1) k_pp_tc(const __grid_constant__
   unsigned char* stage0 = smem + 1024;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __shared__ int err;
-  const int i_begin = cta_off[blockIdx.x], i_end = cta_off[blockIdx.x + 1];
   // items of converged systems are skipped by all three roles alike (the flags do not change
   // during a launch)
   const bool skip = ctl->skip_done != 0;
+  const int i_begin = cta_off[blockIdx.x], i_end = cta_off[blockIdx.x + 1];
 
   if (threadIdx.x == 0) {
     err = 0;
@@ -438,7 +472,6 @@ static std::map<std::string, std::tuple<int, int, float>> g_tile_cache;
 void pnm_prepare_mixed(pnm_ctx* ctx) {
   if (ctx->mixed) return;
   cudaStream_t s = ctx->stream;
-  pnm_need_vpp_f2(ctx);  // the V tiles are split from it
   MixedState* M = new MixedState();
   M->sysctl = ctx->sysctl;
   try {
@@ -522,8 +555,19 @@ void pnm_prepare_mixed(pnm_ctx* ctx) {
       k_to_float<<<(unsigned)((ctx->nxt + 255) / 256), 256, 0, s>>>(ctx->d.x_w, M->xw32, ctx->nxt);
     if (ctx->nxc > 0)
       k_to_float<<<(unsigned)((ctx->nxc + 255) / 256), 256, 0, s>>>(ctx->d.x_v1, M->xv132, ctx->nxc);
-    if (M->nitems > 0)
-      k_pack_v<<<dim3(M->nitems, max_nkb), 256, 0, s>>>(M->items, ctx->vpp_f2, ctx->d.ch_vpp_off, M->vt);
+    if (M->nitems > 0) {
+      std::vector<int2> li;
+      int max_lut = 0;
+      for (const SysInfo& S : ctx->sys) {
+        li.push_back(make_int2(S.lut_len * (S.species == 1 ? 1 : 3), S.species != 1));
+        max_lut = std::max(max_lut, li.back().x);
+      }
+      int2* dli = mdalloc<int2>(ctx, li.size());
+      CUDA_TRY(cudaMemcpyAsync(dli, li.data(), sizeof(int2) * li.size(), cudaMemcpyHostToDevice, s));
+      smem_at_least(k_pack_v, sizeof(long long) * max_lut);
+      k_pack_v<<<dim3(M->nitems, max_nkb), 256, sizeof(long long) * max_lut, s>>>(M->items, ctx->d, ctx->lut_off_d, dli,
+                                                                                  M->vt);
+    }
     CUDA_TRY(cudaGetLastError());
     M->stage_bytes = (2 * A_PLANE + 2 * (uint32_t)max_npad * TC_BK * 2 + 1023) / 1024 * 1024;
     auto smem_for = [&](int nst) { return 1024 + (size_t)nst * M->stage_bytes + 8192; };  // tail guard
@@ -709,14 +753,10 @@ void pnm_apply_pp(pnm_ctx* ctx, int sys, int precision, const double* t, double*
     launch_pp_tc(M->items, M->cta_off, M->grid, M, M->smem, M->nst, ctx->ctl, ctx->ns, s);
     pnm_lad_expand(ctx, M->rpp32, M->ksplit, ctx->ns, out.data());
   } else {
-    if (precision == PNM_PREC_F32PAIR) {
-      pnm_prepare_f2(ctx);
-      pnm_split_cur(ctx, s);
-    }
-    if (precision == PNM_PREC_FP64) pnm_need_vpp64(ctx);
+    pnm_need_vdig(ctx);
     CUDA_TRY(cudaMemsetAsync(ctx->d.rpp, 0, sizeof(double) * std::max<long>(ctx->ns, 1), s));
     // every row: the operator acts on any amplitudes
-    pnm_launch_pp64(ctx, s, false, precision == PNM_PREC_F32PAIR ? ctx->vpp_f2 : nullptr);
+    pnm_launch_pp(ctx, s, false, precision == PNM_PREC_F32PAIR);
     if (precision == PNM_PREC_F32PAIR)
       pnm_lad_expand(ctx, reinterpret_cast<const f2*>(ctx->d.rpp), 1, ctx->ns, out.data());
     else
@@ -771,13 +811,14 @@ void pnm_apply_ph(pnm_ctx* ctx, int sys, int precision, const double* t, double*
     if (ctx->nx > 0) launch_ph_mix(ctx, M->xt32, M->xw32, M->xv132, M->xq32, s);
     k_ph_assemble<float><<<nb, 256, 0, s>>>(ctx->d, M->xq32, ctx->nt, ctx->expand_buf);
   } else {
+    pnm_need_phdig(ctx);
     if (precision == PNM_PREC_F32PAIR) {
       pnm_prepare_f2(ctx);
       pnm_split_cur(ctx, s);
-      if (ctx->nx > 0) launch_ph_f2(ctx, ctx->t_pair, ctx->xw_f2, ctx->xv1_f2, s);
+      if (ctx->nx > 0) launch_ph_f2(ctx, s, s);
       k_ph_assemble<f2><<<nb, 256, 0, s>>>(ctx->d, reinterpret_cast<const f2*>(ctx->d.xq), ctx->nt, ctx->expand_buf);
     } else {
-      if (ctx->nx > 0) launch_ph64(ctx, s);
+      if (ctx->nx > 0) launch_ph64(ctx, s, s, false);
       k_ph_assemble<double><<<nb, 256, 0, s>>>(ctx->d, ctx->d.xq, ctx->nt, ctx->expand_buf);
     }
   }

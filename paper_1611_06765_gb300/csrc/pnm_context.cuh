@@ -7,6 +7,7 @@
 
 struct MixedState;  // mixed-precision operand arenas (mixed.cu)
 struct MlpState;    // learned warm start (mlp.cu)
+struct PhItem;      // work item of the digit ph term (iterate.cu)
 
 // Kernel ids of the per-kernel profiler.
 enum {
@@ -24,37 +25,56 @@ struct pnm_ctx {
 
   // sizes
   int nsp_total = 0, nch = 0, nx = 0, nrows = 0, n_hh_pairs = 0, n_pp_pairs = 0;
-  long nt = 0, nvpp = 0, nvhh = 0, nxt = 0, nxc = 0;
+  long nt = 0, nvhh = 0, nxt = 0, nxc = 0;
   long ns = 0;  // elements of the ladder layout (n_hh x n_lad over the channels with V_pppp)
   int max_x_dim = 0, max_npp = 0, max_nlad = 0;
-  int2* lad_rows = nullptr;  // (channel, ij) rows of the channels with V_pppp (ladder gather)
-  int n_lad_rows = 0;
+  // (channel, ij) rows of the channels with V_pppp (digits of the ladder amplitudes): first those
+  // the updates compute, then the others
+  int2* lad_rows = nullptr;
+  int n_lad_rows = 0, n_lad_rep = 0;
 
   // host copies of the channel metadata
   std::vector<int> h_ch_sys, h_key, h_nhh, h_npp, h_hh_off, h_pp_off, h_vpp;
   std::vector<long> h_t_off, h_x_t_off;
   std::vector<int> h_nlad;               // ladder basis size per channel (0: no V_pppp block)
-  std::vector<long> h_s_off, h_vl_off;   // ladder-layout and ladder-V offsets per channel
+  std::vector<long> h_s_off, h_vd_off;   // ladder-layout and ladder-V offsets per channel
+  long nvdig = 0, ntdig = 0;             // digit words of the ladder V, room for those of the amplitudes
   std::vector<int2> h_rows;
-  std::vector<int> h_x_nph, h_x_nhp, h_x_ph_off, h_x_hp_off;
+  std::vector<int> h_x_nph, h_x_nhp, h_x_ph_off, h_x_hp_off, h_x_sys;
   std::vector<int> h_x_cls;  // spin-flip class of each cross channel (+1, 0, -1)
+  std::vector<int> h_n_urow;    // per channel the rows the updates compute
   std::vector<int> h_row_mode;  // per row (h_rows): 2/1 computed by the updates, 0 a flip
 
   // work lists
-  int2* pp_items = nullptr;   // (channel, first pp column) of the FP64 pp ladder
-  int n_pp_items = 0;
+  // pp ladder: items for the rows the updates compute, and (made on first use) for every row
+  PPItem *pp_items = nullptr, *pp_items_all = nullptr;
+  int n_pp_items = 0, n_pp_all = 0, nsm = 148;
   int4* upd_items = nullptr;  // (channel, ij, first pp column) of the update
   int n_upd_items = 0;
   int *upd_lo_d = nullptr, *upd_hi_d = nullptr;  // per system ranges of the (row, column) items
   int4* grp_items = nullptr;  // (channel, first ij, first pp column, rows) of the update
   int n_grp_items = 0, upd_rows = 1;
   int* ph_list = nullptr;  // cross channels of the ph launches (S_z >= 0, costliest first)
-  // channels of the larger size class (k_ph_big), of the middle and the small class of the CTA
-  // path and of the warp path of k_ph, in that order in ph_list
+  // channels of the larger, the middle and the small size class of the CTA path and of the warp
+  // path, in that order in ph_list
   int n_ph_big = 0, n_ph_mid = 0, n_ph = 0, n_ph_warp = 0;
-  size_t ph_smem64 = 0, ph_smem32 = 0;          // shared memory of a small-class k_ph CTA
-  size_t ph_mid_smem64 = 0, ph_mid_smem32 = 0;  // of a middle-class k_ph CTA
-  size_t ph_big_smem64 = 0, ph_big_smem32 = 0;  // and of a k_ph_big CTA
+  size_t ph_smem32 = 0, ph_mid_smem32 = 0, ph_big_smem32 = 0;  // shared memory per class (FP32)
+  std::vector<int> h_ph_list;
+  // the digit ph term (made on first use, pnm_need_phdig): items in ph_list's order, the n_ph_large
+  // ones with the largest tiles first; W fragments, <kb|v|cj> of the problems, source indices
+  PhItem* ph_items = nullptr;
+  int2* ph_exps = nullptr;
+  int* ph_src = nullptr;
+  uint4* ph_wf = nullptr;
+  long long* ph_v1 = nullptr;
+  double* ph_fixed64 = nullptr;
+  f2* ph_fixed_f2 = nullptr;  // the fixed operands of the smallest channels as element values
+  int n_ph_large = 0;
+  int n_ph_tiny64 = 0, n_ph_tiny_f2 = 0;  // the last items: channels without digits (FP64, FP32-pair results)
+  long* tw_lo = nullptr;                         // first amplitude of each system
+  int* tw_parts = nullptr;
+  int n_tw_parts = 1;
+  size_t ph_large_smem = 0, ph_dig_smem = 0, ph_warp_smem = 0;
   f2* t_pair = nullptr;                          // FP32-pair copy of the current amplitudes
   int *grp_lo_d = nullptr, *grp_hi_d = nullptr;  // per system ranges of the update items
   int *ab_lo_d = nullptr, *ab_hi_d = nullptr;    // per system ranges of the column items
@@ -92,11 +112,9 @@ struct pnm_ctx {
 
   MixedState* mixed = nullptr;
   MlpState* mlp = nullptr;
-  // FP32-pair copies of the ladder-basis V_pppp, V_pphh, W and <kb|v|cj> (made on first use by
-  // the FP32-pair contractions)
-  f2 *vpp_f2 = nullptr, *vpphh_f2 = nullptr, *xw_f2 = nullptr, *xv1_f2 = nullptr;
+  f2* vpphh_f2 = nullptr;  // FP32-pair copy of V_pphh (made on first use by the FP32-pair sweeps)
   // work list of the ladder-basis V (items (channel, first row), per system a run) and the
-  // shared memory of its kernel; the V itself is built on first use (pnm_need_vpp64 / _f2)
+  // shared memory of its kernel; the V itself is built on first use (pnm_need_vdig)
   int2* vl_items = nullptr;
   std::vector<int> vl_sys;
   size_t vl_smem = 0;
@@ -179,9 +197,8 @@ void pnm_reopen(pnm_ctx* ctx);
 void pnm_settle_amplitudes(pnm_ctx* ctx);
 void pnm_mlp_start(pnm_ctx* ctx);
 void pnm_mlp_prepare(pnm_ctx* ctx);
-void pnm_ladder_v(pnm_ctx* ctx, double* out64, f2* out2);
-void pnm_need_vpp64(pnm_ctx* ctx);
-void pnm_need_vpp_f2(pnm_ctx* ctx);
+void pnm_need_vdig(pnm_ctx* ctx);
+void pnm_need_pp_lists(pnm_ctx* ctx);
 void pnm_mlp_enqueue(pnm_ctx* ctx);
 void pnm_drop_solve_graphs(pnm_ctx* ctx);
 void pnm_set_node_priorities(cudaGraph_t body);
@@ -200,8 +217,10 @@ void prof_end(pnm_ctx* ctx);
 void prof_collect(pnm_ctx* ctx);
 FinArgs fin_args(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, bool per_row);
 void pnm_enqueue_stats(pnm_ctx* ctx, bool mixed, bool pair = false);
-void pnm_launch_pp64(pnm_ctx* ctx, cudaStream_t s, bool rep_only = true, const f2* vpp_f2 = nullptr);
-void launch_ph_f2(pnm_ctx* ctx, const f2* tpair, const f2* xw, const f2* xv1, cudaStream_t s);
+void pnm_launch_pp(pnm_ctx* ctx, cudaStream_t s, bool rep_only, bool pair);
+void launch_ph_f2(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny);
+void pnm_need_phdig(pnm_ctx* ctx);
+void pnm_need_digits(pnm_ctx* ctx);
 void pnm_split_f2(const double* a, f2* b, long n, cudaStream_t s);
 void pnm_prepare_f2(pnm_ctx* ctx);
 void pnm_split_cur(pnm_ctx* ctx, cudaStream_t s);
@@ -212,7 +231,7 @@ void pnm_join(pnm_ctx* ctx);
 void pnm_launch_mbpt2_into(const pnm_ctx* ctx, double* partials, double* results);
 void pnm_apply_ph(pnm_ctx* ctx, int sys, int precision, const double* t, double* r, size_t n);
 void pnm_apply_pp(pnm_ctx* ctx, int sys, int precision, const double* t, double* r, size_t n);
-void launch_ph64(pnm_ctx* ctx, cudaStream_t s, bool linear = false);
+void launch_ph64(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny, bool linear);
 void pnm_flip_symmetrise(pnm_ctx* ctx, double* t, cudaStream_t s);
 void pnm_flip_copy(pnm_ctx* ctx, double* t, cudaStream_t s);
 void pnm_flip_copy_current(pnm_ctx* ctx, int iter);

@@ -2,13 +2,13 @@
 //
 // Layout in HBM (all systems of a context concatenated; every index below is global):
 //   states       char4 nvec[n_sp_total] = (n_x, n_y, n_z, s); double eps[], ekin[]
-//   direct chans per channel c: sys, key, n_hh, n_pp, hh_off, pp_off, t_off, vpp_off, vhh_off
+//   direct chans per channel c: sys, key, n_hh, n_pp, hh_off, pp_off, t_off, vhh_off
 //                int2 hh_pair[], pp_pair[] (global state indices, lexicographic per channel)
 //   amplitudes   t[c] is an n_hh x n_pp row-major block (hh rows, pp contiguous): element
 //                (ij, ab) at t_off[c] + ij * n_pp + ab.  v_pphh has the same layout.
 //   V_pppp       only for channels where <ab|v|cd> can be nonzero (not both |S_z| = 2 and
 //                |T_z| = 2: identical nucleons of equal spin do not interact; for neutrons
-//                that leaves S_z = 0): n_pp x n_pp, symmetric, row-major at vpp_off[c].
+//                that leaves S_z = 0): in the ladder basis, as digit words (dig.cuh).
 //   cross chans  per channel x: n_ph rows (a,i), n_hp columns (k,c); T_x/Q_x are
 //                n_ph x n_hp at xt_off[x]; V1_x (<kb|v|cj>) n_hp x n_hp at xc_off[x];
 //                W_x (<kl|v|ce>, n_hp x n_ph) stored transposed (n_ph x n_hp) at xw_off[x].
@@ -72,7 +72,7 @@ struct DevState {
   int* sp_hole;          // 1 for hole states
   // direct channels
   int *ch_sys, *ch_key, *ch_nhh, *ch_npp, *ch_hh_off, *ch_pp_off, *ch_vpp;
-  long *ch_t_off, *ch_vpp_off, *ch_vhh_off;
+  long *ch_t_off, *ch_vhh_off;
   // ladder basis of the pp ladder (channels with a V_pppp block): n_lad vectors per channel,
   // ladder-layout blocks (n_hh x n_lad) at ch_s_off; lad_map per pp pair: its vector and sign
   // as +-(index + 1); lad_mem per vector (at the channel's pp offset): its one or two pairs as
@@ -106,7 +106,16 @@ struct DevState {
   int4* qmap;            // per t element: the four Q positions of P(ij)P(ab) Q (formed positions)
   int *occ_off, *occ_idx; // per state: pair indices (pp for particles, hh for holes)
   // blocks
-  double *v_pphh, *v_pppp, *v_hhhh, *x_v1, *x_w;  // v_pppp: n_lad x n_lad per channel, ladder basis
+  double *v_pphh, *v_hhhh, *x_v1, *x_w;
+  // pp ladder in digit words (dig.cuh): per channel with a V_pppp block the ladder-basis V at
+  // ch_vd_off in fragment order (16-row strips of 16-column steps) with its exponent, and the
+  // ladder-basis amplitudes at ch_td_off, n_hh rows of the padded width, an exponent per hole pair
+  unsigned long long *vdig, *tdig;
+  long *ch_vd_off, *ch_td_off;
+  int *ch_vexp, *texp;
+  // digit words of the current amplitudes and their exponent per system (digit ph term)
+  unsigned long long* twords;
+  int* sys_texp;
   double *den, *inv_den;  // eps_i + eps_j - eps_a - eps_b per amplitude, and its reciprocal
   // iteration state
   double *t0, *t1;       // double buffer, parity = iteration & 1
@@ -115,18 +124,17 @@ struct DevState {
   // v_pphh and v_hhhh copies, chi_hh, the one-body row/column sums and the one-body terms
   float *v32, *vhh32, *chi32, *sij32, *sab32, *dchi32;
   double *rpp, *chi_hh, *dchi, *sab, *sij, *xq;  // rpp: pp ladder in the ladder layout
-  double* s64;           // amplitudes in the ladder basis (input of the FP64 pp ladder)
   double *eparts, *rparts;
   // per-system loop state (converged systems are frozen: later steps skip their work)
   const struct SysCtl* sysctl;
 };
 
-// Work-list items for the grouped pp-ladder launch (FP64 path).
-struct PPItem {
-  int ch;      // direct channel
-  int ab0;     // first pp column of the tile
-  int ij0;     // first hh row of the tile
-  int nij;     // rows in the tile
+// Work item of the pp ladder in digits: a strip of 16 ladder vectors and a pass over up to 8 hole
+// pairs of a channel.
+struct __align__(16) PPItem {
+  int c, strip, n0, nr;  // channel, strip, first row of the pass, rows of the channel
+  int nl, sys;           // ladder vectors and system of the channel
+  long voff;             // digit words of the strip in the arena of V
 };
 
 // Solve-loop control block in device memory (one per context).

@@ -17,6 +17,7 @@
 
 #include <type_traits>
 
+#include "dig.cuh"
 #include "pnm_context.cuh"
 
 namespace {
@@ -733,25 +734,29 @@ __global__ void __launch_bounds__(LAD_THREADS) k_ladder_basis(
   if (threadIdx.x == 0) ch_nlad[c] = base_sh;
 }
 
-// W(c, c') = e e' <rep c|v|rep c'> for VLAD_ROWS rows of one channel per CTA; the channel's
-// representative pair states, their signs and the LUT are staged in shared memory.
+// W(c, c') = e e' <rep c|v|rep c'> for the 16 rows of one strip of a channel per CTA, as digit
+// words (dig.cuh) in the order the ladder kernel's tensor-core fragments read them: per 16-column
+// step four groups (row half + 2 column half) of 32 lanes with two neighbouring columns each
+// (interleaved), zero past the matrix.  The channel's representative pair states, their signs and the
+// interaction table (as integers) are staged in shared memory; no FP64 arithmetic.
+// The BF16 tiles of the mixed ladder (k_pack_v) come from the same integers.
 constexpr int VLAD_ROWS = 16;
-// Out: double (the FP64 ladder V) or f2 (its FP32-pair copy, the element split once).
-template <typename Out>
-__global__ void __launch_bounds__(256) k_v_ladder(const int2* __restrict__ items, const int* __restrict__ ch_pp_off,
-                                                  const int* __restrict__ ch_nlad, const long* __restrict__ ch_vl_off,
-                                                  const int2* __restrict__ lad_mem, const int2* __restrict__ pp_pair,
-                                                  const char4* __restrict__ nvec, const double* __restrict__ lut,
-                                                  int lut_elems, Out* __restrict__ v_lad) {
+__global__ void __launch_bounds__(256) k_v_dig(const int2* __restrict__ items, const int* __restrict__ ch_pp_off,
+                                               const int* __restrict__ ch_nlad, const long* __restrict__ ch_vd_off,
+                                               const int2* __restrict__ lad_mem, const int2* __restrict__ pp_pair,
+                                               const char4* __restrict__ nvec, const double* __restrict__ lut,
+                                               int lut_elems, int species, int* __restrict__ ch_vexp,
+                                               dig_t* __restrict__ vdig) {
   extern __shared__ __align__(16) unsigned char vsm[];
-  double* slut = reinterpret_cast<double*>(vsm);
+  __shared__ int sh_max;
+  long long* xlut = reinterpret_cast<long long*>(vsm);
   int2 it = items[blockIdx.x];
   int c = it.x, r0 = it.y;
   int nl = ch_nlad[c], off = ch_pp_off[c];
-  char4* sa = reinterpret_cast<char4*>(slut + lut_elems);
+  char4* sa = reinterpret_cast<char4*>(xlut + lut_elems);
   char4* sb = sa + nl;
   int* sg = reinterpret_cast<int*>(sb + nl);
-  for (int m = threadIdx.x; m < lut_elems; m += blockDim.x) slut[m] = lut[m];
+  const int e = stage_fixed_lut(lut, lut_elems, species != 1, xlut, &sh_max);
   for (int q = threadIdx.x; q < nl; q += blockDim.x) {
     int m = lad_mem[off + q].x;
     int pos = (m > 0 ? m : -m) - 1;
@@ -760,18 +765,25 @@ __global__ void __launch_bounds__(256) k_v_ladder(const int2* __restrict__ items
     sb[q] = nvec[pr.y];
     sg[q] = m > 0 ? 1 : -1;
   }
+  if (threadIdx.x == 0) ch_vexp[c] = e;
   __syncthreads();
-  int r1 = min(r0 + VLAD_ROWS, nl);
-  for (int row = r0; row < r1; row++) {
-    char4 sc = sa[row], sd = sb[row];
-    int g = sg[row];
-    Out* out = v_lad + ch_vl_off[c] + (long)row * nl;
-    for (int q = threadIdx.x; q < nl; q += blockDim.x) {
-      double v = v_minnesota_as(sa[q], sb[q], sc, sd, slut);
-      v = g * sg[q] > 0 ? v : __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
-      if constexpr (std::is_same<Out, f2>::value) out[q] = Arith<f2>::from_double(v);
-      else out[q] = v;
+  const int steps = (nl + 15) >> 4;
+  uint4* out = reinterpret_cast<uint4*>(vdig + ch_vd_off[c]) + (long)(r0 >> 4) * steps * 128;
+  for (int f = threadIdx.x; f < steps * 128; f += blockDim.x) {
+    const int lane = f & 31, g = (f >> 5) & 3, ks = f >> 7;
+    const int row = r0 + (lane >> 2) + (g & 1) * 8, col = ks * 16 + (lane & 3) * 2 + (g >> 1) * 8;
+    dig_t w[2];
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const int q = col + k;
+      long long v = 0;
+      if (row < nl && q < nl) {
+        v = v_minnesota_fixed(sa[q], sb[q], sa[row], sb[row], xlut);
+        v = sg[row] * sg[q] > 0 ? v : -v;
+      }
+      w[k] = dig_word(v);
     }
+    out[f] = dig_interleave(w[0], w[1]);
   }
 }
 
@@ -852,43 +864,26 @@ struct SysScratch {
   }
 };
 
-// The ladder-basis V_pppp of every system into out64 (FP64) or out2 (FP32 pairs).
-void pnm_ladder_v(pnm_ctx* ctx, double* out64, f2* out2) {
+// The digit words of the ladder-basis V_pppp (the FP64 and FP32-pair pp ladder): built once, on
+// first use.
+void pnm_need_vdig(pnm_ctx* ctx) {
+  if (ctx->d.vdig) return;
   cudaStream_t s = ctx->stream;
   DevState& D = ctx->d;
-  const int nsys = (int)ctx->sys.size();
-  if (out64) smem_at_least(k_v_ladder<double>, ctx->vl_smem);
-  if (out2) smem_at_least(k_v_ladder<f2>, ctx->vl_smem);
-  for (int k = 0; k < nsys; k++) {
+  pnm_need_pp_lists(ctx);
+  D.tdig = ctx_alloc<dig_t>(ctx, ctx->ntdig);
+  D.texp = ctx_alloc<int>(ctx, ctx->n_hh_pairs);
+  D.vdig = ctx_alloc<dig_t>(ctx, std::max<long>(ctx->nvdig, 1));
+  smem_at_least(k_v_dig, ctx->vl_smem);
+  for (int k = 0; k < (int)ctx->sys.size(); k++) {
     const int lo = ctx->vl_sys[k], hi = ctx->vl_sys[k + 1];
     if (hi <= lo) continue;
     const SysInfo& S = ctx->sys[k];
-    const int lut_elems = S.lut_len * (S.species == 1 ? 1 : 3);
-    if (out64)
-      k_v_ladder<double><<<(unsigned)(hi - lo), 256, ctx->vl_smem, s>>>(
-          ctx->vl_items + lo, D.ch_pp_off, D.ch_nlad, D.ch_vpp_off, D.lad_mem, D.pp_pair, D.nvec,
-          D.lut + S.lut_off, lut_elems, out64);
-    if (out2)
-      k_v_ladder<f2><<<(unsigned)(hi - lo), 256, ctx->vl_smem, s>>>(
-          ctx->vl_items + lo, D.ch_pp_off, D.ch_nlad, D.ch_vpp_off, D.lad_mem, D.pp_pair, D.nvec,
-          D.lut + S.lut_off, lut_elems, out2);
+    k_v_dig<<<(unsigned)(hi - lo), 256, ctx->vl_smem, s>>>(
+        ctx->vl_items + lo, D.ch_pp_off, D.ch_nlad, D.ch_vd_off, D.lad_mem, D.pp_pair, D.nvec, D.lut + S.lut_off,
+        S.lut_len * (S.species == 1 ? 1 : 3), S.species, D.ch_vexp, D.vdig);
   }
   CUDA_TRY(cudaGetLastError());
-}
-
-// The FP64 ladder V (the FP64 pp ladder and operator): built once, on first use.
-void pnm_need_vpp64(pnm_ctx* ctx) {
-  if (ctx->d.v_pppp) return;
-  ctx->d.v_pppp = ctx_alloc<double>(ctx, std::max<long>(ctx->nvpp, 1));
-  pnm_ladder_v(ctx, ctx->d.v_pppp, nullptr);
-}
-
-// The FP32-pair ladder V (the refinement sweeps' pp ladder, and the source of the tensor-core
-// ladder's BF16 tiles, whose split starts from the same FP32 rounding): built once.
-void pnm_need_vpp_f2(pnm_ctx* ctx) {
-  if (ctx->vpp_f2) return;
-  ctx->vpp_f2 = ctx_alloc<f2>(ctx, std::max<long>(ctx->nvpp, 1));
-  pnm_ladder_v(ctx, nullptr, ctx->vpp_f2);
 }
 
 void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const double* rhos,
@@ -1128,7 +1123,9 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   D.ch_pp_off = dalloc<int>(C, ctx->owned, s);
   D.ch_vpp = dalloc<int>(C, ctx->owned, s);
   D.ch_t_off = dalloc<long>(C, ctx->owned, s);
-  D.ch_vpp_off = dalloc<long>(C, ctx->owned, s);  // ladder V blocks, set once the basis is known
+  D.ch_vd_off = dalloc<long>(C, ctx->owned, s);  // ladder V blocks, set once the basis is known
+  D.ch_td_off = dalloc<long>(C, ctx->owned, s);
+  D.ch_vexp = dalloc<int>(C, ctx->owned, s);
   D.ch_nlad = dalloc<int>(C, ctx->owned, s);
   D.ch_s_off = dalloc<long>(C, ctx->owned, s);
   D.ch_vhh_off = dalloc<long>(C, ctx->owned, s);
@@ -1147,6 +1144,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
     for (int k = 0; k < nsys; k++)
       for (int x = ctx->sys[k].x_begin; x < ctx->sys[k].x_end; x++) h_x_sys[x] = k;
     h2d(D.x_sys, h_x_sys, s);
+    ctx->h_x_sys = h_x_sys;
   }
   h2d(D.ch_key, h_key, s);
   h2d(D.ch_nhh, h_nhh, s);
@@ -1187,6 +1185,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   D.x_v1 = dalloc<double>(xc_acc, ctx->owned, s);
   D.x_w = dalloc<double>(xt_acc, ctx->owned, s);
   D.t0 = dalloc<double>(t_acc, ctx->owned, s);
+  CUDA_TRY(cudaMemsetAsync(D.t0, 0, sizeof(double) * std::max<long>(t_acc, 1), s));  // held amplitudes of a new context
   D.t1 = dalloc<double>(t_acc, ctx->owned, s);
   D.chi_hh = dalloc<double>(vhh_acc, ctx->owned, s);
   D.sab = dalloc<double>(pp_acc, ctx->owned, s);
@@ -1292,31 +1291,34 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   std::vector<int> h_nlad = d2h(D.ch_nlad, C, s);
   if (d2h(flip_err, 1, s)[0]) throw PnmError{PNM_EINVAL, "spin-flip tables not closed (reference not spin saturated)"};
   ctx->h_x_cls = d2h(D.x_cls, NX, s);
-  std::vector<long> h_s_off(C, 0), h_vl_off(C, -1);
-  long s_acc = 0, vl_acc = 0;
+  std::vector<long> h_s_off(C, 0), h_vd_off(C, -1), h_td_off(C, 0);
+  long s_acc = 0, vd_acc = 0, td_acc = 0;
   int max_nlad = 0;
   std::vector<int2> vl_items;
   for (int c = 0; c < C; c++) {
     h_s_off[c] = s_acc;
     if (!h_vpp[c]) continue;
-    h_vl_off[c] = vl_acc;
+    h_vd_off[c] = vd_acc;
+    h_td_off[c] = td_acc;
+    const long wide = (h_nlad[c] + 15) / 16 * 16;  // rows and columns padded to the tiles of the products
     s_acc += (long)h_nhh[c] * h_nlad[c];
-    vl_acc += (long)h_nlad[c] * h_nlad[c];
+    vd_acc += wide * wide;
+    td_acc += 2 * h_nhh[c] * wide;  // FP16 digits: 16 bytes per element
     max_nlad = std::max(max_nlad, h_nlad[c]);
     for (int r0 = 0; r0 < h_nlad[c]; r0 += VLAD_ROWS) vl_items.push_back(make_int2(c, r0));
   }
   ctx->h_nlad = h_nlad;
   ctx->h_s_off = h_s_off;
-  ctx->h_vl_off = h_vl_off;
+  ctx->h_vd_off = h_vd_off;
   ctx->ns = s_acc;
-  ctx->nvpp = vl_acc;
+  ctx->nvdig = vd_acc;
   h2d(D.ch_s_off, h_s_off, s);
-  h2d(D.ch_vpp_off, h_vl_off, s);
-  D.v_pppp = nullptr;  // the ladder V is built on first use, in the representation a path needs
+  h2d(D.ch_vd_off, h_vd_off, s);
+  h2d(D.ch_td_off, h_td_off, s);
+  D.vdig = nullptr;  // the ladder V is built on first use
   D.rpp = dalloc<double>(s_acc, ctx->owned, s);
-  D.s64 = dalloc<double>(s_acc, ctx->owned, s);
-  // work list of the ladder V (one launch per system: the LUT differs per system), kept for
-  // pnm_ladder_v
+  ctx->ntdig = td_acc;
+  // work list of the ladder V (one launch per system: the LUT differs per system)
   ctx->vl_sys.assign(nsys + 1, 0);
   if (!vl_items.empty()) {
     int max_lut = 0;

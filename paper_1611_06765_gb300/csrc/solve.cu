@@ -206,7 +206,7 @@ int pnm_solve(pnm_ctx* ctx, const pnm_solve_opts& o, double* dE, int* iters, dou
   // refinement sweeps on the FP64 pipe); FP32-pair refinement has its own schedule slot
   const bool fp64_ladder = !mixed || (o.refine_sweeps > 0 && !pair_refine);
   if (fp64_ladder) {
-    pnm_need_vpp64(ctx);
+    pnm_need_digits(ctx);
     pnm_tune_schedule(ctx, PNM_PREC_FP64, o.mix_alpha);
   }
   if (pair_refine) pnm_tune_schedule(ctx, PNM_PREC_FP64 | (1 << 8), o.mix_alpha);
