@@ -177,10 +177,10 @@ __global__ void __launch_bounds__(PP_THREADS, 1) k_pp_tc(const __grid_constant__
   unsigned char* stage0 = smem + 1024;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __shared__ int err;
-  // items of converged systems are skipped by all three roles alike (the flags do not change
-  // during a launch)
+  // items of converged systems are skipped by all three roles alike, and all of them once the loop
+  // has ended (the flags do not change during a launch)
   const bool skip = ctl->skip_done != 0;
-  const int i_begin = cta_off[blockIdx.x], i_end = cta_off[blockIdx.x + 1];
+  const int i_begin = cta_off[blockIdx.x], i_end = skip && ctl->status != 0 ? i_begin : cta_off[blockIdx.x + 1];
 
   if (threadIdx.x == 0) {
     err = 0;

@@ -180,6 +180,7 @@ void pnm_mbpt2_all(pnm_ctx* ctx, double* out);
 int pnm_solve(pnm_ctx* ctx, const pnm_solve_opts& o, double* dE, int* iters, double* resid);
 void pnm_free_mixed(pnm_ctx* ctx);
 void pnm_enqueue_body(pnm_ctx* ctx, int mode, int use_cond, cudaGraphConditionalHandle h);
+void pnm_enqueue_loop_body(pnm_ctx* ctx, int mode, bool refine, cudaGraphConditionalHandle h);
 void pnm_prepare_terms(pnm_ctx* ctx, int terms);
 void pnm_mbpt3_all(pnm_ctx* ctx, double* out);
 // The pp ladder from its ladder layout (planes summed) into host memory in the amplitude layout.

@@ -172,11 +172,11 @@ struct SysCtl {
 constexpr int PNM_DIVERGE_STEPS = 6;
 
 // True inside the solve loop once system `sys` has met its stopping rule (its amplitudes are
-// frozen): the contraction kernels of later steps skip its work, and the update skips it too
+// frozen) or the loop has ended: the contraction kernels of later steps skip its work, and the update skips it too
 // from the second step on (the first one copies the amplitudes into the other buffer, after
 // which both buffers hold them).
 __device__ __forceinline__ bool sys_done(const DevState& D, const LoopCtl* ctl, int sys) {
-  return ctl->skip_done != 0 && D.sysctl != nullptr && D.sysctl[sys].done != 0;
+  return ctl->skip_done != 0 && (ctl->status != 0 || (D.sysctl != nullptr && D.sysctl[sys].done != 0));
 }
 __device__ __forceinline__ bool sys_settled(const SysCtl& S, const LoopCtl* ctl) {
   return ctl->skip_done != 0 && S.done != 0 && ctl->iter >= S.frozen_at + 2;

@@ -80,7 +80,7 @@ struct SolveGraphBuilder {
     CUDA_TRY(cudaStreamEndCapture(s, &out));
     deps = next;
   }
-  void loop(int mode, cudaGraphConditionalHandle h) {
+  void loop(int mode, bool refine, cudaGraphConditionalHandle h) {
     cudaGraphNodeParams cp = {};
     cp.type = cudaGraphNodeTypeConditional;
     cp.conditional.handle = h;
@@ -91,7 +91,7 @@ struct SolveGraphBuilder {
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     CUDA_TRY(cudaStreamBeginCaptureToGraph(ctx->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     try {
-      pnm_enqueue_body(ctx, mode, 1, h);
+      pnm_enqueue_loop_body(ctx, mode, refine, h);
     } catch (...) {
       cudaGraph_t dummy;
       cudaStreamEndCapture(ctx->stream, &dummy);
@@ -128,13 +128,13 @@ static cudaGraphExec_t solve_graph(pnm_ctx* ctx, bool mixed, bool refine, bool p
       pnm_prepare_terms(ctx, terms);
       pnm_loop_begin(ctx, mode1);
     });
-    b.loop(mode1, h1);
+    b.loop(mode1, false, h1);
     b.segment([&] {
       if (mixed) pnm_flip_copy_device(ctx);
       CUDA_TRY(cudaEventRecordWithFlags(ctx->ev[1], s, cudaEventRecordExternal));
       if (refine) pnm_refine_gate(ctx, h2);
     });
-    if (refine) b.loop(PNM_PREC_FP64 | (pair ? 1 << 8 : 0), h2);
+    if (refine) b.loop(PNM_PREC_FP64 | (pair ? 1 << 8 : 0), true, h2);
     b.segment([&] {
       CUDA_TRY(cudaEventRecordWithFlags(ctx->ev[2], s, cudaEventRecordExternal));
       // the control blocks as the loops left them, then t0 = the latest amplitudes
