@@ -151,1016 +151,6 @@ __global__ void k_dchi(DevState D, int nsp_total) {
   }
 }
 
-// ----------------------------------------------------------------------------- ph term
-// Global spin flip: Q is formed for the cross channels with S_z > 0 and for the spin-up rows of
-// the S_z = 0 channels; the update reads every other position at its flip (same value for
-// flip-symmetric amplitudes; qmap holds the formed positions only).  In an
-// S_z = 0 channel, with rows ordered (spin-up rows u, their flips F u) and columns alike,
-// every matrix of the term has the block form [[A, B], [B, A]] (A = M[u][v], B = M[u][F v]);
-// products of such matrices are formed from the half-size sums A + B and differences A - B,
-//   (A_1 + B_1)(A_2 + B_2) = A_3 + B_3,  (A_1 - B_1)(A_2 - B_2) = A_3 - B_3,
-// which is a quarter of the flops of the full channel.
-template <typename T_, int TS>
-struct VecT;
-template <>
-struct VecT<float, 2> {
-  __device__ __forceinline__ static void ld(const float* p, float (&v)[2]) {
-    float2 a = *reinterpret_cast<const float2*>(p);
-    v[0] = a.x; v[1] = a.y;
-  }
-};
-template <>
-struct VecT<float, 4> {
-  __device__ __forceinline__ static void ld(const float* p, float (&v)[4]) {
-    float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-  }
-};
-// Bytes reserved for the index tables at the start of a k_ph CTA's shared memory (R4 + 2 H4
-// ints are used; 2 (R4 + H4) with R4, H4 even keeps the reservation a multiple of 16 bytes).
-__host__ __device__ __forceinline__ size_t ph_index_bytes(int R4, int H4) { return sizeof(int) * 2 * (size_t)(R4 + H4); }
-
-// One CTA (NT threads) per cross channel.  NM = 1: a channel with S_z > 0.  NM = 2: an S_z = 0
-// channel as the pair (sum, difference) of half-size problems, Q written on its spin-up rows.
-// Per problem, in shared memory zero-padded to multiples of TS (R rows (a,i), H columns (k,c)):
-//   Ts = T (R x H), Xt = W^T staged as W (R x H), then T^T (H x R), Cs = C (H x H);
-//   C[(k,c)][(j,b)] = <kb|v|cj> + 1/2 sum_(e,l) <kl|v|ce> t_lj^eb
-//   Q[(a,i)][(j,b)] = sum_(k,c) t_ik^ac C[(k,c)][(j,b)]
-// Each thread accumulates TS x TS outputs of every problem per tile.  Element arithmetic is
-// that of Arith<T_> (FP64, FP32, or FP32 pairs with FP64 results).
-template <typename T_, int NT, int TS, int NM>
-__device__ __forceinline__ void ph_block(const DevState& D, int x, unsigned char* smraw,
-                                         const T_* __restrict__ xt, const T_* __restrict__ xw,
-                                         const T_* __restrict__ xv1, typename Arith<T_>::Out* __restrict__ xq) {
-  using A = Arith<T_>;
-  const int nph = D.x_nph[x], nhp = D.x_nhp[x];
-  const int R = NM == 2 ? nph >> 1 : nph, H = NM == 2 ? nhp >> 1 : nhp;
-  // padded to multiples of the register tile (zeros): the padding costs FMAs in the tiles
-  const int R4 = (R + TS - 1) & ~(TS - 1), H4 = (H + TS - 1) & ~(TS - 1);
-  const int RH = R4 * H4, HH = H4 * H4;
-  // NM = 2: index tables in shared memory first (no chains of dependent global loads below):
-  // sra[u] = spin-up row, sca[v] = spin-up column, scb[v] = its flip
-  int* sra = reinterpret_cast<int*>(smraw);
-  int* sca = sra + R4;
-  int* scb = sca + H4;
-  T_* Ts = reinterpret_cast<T_*>(smraw + ph_index_bytes(R4, H4));
-  T_* Xt = Ts + NM * RH;
-  T_* Cs = Xt + NM * RH;
-  const long to = D.x_t_off[x], wo = D.x_w_off[x], co = D.x_c_off[x];
-  if constexpr (NM == 2) {
-    const int* __restrict__ fcol = D.x_fcol + D.x_hp_off[x];
-    const int* __restrict__ rrow = D.x_rrow + D.x_ph_off[x];
-    const int* __restrict__ rcol = D.x_rcol + D.x_hp_off[x];
-    for (int k = threadIdx.x; k < R4; k += NT) sra[k] = k < R ? rrow[k] : 0;
-    for (int k = threadIdx.x; k < H4; k += NT) {
-      int a = k < H ? rcol[k] : 0;
-      sca[k] = a;
-      scb[k] = k < H ? fcol[a] : 0;
-    }
-    __syncthreads();
-  }
-  // element e = u H4 + s of the staging loops: (u, s) advanced by NT per step without a division
-  const int du = NT / H4, ds = NT % H4;
-  int u = threadIdx.x / H4, s = threadIdx.x % H4;
-#pragma unroll 4
-  for (int e = threadIdx.x; e < RH; e += NT) {
-    T_ t0 = A::zero(), t1 = A::zero(), w0 = A::zero(), w1 = A::zero();
-    if (u < R && s < H) {
-      if constexpr (NM == 1) {
-        long o = (long)u * nhp + s;
-        t0 = xt[to + o];
-        w0 = xw[wo + o];
-      } else {
-        int row = sra[u], ca = sca[s], cb = scb[s];
-        long oa = (long)row * nhp + ca, ob = (long)row * nhp + cb;
-        T_ ta = xt[to + oa], tb = xt[to + ob];
-        t0 = A::add(ta, tb);
-        t1 = A::sub(ta, tb);
-        T_ wa = xw[wo + oa], wb = xw[wo + ob];
-        w0 = A::add(wa, wb);
-        w1 = A::sub(wa, wb);
-      }
-    }
-    Ts[e] = t0;
-    Xt[e] = w0;
-    if constexpr (NM == 2) {
-      Ts[RH + e] = t1;
-      Xt[RH + e] = w1;
-    }
-    u += du;
-    s += ds;
-    if (s >= H4) {
-      s -= H4;
-      u++;
-    }
-  }
-  int r = threadIdx.x / H4, c = threadIdx.x % H4;
-#pragma unroll 4
-  for (int e = threadIdx.x; e < HH; e += NT) {
-    T_ v0 = A::zero(), v1 = A::zero();
-    if (r < H && c < H) {
-      if constexpr (NM == 1) {
-        v0 = xv1[co + (long)r * nhp + c];
-      } else {
-        const long ra = co + (long)sca[r] * nhp;
-        T_ va = xv1[ra + sca[c]], vb = xv1[ra + scb[c]];
-        v0 = A::add(va, vb);
-        v1 = A::sub(va, vb);
-      }
-    }
-    Cs[e] = v0;
-    if constexpr (NM == 2) Cs[HH + e] = v1;
-    r += du;
-    c += ds;
-    if (c >= H4) {
-      c -= H4;
-      r++;
-    }
-  }
-  __syncthreads();
-  const int th = H4 / TS;
-  {
-    // C += 1/2 W^T T (padded rows and columns stay zero)
-    for (int tile = threadIdx.x; tile < NM * th * th; tile += NT) {
-      const int mtx = tile / (th * th), tt = tile % (th * th);
-      const int r0 = (tt / th) * TS, s0 = (tt % th) * TS;
-      const T_* X = Xt + mtx * RH;
-      const T_* Tm = Ts + mtx * RH;
-      T_ acc[TS][TS];
-#pragma unroll
-      for (int i = 0; i < TS; i++)
-#pragma unroll
-        for (int j = 0; j < TS; j++) acc[i][j] = A::zero();
-      for (int u = 0; u < R; u++) {
-        T_ a[TS], b[TS];
-        VecT<T_, TS>::ld(X + u * H4 + r0, a);
-        VecT<T_, TS>::ld(Tm + u * H4 + s0, b);
-#pragma unroll
-        for (int i = 0; i < TS; i++)
-#pragma unroll
-          for (int j = 0; j < TS; j++) A::mac(acc[i][j], a[i], b[j]);
-      }
-      T_* Cm = Cs + mtx * HH;
-#pragma unroll
-      for (int i = 0; i < TS; i++)
-#pragma unroll
-        for (int j = 0; j < TS; j++) {
-          T_& cv = Cm[(r0 + i) * H4 + s0 + j];
-          cv = A::add(cv, A::half(acc[i][j]));
-        }
-    }
-    __syncthreads();
-  }
-  // T transposed into Xt: Xt[s][u] = T[u][s]
-  for (int e = threadIdx.x; e < NM * RH; e += NT) {
-    const int mtx = e / RH, f = e % RH;
-    Xt[mtx * RH + (f % H4) * R4 + f / H4] = Ts[e];
-  }
-  __syncthreads();
-  const int tr = R4 / TS;
-  for (int tile = threadIdx.x; tile < tr * th; tile += NT) {
-    const int r0 = (tile / th) * TS, s0 = (tile % th) * TS;
-    T_ acc[NM][TS][TS];
-#pragma unroll
-    for (int m = 0; m < NM; m++)
-#pragma unroll
-      for (int i = 0; i < TS; i++)
-#pragma unroll
-        for (int j = 0; j < TS; j++) acc[m][i][j] = A::zero();
-    for (int u = 0; u < H; u++) {
-#pragma unroll
-      for (int mtx = 0; mtx < NM; mtx++) {
-        T_ a[TS], b[TS];
-        VecT<T_, TS>::ld(Xt + mtx * RH + u * R4 + r0, a);
-        VecT<T_, TS>::ld(Cs + mtx * HH + u * H4 + s0, b);
-#pragma unroll
-        for (int i = 0; i < TS; i++)
-#pragma unroll
-          for (int j = 0; j < TS; j++) A::mac(acc[mtx][i][j], a[i], b[j]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < TS; i++) {
-      const int r = r0 + i;
-      if (r >= R) continue;
-      if constexpr (NM == 1) {
-        const long qr = to + (long)r * nhp;
-#pragma unroll
-        for (int j = 0; j < TS; j++)
-          if (s0 + j < H) xq[qr + s0 + j] = A::out(acc[0][i][j]);
-      } else {
-        // the spin-up row's two blocks; the flipped rows are never read (see qpos)
-        const long qa = to + (long)sra[r] * nhp;
-#pragma unroll
-        for (int j = 0; j < TS; j++) {
-          const int s = s0 + j;
-          if (s < H) {
-            xq[qa + sca[s]] = A::out(A::half(A::add(acc[0][i][j], acc[1][i][j])));
-            xq[qa + scb[s]] = A::out(A::half(A::sub(acc[0][i][j], acc[1][i][j])));
-          }
-        }
-      }
-    }
-  }
-}
-
-// Cross channels of at most PH_WARP_DIM rows and columns (of their halves for S_z = 0): one
-// warp per channel with its own shared buffers (stride PH_WARP_DIM), no block-wide
-// synchronisation; the same two bodies as the CTA path, one output element per lane and step.
-constexpr int PH_WARPS = PH_THREADS / 32;
-template <typename T_>
-__device__ __forceinline__ void ph_warp_body(const DevState& D, int x, int w, int lane, unsigned char* smraw,
-                                             const T_* __restrict__ xt, const T_* __restrict__ xw,
-                                             const T_* __restrict__ xv1, typename Arith<T_>::Out* __restrict__ xq) {
-  using A = Arith<T_>;
-  constexpr int S = PH_WARP_DIM;
-  const int nph = D.x_nph[x], nhp = D.x_nhp[x];
-  const bool two = D.x_cls[x] == 0;
-  const int nm = two ? 2 : 1;
-  const int R = two ? nph >> 1 : nph, H = two ? nhp >> 1 : nhp;
-  const long to = D.x_t_off[x], wo = D.x_w_off[x], co = D.x_c_off[x];
-  T_* Ts = reinterpret_cast<T_*>(smraw) + (size_t)w * 6 * S * S;  // [m][u][s]
-  T_* Ws = Ts + 2 * S * S;                                         // [m][u][r] = W[u][r]
-  T_* Cs = Ws + 2 * S * S;                                         // [m][r][s]
-  int* sra = reinterpret_cast<int*>(reinterpret_cast<T_*>(smraw) + (size_t)PH_WARPS * 6 * S * S) + w * 3 * S;
-  int* sca = sra + S;
-  int* scb = sca + S;
-  if (two) {
-    const int* __restrict__ fcol = D.x_fcol + D.x_hp_off[x];
-    const int* __restrict__ rrow = D.x_rrow + D.x_ph_off[x];
-    const int* __restrict__ rcol = D.x_rcol + D.x_hp_off[x];
-    if (lane < R) sra[lane] = rrow[lane];
-    if (lane < H) {
-      int a = rcol[lane];
-      sca[lane] = a;
-      scb[lane] = fcol[a];
-    }
-  }
-  __syncwarp();
-  for (int e = lane; e < R * H; e += 32) {
-    int u = e / H, c = e % H;
-    if (two) {
-      long oa = (long)sra[u] * nhp + sca[c], ob = (long)sra[u] * nhp + scb[c];
-      T_ ta = xt[to + oa], tb = xt[to + ob];
-      Ts[u * S + c] = A::add(ta, tb);
-      Ts[S * S + u * S + c] = A::sub(ta, tb);
-      T_ wa = xw[wo + oa], wb = xw[wo + ob];
-      Ws[u * S + c] = A::add(wa, wb);
-      Ws[S * S + u * S + c] = A::sub(wa, wb);
-    } else {
-      long o = (long)u * nhp + c;
-      Ts[u * S + c] = xt[to + o];
-      Ws[u * S + c] = xw[wo + o];
-    }
-  }
-  __syncwarp();
-  for (int e = lane; e < H * H; e += 32) {
-    int r = e / H, c = e % H;
-    for (int m = 0; m < nm; m++) {
-      T_ v;
-      if (two) {
-        const long ra = co + (long)sca[r] * nhp;
-        T_ va = xv1[ra + sca[c]], vb = xv1[ra + scb[c]];
-        v = m == 0 ? A::add(va, vb) : A::sub(va, vb);
-      } else {
-        v = xv1[co + (long)r * nhp + c];
-      }
-      T_ acc = A::zero();
-      for (int u = 0; u < R; u++) A::mac(acc, Ws[m * S * S + u * S + r], Ts[m * S * S + u * S + c]);
-      Cs[m * S * S + r * S + c] = A::add(v, A::half(acc));
-    }
-  }
-  __syncwarp();
-  for (int e = lane; e < R * H; e += 32) {
-    int r = e / H, c = e % H;
-    T_ acc[2] = {A::zero(), A::zero()};
-    for (int m = 0; m < nm; m++)
-      for (int u = 0; u < H; u++) A::mac(acc[m], Ts[m * S * S + r * S + u], Cs[m * S * S + u * S + c]);
-    if (two) {
-      const long qa = to + (long)sra[r] * nhp;
-      xq[qa + sca[c]] = A::out(A::half(A::add(acc[0], acc[1])));
-      xq[qa + scb[c]] = A::out(A::half(A::sub(acc[0], acc[1])));
-    } else {
-      xq[to + (long)r * nhp + c] = A::out(acc[0]);
-    }
-  }
-}
-
-// The ph term over the S_z >= 0 cross channels (xlist): the first nblk CTAs take one channel
-// each (the costliest first), with the S_z > 0 or the S_z = 0 body chosen per channel; the
-// remaining CTAs take PH_WARPS small channels each, one per warp.  (FP32, the mixed iteration.)
-template <typename T_, int NT, int TS>
-__global__ void __launch_bounds__(NT) k_ph(DevState D, const LoopCtl* __restrict__ ctl,
-                                           const int* __restrict__ xlist, int nblk, int nwarp,
-                                           const T_* __restrict__ xt, const T_* __restrict__ xw,
-                                           const T_* __restrict__ xv1, typename Arith<T_>::Out* __restrict__ xq) {
-  static_assert(NT == PH_WARPS * 32, "one warp per small channel");
-  extern __shared__ __align__(16) unsigned char smraw[];
-  if ((int)blockIdx.x < nblk) {
-    const int x = xlist[blockIdx.x];
-    if (sys_done(D, ctl, D.x_sys[x])) return;  // CTA-uniform
-    if (D.x_cls[x] == 0)
-      ph_block<T_, NT, TS, 2>(D, x, smraw, xt, xw, xv1, xq);
-    else
-      ph_block<T_, NT, TS, 1>(D, x, smraw, xt, xw, xv1, xq);
-    return;
-  }
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int idx = ((int)blockIdx.x - nblk) * PH_WARPS + w;
-  if (idx >= nwarp) return;  // whole warps leave; the warp path never synchronises the block
-  const int x = xlist[nblk + idx];
-  if (sys_done(D, ctl, D.x_sys[x])) return;  // warp-uniform
-  ph_warp_body<T_>(D, x, w, lane, smraw, xt, xw, xv1, xq);
-}
-
-static size_t ph_warp_smem(size_t elem) {
-  return (size_t)PH_WARPS * (6 * PH_WARP_DIM * PH_WARP_DIM * elem + 3 * PH_WARP_DIM * sizeof(int));
-}
-
-// Shared memory of a k_ph CTA for channels of at most max_dim (NM = 1) or 2 max_dim (NM = 2)
-// rows and columns: the index tables, then NM problems of Ts, Xt (R x H) and Cs (H x H).
-size_t ph_smem_bytes(int max_dim, int nm, size_t elem) {
-  int m4 = (max_dim + 3) & ~3;
-  return ph_index_bytes(m4, m4) + elem * 3 * (size_t)nm * m4 * m4;
-}
-
-static size_t ph32_smem(const pnm_ctx* ctx) {
-  const size_t b = std::max(std::max(ctx->ph_smem32, ctx->ph_mid_smem32), ctx->ph_big_smem32);
-  return ctx->n_ph_warp > 0 ? std::max(b, ph_warp_smem(sizeof(float))) : b;
-}
-
-// Register tile of the FP32 ph kernel (4 x 4: few shared-memory loads per FMA).
-#ifndef PNM_PH32_TILE
-#define PNM_PH32_TILE 4
-#endif
-
-// Mixed ph: T read from the FP32 cross-channel copy the update scatters, Q in FP32 at its
-// cross-channel positions (the update gathers the four terms of each amplitude).
-void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* xv1, float* xq, cudaStream_t s) {
-  // one launch over the S_z >= 0 cross channels, the costliest first (limited by registers)
-  const int nwb = (ctx->n_ph_warp + PH_WARPS - 1) / PH_WARPS;
-  const int nblk = ctx->n_ph_big + ctx->n_ph_mid + ctx->n_ph;
-  if (nblk + nwb > 0)
-    k_ph<float, PH_THREADS, PNM_PH32_TILE><<<nblk + nwb, PH_THREADS, ph32_smem(ctx), s>>>(
-        ctx->d, ctx->ctl, ctx->ph_list, nblk, ctx->n_ph_warp, xt, xw, xv1, xq);
-}
-
-// ------------------------------------------------------------- ph term, FP64 accuracy (digits)
-// The FP64 and FP32-pair ph term as digit products on the tensor cores (dig.cuh), mma.sync because
-// the matrices are small (N = 66: 17 to 33 rows and columns): per problem (a S_z > 0 channel, or
-// the sum and the difference problem of an S_z = 0 channel)
-//   C[(k,c)][(j,b)] = <kb|v|cj> + 1/2 sum_(e,l) <kl|v|ce> t_lj^eb,   Q[(a,i)][(j,b)] = T C.
-// Operands are integers and their digits from end to end:
-//   - the amplitudes as digit words of one exponent per system (k_tmax, k_twords: two passes over
-//     them per update, where converting at the gather repeated the work for each of the three or
-//     four places of an amplitude and cost two more passes over shared memory);
-//   - W as digits in fragment order, <kb|v|cj> as integers, and the signed amplitude index of every
-//     staged element, fixed per context (k_ph_pack; sums and differences of S_z = 0 formed there);
-//   - T staged as words (sums and differences of S_z = 0 as exact integer sums), two neighbouring
-//     columns interleaved: the k index of the second product; the first reads its k pairs across
-//     rows;
-//   - C as integers, the two terms aligned to the coarser of their units (2^-60 of their bounds or
-//     finer), its digits stored interleaved by row pairs straight from the first product's registers.
-// Only the results leave as floating point.  A group of 32 threads (channels of at most PH_WARP_DIM
-// rows and columns) or of 128 (the others) takes a channel; a warp forms 16 x 8 blocks.
-// What bounds it: instruction issue and its latencies around the products (operand expansion,
-// drains, staging) at twelve warps per SM; without the MMAs it takes 6% less time.  Per launch with
-// the two passes over the amplitudes: N = 66, n^2 <= 42, FP64 149 us against 405 us on the FP64
-// pipe; three densities of N = 66, n^2 <= 36, pairs, 290 against 356 us on the FP32 pipe; symmetric
-// matter, 28 nucleons, n^2 <= 20, FP64 50 against 52 us launched one by one, and shorter beside the
-// ladder in a captured update (no FP64 pipe work to share).
-struct __align__(16) PhItem {
-  int x, sys;                    // cross channel, its system
-  unsigned short R, H, nm, nhp;  // rows, columns of a problem; problems (1: S_z > 0, 2: S_z = 0); channel columns
-  int po, ho;                    // pair offsets
-  // offsets: Q, source indices, W fragments (uint4), <kb|v|cj>, and of the smallest channels W and
-  // <kb|v|cj> as element values
-  unsigned to, src, wf, v1, fx, pad;
-};
-
-__host__ __device__ __forceinline__ int ph_h8(int H) { return (H + 7) & ~7; }
-// Row strides in 16-byte pairs: T's odd, C's 2 modulo 8, so that the fragment loads of the first
-// product (two rows per thread) and of the second spread over the banks.
-__host__ __device__ __forceinline__ int ph_ts(int H) { return ph_h8(H) / 2 + 1; }
-__host__ __device__ __forceinline__ int ph_cs(int H) { return ph_h8(H) + 2; }
-__host__ __device__ __forceinline__ size_t ph_dig_smem(int R, int H, int nm) {
-  return sizeof(uint4) * nm * ((size_t)ph_h8(R) * ph_ts(H) + (size_t)(ph_h8(H) / 2) * ph_cs(H)) +
-         sizeof(int) * ((size_t)ph_h8(R) + 2 * ph_h8(H));
-}
-
-template <int GT>
-__device__ __forceinline__ void group_sync() {
-  if constexpr (GT == 32) __syncwarp();
-  else __syncthreads();
-}
-
-// The term of one channel in FP64 arithmetic (infinities, NaN, or values so large that intermediate
-// results might overflow): the sums of the same expressions in order.
-template <typename Out, int GT>
-__device__ __noinline__ void ph_values(const DevState& D, const PhItem& it, int tid, uint4* Ts, uint4* Cs,
-                                       const int* sra, const int* sca, const int* scb, const double* __restrict__ t,
-                                       const int* __restrict__ src, bool quad, Out* __restrict__ xq) {
-  const int R = it.R, H = it.H, nm = it.nm, H8 = ph_h8(H), TS = ph_ts(H), CS = ph_cs(H);
-  const long TP = (long)ph_h8(R) * TS, CP = (long)(H8 / 2) * CS;
-  auto T = [&](int m, int u, int s) -> double& { return reinterpret_cast<double*>(Ts + m * TP + u * TS + (s >> 1))[s & 1]; };
-  auto C = [&](int m, int r, int c) -> double& { return reinterpret_cast<double*>(Cs + m * CP + (r >> 1) * CS + c)[r & 1]; };
-  auto amp = [&](int c) { return c == 0 ? 0.0 : (c > 0 ? t[c - 1] : -t[-c - 1]); };
-  const double* __restrict__ W = D.x_w + D.x_w_off[it.x];
-  const double* __restrict__ V = D.x_v1 + D.x_c_off[it.x];
-  for (int e = tid; e < R * H; e += GT) {
-    const int u = e / H, s = e % H;
-    if (nm == 1) T(0, u, s) = amp(src[it.src + u * H8 + s]);
-    else {
-      const int2 k = reinterpret_cast<const int2*>(src + it.src)[u * H8 + s];
-      const double a = amp(k.x), b = amp(k.y);
-      T(0, u, s) = a + b;
-      T(1, u, s) = a - b;
-    }
-  }
-  group_sync<GT>();
-  for (int e = tid; e < nm * H * H; e += GT) {
-    const int m = e / (H * H), r = (e % (H * H)) / H, c = e % H;
-    auto pick = [&](const double* __restrict__ M, long row, int col) {  // element of problem m
-      if (nm == 1) return M[row + col];
-      const double a = M[row + sca[col]], b = M[row + scb[col]];
-      return m == 0 ? a + b : a - b;
-    };
-    double acc = 0.0;
-    for (int u = 0; u < R && quad; u++) acc += pick(W, (long)(nm == 1 ? u : sra[u]) * it.nhp, r) * T(m, u, c);
-    C(m, r, c) = pick(V, (long)(nm == 1 ? r : sca[r]) * it.nhp, c) + 0.5 * acc;
-  }
-  group_sync<GT>();
-  for (int e = tid; e < R * H; e += GT) {
-    const int r = e / H, c = e % H;
-    double acc[2] = {0.0, 0.0};
-    for (int m = 0; m < nm; m++)
-      for (int u = 0; u < H; u++) acc[m] += T(m, r, u) * C(m, u, c);
-    if (nm == 1) xq[it.to + (long)r * it.nhp + c] = Arith<Out>::from_double(acc[0]);
-    else {
-      const long q = it.to + (long)sra[r] * it.nhp;
-      xq[q + sca[c]] = Arith<Out>::from_double(0.5 * (acc[0] + acc[1]));
-      xq[q + scb[c]] = Arith<Out>::from_double(0.5 * (acc[0] - acc[1]));
-    }
-  }
-}
-
-// Largest exponent of the amplitudes plus that of W beyond which ph_values is used: C and Q stay
-// finite below.
-constexpr int PH_MAX_EXP = 2900;
-
-// ex: exponents of W and of <kb|v|cj>.
-template <typename Out, int GT, int NM>
-__device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2 ex, unsigned char* smraw,
-                                       const double* __restrict__ t, const int* __restrict__ src,
-                                       const uint4* __restrict__ wf, const long long* __restrict__ v1, bool quad,
-                                       Out* __restrict__ xq) {
-  const int tid = GT == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
-  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, wid = tid >> 5;
-  constexpr int NW = GT / 32;
-  const int R = it.R, H = it.H, R8 = ph_h8(R), H8 = ph_h8(H), TS = ph_ts(H), CS = ph_cs(H);
-  const int TP = R8 * TS, CP = (H8 / 2) * CS;
-  uint4* Ts = reinterpret_cast<uint4*>(smraw);  // [problem][row][column pair]
-  uint4* Cs = Ts + NM * TP;                     // [problem][row pair][column]
-  int* sra = reinterpret_cast<int*>(Cs + NM * CP);
-  int* sca = sra + R8;
-  int* scb = sca + H8;
-  const int et = D.sys_texp[it.sys];
-  if constexpr (NM == 2) {
-    for (int k = tid; k < R; k += GT) sra[k] = D.x_rrow[it.po + k];
-    for (int k = tid; k < H; k += GT) {
-      const int a = D.x_rcol[it.ho + k];
-      sca[k] = a;
-      scb[k] = D.x_fcol[it.ho + a];
-    }
-  }
-  if (et >= DIG_NONFINITE || ex.x >= DIG_NONFINITE || ex.y >= DIG_NONFINITE || et + ex.x > PH_MAX_EXP) {
-    group_sync<GT>();  // the tables; group-uniform branch
-    ph_values<Out, GT>(D, it, tid, Ts, Cs, sra, sca, scb, t, src, quad, xq);
-    return;
-  }
-  // T: two neighbouring columns per step (index rows are padded to H8, rows past R read none)
-  {
-    const dig_t* __restrict__ tw = D.twords;
-    auto word = [&](int c) {
-      if (c == 0) return DIG_BIAS;
-      const dig_t w = tw[c > 0 ? c - 1 : -c - 1];
-      return c < 0 ? dig_neg(w) : w;
-    };
-    const int half = H8 / 2, total = R8 * half, live = R * half, du = GT / half, ds = GT % half;
-    int u = tid / half, s = tid % half;
-#pragma unroll 4
-    for (int f = tid; f < total; f += GT) {
-      uint4* pa = Ts + u * TS + s;
-      if constexpr (NM == 1) {
-        const int2 c = f < live ? reinterpret_cast<const int2*>(src + it.src)[f] : make_int2(0, 0);
-        *pa = dig_interleave(word(c.x), word(c.y));
-      } else {
-        const int4 c = f < live ? reinterpret_cast<const int4*>(src + it.src)[f] : make_int4(0, 0, 0, 0);
-        const dig_t a0 = word(c.x), b0 = word(c.y), a1 = word(c.z), b1 = word(c.w);
-        *pa = dig_interleave(dig_sum(a0, b0), dig_sum(a1, b1));
-        pa[TP] = dig_interleave(dig_diff(a0, b0), dig_diff(a1, b1));
-      }
-      u += du;
-      s += ds;
-      if (s >= half) {
-        s -= half;
-        u++;
-      }
-    }
-  }
-  group_sync<GT>();
-  // C: 16 x 8 blocks of every problem; the fragments of W are requested one step ahead, across
-  // blocks too
-  const int nt = H8 / 8, sc = (H + 15) >> 4, kr = (R + 15) >> 4, blocks = NM * sc * nt;
-  const int p1 = dig_power(ex.x, et) + 14 - 1, pv = ex.y - 1022 - 61;  // units of the two terms (factor 1/2)
-  const int pc = quad ? max(p1, pv) : pv, sx = min(pc - p1, 63), sv = min(pc - pv, 63);
-  const bool small_r = R <= DIG_SMALL_K, small_h = H <= DIG_SMALL_K;
-  uint4 w[4];
-  auto load_w = [&](int b, int ks) {  // block b is strip b / nt of the problems' strips in turn
-    const uint4* __restrict__ wp = wf + it.wf + ((long)(b / nt) * kr + ks) * 128 + lane;
-#pragma unroll
-    for (int r = 0; r < 4; r++) w[r] = __ldg(wp + r * 32);
-  };
-  if (quad && wid < blocks) load_w(wid, 0);
-  for (int b = wid; b < blocks; b += NW) {
-    const int ms = b / nt, m = ms / sc, strip = ms - m * sc, n0 = (b - ms * nt) * 8;
-    const longlong2* __restrict__ vp =
-        reinterpret_cast<const longlong2*>(v1 + it.v1) + (((long)ms * 16 + g) * H8 + n0) / 2 + q;
-    const longlong2 va = __ldg(vp), vb = __ldg(vp + 4 * H8);
-    dig_t c[4] = {(dig_t)(va.x >> sv), (dig_t)(va.y >> sv), (dig_t)(vb.x >> sv), (dig_t)(vb.y >> sv)};
-    if (quad) {
-      float acc[DIG_LEVELS][4] = {};
-      const uint4* tb = Ts + m * TP + (2 * q) * TS + ((n0 + g) >> 1);
-      for (int ks = 0; ks < kr; ks++) {
-        uint32_t a[4][DIG_LEVELS], bb[2][DIG_LEVELS];
-        const bool half = R - ks * 16 <= 8;
-#pragma unroll
-        for (int r = 0; r < 4; r++) dig_expand<DIG_LEVELS>(w[r], a[r]);
-        if (ks + 1 < kr) load_w(b, ks + 1);
-        else if (b + NW < blocks) load_w(b + NW, 0);
-        const uint4* tk = tb + ks * 16 * TS;
-        dig_expand_across(tk[0], tk[TS], g & 1, bb[0]);
-        if (!half) dig_expand_across(tk[8 * TS], tk[9 * TS], g & 1, bb[1]);
-        dig_block(acc, a, bb, half);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const DigSum x = small_r ? dig_drain_small(acc, k) : dig_drain(acc, k);
-        c[k] += (dig_t)(((x.hi << 18) + (x.lo >> 14)) >> sx);  // 2^-54 of the maxima's product or finer
-      }
-    }
-    // digits of the row pairs (g, g ^ 1): the lanes of even g take the block's even columns
-    const bool odd = g & 1;
-    const dig_t r0 = __shfl_xor_sync(0xffffffffu, odd ? c[0] : c[1], 4);
-    const dig_t r1 = __shfl_xor_sync(0xffffffffu, odd ? c[2] : c[3], 4);
-    const dig_t o0 = odd ? c[1] : c[0], o1 = odd ? c[3] : c[2];
-    uint4* pc0 = Cs + m * CP + ((strip * 16 + g) >> 1) * CS + n0 + 2 * q + (odd ? 1 : 0);
-    if (strip * 16 + g < H8)
-      *pc0 = dig_interleave(DIG_BIAS + (odd ? r0 : o0), DIG_BIAS + (odd ? o0 : r0));
-    if (strip * 16 + g + 8 < H8)
-      pc0[4 * CS] = dig_interleave(DIG_BIAS + (odd ? r1 : o1), DIG_BIAS + (odd ? o1 : r1));
-  }
-  group_sync<GT>();
-  // Q
-  const int sr = (R + 15) >> 4, kh = (H + 15) >> 4;
-  const int p2 = 56 + (et - 1022 - 61) + pc - (NM == 2 ? 1 : 0);  // the half of sum and difference
-  for (int b = wid; b < sr * nt; b += NW) {
-    const int m0 = (b / nt) * 16, n0 = (b % nt) * 8;
-    const bool low = m0 + 8 < R;  // rows m0 + 8 ... are stored
-    DigSum x[4] = {}, x0[4];  // the last problem's sums, and those of the one before
-#pragma unroll 1
-    for (int m = 0; m < NM; m++) {
-      float acc[DIG_LEVELS][4] = {};
-      for (int ks = 0; ks < kh; ks++) {
-        uint32_t a[4][DIG_LEVELS], bb[2][DIG_LEVELS];
-        const bool half = H - ks * 16 <= 8;
-        const uint4* ta = Ts + m * TP + (m0 + g) * TS + ks * 8 + q;
-        const uint4* cb = Cs + m * CP + (ks * 8 + q) * CS + n0 + g;
-        const uint4 zero = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-        dig_expand<DIG_LEVELS>(ta[0], a[0]);
-        dig_expand<DIG_LEVELS>(low ? ta[8 * TS] : zero, a[1]);
-        dig_expand<DIG_LEVELS>(cb[0], bb[0]);
-        if (!half) {
-          dig_expand<DIG_LEVELS>(ta[4], a[2]);
-          dig_expand<DIG_LEVELS>(low ? ta[8 * TS + 4] : zero, a[3]);
-          dig_expand<DIG_LEVELS>(cb[4 * CS], bb[1]);
-        }
-        dig_block(acc, a, bb, half);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        x0[k] = x[k];
-        x[k] = small_h ? dig_drain_small(acc, k) : dig_drain(acc, k);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const int r = m0 + g + 8 * (k >> 1), c = n0 + 2 * q + (k & 1);
-      if (r >= R || c >= H) continue;
-      if constexpr (NM == 1) {
-        xq[it.to + (long)r * it.nhp + c] = dig_result<Out>(x[k], p2);
-      } else {
-        // the spin-up row's two blocks; the flipped rows are never read (see qpos)
-        const long o = it.to + (long)sra[r] * it.nhp;
-        xq[o + sca[c]] = dig_result<Out>(DigSum{x0[k].hi + x[k].hi, x0[k].lo + x[k].lo}, p2);
-        xq[o + scb[c]] = dig_result<Out>(DigSum{x0[k].hi - x[k].hi, x0[k].lo - x[k].lo}, p2);
-      }
-    }
-  }
-}
-
-// Digit words of the current amplitudes of every system, of one exponent per system.  TW_PARTS CTAs
-// per system find the largest exponents of their parts (k_tmax); k_twords reduces them (again in
-// every CTA) and converts; part 0 publishes the system's exponent.
-constexpr int TW_THREADS = 256, TW_PARTS = 512;
-__global__ void __launch_bounds__(TW_THREADS) k_tmax(DevState D, const LoopCtl* __restrict__ ctl,
-                                                     const long* __restrict__ t_lo, int* __restrict__ parts) {
-  const int sys = blockIdx.y;
-  if (sys_done(D, ctl, sys)) return;
-  const double* __restrict__ t = cur_t(D, ctl);
-  const long hi = t_lo[sys + 1];
-  int e = 1;
-#pragma unroll 4
-  for (long z = t_lo[sys] + blockIdx.x * TW_THREADS + threadIdx.x; z < hi; z += gridDim.x * TW_THREADS)
-    e = max(e, dig_exp(t[z]));
-  e = __reduce_max_sync(0xffffffffu, e);
-  __shared__ int top;
-  if (threadIdx.x == 0) top = 1;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) atomicMax(&top, e);
-  __syncthreads();
-  if (threadIdx.x == 0) parts[sys * TW_PARTS + blockIdx.x] = top;
-}
-
-__global__ void __launch_bounds__(TW_THREADS) k_twords(DevState D, const LoopCtl* __restrict__ ctl,
-                                                       const long* __restrict__ t_lo, const int* __restrict__ parts,
-                                                       int nparts) {
-  const int sys = blockIdx.y;
-  if (sys_done(D, ctl, sys)) return;
-  int e = 1;
-  for (int k = threadIdx.x & 31; k < nparts; k += 32) e = max(e, parts[sys * TW_PARTS + k]);
-  e = __reduce_max_sync(0xffffffffu, e);
-  if (blockIdx.x == 0 && threadIdx.x == 0) D.sys_texp[sys] = e;
-  if (e >= DIG_NONFINITE) return;  // the term is then formed from the FP64 values
-  const double* __restrict__ t = cur_t(D, ctl);
-  const long hi = t_lo[sys + 1];
-#pragma unroll 4
-  for (long z = t_lo[sys] + blockIdx.x * TW_THREADS + threadIdx.x; z < hi; z += gridDim.x * TW_THREADS)
-    D.twords[z] = dig_word(dig_fixed(t[z], e));
-}
-
-// Channels of at most PH_TINY_DIM (FP32-pair results) or PH_TINY_FP64 (FP64 results) rows and
-// columns per problem, one warp each, in the element arithmetic of the results, the pairs from the
-// pair copy of the amplitudes: a 7 x 7 problem would fill a fifth of a 16 x 8 x 8 block.  120 systems
-// of N = 14, all of whose channels are of this size: 695 us per launch in digits, 145 here (355 with
-// one gather loop per channel in the kernel of the larger channels, at its registers).  In FP64 the
-// line lies lower, the products then share the slow pipe: 28 nucleons, n^2 <= 20, take 94 us per
-// update with a line at 5 and 99 with one at 8; N = 14, n^2 <= 20, whose channels have up to 7 rows,
-// 34.8 and 36.0; n^2 <= 4 (up to 5 rows) 28.5, and in digits 30.
-// fixed: W [problem][row][column] then <kb|v|cj> [problem][row][column] of the channel.
-constexpr int PH_TINY_DIM = 8, PH_TINY_FP64 = 5;
-template <typename T_>
-__device__ __forceinline__ void ph_tiny(const DevState& D, const PhItem& it, T_* Ts,
-                                        const T_* __restrict__ t, const int* __restrict__ src,
-                                        const T_* __restrict__ fixed, bool quad, T_* __restrict__ xq) {
-  using A = Arith<T_>;
-  constexpr int S = PH_TINY_DIM;
-  const int lane = threadIdx.x & 31, R = it.R, H = it.H, nm = it.nm;
-  T_* Ws = Ts + 2 * S * S;  // [problem][row][column], as Ts
-  T_* Cs = Ws + 2 * S * S;
-  const T_* __restrict__ W = fixed + it.fx;
-  const T_* __restrict__ V1 = W + nm * R * H;
-  const int* __restrict__ sp = src + it.src;
-  auto read = [&](int c) {
-    if (c == 0) return A::zero();
-    const T_ v = t[c > 0 ? c - 1 : -c - 1];
-    return c < 0 ? A::neg(v) : v;
-  };
-  for (int e = lane; e < R * H; e += 32) {
-    const int u = e / H, c = e - u * H, k8 = u * ph_h8(H) + c;
-    if (nm == 2) {
-      const int2 k = reinterpret_cast<const int2*>(sp)[k8];
-      const T_ x = read(k.x), y = read(k.y);
-      Ts[u * S + c] = A::add(x, y);
-      Ts[S * S + u * S + c] = A::sub(x, y);
-      if (quad) Ws[S * S + u * S + c] = W[R * H + e];
-    } else {
-      Ts[u * S + c] = read(sp[k8]);
-    }
-    if (quad) Ws[u * S + c] = W[e];
-  }
-  __syncwarp();
-  for (int e = lane; e < nm * H * H; e += 32) {
-    const int m = e >= H * H, f = e - m * H * H, r = f / H, c = f - r * H;
-    T_ acc = A::zero();
-    for (int u = 0; u < R && quad; u++) A::mac(acc, Ws[m * S * S + u * S + r], Ts[m * S * S + u * S + c]);
-    Cs[m * S * S + r * S + c] = A::add(V1[e], A::half(acc));
-  }
-  __syncwarp();
-  for (int e = lane; e < R * H; e += 32) {
-    const int r = e / H, c = e - r * H;
-    T_ acc[2] = {A::zero(), A::zero()};
-    for (int m = 0; m < nm; m++)
-      for (int u = 0; u < H; u++) A::mac(acc[m], Ts[m * S * S + r * S + u], Cs[m * S * S + u * S + c]);
-    if (nm == 2) {
-      const long q = it.to + (long)D.x_rrow[it.po + r] * it.nhp;
-      const int ca = D.x_rcol[it.ho + c], cb = D.x_fcol[it.ho + ca];
-      xq[q + ca] = A::half(A::add(acc[0], acc[1]));
-      xq[q + cb] = A::half(A::sub(acc[0], acc[1]));
-    } else {
-      xq[it.to + (long)r * it.nhp + c] = acc[0];
-    }
-  }
-}
-
-// The first nblk CTAs take one channel each (the costliest first), the others PH_WARPS small
-// channels each, one per warp (stride warp_smem bytes of shared memory).
-template <typename Out>
-__global__ void __launch_bounds__(PH_THREADS, 3) k_ph_dig(DevState D, const LoopCtl* __restrict__ ctl,
-                                                          const PhItem* __restrict__ items, const int2* __restrict__ exps,
-                                                          int nblk, int nwarp, int warp_smem, const int* __restrict__ src,
-                                                          const uint4* __restrict__ wf, const long long* __restrict__ v1,
-                                                          int quad, Out* __restrict__ xq) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const double* __restrict__ t = cur_t(D, ctl);
-  if ((int)blockIdx.x < nblk) {
-    const PhItem it = items[blockIdx.x];
-    if (sys_done(D, ctl, it.sys)) return;  // CTA-uniform
-    const int2 ex = exps[blockIdx.x];
-    if (it.nm == 2) ph_dig<Out, PH_THREADS, 2>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq);
-    else ph_dig<Out, PH_THREADS, 1>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq);
-    return;
-  }
-  const int w = threadIdx.x >> 5, idx = ((int)blockIdx.x - nblk) * PH_WARPS + w;
-  if (idx >= nwarp) return;  // whole warps; the warp path never synchronises the block
-  const PhItem it = items[nblk + idx];
-  if (sys_done(D, ctl, it.sys)) return;
-  const int2 ex = exps[nblk + idx];
-  unsigned char* sm = smraw + (size_t)w * warp_smem;
-  if (it.nm == 2) ph_dig<Out, 32, 2>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq);
-  else ph_dig<Out, 32, 1>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq);
-}
-
-// The smallest channels, one warp each, in a kernel of their own: it needs a third of the registers.
-template <typename T_>
-__global__ void __launch_bounds__(PH_THREADS) k_ph_tiny(DevState D, const LoopCtl* __restrict__ ctl,
-                                                        const PhItem* __restrict__ items, int n,
-                                                        const int* __restrict__ src, const T_* __restrict__ fixed,
-                                                        const f2* __restrict__ tpair, int quad, T_* __restrict__ xq) {
-  __shared__ __align__(16) T_ sm[PH_WARPS][6 * PH_TINY_DIM * PH_TINY_DIM];
-  const int w = threadIdx.x >> 5, idx = blockIdx.x * PH_WARPS + w;
-  if (idx >= n) return;  // whole warps; no block barrier
-  const PhItem it = items[idx];
-  if (sys_done(D, ctl, it.sys)) return;
-  const T_* __restrict__ t;
-  if constexpr (std::is_same<T_, f2>::value) t = tpair;
-  else t = cur_t(D, ctl);
-  ph_tiny<T_>(D, it, sm[w], t, src, fixed, quad != 0, xq);
-}
-
-// The fixed operands of the items (one CTA each): source indices (rows padded to H8), <kb|v|cj> of
-// the problems as integers (padded to whole blocks) and the digits of W, with their exponents.
-__global__ void __launch_bounds__(128) k_ph_pack(DevState D, const PhItem* __restrict__ items, int2* __restrict__ exps,
-                                                 int* __restrict__ src, uint4* __restrict__ wf, long long* __restrict__ v1,
-                                                 double* __restrict__ fixed64, f2* __restrict__ fixed_f2) {
-  __shared__ int top[2];
-  const PhItem it = items[blockIdx.x];
-  const int R = it.R, H = it.H, H8 = ph_h8(H);
-  const int* __restrict__ rr = D.x_rrow + it.po;
-  const int* __restrict__ rc = D.x_rcol + it.ho;
-  const int* __restrict__ fc = D.x_fcol + it.ho;
-  const double* __restrict__ W = D.x_w + D.x_w_off[it.x];
-  const double* __restrict__ V = D.x_v1 + D.x_c_off[it.x];
-  const bool two = it.nm == 2;
-  const bool tiny = max(R, H) <= PH_TINY_DIM;  // element values too
-  auto put = [&](long o, double v) {
-    fixed64[it.fx + o] = v;
-    fixed_f2[it.fx + o] = Arith<f2>::from_double(v);
-  };
-  if (threadIdx.x < 2) top[threadIdx.x] = 1;
-  __syncthreads();
-  int e = 1;
-  for (int f = threadIdx.x; f < R * H8; f += blockDim.x) {
-    const int u = f / H8, s = f % H8, o = u * H + s;
-    if (two) {
-      int2 c = make_int2(0, 0);
-      if (s < H) {
-        const long oa = (long)rr[u] * it.nhp + rc[s], ob = (long)rr[u] * it.nhp + fc[rc[s]];
-        c = make_int2(D.xmap[it.to + oa], D.xmap[it.to + ob]);
-        e = max(e, max(dig_exp(W[oa]), dig_exp(W[ob])));
-        if (tiny) {
-          put(o, W[oa] + W[ob]);
-          put(R * H + o, W[oa] - W[ob]);
-        }
-      }
-      reinterpret_cast<int2*>(src + it.src)[f] = c;
-    } else {
-      src[it.src + f] = s < H ? D.xmap[it.to + o] : 0;
-      if (s < H) {
-        e = max(e, dig_exp(W[o]));
-        if (tiny) put(o, W[o]);
-      }
-    }
-  }
-  e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0) atomicMax(&top[0], e);
-  e = 1;
-  for (int f = threadIdx.x; f < H * H; f += blockDim.x) {
-    const int r = f / H, c = f % H;
-    if (two) {
-      const double a = V[(long)rc[r] * it.nhp + rc[c]], b = V[(long)rc[r] * it.nhp + fc[rc[c]]];
-      e = max(e, max(dig_exp(a), dig_exp(b)));
-      if (tiny) {
-        put(2 * R * H + f, a + b);
-        put(2 * R * H + H * H + f, a - b);
-      }
-    } else {
-      const double a = V[(long)r * it.nhp + c];
-      e = max(e, dig_exp(a));
-      if (tiny) put(R * H + f, a);
-    }
-  }
-  e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0) atomicMax(&top[1], e);
-  __syncthreads();
-  const int ew = top[0], ev = top[1];
-  if (threadIdx.x == 0) exps[blockIdx.x] = make_int2(ew, ev);
-  if (ew >= DIG_NONFINITE || ev >= DIG_NONFINITE) return;
-  const int sc = (H + 15) >> 4, kr = (R + 15) >> 4;
-  for (int f = threadIdx.x; f < sc * 16 * H8; f += blockDim.x) {
-    const int r = f / H8, c = f % H8;
-    long long sum = 0, dif = 0;
-    if (r < H && c < H) {
-      if (two) {
-        const long long a = dig_fixed(V[(long)rc[r] * it.nhp + rc[c]], ev);
-        const long long b = dig_fixed(V[(long)rc[r] * it.nhp + fc[rc[c]]], ev);
-        sum = a + b;
-        dif = a - b;
-      } else {
-        sum = dig_fixed(V[(long)r * it.nhp + c], ev);
-      }
-    }
-    v1[it.v1 + f] = sum;
-    if (two) v1[it.v1 + (long)sc * 16 * H8 + f] = dif;
-  }
-  // fragment order of W as the first operand: rows (k,c), columns (e,l); stored transposed in x_w
-  for (int f = threadIdx.x; f < sc * kr * 128; f += blockDim.x) {
-    const int lane = f & 31, grp = (f >> 5) & 3, ks = (f >> 7) % kr, strip = (f >> 7) / kr;
-    const int r = strip * 16 + (lane >> 2) + (grp & 1) * 8, u0 = ks * 16 + (lane & 3) * 2 + (grp >> 1) * 8;
-    long long sum[2] = {0, 0}, dif[2] = {0, 0};
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-      const int u = u0 + k;
-      if (r >= H || u >= R) continue;
-      if (two) {
-        const long o = (long)rr[u] * it.nhp;
-        const long long a = dig_fixed(W[o + rc[r]], ew), b = dig_fixed(W[o + fc[rc[r]]], ew);
-        sum[k] = a + b;
-        dif[k] = a - b;
-      } else {
-        sum[k] = dig_fixed(W[(long)u * it.nhp + r], ew);
-      }
-    }
-    wf[it.wf + f] = dig_interleave(dig_word(sum[0]), dig_word(sum[1]));
-    if (two) wf[it.wf + (long)sc * kr * 128 + f] = dig_interleave(dig_word(dif[0]), dig_word(dif[1]));
-  }
-}
-
-// Items and fixed operands of the digit ph term (once per context, on first use): the costliest
-// channels first, in ph_list's order; channels whose tiles need more than PH_DIG_SMEM bytes get a
-// launch of their own so that the others keep three CTAs per SM.
-constexpr size_t PH_DIG_SMEM = 72 * 1024;
-void pnm_need_phdig(pnm_ctx* ctx) {
-  if (ctx->ph_items) return;
-  cudaStream_t s = ctx->stream;
-  const int n = ctx->n_ph_big + ctx->n_ph_mid + ctx->n_ph, nw = ctx->n_ph_warp;
-  std::vector<PhItem> items;
-  items.reserve(n + nw);
-  long wf = 0, v1 = 0, src = 0, fixed = 0;
-  ctx->ph_warp_smem = 0;
-  ctx->n_ph_large = 0;
-  ctx->ph_large_smem = ctx->ph_dig_smem = 0;
-  auto add = [&](int x) {
-    PhItem it{};
-    it.x = x;
-    it.sys = ctx->h_x_sys[x];
-    it.nm = ctx->h_x_cls[x] == 0 ? 2 : 1;
-    it.R = ctx->h_x_nph[x] / it.nm;
-    it.H = ctx->h_x_nhp[x] / it.nm;
-    it.nhp = ctx->h_x_nhp[x];
-    it.po = ctx->h_x_ph_off[x];
-    it.ho = ctx->h_x_hp_off[x];
-    it.to = (unsigned)ctx->h_x_t_off[x];
-    it.src = (unsigned)src;
-    src += (long)it.nm * it.R * ph_h8(it.H);
-    it.wf = (unsigned)wf;
-    it.v1 = (unsigned)v1;
-    it.fx = (unsigned)fixed;
-    wf += (long)it.nm * ((it.H + 15) / 16) * ((it.R + 15) / 16) * 128;
-    v1 += (long)it.nm * ((it.H + 15) / 16) * 16 * ph_h8(it.H);
-    const bool tiny = std::max(it.R, it.H) <= PH_TINY_DIM;
-    if (tiny) fixed += (long)it.nm * it.H * (it.R + it.H);
-    items.push_back(it);
-    return ph_dig_smem(it.R, it.H, it.nm);
-  };
-  for (int part = 0; part < 2; part++)
-    for (int k = 0; k < n; k++) {
-      const int x = ctx->h_ph_list[k], nm = ctx->h_x_cls[x] == 0 ? 2 : 1;
-      if ((ph_dig_smem(ctx->h_x_nph[x] / nm, ctx->h_x_nhp[x] / nm, nm) > PH_DIG_SMEM) != (part == 0)) continue;
-      const size_t b = add(x);
-      size_t& most = part == 0 ? ctx->ph_large_smem : ctx->ph_dig_smem;
-      most = std::max(most, b);
-      if (part == 0) ctx->n_ph_large++;
-    }
-  // the warp path by decreasing dimension: the tiny channels of either result type are its end
-  std::vector<int> by_dim[PH_WARP_DIM + 1];
-  for (int k = 0; k < nw; k++) {
-    const int x = ctx->h_ph_list[n + k];
-    by_dim[std::max(ctx->h_x_nph[x], ctx->h_x_nhp[x]) / (ctx->h_x_cls[x] == 0 ? 2 : 1)].push_back(x);
-  }
-  ctx->n_ph_tiny64 = ctx->n_ph_tiny_f2 = 0;
-  for (int d = PH_WARP_DIM; d >= 0; d--) {
-    for (int x : by_dim[d]) ctx->ph_warp_smem = std::max(ctx->ph_warp_smem, (add(x) + 15) / 16 * 16);
-    if (d <= PH_TINY_FP64) ctx->n_ph_tiny64 += (int)by_dim[d].size();
-    if (d <= PH_TINY_DIM) ctx->n_ph_tiny_f2 += (int)by_dim[d].size();
-  }
-  if (std::max(std::max(wf, v1), std::max(src, fixed)) >= (1L << 32))
-    throw PnmError{PNM_EINVAL, "problem too large for 32-bit element maps"};
-  ctx->ph_dig_smem = std::max(ctx->ph_dig_smem, PH_WARPS * ctx->ph_warp_smem);
-  PhItem* d = ctx_alloc<PhItem>(ctx, items.size());
-  ctx->ph_exps = ctx_alloc<int2>(ctx, items.size());
-  ctx->ph_src = ctx_alloc<int>(ctx, src);
-  ctx->ph_wf = ctx_alloc<uint4>(ctx, wf);
-  ctx->ph_v1 = ctx_alloc<long long>(ctx, v1);
-  ctx->ph_fixed64 = ctx_alloc<double>(ctx, fixed);
-  ctx->ph_fixed_f2 = ctx_alloc<f2>(ctx, fixed);
-  if (!items.empty()) {
-    CUDA_TRY(cudaMemcpyAsync(d, items.data(), sizeof(PhItem) * items.size(), cudaMemcpyHostToDevice, s));
-    k_ph_pack<<<(unsigned)items.size(), 128, 0, s>>>(ctx->d, d, ctx->ph_exps, ctx->ph_src, ctx->ph_wf, ctx->ph_v1,
-                                                        ctx->ph_fixed64, ctx->ph_fixed_f2);
-    CUDA_TRY(cudaGetLastError());
-  }
-  const int nsys = (int)ctx->sys.size();
-  std::vector<long> lo(nsys + 1, ctx->nt);
-  long longest = 0;
-  for (int k = 0; k < nsys; k++) {
-    lo[k] = ctx->sys[k].t_begin;
-    longest = std::max(longest, ctx->sys[k].t_end - ctx->sys[k].t_begin);
-  }
-  // parts of about a thousand amplitudes
-  ctx->n_tw_parts = (int)std::max<long>(1, std::min<long>(TW_PARTS, longest / (4 * TW_THREADS)));
-  ctx->tw_lo = ctx_alloc<long>(ctx, nsys + 1);
-  ctx->tw_parts = ctx_alloc<int>(ctx, (size_t)nsys * TW_PARTS);
-  ctx->d.sys_texp = ctx_alloc<int>(ctx, nsys);
-  ctx->d.twords = ctx_alloc<unsigned long long>(ctx, ctx->nt);
-  CUDA_TRY(cudaMemcpyAsync(ctx->tw_lo, lo.data(), sizeof(long) * (nsys + 1), cudaMemcpyHostToDevice, s));
-  const size_t most = std::max(ctx->ph_large_smem, ctx->ph_dig_smem);
-  smem_at_least(k_ph_dig<double>, most);
-  smem_at_least(k_ph_dig<f2>, most);
-  ctx->ph_items = d;
-}
-
-template <typename Out>
-static void launch_ph_dig(pnm_ctx* ctx, bool linear, cudaStream_t s, cudaStream_t s_tiny) {
-  // made before any capture by the host-side callers
-  if (!ctx->ph_items) throw PnmError{PNM_EINVAL, "the ph term's operands have not been built"};
-  constexpr bool pair = std::is_same<Out, f2>::value;
-  const int nl = ctx->n_ph_large, n = ctx->n_ph_big + ctx->n_ph_mid + ctx->n_ph - nl;
-  const int ntiny = pair ? ctx->n_ph_tiny_f2 : ctx->n_ph_tiny64, nw = ctx->n_ph_warp - ntiny;
-  const int nwb = (nw + PH_WARPS - 1) / PH_WARPS, quad = linear ? 0 : 1;
-  Out* xq = reinterpret_cast<Out*>(ctx->d.xq);
-  const PhItem* items = ctx->ph_items;
-  if (nl + n + nw == 0) s_tiny = s;
-  if (nl + n + nw > 0) {
-    const dim3 grid(ctx->n_tw_parts, (unsigned)ctx->sys.size());
-    k_tmax<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts);
-    k_twords<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts, ctx->n_tw_parts);
-  }
-  if (nl > 0)
-    k_ph_dig<Out><<<nl, PH_THREADS, ctx->ph_large_smem, s>>>(ctx->d, ctx->ctl, items, ctx->ph_exps, nl, 0, 0, ctx->ph_src,
-                                                             ctx->ph_wf, ctx->ph_v1, quad, xq);
-  if (n + nwb > 0)
-    k_ph_dig<Out><<<n + nwb, PH_THREADS, ctx->ph_dig_smem, s>>>(ctx->d, ctx->ctl, items + nl, ctx->ph_exps + nl, n, nw,
-                                                                (int)ctx->ph_warp_smem, ctx->ph_src, ctx->ph_wf,
-                                                                ctx->ph_v1, quad, xq);
-  if (ntiny > 0) {
-    const Out* fixed;
-    if constexpr (pair) fixed = ctx->ph_fixed_f2;
-    else fixed = ctx->ph_fixed64;
-    k_ph_tiny<Out><<<(ntiny + PH_WARPS - 1) / PH_WARPS, PH_THREADS, 0, s_tiny>>>(
-        ctx->d, ctx->ctl, items + nl + n + nw, ntiny, ctx->ph_src, fixed, ctx->t_pair, quad, xq);
-  }
-}
-
-// FP64 ph term (linear: without the quadratic part), and the same with its results as FP32 pairs
-// in the 8-byte slots of the FP64 Q (the refinement sweeps with FP32-pair contractions).
-// s_tiny: the stream of the smallest channels, which wait for no digits (a captured update runs them
-// beside the two passes over the amplitudes; in a context without larger channels they keep s).
-void launch_ph64(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny, bool linear) {
-  launch_ph_dig<double>(ctx, linear, s, s_tiny);
-}
-void launch_ph_f2(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny) { launch_ph_dig<f2>(ctx, false, s, s_tiny); }
-
 // ------------------------------------------------------------------------ ladder basis
 // s(ij, q) = sum over the (one or two) pairs of vector q of sign * t(ij, pair) from the current
 // FP64 amplitudes, as digit words of the row's common exponent (dig.cuh), zero words in the
@@ -2339,61 +1329,16 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->sysctl = (SysCtl*)dmalloc(ctx, sizeof(SysCtl) * nsys);
   CUDA_TRY(cudaMemsetAsync(ctx->sysctl, 0, sizeof(SysCtl) * nsys, s));
   ctx->d.sysctl = ctx->sysctl;
-  // cross channels of the ph launch: S_z >= 0 (S_z < 0 ones are read at their flips), costliest first;
-  // shared memory for the largest (NM = 1: rows/columns; NM = 2: those of the halves, twice)
-  // CTA per channel in three size classes (larger than PH_SMALL_DIM: k_ph_big; larger than
-  // PH_MID_DIM; the rest), warp per channel (at most PH_WARP_DIM)
-  std::vector<int> xb, xm, xl, xw;
-  size_t ph_staged = 0;  // three 8-byte matrices of the largest channel: the size limit of a context
-  std::vector<long> xcost(ctx->nx, 0);
+  // three 8-byte matrices of the largest cross channel (of its half-size problems for S_z = 0) and
+  // index tables, in tiles of four: the size limit of a context
+  size_t ph_staged = 0;
   for (int x = 0; x < ctx->nx; x++) {
-    int c = ctx->h_x_cls[x];
-    if (c < 0) continue;
-    long ph = ctx->h_x_nph[x], hp = ctx->h_x_nhp[x];
-    int d = (int)std::max(ph, hp);
-    if (c == 0) {
-      d /= 2;
-      xcost[x] = ph * hp * hp / 4;
-    } else {
-      xcost[x] = ph * hp * hp;
-    }
-    if (d <= PH_WARP_DIM) {
-      xw.push_back(x);
-      continue;
-    }
-    int nm = c == 0 ? 2 : 1;
-    ph_staged = std::max(ph_staged, ph_smem_bytes(d, nm, sizeof(double)));
-    if (d > PH_SMALL_DIM) {
-      ctx->ph_big_smem32 = std::max(ctx->ph_big_smem32, ph_smem_bytes(d, nm, sizeof(float)));
-      xb.push_back(x);
-    } else if (d > PH_MID_DIM) {
-      ctx->ph_mid_smem32 = std::max(ctx->ph_mid_smem32, ph_smem_bytes(d, nm, sizeof(float)));
-      xm.push_back(x);
-    } else {
-      ctx->ph_smem32 = std::max(ctx->ph_smem32, ph_smem_bytes(d, nm, sizeof(float)));
-      xl.push_back(x);
-    }
+    const int nm = ctx->h_x_cls[x] == 0 ? 2 : 1, d = std::max(ctx->h_x_nph[x], ctx->h_x_nhp[x]) / nm;
+    const size_t m4 = (d + 3) & ~3;
+    if (ctx->h_x_cls[x] >= 0 && d > 16) ph_staged = std::max(ph_staged, 4 * m4 * sizeof(int) + sizeof(double) * 3 * nm * m4 * m4);
   }
-  auto costlier = [&](int a, int b) { return xcost[a] != xcost[b] ? xcost[a] > xcost[b] : a < b; };
-  std::sort(xb.begin(), xb.end(), costlier);
-  std::sort(xm.begin(), xm.end(), costlier);
-  std::sort(xl.begin(), xl.end(), costlier);
-  std::sort(xw.begin(), xw.end(), costlier);
-  ctx->n_ph_big = (int)xb.size();
-  ctx->n_ph_mid = (int)xm.size();
-  ctx->n_ph = (int)xl.size();
-  ctx->n_ph_warp = (int)xw.size();
-  // list order: big, middle, small, warp
-  xl.insert(xl.end(), xw.begin(), xw.end());
-  xl.insert(xl.begin(), xm.begin(), xm.end());
-  xl.insert(xl.begin(), xb.begin(), xb.end());
-  ctx->h_ph_list = xl;
-  ctx->ph_list = (int*)dmalloc(ctx, sizeof(int) * std::max<size_t>(1, xl.size()));
-  if (!xl.empty())
-    CUDA_TRY(cudaMemcpyAsync(ctx->ph_list, xl.data(), sizeof(int) * xl.size(), cudaMemcpyHostToDevice, s));
   if (ph_staged > 227 * 1024 || max_nlad > PP_MAX_NLAD)
     throw PnmError{PNM_EINVAL, "channel too large for the shared-memory tiles"};
-  smem_at_least(k_ph<float, PH_THREADS, PNM_PH32_TILE>, ph32_smem(ctx));
   for (int k = 0; k < 2; k++) {
     CUDA_TRY(cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking));
     CUDA_TRY(cudaEventCreateWithFlags(&ctx->ev_join[k], cudaEventDisableTiming));
@@ -2757,11 +1702,6 @@ void pnm_prepare_terms(pnm_ctx* ctx, int terms) {
 // Kernel nodes of a captured update: the ph term at the lowest priority, every other kernel at
 // the highest, so that the shorter branches (pp ladder, one-body sums) are dispatched ahead of
 // the many ph CTAs and run beside them instead of after them.
-static bool is_ph_kernel(const void* f) {
-  return f == (const void*)k_ph<float, PH_THREADS, PNM_PH32_TILE> || f == (const void*)k_ph_dig<double> ||
-         f == (const void*)k_ph_dig<f2> || f == (const void*)k_ph_tiny<double> || f == (const void*)k_ph_tiny<f2>;
-}
-
 void pnm_set_node_priorities(cudaGraph_t body) {
   int least = 0, greatest = 0;
   CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
@@ -2776,7 +1716,7 @@ void pnm_set_node_priorities(cudaGraph_t body) {
     cudaKernelNodeParams kp = {};
     CUDA_TRY(cudaGraphKernelNodeGetParams(nd, &kp));
     cudaKernelNodeAttrValue v = {};
-    v.priority = is_ph_kernel(kp.func) ? least : greatest;
+    v.priority = pnm_is_ph_kernel(kp.func) ? least : greatest;
     CUDA_TRY(cudaGraphKernelNodeSetAttribute(nd, cudaKernelNodeAttributePriority, &v));
   }
 }

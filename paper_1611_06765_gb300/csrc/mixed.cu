@@ -551,10 +551,7 @@ void pnm_prepare_mixed(pnm_ctx* ctx) {
     CUDA_TRY(cudaMemsetAsync(M->xt32, 0, sizeof(float) * std::max<long>(ctx->nxt, 1), s));
     M->xq32 = mdalloc<float>(ctx, ctx->nxt);
     M->aw = mdalloc<double>(ctx, ctx->nt);
-    if (ctx->nxt > 0)
-      k_to_float<<<(unsigned)((ctx->nxt + 255) / 256), 256, 0, s>>>(ctx->d.x_w, M->xw32, ctx->nxt);
-    if (ctx->nxc > 0)
-      k_to_float<<<(unsigned)((ctx->nxc + 255) / 256), 256, 0, s>>>(ctx->d.x_v1, M->xv132, ctx->nxc);
+    pnm_ph_pack32(ctx, M->xw32, M->xv132);
     if (M->nitems > 0) {
       std::vector<int2> li;
       int max_lut = 0;
@@ -664,7 +661,7 @@ void pnm_enqueue_body_mixed(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHand
   pnm_fork(ctx);
   if (ctx->nx > 0) {
     prof_begin(ctx, KID_PH32);
-    launch_ph_mix(ctx, M->xt32, M->xw32, M->xv132, M->xq32, s_ph);
+    launch_ph_mix(ctx, M->xt32, M->xw32, M->xv132, M->xq32, s_ph, ctx->stream);
     prof_end(ctx);
   }
   if (M->nitems > 0) {
@@ -808,7 +805,7 @@ void pnm_apply_ph(pnm_ctx* ctx, int sys, int precision, const double* t, double*
     k_to_float_cur<<<nb, 256, 0, s>>>(ctx->d, ctx->ctl, ctx->nt);
     if (ctx->nxt > 0)
       k_remap_t32<<<(unsigned)((ctx->nxt + 255) / 256), 256, 0, s>>>(ctx->d, ctx->ctl, M->xt32, ctx->nxt);
-    if (ctx->nx > 0) launch_ph_mix(ctx, M->xt32, M->xw32, M->xv132, M->xq32, s);
+    if (ctx->nx > 0) launch_ph_mix(ctx, M->xt32, M->xw32, M->xv132, M->xq32, s, s);
     k_ph_assemble<float><<<nb, 256, 0, s>>>(ctx->d, M->xq32, ctx->nt, ctx->expand_buf);
   } else {
     pnm_need_phdig(ctx);

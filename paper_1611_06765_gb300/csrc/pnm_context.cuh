@@ -7,7 +7,7 @@
 
 struct MixedState;  // mixed-precision operand arenas (mixed.cu)
 struct MlpState;    // learned warm start (mlp.cu)
-struct PhItem;      // work item of the digit ph term (iterate.cu)
+struct PhItem;      // work item of the ph term (ph.cu)
 
 // Kernel ids of the per-kernel profiler.
 enum {
@@ -35,7 +35,7 @@ struct pnm_ctx {
 
   // host copies of the channel metadata
   std::vector<int> h_ch_sys, h_key, h_nhh, h_npp, h_hh_off, h_pp_off, h_vpp;
-  std::vector<long> h_t_off, h_x_t_off;
+  std::vector<long> h_t_off, h_x_t_off, h_x_c_off;
   std::vector<int> h_nlad;               // ladder basis size per channel (0: no V_pppp block)
   std::vector<long> h_s_off, h_vd_off;   // ladder-layout and ladder-V offsets per channel
   long nvdig = 0, ntdig = 0;             // digit words of the ladder V, room for those of the amplitudes
@@ -54,23 +54,19 @@ struct pnm_ctx {
   int *upd_lo_d = nullptr, *upd_hi_d = nullptr;  // per system ranges of the (row, column) items
   int4* grp_items = nullptr;  // (channel, first ij, first pp column, rows) of the update
   int n_grp_items = 0, upd_rows = 1;
-  int* ph_list = nullptr;  // cross channels of the ph launches (S_z >= 0, costliest first)
-  // channels of the larger, the middle and the small size class of the CTA path and of the warp
-  // path, in that order in ph_list
-  int n_ph_big = 0, n_ph_mid = 0, n_ph = 0, n_ph_warp = 0;
-  size_t ph_smem32 = 0, ph_mid_smem32 = 0, ph_big_smem32 = 0;  // shared memory per class (FP32)
-  std::vector<int> h_ph_list;
-  // the digit ph term (made on first use, pnm_need_phdig): items in ph_list's order, the n_ph_large
-  // ones with the largest tiles first; W fragments, <kb|v|cj> of the problems, source indices
+  // ph term: work items (pnm_need_ph_items): n_ph_large + n_ph_cta channels that take a CTA, then
+  // n_ph_warp of the warp path, the last n_ph_tiny (n_ph_tiny64 with FP64 results) of them tiny
   PhItem* ph_items = nullptr;
+  int n_ph_items = 0, n_ph_large = 0, n_ph_cta = 0, n_ph_warp = 0, n_ph_tiny = 0, n_ph_tiny64 = 0;
+  size_t ph32_smem = 0, ph32_warp_smem = 0;  // shared memory per CTA and per warp, FP32
+  // the digit ph term (made on first use, pnm_need_phdig): source indices, W fragments, <kb|v|cj>
+  long ph_sizes[4] = {0, 0, 0, 0};
   int2* ph_exps = nullptr;
   int* ph_src = nullptr;
   uint4* ph_wf = nullptr;
   long long* ph_v1 = nullptr;
   double* ph_fixed64 = nullptr;
   f2* ph_fixed_f2 = nullptr;  // the fixed operands of the smallest channels as element values
-  int n_ph_large = 0;
-  int n_ph_tiny64 = 0, n_ph_tiny_f2 = 0;  // the last items: channels without digits (FP64, FP32-pair results)
   long* tw_lo = nullptr;                         // first amplitude of each system
   int* tw_parts = nullptr;
   int n_tw_parts = 1;
@@ -225,7 +221,6 @@ void pnm_need_digits(pnm_ctx* ctx);
 void pnm_split_f2(const double* a, f2* b, long n, cudaStream_t s);
 void pnm_prepare_f2(pnm_ctx* ctx);
 void pnm_split_cur(pnm_ctx* ctx, cudaStream_t s);
-size_t ph_smem_bytes(int max_dim, int nm, size_t elem);
 void pnm_mixed_pack_initial(pnm_ctx* ctx, double alpha);
 void pnm_fork(pnm_ctx* ctx);
 void pnm_join(pnm_ctx* ctx);
@@ -236,7 +231,11 @@ void launch_ph64(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny, bool linear)
 void pnm_flip_symmetrise(pnm_ctx* ctx, double* t, cudaStream_t s);
 void pnm_flip_copy(pnm_ctx* ctx, double* t, cudaStream_t s);
 void pnm_flip_copy_current(pnm_ctx* ctx, int iter);
-void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* xv1, float* xq, cudaStream_t s);
+void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* xv1, float* xq, cudaStream_t s,
+                   cudaStream_t s_tiny);
+void pnm_ph_pack32(pnm_ctx* ctx, float* xw, float* xv1);
+void pnm_need_ph_items(pnm_ctx* ctx);
+bool pnm_is_ph_kernel(const void* f);
 void launch_update64(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, bool pair = false);
 void launch_update_mix(pnm_ctx* ctx, const float* rpp, const float* xq, const double* aw, float* xt, int use_cond,
                        cudaGraphConditionalHandle h, int nplanes, long pstride);

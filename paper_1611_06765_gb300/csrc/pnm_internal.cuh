@@ -9,9 +9,12 @@
 //   V_pppp       only for channels where <ab|v|cd> can be nonzero (not both |S_z| = 2 and
 //                |T_z| = 2: identical nucleons of equal spin do not interact; for neutrons
 //                that leaves S_z = 0): in the ladder basis, as digit words (dig.cuh).
-//   cross chans  per channel x: n_ph rows (a,i), n_hp columns (k,c); T_x/Q_x are
-//                n_ph x n_hp at xt_off[x]; V1_x (<kb|v|cj>) n_hp x n_hp at xc_off[x];
-//                W_x (<kl|v|ce>, n_hp x n_ph) stored transposed (n_ph x n_hp) at xw_off[x].
+//   cross chans  per channel x: n_ph rows (a,i), n_hp columns (k,c).  Held in formed layout: only
+//                the elements the ph term forms, S_z > 0 channels whole (R = n_ph, H = n_hp, one
+//                block), S_z = 0 ones on their spin-up rows (R = n_ph / 2, H = n_hp / 2, the block of
+//                the spin-up columns and the block of their flips), S_z < 0 none.  A block of T_x, Q_x
+//                and W_x (<kl|v|ce>, transposed) is R rows of stride formed_width(H) at x_t_off[x],
+//                one of V1_x (<kb|v|cj>) H such rows at x_c_off[x]; the padding holds zeros.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -87,7 +90,7 @@ struct DevState {
   // cross channels
   int *x_nph, *x_nhp;
   int* x_sys;            // cross channel -> system
-  long *x_t_off, *x_c_off, *x_w_off;
+  long *x_t_off, *x_c_off;
   int2 *ph_pair, *hp_pair;
   int* x_ph_off;
   int* x_hp_off;
@@ -102,7 +105,7 @@ struct DevState {
   int* ch_uoff;          // per direct channel its run of upd_row (nch + 1 offsets)
   UpdRow* upd_rowinfo;   // per update item UPD_ROWS rows (rows past the item's last repeat it)
   // maps
-  int* xmap;             // per T element: sign * (t index + 1), 0 = structurally zero
+  int* xmap;             // per formed T element: sign * (t index + 1), 0 = structurally zero
   int4* qmap;            // per t element: the four Q positions of P(ij)P(ab) Q (formed positions)
   int *occ_off, *occ_idx; // per state: pair indices (pp for particles, hh for holes)
   // blocks
@@ -128,6 +131,9 @@ struct DevState {
   // per-system loop state (converged systems are frozen: later steps skip their work)
   const struct SysCtl* sysctl;
 };
+
+// Row stride of the formed matrices of a cross channel: 16-byte groups of FP32.
+__host__ __device__ __forceinline__ int formed_width(int H) { return (H + 3) & ~3; }
 
 // Work item of the pp ladder in digits: a strip of 16 ladder vectors and a pass over up to 8 hole
 // pairs of a channel.
@@ -212,12 +218,7 @@ struct FinArgs {
 constexpr int UPD_ROWS = PNM_UPD_ROWS, UPD_MAX_NHH = 128, UPD_BATCH = PNM_UPD_BATCH;
 constexpr int UPD_MIN_BLOCKS = PNM_UPD_MIN_BLOCKS;
 
-// Threads of a ph-term CTA (one cross channel each); channels of at most PH_WARP_DIM rows and
-// columns (of their halves for S_z = 0) take one warp each.
-// Channels with more than PH_SMALL_DIM rows or columns go to the larger size class, those with
-// more than PH_MID_DIM to the middle one (each class with its own launch and shared-memory
-// size, so that the many smaller channels keep more CTAs per SM).
-constexpr int PH_THREADS = 128, PH_WARP_DIM = 16, PH_SMALL_DIM = 32, PH_MID_DIM = 24;
+constexpr int PH_THREADS = 128;  // threads of a ph-term CTA
 
 // pp ladder of amplitude (ij, ab) of channel c from its ladder-layout value (planes summed by
 // the caller where there are several).

@@ -389,25 +389,43 @@ __device__ __forceinline__ int t_code(int p1, int p2, int h1, int h2, const char
   return sgn * (int)(idx + 1);
 }
 
-// T_x[(a,i)][(k,c)] = t_ik^ac, read from the restricted direct block with its sign.
-// Encoded as sign * (t index + 1); 0 where the element vanishes (a = c or i = k).
+// Row and column of a cross channel behind element (m, u, v) of its formed matrices: S_z > 0 rows
+// and columns as they are (m = 0); S_z = 0 the u-th spin-up row, and of the v-th spin-up column
+// (m = 0) or of its flip (m = 1).
+struct FormedChannel {
+  int nm, R, H, W;  // problems, rows, columns, row stride
+  const int *rrow, *rcol, *fcol;
+  __device__ FormedChannel(int cls, int nph, int nhp, const int* rrow_, const int* rcol_, const int* fcol_)
+      : nm(cls < 0 ? 0 : (cls == 0 ? 2 : 1)), R(cls == 0 ? nph >> 1 : nph), H(cls == 0 ? nhp >> 1 : nhp),
+        W(formed_width(H)), rrow(rrow_), rcol(rcol_), fcol(fcol_) {}
+  __device__ int row(int u) const { return nm == 2 ? rrow[u] : u; }
+  __device__ int col(int m, int v) const { return nm == 2 ? (m ? fcol[rcol[v]] : rcol[v]) : v; }
+};
+
+// T_x[(a,i)][(k,c)] = t_ik^ac of the formed elements, read from the restricted direct block with its
+// sign.  Encoded as sign * (t index + 1); 0 where the element vanishes (a = c or i = k) and in the
+// padding.
 __global__ void k_xmap(int x0, const int* __restrict__ x_nph, const int* __restrict__ x_nhp,
-                       const long* __restrict__ x_t_off, const int* __restrict__ x_ph_off,
-                       const int* __restrict__ x_hp_off, const int2* __restrict__ ph_pair,
-                       const int2* __restrict__ hp_pair, const char4* __restrict__ nvec,
-                       int sp_off, int N, int nsp, int m, int M, int species,
+                       const int* __restrict__ x_cls, const int* __restrict__ x_rrow, const int* __restrict__ x_rcol,
+                       const int* __restrict__ x_fcol, const long* __restrict__ x_t_off,
+                       const int* __restrict__ x_ph_off, const int* __restrict__ x_hp_off,
+                       const int2* __restrict__ ph_pair, const int2* __restrict__ hp_pair,
+                       const char4* __restrict__ nvec, int sp_off, int N, int nsp, int m, int M, int species,
                        const int* __restrict__ key2ch, int ch0, const long* __restrict__ ch_t_off,
                        const int* __restrict__ ch_npp, const int* __restrict__ pos_hh,
                        const int* __restrict__ pos_pp, int* __restrict__ xmap) {
-  int x = x0 + blockIdx.x;
-  int nph = x_nph[x], nhp = x_nhp[x];
-  long base = x_t_off[x];
-  for (int e = threadIdx.x; e < nph * nhp; e += blockDim.x) {
-    int rr = e / nhp, ss = e % nhp;
-    int2 ai = ph_pair[x_ph_off[x] + rr], kc = hp_pair[x_hp_off[x] + ss];
-    int a = ai.x - sp_off, i = ai.y - sp_off, k = kc.x - sp_off, c = kc.y - sp_off;
-    xmap[base + e] = t_code(a, c, i, k, nvec + sp_off, N, nsp - N, m, M, species, key2ch, ch0, ch_t_off,
-                            ch_npp, pos_hh, pos_pp);
+  const int x = x0 + blockIdx.x, po = x_ph_off[x], ho = x_hp_off[x];
+  const FormedChannel f(x_cls[x], x_nph[x], x_nhp[x], x_rrow + po, x_rcol + ho, x_fcol + ho);
+  const long base = x_t_off[x];
+  for (int e = threadIdx.x; e < f.nm * f.R * f.W; e += blockDim.x) {
+    const int mu = e / f.W, v = e - mu * f.W, mm = mu >= f.R, u = mu - mm * f.R;
+    int code = 0;
+    if (v < f.H) {
+      const int2 ai = ph_pair[po + f.row(u)], kc = hp_pair[ho + f.col(mm, v)];
+      code = t_code(ai.x - sp_off, kc.y - sp_off, ai.y - sp_off, kc.x - sp_off, nvec + sp_off, N, nsp - N, m, M,
+                    species, key2ch, ch0, ch_t_off, ch_npp, pos_hh, pos_pp);
+    }
+    xmap[base + e] = code;
   }
 }
 
@@ -417,36 +435,43 @@ __global__ void k_xmap(int x0, const int* __restrict__ x_nph, const int* __restr
 // cross channels with S_z >= 0 and, in those with S_z = 0, only in the rows of a spin-up
 // particle; every other position is replaced by that of its spin flip
 // Q_F(x)[(Fp,Fh)][(Fh2,Fp2)], which holds the same value for flip-symmetric amplitudes.
-__device__ __forceinline__ int qpos(int p, int h, int h2, int p2, int N, int np,
-                                    const int* __restrict__ phch, const int* __restrict__ phpos,
-                                    const int* __restrict__ hppos, int x0,
-                                    const long* __restrict__ x_t_off,
-                                    const int* __restrict__ x_nhp, const int* __restrict__ x_cls,
+struct CrossTables {
+  const int *phch, *phpos, *hppos, *x_nph, *x_nhp, *x_cls, *x_ph_off, *x_hp_off, *x_rinv, *x_cinv;
+  const long* x_t_off;
+  int x0;
+};
+__device__ __forceinline__ int qpos(int p, int h, int h2, int p2, int N, int np, const CrossTables& X,
                                     const char4* __restrict__ nv, const int* __restrict__ idx3, int r,
                                     int species) {
   size_t u = (size_t)(p - N) * N + h;
-  int x = phch[u];
+  int x = X.phch[u];
   if (x < 0) return -1;
-  int g = x0 + x;
-  if (x_cls[g] < 0 || (x_cls[g] == 0 && spin_of(nv[p].w, species) < 0)) {
+  int g = X.x0 + x;
+  if (X.x_cls[g] < 0 || (X.x_cls[g] == 0 && spin_of(nv[p].w, species) < 0)) {
     p = flip_state(nv, idx3, r, p, species);
     h = flip_state(nv, idx3, r, h, species);
     h2 = flip_state(nv, idx3, r, h2, species);
     p2 = flip_state(nv, idx3, r, p2, species);
     u = (size_t)(p - N) * N + h;
-    g = x0 + phch[u];
+    g = X.x0 + X.phch[u];
   }
-  return (int)(x_t_off[g] + (long)phpos[u] * x_nhp[g] + hppos[(size_t)h2 * np + (p2 - N)]);
+  const bool zero = X.x_cls[g] == 0;
+  const int R = zero ? X.x_nph[g] >> 1 : X.x_nph[g], W = formed_width(zero ? X.x_nhp[g] >> 1 : X.x_nhp[g]);
+  int row = X.phpos[u], col = X.hppos[(size_t)h2 * np + (p2 - N)], m = 0;
+  if (zero) {
+    row = X.x_rinv[X.x_ph_off[g] + row];
+    col = X.x_cinv[X.x_hp_off[g] + col];
+    m = col < 0;
+    if (m) col = -col - 1;
+  }
+  return (int)(X.x_t_off[g] + (long)(m * R + row) * W + col);
 }
 
 __global__ void k_qmap(int row0, const int2* __restrict__ row_item,
                        const int* __restrict__ ch_hh_off, const int* __restrict__ ch_pp_off,
                        const int* __restrict__ ch_npp, const long* __restrict__ ch_t_off,
                        const int2* __restrict__ hh_pair, const int2* __restrict__ pp_pair,
-                       int sp_off, int N, int nsp, const int* __restrict__ phch,
-                       const int* __restrict__ phpos, const int* __restrict__ hppos, int x0,
-                       const long* __restrict__ x_t_off, const int* __restrict__ x_nhp,
-                       const int* __restrict__ x_cls, const char4* __restrict__ nvec,
+                       int sp_off, int N, int nsp, CrossTables X, const char4* __restrict__ nvec,
                        const int* __restrict__ idx3, int r, int species, int4* __restrict__ qmap) {
   int2 it = row_item[row0 + blockIdx.x];
   int c = it.x, ij = it.y;
@@ -460,10 +485,10 @@ __global__ void k_qmap(int row0, const int2* __restrict__ row_item,
     int2 pb = pp_pair[ch_pp_off[c] + ab];
     int a = pb.x - sp_off, b = pb.y - sp_off;
     int4 q;
-    q.x = qpos(a, i, j, b, N, np, phch, phpos, hppos, x0, x_t_off, x_nhp, x_cls, nv, idx3, r, species);
-    q.y = qpos(a, j, i, b, N, np, phch, phpos, hppos, x0, x_t_off, x_nhp, x_cls, nv, idx3, r, species);
-    q.z = qpos(b, i, j, a, N, np, phch, phpos, hppos, x0, x_t_off, x_nhp, x_cls, nv, idx3, r, species);
-    q.w = qpos(b, j, i, a, N, np, phch, phpos, hppos, x0, x_t_off, x_nhp, x_cls, nv, idx3, r, species);
+    q.x = qpos(a, i, j, b, N, np, X, nv, idx3, r, species);
+    q.y = qpos(a, j, i, b, N, np, X, nv, idx3, r, species);
+    q.z = qpos(b, i, j, a, N, np, X, nv, idx3, r, species);
+    q.w = qpos(b, j, i, a, N, np, X, nv, idx3, r, species);
     qmap[base + ab] = q;
   }
 }
@@ -479,7 +504,9 @@ __global__ void k_qmap(int row0, const int2* __restrict__ row_item,
 //           reads the flipped channel F(x) instead, see qpos);
 //   x_fcol  per column (k,c) the column of (F k, F c) in F(x);
 //   x_rrow / x_rcol (S_z = 0)  the rows (a,i) and columns (k,c) with spin-up a and k, in order
-//           (half of each: the other half are their flips).
+//           (half of each: the other half are their flips);
+//   x_rinv / x_cinv  their inverses: the place of a spin-up row, and of a column v (spin-up) or
+//           -v - 1 (the flip of the v-th spin-up column).
 // Sets *err when the rows or columns of a channel do not map onto one channel F(x) (a
 // reference that is not spin saturated).
 // One warp per channel; the spin-up rows and columns are compacted in order with ballots.
@@ -490,7 +517,8 @@ __global__ void k_xflip(int x0, int nxs, const int* __restrict__ x_nph, const in
                         int sp_off, int N, int nsp, const int* __restrict__ phpos,
                         const int* __restrict__ phch, const int* __restrict__ hppos, int* __restrict__ x_cls,
                         int* __restrict__ x_fcol,
-                        int* __restrict__ x_rrow, int* __restrict__ x_rcol, int* __restrict__ err) {
+                        int* __restrict__ x_rrow, int* __restrict__ x_rcol, int* __restrict__ x_rinv,
+                        int* __restrict__ x_cinv, int* __restrict__ err) {
   const int xl = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (xl >= nxs) return;  // warp-uniform
@@ -525,7 +553,11 @@ __global__ void k_xflip(int x0, int nxs, const int* __restrict__ x_nph, const in
     if (mir < 0) mir = __shfl_sync(0xffffffffu, ch, 0);
     bad = __any_sync(0xffffffffu, lbad || (k < nph && ch != mir));
     unsigned bu = __ballot_sync(0xffffffffu, up);
-    if (up) x_rrow[po + nr + __popc(bu & lt)] = k;
+    if (up) {
+      const int v = nr + __popc(bu & lt);
+      x_rrow[po + v] = k;
+      x_rinv[po + k] = v;
+    }
     nr += __popc(bu);
   }
   for (int k0 = 0; k0 < nhp && !bad; k0 += 32) {
@@ -544,7 +576,12 @@ __global__ void k_xflip(int x0, int nxs, const int* __restrict__ x_nph, const in
     }
     bad = __any_sync(0xffffffffu, lbad);
     unsigned bu = __ballot_sync(0xffffffffu, up);
-    if (up) x_rcol[ho + nc + __popc(bu & lt)] = k;
+    if (up) {
+      const int v = nc + __popc(bu & lt);
+      x_rcol[ho + v] = k;
+      x_cinv[ho + k] = v;
+      x_cinv[ho + x_fcol[ho + k]] = -v - 1;
+    }
     nc += __popc(bu);
   }
   if (lane != 0) return;
@@ -800,23 +837,35 @@ __global__ void k_v_hhhh(int c0, const int* __restrict__ ch_hh_off,
   }
 }
 
-// V1_x[(k,c)][(j,b)] = <kb|v|cj>,  W_x[(k,c)][(e,l)] = <kl|v|ce> (stored as W_x^T).
+// V1_x[(k,c)][(j,b)] = <kb|v|cj>,  W_x[(k,c)][(e,l)] = <kl|v|ce> (stored as W_x^T), formed elements
+// only, zero in the padding.
 __global__ void k_v_cross(int x0, const int* __restrict__ x_nph, const int* __restrict__ x_nhp,
-                          const long* __restrict__ x_c_off, const long* __restrict__ x_w_off,
-                          const int* __restrict__ x_ph_off, const int* __restrict__ x_hp_off,
-                          const int2* __restrict__ ph_pair, const int2* __restrict__ hp_pair,
-                          const char4* __restrict__ nvec, const double* __restrict__ lut,
-                          double* __restrict__ x_v1, double* __restrict__ x_w) {
-  int x = x0 + blockIdx.x;
-  int nph = x_nph[x], nhp = x_nhp[x];
-  for (int e = threadIdx.x; e < nhp * nhp; e += blockDim.x) {
-    int2 kc = hp_pair[x_hp_off[x] + e / nhp], jb = hp_pair[x_hp_off[x] + e % nhp];
-    x_v1[x_c_off[x] + e] = v_minnesota_as(nvec[kc.x], nvec[jb.y], nvec[kc.y], nvec[jb.x], lut);
+                          const int* __restrict__ x_cls, const int* __restrict__ x_rrow, const int* __restrict__ x_rcol,
+                          const int* __restrict__ x_fcol, const long* __restrict__ x_c_off,
+                          const long* __restrict__ x_t_off, const int* __restrict__ x_ph_off,
+                          const int* __restrict__ x_hp_off, const int2* __restrict__ ph_pair,
+                          const int2* __restrict__ hp_pair, const char4* __restrict__ nvec,
+                          const double* __restrict__ lut, double* __restrict__ x_v1, double* __restrict__ x_w) {
+  const int x = x0 + blockIdx.x, po = x_ph_off[x], ho = x_hp_off[x];
+  const FormedChannel f(x_cls[x], x_nph[x], x_nhp[x], x_rrow + po, x_rcol + ho, x_fcol + ho);
+  for (int e = threadIdx.x; e < f.nm * f.H * f.W; e += blockDim.x) {
+    const int mr = e / f.W, v = e - mr * f.W, m = mr >= f.H, r = mr - m * f.H;
+    double y = 0.0;
+    if (v < f.H) {
+      const int2 kc = hp_pair[ho + f.col(0, r)], jb = hp_pair[ho + f.col(m, v)];
+      y = v_minnesota_as(nvec[kc.x], nvec[jb.y], nvec[kc.y], nvec[jb.x], lut);
+    }
+    x_v1[x_c_off[x] + e] = y;
   }
   // stored transposed, W^T[(e,l)][(k,c)], so the ph kernel stages it with coalesced loads
-  for (int e = threadIdx.x; e < nph * nhp; e += blockDim.x) {
-    int2 el = ph_pair[x_ph_off[x] + e / nhp], kc = hp_pair[x_hp_off[x] + e % nhp];
-    x_w[x_w_off[x] + e] = v_minnesota_as(nvec[kc.x], nvec[el.y], nvec[kc.y], nvec[el.x], lut);
+  for (int e = threadIdx.x; e < f.nm * f.R * f.W; e += blockDim.x) {
+    const int mu = e / f.W, v = e - mu * f.W, m = mu >= f.R, u = mu - m * f.R;
+    double y = 0.0;
+    if (v < f.H) {
+      const int2 el = ph_pair[po + f.row(u)], kc = hp_pair[ho + f.col(m, v)];
+      y = v_minnesota_as(nvec[kc.x], nvec[el.y], nvec[kc.y], nvec[el.x], lut);
+    }
+    x_w[x_t_off[x] + e] = y;
   }
 }
 
@@ -1037,8 +1086,9 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   std::vector<int2> h_rows;
   std::vector<std::vector<int>> h_lad_chans(nsys);  // per system: channels with a V_pppp block
   std::vector<int> h_x_nph, h_x_nhp, h_x_ph_off, h_x_hp_off;
-  std::vector<long> h_x_t_off, h_x_c_off, h_x_w_off;
-  long t_acc = 0, vhh_acc = 0, xt_acc = 0, xc_acc = 0;
+  std::vector<long> h_x_t_off, h_x_c_off;
+  std::vector<int> h_x_cls;
+  long t_acc = 0, vhh_acc = 0, xt_acc = 0, xc_acc = 0, xt_full = 0;
   int hh_acc = 0, pp_acc = 0, ph_acc = 0, hp_acc = 0;
   for (int k = 0; k < nsys; k++) {
     SysInfo& S = sys[k];
@@ -1080,15 +1130,22 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
       h_x_hp_off.push_back(hp_acc);
       h_x_t_off.push_back(xt_acc);
       h_x_c_off.push_back(xc_acc);
-      h_x_w_off.push_back(xt_acc);  // W_x has n_hp x n_ph entries, as many as T_x
+      // the formed matrices of the ph term: S_z > 0 whole, S_z = 0 the spin-up rows (the spin of a
+      // key's charge slot is that of its first index)
+      const int K = X.xkeys[x], cls = (S.species == 1 ? K % 3 : (K % 9) / 3) - 1;
+      h_x_cls.push_back(cls);
       ph_acc += X.xnph[x];
       hp_acc += X.xnhp[x];
-      xt_acc += (long)X.xnph[x] * X.xnhp[x];
-      xc_acc += (long)X.xnhp[x] * X.xnhp[x];
+      xt_full += (long)X.xnph[x] * X.xnhp[x];
+      if (cls >= 0) {
+        const int nm = cls == 0 ? 2 : 1, R = X.xnph[x] / nm, H = X.xnhp[x] / nm;
+        xt_acc += (long)nm * R * formed_width(H);
+        xc_acc += (long)nm * H * formed_width(H);
+      }
     }
     S.x_end = (int)h_x_nph.size();
   }
-  if (t_acc >= (1L << 31) - 2 || xt_acc >= (1L << 31) - 2)
+  if (t_acc >= (1L << 31) - 2 || xt_full >= (1L << 31) - 2)
     throw PnmError{PNM_EINVAL, "problem too large for 32-bit element maps"};
   ctx->nch = (int)h_key.size();
   ctx->nx = (int)h_x_nph.size();
@@ -1109,6 +1166,8 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   ctx->h_x_nph = h_x_nph;
   ctx->h_x_nhp = h_x_nhp;
   ctx->h_x_t_off = h_x_t_off;
+  ctx->h_x_c_off = h_x_c_off;
+  ctx->h_x_cls = h_x_cls;
   ctx->h_x_ph_off = h_x_ph_off;
   ctx->h_x_hp_off = h_x_hp_off;
   ctx->h_hh_off = h_hh_off;
@@ -1137,7 +1196,6 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   D.x_hp_off = dalloc<int>(NX, ctx->owned, s);
   D.x_t_off = dalloc<long>(NX, ctx->owned, s);
   D.x_c_off = dalloc<long>(NX, ctx->owned, s);
-  D.x_w_off = dalloc<long>(NX, ctx->owned, s);
   h2d(D.ch_sys, h_ch_sys, s);
   {
     std::vector<int> h_x_sys(NX);
@@ -1161,7 +1219,6 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   h2d(D.x_hp_off, h_x_hp_off, s);
   h2d(D.x_t_off, h_x_t_off, s);
   h2d(D.x_c_off, h_x_c_off, s);
-  h2d(D.x_w_off, h_x_w_off, s);
 
   D.hh_pair = dalloc<int2>(hh_acc, ctx->owned, s);
   D.pp_pair = dalloc<int2>(pp_acc, ctx->owned, s);
@@ -1171,6 +1228,14 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   D.x_rrow = dalloc<int>(ph_acc, ctx->owned, s);
   D.x_fcol = dalloc<int>(hp_acc, ctx->owned, s);
   D.x_rcol = dalloc<int>(hp_acc, ctx->owned, s);
+  int* x_rinv = dalloc<int>(ph_acc, scr[0].owned, s);
+  int* x_cinv = dalloc<int>(hp_acc, scr[0].owned, s);
+  // valid indices also where a channel that does not map onto one (flip_err) leaves gaps
+  CUDA_TRY(cudaMemsetAsync(D.x_rrow, 0, sizeof(int) * std::max(ph_acc, 1), s));
+  CUDA_TRY(cudaMemsetAsync(D.x_fcol, 0, sizeof(int) * std::max(hp_acc, 1), s));
+  CUDA_TRY(cudaMemsetAsync(D.x_rcol, 0, sizeof(int) * std::max(hp_acc, 1), s));
+  CUDA_TRY(cudaMemsetAsync(x_rinv, 0, sizeof(int) * std::max(ph_acc, 1), s));
+  CUDA_TRY(cudaMemsetAsync(x_cinv, 0, sizeof(int) * std::max(hp_acc, 1), s));
   D.fmap = dalloc<int>(t_acc, ctx->owned, s);
   int* flip_err = dalloc<int>(1, ctx->owned, s);
   CUDA_TRY(cudaMemsetAsync(flip_err, 0, sizeof(int), s));
@@ -1219,24 +1284,25 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
           D.nvec + S.sp_off, X.idx3, S.r, S.m, S.M, S.species, S.N, S.nsp, S.sp_off, nxs, xk,
           D.x_ph_off + S.x_begin, D.x_hp_off + S.x_begin, D.ph_pair, D.hp_pair, X.phpos, X.phch,
           X.hppos);
-      k_xmap<<<nxs, 256, 0, s>>>(S.x_begin, D.x_nph, D.x_nhp, D.x_t_off, D.x_ph_off, D.x_hp_off,
-                                 D.ph_pair, D.hp_pair, D.nvec, S.sp_off, S.N, S.nsp, S.m, S.M,
-                                 S.species, X.key2ch, S.ch_begin, D.ch_t_off, D.ch_npp, X.pos_hh, X.pos_pp,
-                                 D.xmap);
       k_xflip<<<(nxs * 32 + 255) / 256, 256, 0, s>>>(S.x_begin, nxs, D.x_nph, D.x_nhp, D.x_ph_off, D.x_hp_off,
                                                 D.ph_pair, D.hp_pair, D.nvec, X.idx3, S.r, S.species,
                                                 S.sp_off, S.N, S.nsp, X.phpos, X.phch, X.hppos, D.x_cls,
-                                                D.x_fcol, D.x_rrow, D.x_rcol, flip_err);
-      k_v_cross<<<nxs, 256, 0, s>>>(S.x_begin, D.x_nph, D.x_nhp, D.x_c_off, D.x_w_off,
-                                    D.x_ph_off, D.x_hp_off, D.ph_pair, D.hp_pair, D.nvec,
+                                                D.x_fcol, D.x_rrow, D.x_rcol, x_rinv, x_cinv, flip_err);
+      k_xmap<<<nxs, 256, 0, s>>>(S.x_begin, D.x_nph, D.x_nhp, D.x_cls, D.x_rrow, D.x_rcol, D.x_fcol, D.x_t_off,
+                                 D.x_ph_off, D.x_hp_off, D.ph_pair, D.hp_pair, D.nvec, S.sp_off, S.N, S.nsp, S.m,
+                                 S.M, S.species, X.key2ch, S.ch_begin, D.ch_t_off, D.ch_npp, X.pos_hh, X.pos_pp,
+                                 D.xmap);
+      k_v_cross<<<nxs, 256, 0, s>>>(S.x_begin, D.x_nph, D.x_nhp, D.x_cls, D.x_rrow, D.x_rcol, D.x_fcol, D.x_c_off,
+                                    D.x_t_off, D.x_ph_off, D.x_hp_off, D.ph_pair, D.hp_pair, D.nvec,
                                     D.lut + S.lut_off, D.x_v1, D.x_w);
     }
     int nrows = S.row_end - S.row_begin;
     if (nrows > 0) {
       k_qmap<<<nrows, 128, 0, s>>>(S.row_begin, D.row_item, D.ch_hh_off, D.ch_pp_off, D.ch_npp,
                                    D.ch_t_off, D.hh_pair, D.pp_pair, S.sp_off, S.N, S.nsp,
-                                   X.phch, X.phpos, X.hppos, S.x_begin, D.x_t_off, D.x_nhp,
-                                   D.x_cls, D.nvec, X.idx3, S.r, S.species, D.qmap);
+                                   CrossTables{X.phch, X.phpos, X.hppos, D.x_nph, D.x_nhp, D.x_cls, D.x_ph_off,
+                                               D.x_hp_off, x_rinv, x_cinv, D.x_t_off, S.x_begin},
+                                   D.nvec, X.idx3, S.r, S.species, D.qmap);
       k_fmap<<<nrows, 128, 0, s>>>(S.row_begin, D.row_item, D.ch_hh_off, D.ch_pp_off, D.ch_npp, D.ch_t_off,
                                    D.hh_pair, D.pp_pair, D.nvec, X.idx3, S.r, S.species, S.sp_off, S.N,
                                    S.nsp, S.m, S.M, X.key2ch, S.ch_begin, X.pos_hh, X.pos_pp, D.fmap,
@@ -1290,7 +1356,6 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   }
   std::vector<int> h_nlad = d2h(D.ch_nlad, C, s);
   if (d2h(flip_err, 1, s)[0]) throw PnmError{PNM_EINVAL, "spin-flip tables not closed (reference not spin saturated)"};
-  ctx->h_x_cls = d2h(D.x_cls, NX, s);
   std::vector<long> h_s_off(C, 0), h_vd_off(C, -1), h_td_off(C, 0);
   long s_acc = 0, vd_acc = 0, td_acc = 0;
   int max_nlad = 0;

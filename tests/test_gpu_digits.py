@@ -72,6 +72,19 @@ def test_operators_against_oracle(pkg, N, Z, rho, n2, spread):
     g.close()
 
 
+@pytest.mark.parametrize("N,Z,rho,n2", [s for s in SYSTEMS if not s[1]])
+def test_mixed_ph_operator(pkg, N, Z, rho, n2):
+    """The FP32 ph term over channels of 1 to 33 rows and columns (a part of a warp, a warp, a CTA each):
+    two chained FP32 products over at most 33 terms, 2 * 33 * 2^-24 < 4e-6 of the element's sum of
+    absolute products, and the rounding of the operands, 3 * 2^-24."""
+    g, o = _pair(pkg, N, Z, rho, n2)
+    t = random_amplitudes(len(g.amplitude_labels()), seed=17)
+    ts = spinflip.symmetrise(t, spinflip.flip_permutation(g.amplitude_labels(), o.states()))
+    ref, bound = o.ph_apply(ts), o.ph_apply(ts, absval=True)
+    assert np.all(np.abs(g.apply_ph_term(t, precision=pkg.PNM_PREC_BF16X3) - ref) <= 5e-6 * bound + 1e-30)
+    g.close()
+
+
 @pytest.mark.parametrize("N,Z,rho,n2", [(14, 0, 0.08, 9), (66, 0, 0.16, 14), (14, 14, 0.16, 6)])
 def test_power_of_two_scaling_is_exact(pkg, N, Z, rho, n2):
     """The ladder is linear and its digits carry one exponent per row: scaled amplitudes give the
