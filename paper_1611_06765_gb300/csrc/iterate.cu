@@ -579,7 +579,7 @@ __device__ void last_block_finalize(const FinArgs& f, LoopCtl* ctl) {
 // denominator, residual, step (alpha / eps_ij^ab prepared per solve, aw) and energy stay FP64.
 template <typename T_>
 __global__ void __launch_bounds__(128) k_update(DevState D, LoopCtl* __restrict__ ctl,
-                                                const int4* __restrict__ items, FinArgs fa,
+                                                const UpdItem* __restrict__ items, FinArgs fa,
                                                 const T_* __restrict__ tpair, const double* __restrict__ aw) {
   constexpr bool PAIR = std::is_same<T_, f2>::value;
   using A = Arith<T_>;
@@ -590,12 +590,10 @@ __global__ void __launch_bounds__(128) k_update(DevState D, LoopCtl* __restrict_
   __shared__ int row_ij[UPD_ROWS];
   __shared__ double sh32[32];
   if (ctl->status != 0) return;  // the loop has ended within its body (see pnm_enqueue_loop_body)
-  int4 it = items[blockIdx.x];
-  int c = it.x, ng = it.w;
-  int npp = D.ch_npp[c], nh = D.ch_nhh[c];
-  int ab = it.z + threadIdx.x;
-  bool frozen = fa.sc[D.ch_sys[c]].done != 0;
-  if (sys_settled(fa.sc[D.ch_sys[c]], ctl)) {
+  const UpdItem it = items[blockIdx.x];
+  const int c = it.c, ng = it.ng, npp = it.npp, nh = it.nh, ab = it.ab0 + threadIdx.x;
+  const bool frozen = fa.sc[it.sys].done != 0;
+  if (sys_settled(fa.sc[it.sys], ctl)) {
     // converged at least two steps ago: both amplitude buffers already hold its values
     if (threadIdx.x == 0) {
       D.eparts[blockIdx.x] = 0.0;
@@ -604,12 +602,11 @@ __global__ void __launch_bounds__(128) k_update(DevState D, LoopCtl* __restrict_
     last_block_finalize(fa, ctl);
     return;
   }
-  bool has_vpp = D.ch_vpp[c] != 0;
+  const bool has_vpp = it.nl != 0;
   double alpha = ctl->alpha;
   const double* __restrict__ t = cur_t(D, ctl);
   double* __restrict__ tn = next_t(D, ctl);
-  long base = D.ch_t_off[c];
-  long vho = D.ch_vhh_off[c];
+  const long base = it.base, vho = it.vhh_off;
   const UpdRow* __restrict__ rt = D.upd_rowinfo + (long)blockIdx.x * UPD_ROWS;
   if ((int)threadIdx.x < UPD_ROWS) {
     const UpdRow ri = rt[threadIdx.x];
@@ -736,41 +733,54 @@ void launch_update64(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, b
 //               table (bit for bit the stored element, one FP64 addition) instead of streamed
 // Arrays read once per update (t, alpha / eps, flip and Q maps) and the FP64 amplitudes written
 // for the next update are streamed with the evict-first policy, so that the ph term's T and Q
-// (50 MB each for the held-out batch, read and written at random) and the FP32 amplitudes the
+// (25 MB each for the held-out batch, read and written at random) and the FP32 amplitudes the
 // next update's contractions read stay in L2.
 // The FP64 unit of a GB300 runs at about 1/64 of its FP32 rate, so the FP64 work is held to
 // eight instructions per amplitude; the new amplitude goes to t (FP64) for itself and to t32 for
 // itself and, sign applied, for its spin flip.  The FP64 flips are not read before the mixed
 // iteration ends (the update reads t at the amplitudes it computes only); one flip copy of the
-// current buffer fills them then (pnm_flip_copy_current).  Rows go in batches of UPD_BATCH with
-// all loads of a batch issued before any store (rows past ng repeat the last row and are
+// current buffer fills them then (pnm_flip_copy_current).
+// What bounds it is a chain of dependent round trips per CTA at 24 warps per SM, so the chain is kept
+// short: the item carries the channel's metadata, and the Q positions of all rows are copied
+// asynchronously into the thread's own places of shared memory before the row setup (they wait for
+// nothing else), which leaves one round trip per batch of UPD_BATCH rows (the streams and the four Q
+// gathers together) instead of two.  One update of three N=66, N_max=36 systems: 121 us with metadata
+// by index and positions loaded per batch, 113 us here; 120 twisted N=14, N_max=20 systems 200, 190 us.
+// The t32 column of the hh ladder staged the same way costs more shared memory than it hides: 162 us.
+// All loads of a batch are issued before any store (rows past ng repeat the last row and are
 // discarded).
 __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, LoopCtl* __restrict__ ctl,
-                                                    const int4* __restrict__ items, FinArgs fa,
+                                                    const UpdItem* __restrict__ items, FinArgs fa,
                                                     const float* __restrict__ rpp, const float* __restrict__ xq,
                                                     const double* __restrict__ aw, float* __restrict__ xt,
-                                                    const int* __restrict__ lut_off, int nplanes, long pstride) {
-  __shared__ float chs[UPD_MAX_NHH * UPD_ROWS];  // chi32[kl][ij of row g] at kl * UPD_ROWS + g
+                                                    int nplanes, long pstride) {
+  // dynamic: Q positions [row][column], chi32[kl][ij of row g] at kl * UPD_ROWS + g
+  extern __shared__ __align__(16) unsigned char upd_sm[];
   __shared__ float row_dij[UPD_ROWS];
   __shared__ double row_eij[UPD_ROWS];
   __shared__ int row_ij[UPD_ROWS];
   __shared__ char4 row_si[UPD_ROWS], row_sj[UPD_ROWS];
   __shared__ double red[2][128];
   if (ctl->status != 0) return;  // the loop has ended within its body (see pnm_enqueue_loop_body)
-  int4 it = items[blockIdx.x];
-  int c = it.x, ng = it.w;
-  int npp = D.ch_npp[c], nh = D.ch_nhh[c];
-  int ab = it.z + threadIdx.x;
+  const UpdItem it = items[blockIdx.x];
+  const int ng = it.ng, npp = it.npp, nh = it.nh, ab = it.ab0 + threadIdx.x;
+  int4* qsm = reinterpret_cast<int4*>(upd_sm) + threadIdx.x;
+  float* chs = reinterpret_cast<float*>(upd_sm + sizeof(int4) * 128 * UPD_ROWS);
   const bool col = ab < npp;
-  const bool has_vpp = D.ch_vpp[c] != 0;
+  const long base = it.base;
+  const float* __restrict__ t32 = cur_t32(D, ctl);
+  const UpdRow* __restrict__ rt = D.upd_rowinfo + (long)blockIdx.x * UPD_ROWS;
   // the column's pair data does not depend on the rows: loaded beside the row setup
   int2 p = make_int2(0, 0);
   int lmap = 0;
   if (col) {
-    p = D.pp_pair[D.ch_pp_off[c] + ab];
-    if (has_vpp) lmap = D.lad_map[D.ch_pp_off[c] + ab];
+    for (int g = 0; g < ng; g++)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(qsm + g * 128)),
+                   "l"(D.qmap + base + (long)rt[g].ij * npp + ab)
+                   : "memory");
+    p = D.pp_pair[it.pp_off + ab];
+    if (it.nl) lmap = D.lad_map[it.pp_off + ab];
   }
-  const UpdRow* __restrict__ rt = D.upd_rowinfo + (long)blockIdx.x * UPD_ROWS;
   if ((int)threadIdx.x < UPD_ROWS) {
     const UpdRow ri = rt[threadIdx.x];
     row_ij[threadIdx.x] = ri.ij;
@@ -788,31 +798,31 @@ __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, 
     sa = D.nvec[p.x];
     sb = D.nvec[p.y];
   }
-  const bool frozen = fa.sc[D.ch_sys[c]].done != 0;
-  if (sys_settled(fa.sc[D.ch_sys[c]], ctl)) {
+  const bool frozen = fa.sc[it.sys].done != 0;
+  if (sys_settled(fa.sc[it.sys], ctl)) {
     // converged at least two steps ago: both amplitude buffers already hold its values
     if (threadIdx.x == 0) {
       D.eparts[blockIdx.x] = 0.0;
       D.rparts[blockIdx.x] = 0.0;
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     last_block_finalize(fa, ctl);
     return;
   }
   // chi's columns of the item's rows, their indices read from the row table (no wait for the
   // row setup above: one barrier covers both)
   if (!frozen) {
-    const float* __restrict__ chi = D.chi32 + D.ch_vhh_off[c];
+    const float* __restrict__ chi = D.chi32 + it.vhh_off;
     for (int e = threadIdx.x; e < nh * UPD_ROWS; e += blockDim.x) {
       const int kl = e / UPD_ROWS, g = e % UPD_ROWS;
       chs[e] = g < ng ? chi[(long)kl * nh + rt[g].ij] : 0.0f;
     }
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   const double* __restrict__ t = cur_t(D, ctl);
-  const float* __restrict__ t32 = cur_t32(D, ctl);
   double* __restrict__ tn = next_t(D, ctl);
   float* __restrict__ t32n = next_t32(D, ctl);
-  const long base = D.ch_t_off[c];
   // energy and residual sums of the amplitudes whose spin flip is another amplitude (counted
   // twice) and of those that are their own flip (counted once)
   double e2 = 0.0, e1 = 0.0, r2 = 0.0, r1 = 0.0;
@@ -821,10 +831,9 @@ __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, 
 #pragma unroll
     for (int g = 0; g < UPD_ROWS; g++) hh[g] = 0.0f;
     if (!frozen) {
-      const float* __restrict__ tc = t32 + base + ab;
 #pragma unroll UPD_HH_UNROLL
       for (int kl = 0; kl < nh; kl++) {
-        const float tk = tc[(long)kl * npp];
+        const float tk = t32[base + ab + (long)kl * npp];
         const float4 c0 = *reinterpret_cast<const float4*>(chs + kl * UPD_ROWS);
         const float4 c1 = *reinterpret_cast<const float4*>(chs + kl * UPD_ROWS + 4);
         hh[0] = fmaf(tk, c0.x, hh[0]); hh[1] = fmaf(tk, c0.y, hh[1]);
@@ -833,25 +842,18 @@ __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, 
         hh[6] = fmaf(tk, c1.z, hh[6]); hh[7] = fmaf(tk, c1.w, hh[7]);
       }
     }
-    const double* __restrict__ lut = D.lut + lut_off[D.ch_sys[c]];
+    const double* __restrict__ lut = D.lut + it.lut_off;
     // the pp ladder's element in the ladder layout: s_off + ij * n_lad + |m| - 1, sign of m
-    long lad0 = 0;
-    int nl = 0;
-    bool lneg = false;
-    if (has_vpp) {
-      const int m = lmap;
-      lneg = m < 0;
-      nl = D.ch_nlad[c];
-      lad0 = D.ch_s_off[c] + ((m > 0 ? m : -m) - 1);
-    }
+    const int nl = it.nl;
+    const bool has_vpp = nl != 0, lneg = lmap < 0;
+    const long lad0 = it.s_off + ((lmap > 0 ? lmap : -lmap) - 1);
 #pragma unroll
     for (int gb = 0; gb < UPD_ROWS; gb += UPD_BATCH) {
       if (gb >= ng) break;
       long z[UPD_BATCH];
       double tz[UPD_BATCH], wz[UPD_BATCH];
       int fc[UPD_BATCH];
-      float t32z[UPD_BATCH], part[UPD_BATCH], qs[UPD_BATCH];
-      int4 qm[UPD_BATCH];
+      float part[UPD_BATCH], qs[UPD_BATCH], t32z[UPD_BATCH];
 #pragma unroll
       for (int j = 0; j < UPD_BATCH; j++) {
         const int g = min(gb + j, ng - 1);
@@ -860,7 +862,6 @@ __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, 
         wz[j] = __ldcs(aw + z[j]);
         fc[j] = __ldcs(D.fmap + z[j]);
         t32z[j] = t32[z[j]];
-        qm[j] = __ldcs(D.qmap + z[j]);
         float rl = 0.0f;
         if (has_vpp) {
           const long zl = lad0 + (long)row_ij[g] * nl;
@@ -868,12 +869,10 @@ __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, 
           if (lneg) rl = -rl;
         }
         part[j] = rl;
-      }
-#pragma unroll
-      for (int j = 0; j < UPD_BATCH; j++) {
         // P(ij)P(ab) Q: Q_ij^ab - Q_ji^ab - Q_ij^ba + Q_ji^ba from the cross-channel layout
-        const float a0 = qm[j].x >= 0 ? xq[qm[j].x] : 0.0f, a1 = qm[j].y >= 0 ? xq[qm[j].y] : 0.0f;
-        const float a2 = qm[j].z >= 0 ? xq[qm[j].z] : 0.0f, a3 = qm[j].w >= 0 ? xq[qm[j].w] : 0.0f;
+        const int4 qm = qsm[g * 128];
+        const float a0 = qm.x >= 0 ? xq[qm.x] : 0.0f, a1 = qm.y >= 0 ? xq[qm.y] : 0.0f;
+        const float a2 = qm.z >= 0 ? xq[qm.z] : 0.0f, a3 = qm.w >= 0 ? xq[qm.w] : 0.0f;
         qs[j] = (a0 - a1) - (a2 - a3);
       }
 #pragma unroll
@@ -904,10 +903,11 @@ __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, 
         if (!frozen) {
           // the T positions of t_ij^ab, t_ji^ab, t_ij^ba, t_ji^ba (the Q positions of the same
           // amplitude; stores only, nothing waits on them)
-          if (qm[j].x >= 0) xt[qm[j].x] = o32;
-          if (qm[j].y >= 0) xt[qm[j].y] = -o32;
-          if (qm[j].z >= 0) xt[qm[j].z] = -o32;
-          if (qm[j].w >= 0) xt[qm[j].w] = o32;
+          const int4 qm = qsm[g * 128];
+          if (qm.x >= 0) xt[qm.x] = o32;
+          if (qm.y >= 0) xt[qm.y] = -o32;
+          if (qm.z >= 0) xt[qm.z] = -o32;
+          if (qm.w >= 0) xt[qm.w] = o32;
         }
       }
     }
@@ -929,11 +929,15 @@ __global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, 
   last_block_finalize(fa, ctl);
 }
 
+static size_t upd_mix_smem(const pnm_ctx* ctx) {
+  return sizeof(int4) * 128 * UPD_ROWS + sizeof(float) * UPD_ROWS * (size_t)ctx->max_nhh;
+}
+
 void launch_update_mix(pnm_ctx* ctx, const float* rpp, const float* xq, const double* aw, float* xt, int use_cond,
                        cudaGraphConditionalHandle h, int nplanes, long pstride) {
-  k_update_mix<<<ctx->n_grp_items, 128, 0, ctx->stream>>>(ctx->d, ctx->ctl, ctx->grp_items,
-                                                         fin_args(ctx, use_cond, h, false), rpp, xq, aw, xt,
-                                                         ctx->lut_off_d, nplanes, pstride);
+  k_update_mix<<<ctx->n_grp_items, 128, upd_mix_smem(ctx), ctx->stream>>>(ctx->d, ctx->ctl, ctx->grp_items,
+                                                                          fin_args(ctx, use_cond, h, false), rpp, xq, aw,
+                                                                          xt, nplanes, pstride);
 }
 
 // alpha / eps_ij^ab per amplitude (the step of the mixed update).
@@ -1104,11 +1108,11 @@ __global__ void k_start(const double* __restrict__ parts, const int* __restrict_
 static void* dmalloc(pnm_ctx* ctx, size_t bytes) { return pnm_ctx_alloc(ctx, bytes); }
 
 // Static row data of the update items: row g of item i is the (min(g, ng - 1))-th row of its run.
-__global__ void k_rowinfo(DevState D, const int4* __restrict__ items, UpdRow* __restrict__ out) {
+__global__ void k_rowinfo(DevState D, const UpdItem* __restrict__ items, UpdRow* __restrict__ out) {
   const int g = threadIdx.x;
   if (g >= UPD_ROWS) return;
-  const int4 it = items[blockIdx.x];
-  const int c = it.x, ij = D.upd_row[it.y + min(g, it.w - 1)];
+  const UpdItem it = items[blockIdx.x];
+  const int c = it.c, ij = D.upd_row[it.r0 + min(g, it.ng - 1)];
   const int2 h = D.hh_pair[D.ch_hh_off[c] + ij];
   UpdRow r;
   r.ij = ij;
@@ -1241,7 +1245,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
     CUDA_TRY(cudaMemcpyAsync(ctx->d.upd_row, urow.data(), sizeof(int) * urow.size(), cudaMemcpyHostToDevice, s));
   ctx->d.ch_uoff = (int*)dmalloc(ctx, sizeof(int) * (ctx->nch + 1));
   CUDA_TRY(cudaMemcpyAsync(ctx->d.ch_uoff, uoff.data(), sizeof(int) * (ctx->nch + 1), cudaMemcpyHostToDevice, s));
-  auto group_items = [&](int G, std::vector<int4>* out, std::vector<int>* glo, std::vector<int>* ghi) {
+  auto group_items = [&](int G, std::vector<UpdItem>* out, std::vector<int>* glo, std::vector<int>* ghi) {
     size_t n = 0;
     for (int k = 0; k < nsys; k++) {
       if (glo) (*glo)[k] = (int)(out ? out->size() : n);
@@ -1249,7 +1253,10 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
         int nr = uoff[c + 1] - uoff[c], np = ctx->h_npp[c];
         for (int r0 = 0; r0 < nr; r0 += G)
           for (int ab0 = 0; ab0 < np; ab0 += 128) {
-            if (out) out->push_back(make_int4(c, uoff[c] + r0, ab0, std::min(G, nr - r0)));
+            if (out)
+              out->push_back(UpdItem{c, uoff[c] + r0, ab0, std::min(G, nr - r0), np, ctx->h_nhh[c], k,
+                                     ctx->h_vpp[c] ? ctx->h_nlad[c] : 0, ctx->h_pp_off[c], lut[k], ctx->h_t_off[c],
+                                     ctx->h_vhh_off[c], ctx->h_s_off[c]});
             n++;
           }
       }
@@ -1259,7 +1266,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   };
   int G = UPD_ROWS;
   while (G > 1 && group_items(G, nullptr, nullptr, nullptr) < (size_t)8 * nsm) G >>= 1;
-  std::vector<int4> grp;
+  std::vector<UpdItem> grp;
   std::vector<int> glo(nsys), ghi(nsys);
   group_items(G, &grp, &glo, &ghi);
   // static row data of every update item, filled on the device (pairs and energies live there)
@@ -1304,9 +1311,9 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->upd_lo_d = ud;
   ctx->upd_hi_d = ud + nsys;
   ctx->n_grp_items = (int)grp.size();
-  ctx->grp_items = (int4*)dmalloc(ctx, sizeof(int4) * std::max<size_t>(1, grp.size()));
+  ctx->grp_items = (UpdItem*)dmalloc(ctx, sizeof(UpdItem) * std::max<size_t>(1, grp.size()));
   if (!grp.empty()) {
-    CUDA_TRY(cudaMemcpyAsync(ctx->grp_items, grp.data(), sizeof(int4) * grp.size(),
+    CUDA_TRY(cudaMemcpyAsync(ctx->grp_items, grp.data(), sizeof(UpdItem) * grp.size(),
                              cudaMemcpyHostToDevice, s));
     k_rowinfo<<<(unsigned)grp.size(), 32, 0, s>>>(ctx->d, ctx->grp_items, ctx->d.upd_rowinfo);
     CUDA_TRY(cudaGetLastError());
@@ -1345,6 +1352,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   }
   CUDA_TRY(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
   smem_at_least(k_tdig, sizeof(double) * max_nlad);
+  smem_at_least(k_update_mix, upd_mix_smem(ctx));
   smem_at_least(k_pp<double>, PP_SMEM);
   smem_at_least(k_pp<f2>, PP_SMEM);
   CUDA_TRY(cudaStreamSynchronize(s));

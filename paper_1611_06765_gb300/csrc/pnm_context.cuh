@@ -35,7 +35,7 @@ struct pnm_ctx {
 
   // host copies of the channel metadata
   std::vector<int> h_ch_sys, h_key, h_nhh, h_npp, h_hh_off, h_pp_off, h_vpp;
-  std::vector<long> h_t_off, h_x_t_off, h_x_c_off;
+  std::vector<long> h_t_off, h_vhh_off, h_x_t_off, h_x_c_off;
   std::vector<int> h_nlad;               // ladder basis size per channel (0: no V_pppp block)
   std::vector<long> h_s_off, h_vd_off;   // ladder-layout and ladder-V offsets per channel
   long nvdig = 0, ntdig = 0;             // digit words of the ladder V, room for those of the amplitudes
@@ -52,7 +52,7 @@ struct pnm_ctx {
   int4* upd_items = nullptr;  // (channel, ij, first pp column) of the update
   int n_upd_items = 0;
   int *upd_lo_d = nullptr, *upd_hi_d = nullptr;  // per system ranges of the (row, column) items
-  int4* grp_items = nullptr;  // (channel, first ij, first pp column, rows) of the update
+  UpdItem* grp_items = nullptr;  // items of the updates
   int n_grp_items = 0, upd_rows = 1;
   // ph term: work items (pnm_need_ph_items): n_ph_large + n_ph_cta channels that take a CTA, then
   // n_ph_warp of the warp path, the last n_ph_tiny (n_ph_tiny64 with FP64 results) of them tiny

@@ -66,6 +66,15 @@ struct __align__(16) UpdRow {
   double eij;
 };
 
+// Work item of the update kernels: up to UPD_ROWS rows of the list upd_row and 128 pp columns of a
+// channel, with what its CTA would otherwise look up in the channel tables.
+struct __align__(16) UpdItem {
+  int c, r0, ab0, ng;          // channel, first entry of upd_row, first column, rows
+  int npp, nh, sys, nl;        // sizes of the channel, its system, ladder vectors (0: no V_pppp block)
+  int pp_off, lut_off;         // pairs of the channel, interaction table of the system
+  long base, vhh_off, s_off;   // amplitudes, chi_hh, ladder layout
+};
+
 // Device arena pointers; all arrays are global over the systems of the context.
 struct DevState {
   // states

@@ -1161,6 +1161,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   ctx->h_nhh = h_nhh;
   ctx->h_npp = h_npp;
   ctx->h_t_off = h_t_off;
+  ctx->h_vhh_off = h_vhh_off;
   ctx->h_vpp = h_vpp;
   ctx->h_rows = h_rows;
   ctx->h_x_nph = h_x_nph;
