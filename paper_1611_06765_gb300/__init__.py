@@ -176,7 +176,7 @@ class Context:
     def get_amplitudes(self, sys=0):
         n = C.c_size_t()
         _lib.check(_lib.load().pnm_amplitude_labels(self._h, sys, C.byref(n), None))
-        t = np.zeros(n.value)
+        t = np.empty(n.value)  # filled by the call: zeroing 8 MB first cost as much again as copying it
         _lib.check(_lib.load().pnm_get_amplitudes(self._h, sys, _ptr(t), n.value))
         return t
 
@@ -187,14 +187,14 @@ class Context:
     def apply_pp_ladder(self, t, precision=PNM_PREC_FP64, sys=0):
         """pnm_apply_pp_ladder: the pp-ladder term alone applied to amplitudes t."""
         t = np.ascontiguousarray(t, dtype=np.float64)
-        r = np.zeros_like(t)
+        r = np.empty_like(t)
         _lib.check(_lib.load().pnm_apply_pp_ladder(self._h, sys, precision, _ptr(t), _ptr(r), t.size))
         return r
 
     def apply_ph_term(self, t, precision=PNM_PREC_FP64, sys=0):
         """pnm_apply_ph_term: the ph term (linear and quadratic) alone applied to amplitudes t."""
         t = np.ascontiguousarray(t, dtype=np.float64)
-        r = np.zeros_like(t)
+        r = np.empty_like(t)
         _lib.check(_lib.load().pnm_apply_ph_term(self._h, sys, precision, _ptr(t), _ptr(r), t.size))
         return r
 

@@ -1505,26 +1505,24 @@ FinArgs fin_args(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, bool 
 }
 
 template <typename T_>
-static void lad_expand(pnm_ctx* ctx, const T_* rs, int planes, long pstride, double* host_out) {
+static void lad_expand(pnm_ctx* ctx, const T_* rs, int planes, long pstride) {
   cudaStream_t s = ctx->stream;
   if (!ctx->expand_buf) ctx->expand_buf = (double*)dmalloc(ctx, sizeof(double) * std::max<long>(ctx->nt, 1));
   if (ctx->nrows > 0)
     k_lad_expand<T_><<<ctx->nrows, 128, 0, s>>>(ctx->d, rs, planes, pstride, ctx->expand_buf);
   CUDA_TRY(cudaGetLastError());
-  CUDA_TRY(cudaMemcpyAsync(host_out, ctx->expand_buf, sizeof(double) * ctx->nt, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(cudaStreamSynchronize(s));
 }
 
-void pnm_lad_expand(pnm_ctx* ctx, const float* rs, int planes, long pstride, double* host_out) {
-  lad_expand(ctx, rs, planes, pstride, host_out);
+void pnm_lad_expand(pnm_ctx* ctx, const float* rs, int planes, long pstride) {
+  lad_expand(ctx, rs, planes, pstride);
 }
 
-void pnm_lad_expand(pnm_ctx* ctx, const double* rs, int planes, long pstride, double* host_out) {
-  lad_expand(ctx, rs, planes, pstride, host_out);
+void pnm_lad_expand(pnm_ctx* ctx, const double* rs, int planes, long pstride) {
+  lad_expand(ctx, rs, planes, pstride);
 }
 
-void pnm_lad_expand(pnm_ctx* ctx, const f2* rs, int planes, long pstride, double* host_out) {
-  lad_expand(ctx, rs, planes, pstride, host_out);
+void pnm_lad_expand(pnm_ctx* ctx, const f2* rs, int planes, long pstride) {
+  lad_expand(ctx, rs, planes, pstride);
 }
 
 // The pp ladder in the ladder basis: the digits of the amplitudes, then the digit products

@@ -82,8 +82,8 @@ struct pnm_ctx {
   int *row_lo_d = nullptr, *row_hi_d = nullptr, *lut_off_d = nullptr;  // per system
   LoopCtl* ctl = nullptr;     // device
   double* small = nullptr;    // device scratch for single-value queries
-  double* mbpt3_buf = nullptr;
-  double* expand_buf = nullptr;  // the pp ladder in the amplitude layout (operator call)  // per-row partials and per-system results of pnm_mbpt3
+  double* mbpt3_buf = nullptr;   // per-row partials and per-system results of pnm_mbpt3
+  double* expand_buf = nullptr;  // the pp ladder or ph term in the amplitude layout (operator calls)
   SysCtl* sysctl = nullptr;   // device, one per system
   double* hist = nullptr;     // device, (hist_cap) per system
   int hist_cap = 0;
@@ -180,9 +180,9 @@ void pnm_enqueue_loop_body(pnm_ctx* ctx, int mode, bool refine, cudaGraphConditi
 void pnm_prepare_terms(pnm_ctx* ctx, int terms);
 void pnm_mbpt3_all(pnm_ctx* ctx, double* out);
 // The pp ladder from its ladder layout (planes summed) into host memory in the amplitude layout.
-void pnm_lad_expand(pnm_ctx* ctx, const float* rs, int planes, long pstride, double* host_out);
-void pnm_lad_expand(pnm_ctx* ctx, const double* rs, int planes, long pstride, double* host_out);
-void pnm_lad_expand(pnm_ctx* ctx, const f2* rs, int planes, long pstride, double* host_out);
+void pnm_lad_expand(pnm_ctx* ctx, const float* rs, int planes, long pstride);
+void pnm_lad_expand(pnm_ctx* ctx, const double* rs, int planes, long pstride);
+void pnm_lad_expand(pnm_ctx* ctx, const f2* rs, int planes, long pstride);
 // alpha / eps_ij^ab of the current mixed solve (the step of the mixed and refinement updates)
 const double* pnm_mixed_aw(const pnm_ctx* ctx);
 void pnm_enqueue_body_mixed(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h);
