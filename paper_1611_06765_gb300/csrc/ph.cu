@@ -20,8 +20,8 @@
 
 constexpr int PH_WARPS = PH_THREADS / 32;
 // Channels of at most PH_WARP_DIM rows and columns per problem take one warp, the others a CTA; of at
-// most PH_TINY_DIM (FP32, FP32-pair results) or PH_TINY_FP64 (FP64 results) a part of a warp or a warp
-// of the tiny kernels.
+// most PH_TINY_DIM (FP32, FP32-pair results) or PH_TINY_FP64 (FP64 results beside larger channels) a
+// part of a warp or a warp of the tiny kernels.
 constexpr int PH_WARP_DIM = 16, PH_TINY_DIM = 8, PH_TINY_FP64 = 5;
 
 // One cross channel of the term: a problem (S_z > 0) or two of half size (S_z = 0).
@@ -580,13 +580,13 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
 constexpr int TW_THREADS = 256, TW_PARTS = 512;
 __global__ void __launch_bounds__(TW_THREADS) k_tmax(DevState D, const LoopCtl* __restrict__ ctl,
                                                      const long* __restrict__ t_lo, int* __restrict__ parts) {
-  const int sys = blockIdx.y;
+  const int sys = blockIdx.x;
   if (sys_done(D, ctl, sys)) return;
   const double* __restrict__ t = cur_t(D, ctl);
   const long hi = t_lo[sys + 1];
   int e = 1;
 #pragma unroll 4
-  for (long z = t_lo[sys] + blockIdx.x * TW_THREADS + threadIdx.x; z < hi; z += gridDim.x * TW_THREADS)
+  for (long z = t_lo[sys] + blockIdx.y * TW_THREADS + threadIdx.x; z < hi; z += gridDim.y * TW_THREADS)
     e = max(e, dig_exp(t[z]));
   e = __reduce_max_sync(0xffffffffu, e);
   __shared__ int top;
@@ -594,23 +594,23 @@ __global__ void __launch_bounds__(TW_THREADS) k_tmax(DevState D, const LoopCtl* 
   __syncthreads();
   if ((threadIdx.x & 31) == 0) atomicMax(&top, e);
   __syncthreads();
-  if (threadIdx.x == 0) parts[sys * TW_PARTS + blockIdx.x] = top;
+  if (threadIdx.x == 0) parts[sys * TW_PARTS + blockIdx.y] = top;
 }
 
 __global__ void __launch_bounds__(TW_THREADS) k_twords(DevState D, const LoopCtl* __restrict__ ctl,
                                                        const long* __restrict__ t_lo, const int* __restrict__ parts,
                                                        int nparts) {
-  const int sys = blockIdx.y;
+  const int sys = blockIdx.x;
   if (sys_done(D, ctl, sys)) return;
   int e = 1;
   for (int k = threadIdx.x & 31; k < nparts; k += 32) e = max(e, parts[sys * TW_PARTS + k]);
   e = __reduce_max_sync(0xffffffffu, e);
-  if (blockIdx.x == 0 && threadIdx.x == 0) D.sys_texp[sys] = e;
+  if (blockIdx.y == 0 && threadIdx.x == 0) D.sys_texp[sys] = e;
   if (e >= DIG_NONFINITE) return;  // the term is then formed from the FP64 values
   const double* __restrict__ t = cur_t(D, ctl);
   const long hi = t_lo[sys + 1];
 #pragma unroll 4
-  for (long z = t_lo[sys] + blockIdx.x * TW_THREADS + threadIdx.x; z < hi; z += gridDim.x * TW_THREADS)
+  for (long z = t_lo[sys] + blockIdx.y * TW_THREADS + threadIdx.x; z < hi; z += gridDim.y * TW_THREADS)
     D.twords[z] = dig_word(dig_fixed(t[z], e));
 }
 
@@ -619,9 +619,8 @@ __global__ void __launch_bounds__(TW_THREADS) k_twords(DevState D, const LoopCtl
 // pair copy of the amplitudes: a 7 x 7 problem would fill a fifth of a 16 x 8 x 8 block.  120 systems
 // of N = 14, all of whose channels are of this size: 695 us per launch in digits, 145 here (355 with
 // one gather loop per channel in the kernel of the larger channels, at its registers).  In FP64 the
-// line lies lower, the products then share the slow pipe: 28 nucleons, n^2 <= 20, take 94 us per
-// update with a line at 5 and 99 with one at 8; N = 14, n^2 <= 20, whose channels have up to 7 rows,
-// 34.8 and 36.0; n^2 <= 4 (up to 5 rows) 28.5, and in digits 30.
+// line lies lower where larger channels take the digit kernel anyway, the products then share the
+// slow pipe: 28 nucleons, n^2 <= 20, take 94 us per update with a line at 5 and 99 with one at 8.
 // fixed: W [problem][row][column] then <kb|v|cj> [problem][row][column] of the channel.
 template <typename T_>
 __device__ __forceinline__ void ph_tiny(const DevState& D, const PhItem& it, T_* Ts,
@@ -860,16 +859,23 @@ void pnm_need_ph_items(pnm_ctx* ctx) {
     most = std::max(most, dig);
     ctx->ph32_smem = std::max(ctx->ph32_smem, f32);
   }
+  // FP64 results: where no channel is larger than PH_TINY_DIM all take the tiny kernel, which saves
+  // the passes that make the digits (N = 14: the operator call 96 -> 73 us, a solve of one
+  // n^2 <= 24 system 955 -> 852 us, of sixteen 4.82 -> 4.22 ms); beside larger channels the digit
+  // kernel is the faster one from PH_TINY_FP64 + 1 on.
+  bool larger = !cta.empty();
+  for (int d = PH_TINY_DIM + 1; d <= PH_WARP_DIM; d++) larger = larger || !by_dim[d].empty();
+  const int tiny64 = larger ? PH_TINY_FP64 : PH_TINY_DIM;
   for (int d = PH_WARP_DIM; d >= 0; d--) {
     const int n = (int)by_dim[d].size();
     for (int x : by_dim[d]) {
       add(x);
-      if (d > PH_TINY_FP64) ctx->ph_warp_smem = std::max(ctx->ph_warp_smem, dig);
+      if (d > tiny64) ctx->ph_warp_smem = std::max(ctx->ph_warp_smem, dig);
       if (d > PH_TINY_DIM) ctx->ph32_warp_smem = std::max(ctx->ph32_warp_smem, f32);
     }
     ctx->n_ph_warp += n;
     if (d <= PH_TINY_DIM) ctx->n_ph_tiny += n;
-    if (d <= PH_TINY_FP64) ctx->n_ph_tiny64 += n;
+    if (d <= tiny64) ctx->n_ph_tiny64 += n;
   }
   if (std::max(std::max(wf, v1), std::max(src, fixed)) >= (1UL << 32))
     throw PnmError{PNM_EINVAL, "problem too large for 32-bit element maps"};
@@ -932,7 +938,7 @@ static void launch_ph_dig(pnm_ctx* ctx, bool linear, cudaStream_t s, cudaStream_
   const PhItem* items = ctx->ph_items;
   if (nl + n + nw == 0) s_tiny = s;
   if (nl + n + nw > 0) {
-    const dim3 grid(ctx->n_tw_parts, (unsigned)ctx->sys.size());
+    const dim3 grid((unsigned)ctx->sys.size(), ctx->n_tw_parts);
     k_tmax<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts);
     k_twords<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts, ctx->n_tw_parts);
   }
