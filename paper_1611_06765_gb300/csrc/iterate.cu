@@ -952,20 +952,6 @@ void pnm_alpha_inv(pnm_ctx* ctx, double alpha, double* aw) {
   CUDA_TRY(cudaGetLastError());
 }
 
-// Per row (channel, ij) of the amplitudes: 2 if the spin flip maps it onto a later row (it is
-// computed by the updates), 0 onto an earlier one (written by that row's update), 1 onto
-// itself (its columns are paired among themselves).
-__global__ void k_row_mode(DevState D, int nrows, int* __restrict__ mode) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrows) return;
-  int2 it = D.row_item[r];
-  int npp = D.ch_npp[it.x];
-  long z0 = D.ch_t_off[it.x] + (long)it.y * npp;
-  int cd = D.fmap[z0];
-  long f0 = (long)(cd > 0 ? cd : -cd) - 1;
-  mode[r] = (f0 >= z0 && f0 < z0 + npp) ? 1 : (f0 > z0 ? 2 : 0);
-}
-
 // t <- (t + F t) / 2 under the global spin flip F (fmap).  The solution is flip-symmetric
 // and the ph term is formed for flip-symmetric amplitudes, so kept and learned starts are
 // symmetrised first (MBPT2 and zero starts are symmetric already).  A pair (z, F z) is handled
@@ -1218,14 +1204,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   // rows the updates compute: of two rows that the spin flip maps onto each other the one
   // whose amplitudes come first, and the rows it maps onto themselves (half of their
   // columns); per channel a run of the list upd_row, which update items index
-  std::vector<int> rmode(ctx->nrows, 2);
-  if (ctx->nrows > 0) {
-    int* dm = (int*)dmalloc(ctx, sizeof(int) * ctx->nrows);
-    k_row_mode<<<(ctx->nrows + 255) / 256, 256, 0, s>>>(ctx->d, ctx->nrows, dm);
-    CUDA_TRY(cudaMemcpyAsync(rmode.data(), dm, sizeof(int) * ctx->nrows, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-  }
-  ctx->h_row_mode = rmode;
+  const std::vector<int>& rmode = ctx->h_row_mode;
   std::vector<int> urow, uoff(ctx->nch + 1, 0), ucnt(ctx->nch, 0);
   for (int r = 0; r < ctx->nrows; r++)
     if (rmode[r]) ucnt[ctx->h_rows[r].x]++;

@@ -109,10 +109,10 @@ struct pnm_ctx {
   MixedState* mixed = nullptr;
   MlpState* mlp = nullptr;
   f2* vpphh_f2 = nullptr;  // FP32-pair copy of V_pphh (made on first use by the FP32-pair sweeps)
-  // work list of the ladder-basis V (items (channel, first row), per system a run) and the
+  // work list of the ladder-basis V (channel, first row, interaction table and its size) and the
   // shared memory of its kernel; the V itself is built on first use (pnm_need_vdig)
-  int2* vl_items = nullptr;
-  std::vector<int> vl_sys;
+  int4* vl_items = nullptr;
+  int n_vl_items = 0;
   size_t vl_smem = 0;
   double hbar2_2m = 0.0;
   int mlp_fallback = 0;  // 1 when the last learned start was replaced by the MBPT2 start

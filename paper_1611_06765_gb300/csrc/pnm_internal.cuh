@@ -96,17 +96,8 @@ struct DevState {
   int2 *hh_pair, *pp_pair;
   // rows (channel, ij) for the update and energy partials
   int2* row_item;        // (channel, ij)
-  // cross channels
-  int *x_nph, *x_nhp;
-  int* x_sys;            // cross channel -> system
-  long *x_t_off, *x_c_off;
+  // pairs of the cross channels
   int2 *ph_pair, *hp_pair;
-  int* x_ph_off;
-  int* x_hp_off;
-  // global spin flip F: class of each cross channel (+1: S_z > 0, formed in full; 0: S_z = 0,
-  // formed on its spin-up rows; -1: S_z < 0, not formed), the flipped column of every hp
-  // column, and for S_z = 0 channels the spin-up rows and columns (first half of the slots)
-  int *x_cls, *x_fcol, *x_rrow, *x_rcol;
   int* fmap;             // per t element: sign * (index + 1) of its spin-flipped element
   // mixed and FP64 updates: the hole-pair rows they compute (flip representatives), per item
   // a run of this list (items hold (channel, first entry, first column, rows))
