@@ -29,6 +29,7 @@
 #ifndef PNM_UPD_HH_UNROLL
 #define PNM_UPD_HH_UNROLL 4
 #endif
+constexpr int UPD_MIX_UNROLL = 2;  // chunks of a warp of the mixed update in flight
 constexpr int UPD_HH_UNROLL = PNM_UPD_HH_UNROLL;  // loads of the mixed update's hh-ladder pass in flight
 
 
@@ -106,7 +107,10 @@ __global__ void __launch_bounds__(128) k_tstats(DevState D, const LoopCtl* __res
       }
       if (lane == 0) {
         long e = D.ch_vhh_off[c] + (long)kl * nh + ij;
-        io.chi[e] = io.vhh[e] + acc;
+        const T_ chi = io.vhh[e] + acc;
+        // the pair update reads chi as pairs, in the same 8-byte slots
+        if constexpr (PAIR) reinterpret_cast<f2*>(io.chi)[e] = Arith<f2>::from_double(chi);
+        else io.chi[e] = chi;
       }
     }
   } else {
@@ -447,15 +451,12 @@ void pnm_split_f2(const double* a, f2* b, long n, cudaStream_t s) {
 // End of one update: energy (Eq. ccdcorr, sum of v t over restricted amplitudes) and
 // residual norm per system from the block partials in a fixed order, the |dE| test, the
 // energy history, and the loop condition of the device-side loop.
-// It runs alone on one SM after the last block of the update, so its time adds to every update:
-// a chain of dependent round trips, not bandwidth.  Batches of at least FIN_WARP_SYSTEMS systems
-// take one warp per system (no block barrier between systems); fewer take the whole block per
-// system, which reads the several thousand partials of a large system with four times the loads
-// in flight.  FIN_UNROLL partial pairs are requested before the first is added.  120 systems of
-// 27 partials each, mixed solve of 20 updates read back whole: 21.0 -> 16.4 ms against the block
-// taking the systems one after the other (two reductions and three barriers each); a single
-// system of 66 states, 39 updates: 1.143 -> 1.122 ms from the earlier loads.
-constexpr int FIN_WARP_SYSTEMS = 4, FIN_UNROLL = 8;
+// The last CTA of a system closes that system, the last of these the update: a chain of dependent
+// round trips, not bandwidth, that adds to every update, so the systems of a batch go side by side
+// (one CTA closing all 120 systems of 22 partials each, a warp per system, left the GPU idle for half
+// of the update: 141 us, 79 us so).  FIN_UNROLL partial pairs are requested before the first
+// is added.
+constexpr int FIN_UNROLL = 8;
 
 __device__ __forceinline__ void sum_partials(const FinArgs& f, int s, int first, int step, double& e, double& r) {
   const int hi = f.hi[s];
@@ -482,9 +483,10 @@ __device__ __forceinline__ void sum_partials(const FinArgs& f, int s, int first,
 }
 
 // One system's control block from its energy and squared residual (one thread).  S and the loop
-// control c are copies read before the sums, so that their loads overlap the partials'.
-__device__ __forceinline__ void finalize_one(const FinArgs& f, SysCtl S, const LoopCtl& c, int s, double e, double r,
-                                             bool& all_done, bool& bad) {
+// control c are copies read before the sums, so that their loads overlap the partials'.  Returns
+// whether the system has diverged.
+__device__ __forceinline__ bool finalize_one(const FinArgs& f, SysCtl& S, const LoopCtl& c, int s, double e, double r) {
+  bool bad = false;
   if (!S.done) {
     S.iters += 1;
     S.e_new = e;
@@ -494,450 +496,322 @@ __device__ __forceinline__ void finalize_one(const FinArgs& f, SysCtl S, const L
     S.e_old = e;
     S.grow = (diff > 2.0 * S.d_old && diff > S.tol) ? S.grow + 1 : 0;
     S.d_old = diff;
-    bad = bad || !isfinite(e) || !isfinite(r) || S.grow >= PNM_DIVERGE_STEPS;
+    bad = !isfinite(e) || !isfinite(r) || S.grow >= PNM_DIVERGE_STEPS;
     if (diff < S.tol && c.iter + 1 >= c.min_iter) {
       S.done = 1;
       S.frozen_at = c.iter;
     }
     f.sc[s] = S;
   }
-  all_done = all_done && S.done;
+  return bad;
 }
 
-__device__ void finalize_systems(const FinArgs& f, LoopCtl* ctl) {
-  __shared__ double sh32f[32];
-  const LoopCtl c = *ctl;
-  bool all_done = true, bad = false;  // of the systems this thread closes
-  double e, r;
-  if (f.nsys >= FIN_WARP_SYSTEMS) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int s = warp; s < f.nsys; s += nw) {
-      SysCtl S;
-      if (lane == 0) S = f.sc[s];
-      sum_partials(f, s, lane, 32, e, r);
-      e = warp_sum(e);
-      r = warp_sum(r);
-      if (lane == 0) finalize_one(f, S, c, s, e, r, all_done, bad);
-    }
-    all_done = __syncthreads_and(all_done);
-    bad = __syncthreads_or(bad);
-  } else {
-    for (int s = 0; s < f.nsys; s++) {
-      SysCtl S;
-      if (threadIdx.x == 0) S = f.sc[s];
-      sum_partials(f, s, threadIdx.x, blockDim.x, e, r);
-      block_sum2(e, r, sh32f);
-      if (threadIdx.x == 0) finalize_one(f, S, c, s, e, r, all_done, bad);
-    }
-  }
-  if (threadIdx.x == 0) {
-    ctl->iter = c.iter + 1;
-    int cont = 1;
-    if (c.dev_error) {
-      ctl->status = PNM_ETIMEOUT;
-      cont = 0;
-    } else if (bad) {
-      ctl->status = PNM_EDIVERGED;
-      cont = 0;
-    } else if (all_done) {
-      ctl->status = 1;
-      cont = 0;
-    } else if (c.iter + 1 >= c.max_iter) {
-      ctl->status = PNM_ENOTCONV;
-      cont = 0;
-    }
-    if (f.use_cond) cudaGraphSetConditional(f.handle, cont ? 1u : 0u);
-  }
-}
-
-// The last block of a grid to finish runs the finalize step (no waiting: the blocks count
-// themselves out with an atomic after a fence, as in the CUDA threadfence reduction).
-__device__ void last_block_finalize(const FinArgs& f, LoopCtl* ctl) {
-  // only thread 0 wrote the block's partials: its fence orders them before the count
+// The last CTA of system s to finish closes it, and the last system the update (no waiting: CTAs and
+// systems count themselves out with atomics after a fence, as in the CUDA threadfence reduction).
+// Every counter is left at zero for the next update.
+__device__ void finalize_system(const FinArgs& f, LoopCtl* ctl, int s) {
   __shared__ int is_last;
+  __shared__ double sh32f[32];
+  const int ctas = f.hi[s] - f.lo[s];
   __syncthreads();
   if (threadIdx.x == 0) {
+    // only thread 0 wrote the block's partials: its fence orders them before the count
     __threadfence();
-    is_last = (atomicAdd(&ctl->blocks_done, 1) == (int)gridDim.x - 1);
+    is_last = atomicAdd(f.blocks_done + s, 1) == ctas - 1;
   }
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  finalize_systems(f, ctl);
-  if (threadIdx.x == 0) ctl->blocks_done = 0;
+  const LoopCtl c = *ctl;
+  SysCtl S;
+  if (threadIdx.x == 0) S = f.sc[s];
+  double e, r;
+  sum_partials(f, s, threadIdx.x, blockDim.x, e, r);
+  block_sum2(e, r, sh32f);
+  if (threadIdx.x != 0) return;
+  f.blocks_done[s] = 0;
+  bool bad = finalize_one(f, S, c, s, e, r), all_done = S.done;
+  if (f.nsys > 1) {
+    // systems closed, converged and diverged, counted in 21 bits each
+    const unsigned long long one = 1ull | (unsigned long long)(S.done != 0) << 21 | (unsigned long long)bad << 42;
+    const unsigned long long now = atomicAdd(&ctl->closed, one) + one;
+    if ((now & 0x1fffff) != (unsigned)f.nsys) return;
+    ctl->closed = 0;
+    all_done = (now >> 21 & 0x1fffff) == (unsigned)f.nsys;
+    bad = now >> 42 != 0;
+  }
+  ctl->iter = c.iter + 1;
+  int cont = 1;
+  if (c.dev_error) {
+    ctl->status = PNM_ETIMEOUT;
+    cont = 0;
+  } else if (bad) {
+    ctl->status = PNM_EDIVERGED;
+    cont = 0;
+  } else if (all_done) {
+    ctl->status = 1;
+    cont = 0;
+  } else if (c.iter + 1 >= c.max_iter) {
+    ctl->status = PNM_ENOTCONV;
+    cont = 0;
+  }
+  if (f.use_cond) cudaGraphSetConditional(f.handle, cont ? 1u : 0u);
 }
 
 // ---------------------------------------------------------------------------- update
-// One CTA per item (channel, up to UPD_ROWS hole pairs ij, 128 pp columns).  Jacobi step of
-// Eq. (ccd3): the bracket collects v, the non-eps parts of the one-body terms, the pp and hh
-// ladders and P(ij)P(ab) Q; then t_new = bracket / eps_ij^ab and t = alpha t_new + (1 - alpha) t_old.
-// The residual of the amplitude equation is R = bracket - eps_ij^ab t.  The hh ladder is
-// summed in the element arithmetic of T_: FP64, or FP32 pairs from the pair copy of the
-// amplitudes (the sweeps with FP32-pair contractions); everything else is FP64.
-// With FP32 pairs the pp ladder, the hh ladder and the ph term arrive as pairs (the 8-byte
-// slots of rpp and xq) and their sum is formed on the FP32 pipe and converted to FP64 once; the
-// denominator, residual, step (alpha / eps_ij^ab prepared per solve, aw) and energy stay FP64.
-template <typename T_>
-__global__ void __launch_bounds__(128) k_update(DevState D, LoopCtl* __restrict__ ctl,
-                                                const UpdItem* __restrict__ items, FinArgs fa,
-                                                const T_* __restrict__ tpair, const double* __restrict__ aw) {
+// Jacobi step of Eq. (ccd3): the bracket collects v, the non-eps parts of the one-body terms, the pp
+// and hh ladders and P(ij)P(ab) Q; then t_new = bracket / eps_ij^ab and t = alpha t_new + (1 - alpha)
+// t_old.  The residual of the amplitude equation is R = bracket - eps_ij^ab t.
+// One amplitude of each spin-flip pair is computed (the one with the smaller index) and written to
+// both; the pair counts twice in the energy and the residual norm.
+//
+// One thread per amplitude of the rows the updates compute, in the order of the list upd_z (chunks of
+// 32 in one channel, UpdItem; a CTA's chunks in one system), U chunks per warp.  What bounds an update
+// is a chain of dependent round trips, so the chain is three long: the amplitude's index and the
+// chunk's metadata; the streams (t, v, eps, maps), the pair's states and the hh ladder's column; the Q,
+// ladder and one-body values behind them.  A thread per column that goes through eight rows of a
+// channel, as before, has the hh ladder's t column once for eight rows, but idles where a channel has
+// less than 128 columns and walks the chain once for every row or two; the column is a coalesced load
+// that L1 and L2 serve.
+struct UpdSums {  // energy and residual norm, amplitudes with and without a flip of their own
+  double e2 = 0.0, e1 = 0.0, r2 = 0.0, r1 = 0.0;
+  __device__ __forceinline__ void add(bool flip, double v, double out, double R) {
+    if (flip) {
+      e2 = fma(v, out, e2);
+      r2 = fma(R, R, r2);
+    } else {
+      e1 = fma(v, out, e1);
+      r1 = fma(R, R, r1);
+    }
+  }
+};
+
+// Block sums of the energy and the residual norm into the CTA's partials.  The first exchange leaves
+// the energies in one half of the warp and the residuals in the other, so that both are reduced by
+// five additions of the slow FP64 pipe instead of ten.
+__device__ __forceinline__ void upd_partials(const DevState& D, const UpdSums& S) {
+  __shared__ double red[UPD_THREADS / 32][2];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool low = lane < 16;
+  const double e = fma(2.0, S.e2, S.e1), r = fma(2.0, S.r2, S.r1);
+  double x = (low ? e : r) + __shfl_xor_sync(0xffffffffu, low ? r : e, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if ((lane & 15) == 0) red[w][lane >> 4] = x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    D.eparts[blockIdx.x] = (red[0][0] + red[1][0]) + (red[2][0] + red[3][0]);
+    D.rparts[blockIdx.x] = (red[0][1] + red[1][1]) + (red[2][1] + red[3][1]);
+  }
+}
+
+// FP64 update, or (T_ = f2) the update of the sweeps with FP32-pair contractions: the pp ladder, the
+// hh ladder (from the pair copy of the amplitudes) and the ph term are pairs then (the 8-byte slots of
+// rpp and xq) and their sum is formed on the FP32 pipe and converted to FP64 once; the denominator,
+// residual, step (alpha / eps_ij^ab prepared per solve, aw) and energy stay FP64.
+// One FP64 update with the thread-per-column layout and here: N=66, N_max=42 93, 69 us (the FP64 pipe
+// busy for 72% of the time the SMs are); 28 nucleons, N_max=20 27.8, 18.4; N=14, N_max=4 16.4, 12.3.
+template <typename T_, int U>
+__global__ void __launch_bounds__(UPD_THREADS) k_update(DevState D, LoopCtl* __restrict__ ctl,
+                                                        const UpdItem* __restrict__ items,
+                                                        const int* __restrict__ upd_z, FinArgs fa,
+                                                        const T_* __restrict__ tpair, const double* __restrict__ aw) {
   constexpr bool PAIR = std::is_same<T_, f2>::value;
   using A = Arith<T_>;
-  // the hh-ladder factor chi_kl^ij of the item's rows: chs[kl][g], zero for rows past ng;
-  // per row: its hole pair ij and d_i + d_j of the one-body term
-  __shared__ T_ chs[UPD_MAX_NHH][UPD_ROWS];
-  __shared__ double row_dij[UPD_ROWS];
-  __shared__ int row_ij[UPD_ROWS];
-  __shared__ double sh32[32];
   if (ctl->status != 0) return;  // the loop has ended within its body (see pnm_enqueue_loop_body)
-  const UpdItem it = items[blockIdx.x];
-  const int c = it.c, ng = it.ng, npp = it.npp, nh = it.nh, ab = it.ab0 + threadIdx.x;
-  const bool frozen = fa.sc[it.sys].done != 0;
-  if (sys_settled(fa.sc[it.sys], ctl)) {
-    // converged at least two steps ago: both amplitude buffers already hold its values
-    if (threadIdx.x == 0) {
-      D.eparts[blockIdx.x] = 0.0;
-      D.rparts[blockIdx.x] = 0.0;
-    }
-    last_block_finalize(fa, ctl);
-    return;
-  }
-  const bool has_vpp = it.nl != 0;
-  double alpha = ctl->alpha;
-  const double* __restrict__ t = cur_t(D, ctl);
-  double* __restrict__ tn = next_t(D, ctl);
-  const long base = it.base, vho = it.vhh_off;
-  const UpdRow* __restrict__ rt = D.upd_rowinfo + (long)blockIdx.x * UPD_ROWS;
-  if ((int)threadIdx.x < UPD_ROWS) {
-    const UpdRow ri = rt[threadIdx.x];
-    row_ij[threadIdx.x] = ri.ij;
-    row_dij[threadIdx.x] = D.dchi[ri.hx] + D.dchi[ri.hy];
-  }
-  // chi's columns of the item's rows from the row table (one barrier covers both)
-  for (int e = threadIdx.x; e < nh * UPD_ROWS; e += blockDim.x) {
-    int kl = e / UPD_ROWS, g = e % UPD_ROWS;
-    chs[kl][g] = g < ng ? A::from_double(D.chi_hh[vho + (long)kl * nh + rt[g].ij]) : A::zero();
-  }
-  __syncthreads();
-  double esum = 0.0, rsum = 0.0;
-  if (ab < npp) {
-    // hh ladder sum_kl t_ab^kl chi_kl^ij for all rows of the item: one pass over the t column
-    T_ hs[UPD_ROWS];
+  const long chunk0 = (long)blockIdx.x * (U * UPD_THREADS / 32);
+  const int sys = items[chunk0].sys;
+  UpdSums S;
+  // converged at least two steps ago: both amplitude buffers already hold its values, and its sums
+  // are not read any more
+  if (!sys_settled(fa.sc[sys], ctl)) {
+    const bool frozen = fa.sc[sys].done != 0;
+    const double alpha = ctl->alpha;
+    const double* __restrict__ t = cur_t(D, ctl);
+    double* __restrict__ tn = next_t(D, ctl);
+    const T_* __restrict__ tc;
+    if constexpr (PAIR) tc = tpair;
+    else tc = t;
+    const T_* __restrict__ rp = reinterpret_cast<const T_*>(D.rpp);
+    const T_* __restrict__ xq = reinterpret_cast<const T_*>(D.xq);
 #pragma unroll
-    for (int g = 0; g < UPD_ROWS; g++) hs[g] = A::zero();
-    if (!frozen) {
-      const long col = base + ab;
-      const T_* __restrict__ tc;
-      if constexpr (PAIR) tc = tpair;
-      else tc = t;
-#pragma unroll 4
-      for (int kl = 0; kl < nh; kl++) {
-        const T_ tk = tc[col + (long)kl * npp];
-#pragma unroll
-        for (int g = 0; g < UPD_ROWS; g++) A::mac(hs[g], tk, chs[kl][g]);
-      }
-    }
-    int2 p = D.pp_pair[D.ch_pp_off[c] + ab];
-    // one-body part of the bracket: (d_a + d_b - d_i - d_j) t with d_p = chi_p - eps_p
-    double da = D.dchi[p.x] + D.dchi[p.y];
-#pragma unroll
-    for (int g = 0; g < UPD_ROWS; g++) {
-      if (g >= ng) break;
-      long z = base + (long)row_ij[g] * npp + ab;
-      // one amplitude of each spin-flip pair is computed (the one with the smaller index) and
-      // written to both; the pair counts twice in the energy and the residual norm
+    for (int u = 0; u < U; u++) {
+      const long chunk = chunk0 + u * (UPD_THREADS / 32) + (threadIdx.x >> 5);
+      const UpdItem it = items[chunk];
+      const int zi = upd_z[chunk * 32 + (threadIdx.x & 31)];
+      if (zi < 0) continue;  // padding
+      const long z = zi;
       const int fc = D.fmap[z];
       const long f = (long)(fc > 0 ? fc : -fc) - 1;
       if (f < z) continue;
-      const double wgt = f == z ? 1.0 : 2.0;
-      double tz = t[z];
-      double out = tz;
-      double v = D.v_pphh[z];
+      const int e = (int)(z - it.base), ij = e / it.npp, ab = e - ij * it.npp, nh = it.nh, npp = it.npp;
+      const double tz = t[z], v = D.v_pphh[z];
+      double out = tz, R = 0.0;
       if (!frozen) {
-        int4 q = D.qmap[z];
+        const int4 q = D.qmap[z];
+        const int2 p = D.pp_pair[it.pp_off + ab], h = D.hh_pair[it.hh_off + ij];
+        const double den = D.den[z], step = PAIR ? aw[z] : D.inv_den[z];
+        T_ rl = A::zero();
+        if (it.nl) {
+          const int m = D.lad_map[it.pp_off + ab];
+          rl = rp[it.s_off + (long)ij * it.nl + ((m > 0 ? m : -m) - 1)];
+          if (m < 0) rl = A::neg(rl);
+        }
+        const T_ q0 = q.x >= 0 ? xq[q.x] : A::zero(), q1 = q.y >= 0 ? xq[q.y] : A::zero();
+        const T_ q2 = q.z >= 0 ? xq[q.z] : A::zero(), q3 = q.w >= 0 ? xq[q.w] : A::zero();
+        // one-body part of the bracket: (d_a + d_b - d_i - d_j) t with d_p = chi_p - eps_p
+        const double d = (D.dchi[p.x] + D.dchi[p.y]) - (D.dchi[h.x] + D.dchi[h.y]);
+        // hh ladder sum_kl t_ab^kl chi_kl^ij
+        T_ hs = A::zero();
+        const T_* __restrict__ col = tc + it.base + ab;
+        const T_* __restrict__ chi = reinterpret_cast<const T_*>(D.chi_hh) + it.vhh_off + ij;
+#pragma unroll 4
+        for (int kl = 0; kl < nh; kl++) A::mac(hs, col[(long)kl * npp], chi[(long)kl * nh]);
         if constexpr (PAIR) {
           // pp ladder + hh ladder + P(ij)P(ab) Q in FP32 pairs, converted once
-          const f2* __restrict__ rp = reinterpret_cast<const f2*>(D.rpp);
-          const f2* __restrict__ xqp = reinterpret_cast<const f2*>(D.xq);
-          f2 corr = hs[g];
-          if (has_vpp) {
-            int sg;
-            const f2 rl = rp[lad_index(D, c, row_ij[g], ab, sg)];
-            corr = A::add(corr, sg > 0 ? rl : A::neg(rl));
-          }
-          if (q.x >= 0) corr = A::add(corr, xqp[q.x]);
-          if (q.y >= 0) corr = A::sub(corr, xqp[q.y]);
-          if (q.z >= 0) corr = A::sub(corr, xqp[q.z]);
-          if (q.w >= 0) corr = A::add(corr, xqp[q.w]);
-          const double num = fma(da - row_dij[g], tz, v) + A::to_double(corr);
-          const double R = fma(-D.den[z], tz, num);  // bracket - eps_ij^ab t
-          rsum = fma(wgt * R, R, rsum);
-          out = fma(R, aw[z], tz);                   // t + alpha R / eps_ij^ab
+          const f2 corr = A::add(A::sub(A::sub(A::add(A::add(hs, rl), q0), q1), q2), q3);
+          const double num = fma(d, tz, v) + A::to_double(corr);
+          R = fma(-den, tz, num);  // bracket - eps_ij^ab t
+          out = fma(R, step, tz);  // t + alpha R / eps_ij^ab
         } else {
-          double num = v + (da - row_dij[g]) * tz;
-          if (has_vpp) {
-            int sg;
-            double rl = D.rpp[lad_index(D, c, row_ij[g], ab, sg)];
-            num += sg > 0 ? rl : -rl;
-          }
-          num += A::to_double(hs[g]);
-          double ph = 0.0;
-          if (q.x >= 0) ph += D.xq[q.x];
-          if (q.y >= 0) ph -= D.xq[q.y];
-          if (q.z >= 0) ph -= D.xq[q.z];
-          if (q.w >= 0) ph += D.xq[q.w];
-          num += ph;
-          double tnew = num * D.inv_den[z];
-          double R = num - D.den[z] * tz;
-          rsum += wgt * (R * R);
-          out = alpha * tnew + (1.0 - alpha) * tz;
+          const double num = ((fma(d, tz, v) + rl) + hs) + (((q0 - q1) - q2) + q3);
+          R = fma(-den, tz, num);
+          out = fma(alpha, num * step, (1.0 - alpha) * tz);
         }
       }
       tn[z] = out;
       if (f != z) tn[f] = fc > 0 ? out : -out;
-      esum = fma(wgt * v, out, esum);
+      S.add(f != z, v, out, R);
     }
+    upd_partials(D, S);
   }
-  block_sum2(esum, rsum, sh32);
-  if (threadIdx.x == 0) {
-    D.eparts[blockIdx.x] = esum;
-    D.rparts[blockIdx.x] = rsum;
-  }
-  last_block_finalize(fa, ctl);
+  finalize_system(fa, ctl, sys);
+}
+
+template <typename T_>
+static void launch_update(pnm_ctx* ctx, const FinArgs& fa, const T_* tpair, const double* aw) {
+  auto go = [&](auto k) {
+    k<<<ctx->n_upd_ctas, UPD_THREADS, 0, ctx->stream>>>(ctx->d, ctx->ctl, ctx->upd_chunks, ctx->upd_z, fa, tpair, aw);
+  };
+  if (ctx->upd_per_warp == 1) go(k_update<T_, 1>);
+  else if (ctx->upd_per_warp == 2) go(k_update<T_, 2>);
+  else go(k_update<T_, 4>);
 }
 
 void launch_update64(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, bool pair) {
-  if (pair)
-    k_update<f2><<<ctx->n_grp_items, 128, 0, ctx->stream>>>(ctx->d, ctx->ctl, ctx->grp_items,
-                                                            fin_args(ctx, use_cond, h, false), ctx->t_pair,
-                                                            pnm_mixed_aw(ctx));
-  else
-    k_update<double><<<ctx->n_grp_items, 128, 0, ctx->stream>>>(ctx->d, ctx->ctl, ctx->grp_items,
-                                                                fin_args(ctx, use_cond, h, false), nullptr,
-                                                                nullptr);
+  const FinArgs fa = fin_args(ctx, use_cond, h);
+  if (pair) launch_update<f2>(ctx, fa, ctx->t_pair, pnm_mixed_aw(ctx));
+  else launch_update<double>(ctx, fa, nullptr, nullptr);
 }
 
-// Mixed-precision update.  One CTA per item (channel, up to UPD_ROWS hole pairs ij of the rows
-// the updates compute, 128 pp columns); each thread owns one column ab and the item's rows.
-//   hh ladder   sum_kl t_ab^kl chi_kl^ij in FP32 for all rows of the item from one pass over
-//               the FP32 t column (chi's columns of the item's rows staged in shared memory)
+// Mixed-precision update, in the same layout:
+//   hh ladder   sum_kl t_ab^kl chi_kl^ij in FP32 from the FP32 copies
 //   bracket     corrections in FP32: one-body (d_a + d_b - d_i - d_j) t, pp ladder (ladder
 //               layout, k-split planes summed), hh ladder, and the ph term
 //               Q_ij^ab - Q_ji^ab - Q_ij^ba + Q_ji^ba gathered from the cross-channel Q (qmap)
 //   T scatter   the new FP32 amplitude to its four places in the ph term's T (the positions of
 //               the four Q terms, qmap; formed positions only, so the same for the amplitude
 //               and its spin flip), which the next ph kernel reads row by row
-//   FP64        denominator eps_a + eps_b - eps_i - eps_j, residual R = v + bracket - eps_ij^ab t,
-//               step t + alpha R / eps_ij^ab (alpha / eps_ij^ab prepared per solve), energy and
-//               residual partial sums; v = <ab|v|ij> regenerated from the system's interaction
-//               table (bit for bit the stored element, one FP64 addition) instead of streamed
-// Arrays read once per update (t, alpha / eps, flip and Q maps) and the FP64 amplitudes written
-// for the next update are streamed with the evict-first policy, so that the ph term's T and Q
+//   FP64        residual R = v + bracket - eps_ij^ab t, step t + alpha R / eps_ij^ab (alpha / eps_ij^ab
+//               prepared per solve), energy and residual partial sums
+// Arrays read once per update (t, v, eps, alpha / eps, flip and Q maps) and the FP64 amplitudes
+// written for the next update are streamed with the evict-first policy, so that the ph term's T and Q
 // (25 MB each for the held-out batch, read and written at random) and the FP32 amplitudes the
 // next update's contractions read stay in L2.
 // The FP64 unit of a GB300 runs at about 1/64 of its FP32 rate, so the FP64 work is held to
-// eight instructions per amplitude; the new amplitude goes to t (FP64) for itself and to t32 for
-// itself and, sign applied, for its spin flip.  The FP64 flips are not read before the mixed
+// six instructions and two conversions per amplitude (v and eps are read: forming them from the
+// states took three more and two more round trips); the new amplitude goes to t (FP64) for itself and
+// to t32 for itself and, sign applied, for its spin flip.  The FP64 flips are not read before the mixed
 // iteration ends (the update reads t at the amplitudes it computes only); one flip copy of the
 // current buffer fills them then (pnm_flip_copy_current).
-// What bounds it is a chain of dependent round trips per CTA at 24 warps per SM, so the chain is kept
-// short: the item carries the channel's metadata, and the Q positions of all rows are copied
-// asynchronously into the thread's own places of shared memory before the row setup (they wait for
-// nothing else), which leaves one round trip per batch of UPD_BATCH rows (the streams and the four Q
-// gathers together) instead of two.  One update of three N=66, N_max=36 systems: 121 us with metadata
-// by index and positions loaded per batch, 113 us here; 120 twisted N=14, N_max=20 systems 200, 190 us.
-// The t32 column of the hh ladder staged the same way costs more shared memory than it hides: 162 us.
-// All loads of a batch are issued before any store (rows past ng repeat the last row and are
-// discarded).
-__global__ void __launch_bounds__(128, UPD_MIN_BLOCKS) k_update_mix(DevState D, LoopCtl* __restrict__ ctl,
-                                                    const UpdItem* __restrict__ items, FinArgs fa,
-                                                    const float* __restrict__ rpp, const float* __restrict__ xq,
-                                                    const double* __restrict__ aw, float* __restrict__ xt,
-                                                    int nplanes, long pstride) {
-  // dynamic: Q positions [row][column], chi32[kl][ij of row g] at kl * UPD_ROWS + g
-  extern __shared__ __align__(16) unsigned char upd_sm[];
-  __shared__ float row_dij[UPD_ROWS];
-  __shared__ double row_eij[UPD_ROWS];
-  __shared__ int row_ij[UPD_ROWS];
-  __shared__ char4 row_si[UPD_ROWS], row_sj[UPD_ROWS];
-  __shared__ double red[2][128];
+// One update with the thread-per-column layout and here: three N=66, N_max=36 systems 113, 90 us; 120
+// twisted N=14, N_max=20 systems 190, 79; one of these 14.3, 12.3.
+template <int U>
+__global__ void __launch_bounds__(UPD_THREADS, UPD_MIN_BLOCKS) k_update_mix(
+    DevState D, LoopCtl* __restrict__ ctl, const UpdItem* __restrict__ items, const int* __restrict__ upd_z, FinArgs fa,
+    const float* __restrict__ rpp, const float* __restrict__ xq, const double* __restrict__ aw, float* __restrict__ xt,
+    int nplanes, long pstride) {
   if (ctl->status != 0) return;  // the loop has ended within its body (see pnm_enqueue_loop_body)
-  const UpdItem it = items[blockIdx.x];
-  const int ng = it.ng, npp = it.npp, nh = it.nh, ab = it.ab0 + threadIdx.x;
-  int4* qsm = reinterpret_cast<int4*>(upd_sm) + threadIdx.x;
-  float* chs = reinterpret_cast<float*>(upd_sm + sizeof(int4) * 128 * UPD_ROWS);
-  const bool col = ab < npp;
-  const long base = it.base;
-  const float* __restrict__ t32 = cur_t32(D, ctl);
-  const UpdRow* __restrict__ rt = D.upd_rowinfo + (long)blockIdx.x * UPD_ROWS;
-  // the column's pair data does not depend on the rows: loaded beside the row setup
-  int2 p = make_int2(0, 0);
-  int lmap = 0;
-  if (col) {
-    for (int g = 0; g < ng; g++)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(qsm + g * 128)),
-                   "l"(D.qmap + base + (long)rt[g].ij * npp + ab)
-                   : "memory");
-    p = D.pp_pair[it.pp_off + ab];
-    if (it.nl) lmap = D.lad_map[it.pp_off + ab];
-  }
-  if ((int)threadIdx.x < UPD_ROWS) {
-    const UpdRow ri = rt[threadIdx.x];
-    row_ij[threadIdx.x] = ri.ij;
-    row_dij[threadIdx.x] = D.dchi32[ri.hx] + D.dchi32[ri.hy];
-    row_eij[threadIdx.x] = ri.eij;
-    row_si[threadIdx.x] = ri.si;
-    row_sj[threadIdx.x] = ri.sj;
-  }
-  float dab = 0.0f;
-  double eab = 0.0;
-  char4 sa = make_char4(0, 0, 0, 0), sb = sa;
-  if (col) {
-    dab = D.dchi32[p.x] + D.dchi32[p.y];
-    eab = D.eps[p.x] + D.eps[p.y];
-    sa = D.nvec[p.x];
-    sb = D.nvec[p.y];
-  }
-  const bool frozen = fa.sc[it.sys].done != 0;
-  if (sys_settled(fa.sc[it.sys], ctl)) {
-    // converged at least two steps ago: both amplitude buffers already hold its values
-    if (threadIdx.x == 0) {
-      D.eparts[blockIdx.x] = 0.0;
-      D.rparts[blockIdx.x] = 0.0;
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    last_block_finalize(fa, ctl);
-    return;
-  }
-  // chi's columns of the item's rows, their indices read from the row table (no wait for the
-  // row setup above: one barrier covers both)
-  if (!frozen) {
-    const float* __restrict__ chi = D.chi32 + it.vhh_off;
-    for (int e = threadIdx.x; e < nh * UPD_ROWS; e += blockDim.x) {
-      const int kl = e / UPD_ROWS, g = e % UPD_ROWS;
-      chs[e] = g < ng ? chi[(long)kl * nh + rt[g].ij] : 0.0f;
-    }
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
-  const double* __restrict__ t = cur_t(D, ctl);
-  double* __restrict__ tn = next_t(D, ctl);
-  float* __restrict__ t32n = next_t32(D, ctl);
-  // energy and residual sums of the amplitudes whose spin flip is another amplitude (counted
-  // twice) and of those that are their own flip (counted once)
-  double e2 = 0.0, e1 = 0.0, r2 = 0.0, r1 = 0.0;
-  if (col) {
-    float hh[UPD_ROWS];
-#pragma unroll
-    for (int g = 0; g < UPD_ROWS; g++) hh[g] = 0.0f;
-    if (!frozen) {
+  const long chunk0 = (long)blockIdx.x * (U * UPD_THREADS / 32);
+  const int sys = items[chunk0].sys;
+  UpdSums S;
+  // converged at least two steps ago: both amplitude buffers already hold its values, and its sums
+  // are not read any more
+  if (!sys_settled(fa.sc[sys], ctl)) {
+    const bool frozen = fa.sc[sys].done != 0;
+    const double* __restrict__ t = cur_t(D, ctl);
+    const float* __restrict__ t32 = cur_t32(D, ctl);
+    double* __restrict__ tn = next_t(D, ctl);
+    float* __restrict__ t32n = next_t32(D, ctl);
+#pragma unroll (U < UPD_MIX_UNROLL ? U : UPD_MIX_UNROLL)
+    for (int u = 0; u < U; u++) {
+      const long chunk = chunk0 + u * (UPD_THREADS / 32) + (threadIdx.x >> 5);
+      const UpdItem it = items[chunk];
+      const int zi = upd_z[chunk * 32 + (threadIdx.x & 31)];
+      if (zi < 0) continue;  // padding
+      const long z = zi;
+      const int e = (int)(z - it.base), ij = e / it.npp, ab = e - ij * it.npp, nh = it.nh, npp = it.npp;
+      const double tz = __ldcs(t + z), wz = __ldcs(aw + z), v = __ldcs(D.v_pphh + z), den = __ldcs(D.den + z);
+      const int fc = __ldcs(D.fmap + z);
+      const int4 qm = __ldcs(D.qmap + z);
+      const float t32z = t32[z];
+      const int2 p = D.pp_pair[it.pp_off + ab], h = D.hh_pair[it.hh_off + ij];
+      float rl = 0.0f;
+      if (it.nl) {
+        const int m = D.lad_map[it.pp_off + ab];
+        const long zl = it.s_off + (long)ij * it.nl + ((m > 0 ? m : -m) - 1);
+        for (int pl = 0; pl < nplanes; pl++) rl += rpp[pl * pstride + zl];
+        if (m < 0) rl = -rl;
+      }
+      // P(ij)P(ab) Q: Q_ij^ab - Q_ji^ab - Q_ij^ba + Q_ji^ba from the cross-channel layout
+      const float a0 = qm.x >= 0 ? xq[qm.x] : 0.0f, a1 = qm.y >= 0 ? xq[qm.y] : 0.0f;
+      const float a2 = qm.z >= 0 ? xq[qm.z] : 0.0f, a3 = qm.w >= 0 ? xq[qm.w] : 0.0f;
+      const float d = (D.dchi32[p.x] + D.dchi32[p.y]) - (D.dchi32[h.x] + D.dchi32[h.y]);
+      float hh = 0.0f;
+      if (!frozen) {
+        const float* __restrict__ col = t32 + it.base + ab;
+        const float* __restrict__ chi = D.chi32 + it.vhh_off + ij;
 #pragma unroll UPD_HH_UNROLL
-      for (int kl = 0; kl < nh; kl++) {
-        const float tk = t32[base + ab + (long)kl * npp];
-        const float4 c0 = *reinterpret_cast<const float4*>(chs + kl * UPD_ROWS);
-        const float4 c1 = *reinterpret_cast<const float4*>(chs + kl * UPD_ROWS + 4);
-        hh[0] = fmaf(tk, c0.x, hh[0]); hh[1] = fmaf(tk, c0.y, hh[1]);
-        hh[2] = fmaf(tk, c0.z, hh[2]); hh[3] = fmaf(tk, c0.w, hh[3]);
-        hh[4] = fmaf(tk, c1.x, hh[4]); hh[5] = fmaf(tk, c1.y, hh[5]);
-        hh[6] = fmaf(tk, c1.z, hh[6]); hh[7] = fmaf(tk, c1.w, hh[7]);
+        for (int kl = 0; kl < nh; kl++) hh = fmaf(col[(long)kl * npp], chi[(long)kl * nh], hh);
+      }
+      // one amplitude of each spin-flip pair is computed (the smaller index) and written to both
+      const long f = (long)(fc > 0 ? fc : -fc) - 1;
+      if (f < z) continue;
+      double out = tz, R = 0.0;
+      if (!frozen) {
+        const float corr = d * t32z + (rl + hh) + ((a0 - a1) - (a2 - a3));
+        R = fma(-den, tz, v) + (double)corr;  // bracket - eps_ij^ab t
+        out = fma(R, wz, tz);
+      }
+      const float o32 = (float)out;
+      __stcs(tn + z, out);
+      t32n[z] = o32;
+      if (f != z) t32n[f] = fc < 0 ? -o32 : o32;
+      S.add(f != z, v, out, R);
+      if (!frozen) {
+        // the T positions of t_ij^ab, t_ji^ab, t_ij^ba, t_ji^ba (the Q positions of the same
+        // amplitude; stores only, nothing waits on them)
+        if (qm.x >= 0) xt[qm.x] = o32;
+        if (qm.y >= 0) xt[qm.y] = -o32;
+        if (qm.z >= 0) xt[qm.z] = -o32;
+        if (qm.w >= 0) xt[qm.w] = o32;
       }
     }
-    const double* __restrict__ lut = D.lut + it.lut_off;
-    // the pp ladder's element in the ladder layout: s_off + ij * n_lad + |m| - 1, sign of m
-    const int nl = it.nl;
-    const bool has_vpp = nl != 0, lneg = lmap < 0;
-    const long lad0 = it.s_off + ((lmap > 0 ? lmap : -lmap) - 1);
-#pragma unroll
-    for (int gb = 0; gb < UPD_ROWS; gb += UPD_BATCH) {
-      if (gb >= ng) break;
-      long z[UPD_BATCH];
-      double tz[UPD_BATCH], wz[UPD_BATCH];
-      int fc[UPD_BATCH];
-      float part[UPD_BATCH], qs[UPD_BATCH], t32z[UPD_BATCH];
-#pragma unroll
-      for (int j = 0; j < UPD_BATCH; j++) {
-        const int g = min(gb + j, ng - 1);
-        z[j] = base + (long)row_ij[g] * npp + ab;
-        tz[j] = __ldcs(t + z[j]);
-        wz[j] = __ldcs(aw + z[j]);
-        fc[j] = __ldcs(D.fmap + z[j]);
-        t32z[j] = t32[z[j]];
-        float rl = 0.0f;
-        if (has_vpp) {
-          const long zl = lad0 + (long)row_ij[g] * nl;
-          for (int pl = 0; pl < nplanes; pl++) rl += rpp[pl * pstride + zl];
-          if (lneg) rl = -rl;
-        }
-        part[j] = rl;
-        // P(ij)P(ab) Q: Q_ij^ab - Q_ji^ab - Q_ij^ba + Q_ji^ba from the cross-channel layout
-        const int4 qm = qsm[g * 128];
-        const float a0 = qm.x >= 0 ? xq[qm.x] : 0.0f, a1 = qm.y >= 0 ? xq[qm.y] : 0.0f;
-        const float a2 = qm.z >= 0 ? xq[qm.z] : 0.0f, a3 = qm.w >= 0 ? xq[qm.w] : 0.0f;
-        qs[j] = (a0 - a1) - (a2 - a3);
-      }
-#pragma unroll
-      for (int j = 0; j < UPD_BATCH; j++) {
-        const int g = gb + j;
-        if (g >= ng) break;
-        // one amplitude of each spin-flip pair is computed (the smaller index) and written to both
-        const long f = (long)(fc[j] > 0 ? fc[j] : -fc[j]) - 1;
-        if (f < z[j]) continue;
-        const double v = v_minnesota_as(sa, sb, row_si[g], row_sj[g], lut);
-        double out = tz[j], R = 0.0;
-        if (!frozen) {
-          const float corr = (dab - row_dij[g]) * t32z[j] + (part[j] + hh[g]) + qs[j];
-          R = fma(eab - row_eij[g], tz[j], v) + (double)corr;  // bracket - eps_ij^ab t
-          out = fma(R, wz[j], tz[j]);
-        }
-        const float o32 = (float)out;
-        __stcs(tn + z[j], out);
-        t32n[z[j]] = o32;
-        if (f != z[j]) {
-          t32n[f] = fc[j] < 0 ? -o32 : o32;
-          e2 = fma(v, out, e2);
-          r2 = fma(R, R, r2);
-        } else {
-          e1 = fma(v, out, e1);
-          r1 = fma(R, R, r1);
-        }
-        if (!frozen) {
-          // the T positions of t_ij^ab, t_ji^ab, t_ij^ba, t_ji^ba (the Q positions of the same
-          // amplitude; stores only, nothing waits on them)
-          const int4 qm = qsm[g * 128];
-          if (qm.x >= 0) xt[qm.x] = o32;
-          if (qm.y >= 0) xt[qm.y] = -o32;
-          if (qm.z >= 0) xt[qm.z] = -o32;
-          if (qm.w >= 0) xt[qm.w] = o32;
-        }
-      }
-    }
+    upd_partials(D, S);
   }
-  // block sums: per thread in FP64, then 128 values per sum added by one warp
-  red[0][threadIdx.x] = fma(2.0, e2, e1);
-  red[1][threadIdx.x] = fma(2.0, r2, r1);
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double es = (red[0][threadIdx.x] + red[0][threadIdx.x + 32]) + (red[0][threadIdx.x + 64] + red[0][threadIdx.x + 96]);
-    double rs = (red[1][threadIdx.x] + red[1][threadIdx.x + 32]) + (red[1][threadIdx.x + 64] + red[1][threadIdx.x + 96]);
-    es = warp_sum(es);
-    rs = warp_sum(rs);
-    if (threadIdx.x == 0) {
-      D.eparts[blockIdx.x] = es;
-      D.rparts[blockIdx.x] = rs;
-    }
-  }
-  last_block_finalize(fa, ctl);
-}
-
-static size_t upd_mix_smem(const pnm_ctx* ctx) {
-  return sizeof(int4) * 128 * UPD_ROWS + sizeof(float) * UPD_ROWS * (size_t)ctx->max_nhh;
+  finalize_system(fa, ctl, sys);
 }
 
 void launch_update_mix(pnm_ctx* ctx, const float* rpp, const float* xq, const double* aw, float* xt, int use_cond,
                        cudaGraphConditionalHandle h, int nplanes, long pstride) {
-  k_update_mix<<<ctx->n_grp_items, 128, upd_mix_smem(ctx), ctx->stream>>>(ctx->d, ctx->ctl, ctx->grp_items,
-                                                                          fin_args(ctx, use_cond, h, false), rpp, xq, aw,
-                                                                          xt, nplanes, pstride);
+  const FinArgs fa = fin_args(ctx, use_cond, h);
+  auto go = [&](auto k) {
+    k<<<ctx->n_upd_ctas, UPD_THREADS, 0, ctx->stream>>>(ctx->d, ctx->ctl, ctx->upd_chunks, ctx->upd_z, fa, rpp, xq, aw, xt,
+                                                        nplanes, pstride);
+  };
+  if (ctx->upd_per_warp == 1) go(k_update_mix<1>);
+  else if (ctx->upd_per_warp == 2) go(k_update_mix<2>);
+  else go(k_update_mix<4>);
 }
 
 // alpha / eps_ij^ab per amplitude (the step of the mixed update).
@@ -1063,9 +937,9 @@ __global__ void k_reduce_rows(const double* __restrict__ parts, const int* __res
 __global__ void k_start(const double* __restrict__ parts, const int* __restrict__ row_lo,
                         const int* __restrict__ row_hi, int nsys, SysCtl* __restrict__ sc,
                         LoopCtl* __restrict__ ctl, double* __restrict__ hist, int hist_cap) {
-  // one warp per system in batches (as in finalize_systems), else the whole block
+  // one warp per system in batches, else the whole block
   __shared__ double sh32[32];
-  const bool by_warp = nsys >= FIN_WARP_SYSTEMS;
+  const bool by_warp = nsys >= 4;
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int s = by_warp ? threadIdx.x >> 5 : 0; s < nsys; s += by_warp ? nw : 1) {
     double acc = 0.0;
@@ -1084,7 +958,6 @@ __global__ void k_start(const double* __restrict__ parts, const int* __restrict_
   if (threadIdx.x == 0) {
     ctl->iter = 0;
     ctl->status = 0;
-    ctl->blocks_done = 0;
     ctl->dev_error = 0;
   }
 }
@@ -1093,22 +966,13 @@ __global__ void k_start(const double* __restrict__ parts, const int* __restrict_
 
 static void* dmalloc(pnm_ctx* ctx, size_t bytes) { return pnm_ctx_alloc(ctx, bytes); }
 
-// Static row data of the update items: row g of item i is the (min(g, ng - 1))-th row of its run.
-__global__ void k_rowinfo(DevState D, const UpdItem* __restrict__ items, UpdRow* __restrict__ out) {
-  const int g = threadIdx.x;
-  if (g >= UPD_ROWS) return;
-  const UpdItem it = items[blockIdx.x];
-  const int c = it.c, ij = D.upd_row[it.r0 + min(g, it.ng - 1)];
-  const int2 h = D.hh_pair[D.ch_hh_off[c] + ij];
-  UpdRow r;
-  r.ij = ij;
-  r.hx = h.x;
-  r.hy = h.y;
-  r.pad = 0;
-  r.si = D.nvec[h.x];
-  r.sj = D.nvec[h.y];
-  r.eij = D.eps[h.x] + D.eps[h.y];
-  out[(long)blockIdx.x * UPD_ROWS + g] = r;
+// Amplitudes of the update chunks: rows of the channel's run of upd_row one after the other.
+__global__ void k_upd_list(DevState D, const UpdItem* __restrict__ items, long n, int* __restrict__ upd_z) {
+  const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const UpdItem it = items[k >> 5];
+  const int e = it.e0 + (int)(k & 31), r = e / it.npp;
+  upd_z[k] = e < it.ne ? (int)(it.base + (long)D.upd_row[it.uoff + r] * it.npp + (e - r * it.npp)) : -1;
 }
 
 // pp items of nr[c] rows per channel in the order of decreasing work, so that the last CTAs are
@@ -1188,8 +1052,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
     max_nlad = std::max(max_nlad, nl);
   }
   // per-row items (channel, ij, first column), 128 columns each, grouped by system (the
-  // learned-start kernels); update items (channel, first ij, first column, rows) with up to
-  // UPD_ROWS hole pairs each, fewer when the grid would not fill the GPU
+  // learned-start kernels)
   for (int k = 0; k < nsys; k++) {
     ulo[k] = (int)upd.size();
     for (int r = ctx->sys[k].row_begin; r < ctx->sys[k].row_end; r++) {
@@ -1224,33 +1087,32 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
     CUDA_TRY(cudaMemcpyAsync(ctx->d.upd_row, urow.data(), sizeof(int) * urow.size(), cudaMemcpyHostToDevice, s));
   ctx->d.ch_uoff = (int*)dmalloc(ctx, sizeof(int) * (ctx->nch + 1));
   CUDA_TRY(cudaMemcpyAsync(ctx->d.ch_uoff, uoff.data(), sizeof(int) * (ctx->nch + 1), cudaMemcpyHostToDevice, s));
-  auto group_items = [&](int G, std::vector<UpdItem>* out, std::vector<int>* glo, std::vector<int>* ghi) {
-    size_t n = 0;
-    for (int k = 0; k < nsys; k++) {
-      if (glo) (*glo)[k] = (int)(out ? out->size() : n);
-      for (int c = ctx->sys[k].ch_begin; c < ctx->sys[k].ch_end; c++) {
-        int nr = uoff[c + 1] - uoff[c], np = ctx->h_npp[c];
-        for (int r0 = 0; r0 < nr; r0 += G)
-          for (int ab0 = 0; ab0 < np; ab0 += 128) {
-            if (out)
-              out->push_back(UpdItem{c, uoff[c] + r0, ab0, std::min(G, nr - r0), np, ctx->h_nhh[c], k,
-                                     ctx->h_vpp[c] ? ctx->h_nlad[c] : 0, ctx->h_pp_off[c], lut[k], ctx->h_t_off[c],
-                                     ctx->h_vhh_off[c], ctx->h_s_off[c]});
-            n++;
-          }
-      }
-      if (ghi) (*ghi)[k] = (int)(out ? out->size() : n);
-    }
-    return n;
-  };
-  int G = UPD_ROWS;
-  while (G > 1 && group_items(G, nullptr, nullptr, nullptr) < (size_t)8 * nsm) G >>= 1;
-  std::vector<UpdItem> grp;
+  // Chunks of the updates: 32 amplitudes of one channel each (its last is padded), a CTA's in one
+  // system (padded chunks past its end).  A warp takes more than one where the GPU stays full: fewer
+  // partial sums for the last CTA to add, and the block sums' FP64 additions count for more amplitudes.
+  std::vector<UpdItem> chunks;
   std::vector<int> glo(nsys), ghi(nsys);
-  group_items(G, &grp, &glo, &ghi);
-  // static row data of every update item, filled on the device (pairs and energies live there)
-  ctx->d.upd_rowinfo = (UpdRow*)dmalloc(ctx, sizeof(UpdRow) * UPD_ROWS * std::max<size_t>(1, grp.size()));
-  ctx->upd_rows = G;
+  long n_chunks = 0;
+  for (int c = 0; c < ctx->nch; c++) n_chunks += ((long)(uoff[c + 1] - uoff[c]) * ctx->h_npp[c] + 31) / 32;
+  const int warps = UPD_THREADS / 32;
+  ctx->upd_per_warp = 4;
+  while (ctx->upd_per_warp > 1 && n_chunks < (long)UPD_FULL * nsm * warps * ctx->upd_per_warp) ctx->upd_per_warp >>= 1;
+  const int per_cta = warps * ctx->upd_per_warp;
+  chunks.reserve(n_chunks + (size_t)per_cta * nsys);
+  for (int k = 0; k < nsys; k++) {
+    glo[k] = (int)(chunks.size() / per_cta);
+    for (int c = ctx->sys[k].ch_begin; c < ctx->sys[k].ch_end; c++) {
+      const int np = ctx->h_npp[c], ne = (uoff[c + 1] - uoff[c]) * np;
+      for (int e0 = 0; e0 < ne; e0 += 32)
+        chunks.push_back(UpdItem{e0, ne, uoff[c], np, ctx->h_nhh[c], k, ctx->h_vpp[c] ? ctx->h_nlad[c] : 0,
+                                 ctx->h_pp_off[c], ctx->h_hh_off[c], 0, ctx->h_t_off[c], ctx->h_vhh_off[c],
+                                 ctx->h_s_off[c]});
+    }
+    // at least one CTA per system: it closes the system's update
+    while (chunks.size() % per_cta || (int)(chunks.size() / per_cta) == glo[k]) chunks.push_back(UpdItem{0, 0, 0, 1, 0, k, 0, 0, 0, 0, 0, 0, 0});
+    ghi[k] = (int)(chunks.size() / per_cta);
+  }
+  ctx->n_upd_ctas = (int)(chunks.size() / per_cta);
   ctx->max_npp = max_npp;
   ctx->max_nlad = max_nlad;
   std::vector<int> alo(nsys), ahi(nsys);
@@ -1289,12 +1151,12 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   CUDA_TRY(cudaMemcpyAsync(ud + nsys, uhi.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, s));
   ctx->upd_lo_d = ud;
   ctx->upd_hi_d = ud + nsys;
-  ctx->n_grp_items = (int)grp.size();
-  ctx->grp_items = (UpdItem*)dmalloc(ctx, sizeof(UpdItem) * std::max<size_t>(1, grp.size()));
-  if (!grp.empty()) {
-    CUDA_TRY(cudaMemcpyAsync(ctx->grp_items, grp.data(), sizeof(UpdItem) * grp.size(),
-                             cudaMemcpyHostToDevice, s));
-    k_rowinfo<<<(unsigned)grp.size(), 32, 0, s>>>(ctx->d, ctx->grp_items, ctx->d.upd_rowinfo);
+  ctx->upd_chunks = (UpdItem*)dmalloc(ctx, sizeof(UpdItem) * std::max<size_t>(1, chunks.size()));
+  ctx->upd_z = (int*)dmalloc(ctx, sizeof(int) * 32 * std::max<size_t>(1, chunks.size()));
+  if (!chunks.empty()) {
+    const long n = 32 * (long)chunks.size();
+    CUDA_TRY(cudaMemcpyAsync(ctx->upd_chunks, chunks.data(), sizeof(UpdItem) * chunks.size(), cudaMemcpyHostToDevice, s));
+    k_upd_list<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ctx->d, ctx->upd_chunks, n, ctx->upd_z);
     CUDA_TRY(cudaGetLastError());
   }
   int* gd = (int*)dmalloc(ctx, sizeof(int) * 2 * nsys);
@@ -1303,7 +1165,7 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->grp_lo_d = gd;
   ctx->grp_hi_d = gd + nsys;
   // partial sums: one per update item (at least one per row for init/MBPT2)
-  size_t nparts = std::max<size_t>(upd.size(), (size_t)ctx->nrows);
+  size_t nparts = std::max<size_t>(std::max<size_t>(upd.size(), ctx->n_upd_ctas), (size_t)ctx->nrows);
   ctx->d.eparts = (double*)dmalloc(ctx, sizeof(double) * nparts);
   ctx->d.rparts = (double*)dmalloc(ctx, sizeof(double) * nparts);
   int mx = 0;
@@ -1311,6 +1173,8 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->max_x_dim = mx;
   ctx->ctl = (LoopCtl*)dmalloc(ctx, sizeof(LoopCtl));
   CUDA_TRY(cudaMemsetAsync(ctx->ctl, 0, sizeof(LoopCtl), s));
+  ctx->blocks_done = (int*)dmalloc(ctx, sizeof(int) * nsys);
+  CUDA_TRY(cudaMemsetAsync(ctx->blocks_done, 0, sizeof(int) * nsys, s));
   ctx->small = (double*)dmalloc(ctx, sizeof(double) * 8);
   ctx->sysctl = (SysCtl*)dmalloc(ctx, sizeof(SysCtl) * nsys);
   CUDA_TRY(cudaMemsetAsync(ctx->sysctl, 0, sizeof(SysCtl) * nsys, s));
@@ -1331,7 +1195,6 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   }
   CUDA_TRY(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
   smem_at_least(k_tdig, sizeof(double) * max_nlad);
-  smem_at_least(k_update_mix, upd_mix_smem(ctx));
   smem_at_least(k_pp<double>, PP_SMEM);
   smem_at_least(k_pp<f2>, PP_SMEM);
   CUDA_TRY(cudaStreamSynchronize(s));
@@ -1467,14 +1330,14 @@ void pnm_launch_mbpt2_into(const pnm_ctx* ctx, double* partials, double* results
 }
 
 // The body of one update, enqueued on the context stream (FP64 path).
-// per_row: partials of the per-row mixed update (items upd_items), else of the grouped update.
-FinArgs fin_args(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, bool per_row) {
+FinArgs fin_args(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h) {
   FinArgs f;
   f.eparts = ctx->d.eparts;
   f.rparts = ctx->d.rparts;
-  f.lo = per_row ? ctx->upd_lo_d : ctx->grp_lo_d;
-  f.hi = per_row ? ctx->upd_hi_d : ctx->grp_hi_d;
+  f.lo = ctx->grp_lo_d;
+  f.hi = ctx->grp_hi_d;
   f.nsys = (int)ctx->sys.size();
+  f.blocks_done = ctx->blocks_done;
   f.sc = ctx->sysctl;
   f.hist = ctx->hist;
   f.hist_cap = ctx->hist_cap;

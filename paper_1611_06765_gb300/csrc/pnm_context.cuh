@@ -52,8 +52,9 @@ struct pnm_ctx {
   int4* upd_items = nullptr;  // (channel, ij, first pp column) of the update
   int n_upd_items = 0;
   int *upd_lo_d = nullptr, *upd_hi_d = nullptr;  // per system ranges of the (row, column) items
-  UpdItem* grp_items = nullptr;  // items of the updates
-  int n_grp_items = 0, upd_rows = 1;
+  UpdItem* upd_chunks = nullptr;  // of the updates: chunks of 32 amplitudes, and the amplitudes
+  int* upd_z = nullptr;
+  int n_upd_ctas = 0, upd_per_warp = 1;
   // ph term: work items (pnm_need_ph_items): n_ph_large + n_ph_cta channels that take a CTA, then
   // n_ph_warp of the warp path, the last n_ph_tiny (n_ph_tiny64 with FP64 results) of them tiny
   PhItem* ph_items = nullptr;
@@ -85,6 +86,7 @@ struct pnm_ctx {
   double* mbpt3_buf = nullptr;   // per-row partials and per-system results of pnm_mbpt3
   double* expand_buf = nullptr;  // the pp ladder or ph term in the amplitude layout (operator calls)
   SysCtl* sysctl = nullptr;   // device, one per system
+  int* blocks_done = nullptr; // device, one per system
   double* hist = nullptr;     // device, (hist_cap) per system
   int hist_cap = 0;
   int last_iters_host = 0;
@@ -212,7 +214,7 @@ int* pnm_mlp_err(pnm_ctx* ctx);
 void prof_begin(pnm_ctx* ctx, int kid);
 void prof_end(pnm_ctx* ctx);
 void prof_collect(pnm_ctx* ctx);
-FinArgs fin_args(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h, bool per_row);
+FinArgs fin_args(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h);
 void pnm_enqueue_stats(pnm_ctx* ctx, bool mixed, bool pair = false);
 void pnm_launch_pp(pnm_ctx* ctx, cudaStream_t s, bool rep_only, bool pair);
 void launch_ph_f2(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny);

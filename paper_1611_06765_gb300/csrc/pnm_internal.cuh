@@ -58,20 +58,12 @@ struct SysInfo {
   double phi[3];          // twist theta / (2 pi) per axis; all zero = periodic
 };
 
-// Static data of one row (hole pair ij) of an update item: the pair's states, their spin labels
-// and eps_i + eps_j, so that an update's row setup is one load and the one-body gathers.
-struct __align__(16) UpdRow {
-  int ij, hx, hy, pad;
-  char4 si, sj;
-  double eij;
-};
-
-// Work item of the update kernels: up to UPD_ROWS rows of the list upd_row and 128 pp columns of a
-// channel, with what its CTA would otherwise look up in the channel tables.
+// 32 amplitudes of a channel's computed rows (a chunk of the update kernels), with what its warp would
+// otherwise look up in the channel tables.
 struct __align__(16) UpdItem {
-  int c, r0, ab0, ng;          // channel, first entry of upd_row, first column, rows
+  int e0, ne, uoff;            // first element, elements of the channel's run of upd_row, its start
   int npp, nh, sys, nl;        // sizes of the channel, its system, ladder vectors (0: no V_pppp block)
-  int pp_off, lut_off;         // pairs of the channel, interaction table of the system
+  int pp_off, hh_off, pad;     // pairs of the channel
   long base, vhh_off, s_off;   // amplitudes, chi_hh, ladder layout
 };
 
@@ -99,11 +91,9 @@ struct DevState {
   // pairs of the cross channels
   int2 *ph_pair, *hp_pair;
   int* fmap;             // per t element: sign * (index + 1) of its spin-flipped element
-  // mixed and FP64 updates: the hole-pair rows they compute (flip representatives), per item
-  // a run of this list (items hold (channel, first entry, first column, rows))
+  // the hole-pair rows the updates compute (flip representatives), per channel a run of this list
   int* upd_row;
   int* ch_uoff;          // per direct channel its run of upd_row (nch + 1 offsets)
-  UpdRow* upd_rowinfo;   // per update item UPD_ROWS rows (rows past the item's last repeat it)
   // maps
   int* xmap;             // per formed T element: sign * (t index + 1), 0 = structurally zero
   int4* qmap;            // per t element: the four Q positions of P(ij)P(ab) Q (formed positions)
@@ -146,7 +136,6 @@ struct __align__(16) PPItem {
 // Solve-loop control block in device memory (one per context).
 struct LoopCtl {
   int iter;          // updates made in the current solve
-  int blocks_done;   // blocks of the current update that have finished (last-block finalize)
   int dev_error;     // set by a kernel whose bounded wait ran out (the loop then stops)
   int max_iter;
   int status;        // 0 running, 1 converged, PNM_ENOTCONV, PNM_EDIVERGED
@@ -154,6 +143,7 @@ struct LoopCtl {
   int min_iter;      // no system counts as converged before this many updates
   int skip_done;     // 1 inside the solve loop: kernels skip the work of converged systems
   double alpha;
+  unsigned long long closed;  // systems whose last CTA of the current update has finished (finalize_system)
 };
 
 // Run-time parameters of a whole-solve graph, copied from pinned host memory by its first node.
@@ -195,6 +185,7 @@ struct FinArgs {
   const int* lo;        // per system: first partial
   const int* hi;        // per system: one past the last partial
   int nsys;
+  int* blocks_done;     // per system: CTAs of the current update that have finished
   SysCtl* sc;
   double* hist;
   int hist_cap;
@@ -202,21 +193,17 @@ struct FinArgs {
   cudaGraphConditionalHandle handle;
 };
 
-// The update kernels: at most UPD_ROWS hole pairs per CTA (the FP64 update shares one pass
-// over a t column for the hh ladder among them), loads issued in batches of UPD_BATCH rows,
-// at least UPD_MIN_BLOCKS CTAs of the mixed update per SM; channels may hold at most
-// UPD_MAX_NHH hole pairs.  The PNM_UPD_* macros override the tuning constants at build time.
-#ifndef PNM_UPD_ROWS
-#define PNM_UPD_ROWS 8
-#endif
-#ifndef PNM_UPD_BATCH
-#define PNM_UPD_BATCH 2
-#endif
+// The update kernels: threads of a CTA, CTAs of the mixed update per SM at least, CTAs per SM above
+// which a warp takes more than one chunk; channels may hold at most UPD_MAX_NHH hole pairs.  The
+// PNM_UPD_* macros override the tuning constants at build time.
 #ifndef PNM_UPD_MIN_BLOCKS
-#define PNM_UPD_MIN_BLOCKS 6
+#define PNM_UPD_MIN_BLOCKS 7
 #endif
-constexpr int UPD_ROWS = PNM_UPD_ROWS, UPD_MAX_NHH = 128, UPD_BATCH = PNM_UPD_BATCH;
-constexpr int UPD_MIN_BLOCKS = PNM_UPD_MIN_BLOCKS;
+#ifndef PNM_UPD_FULL
+#define PNM_UPD_FULL 16
+#endif
+constexpr int UPD_THREADS = 128, UPD_MAX_NHH = 128;
+constexpr int UPD_MIN_BLOCKS = PNM_UPD_MIN_BLOCKS, UPD_FULL = PNM_UPD_FULL;
 
 constexpr int PH_THREADS = 128;  // threads of a ph-term CTA
 
