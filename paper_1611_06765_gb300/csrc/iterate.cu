@@ -869,68 +869,66 @@ void pnm_flip_symmetrise(pnm_ctx* ctx, double* t, cudaStream_t s) {
     k_flip_sym<<<(unsigned)((ctx->nt + 255) / 256), 256, 0, s>>>(ctx->d.fmap, t, ctx->nt);
 }
 
-// Initial amplitudes (MBPT2 guess or zero) into t0 with energy partials.
-__global__ void __launch_bounds__(128) k_init(DevState D, int init) {
+// v / eps from the reciprocal held beside eps: one product and Markstein's correction step (IBM J.
+// Res. Dev. 34 (1990) 111: with y = 1 / eps correctly rounded and q = v y, q + y (v - q eps) is the
+// correctly rounded quotient whenever q is within one last place of it), three FP64 instructions
+// where a division takes a dozen.
+__device__ __forceinline__ double div_by_eps(double v, double den, double inv) {
+  if (!isfinite(inv)) return v / den;
+  const double q = v * inv;
+  return fma(fma(-q, den, v), inv, q);
+}
+
+// MBPT2 energy partials sum v t over restricted amplitudes per row (channel, ij), and with WRITE the
+// start amplitudes (MBPT2 guess, zero, or as they are) into t0.  One amplitude of each spin-flip pair
+// is formed, written to both and counted twice; the rows that the flip maps onto earlier ones are
+// theirs.  Bound by the FP64 pipe when every amplitude was formed from its states and divided (122 us
+// for three N=66, N_max=36 systems; 33 so).
+template <bool WRITE>
+__global__ void __launch_bounds__(128) k_mbpt2(DevState D, int init) {
   __shared__ double sh32[32];
-  int2 it = D.row_item[blockIdx.x];
-  int c = it.x, ij = it.y;
-  int npp = D.ch_npp[c];
-  long row = D.ch_t_off[c] + (long)ij * npp;
-  int2 h = D.hh_pair[D.ch_hh_off[c] + ij];
-  double ei = D.eps[h.x], ej = D.eps[h.y];
-  double esum = 0.0;
-  for (int ab = threadIdx.x; ab < npp; ab += blockDim.x) {
-    long z = row + ab;
-    double v = D.v_pphh[z];
-    double t;
-    if (init == PNM_INIT_MBPT2) {
-      int2 p = D.pp_pair[D.ch_pp_off[c] + ab];
-      t = v / (ei + ej - D.eps[p.x] - D.eps[p.y]);
-      D.t0[z] = t;
-    } else if (init == PNM_INIT_ZERO) {
-      t = 0.0;
-      D.t0[z] = t;
-    } else {
-      t = D.t0[z];
+  const int2 it = D.row_item[blockIdx.x];
+  const int npp = D.ch_npp[it.x];
+  const long row = D.ch_t_off[it.x] + (long)it.y * npp;
+  const int first = D.fmap[row];
+  double e2 = 0.0, e1 = 0.0;
+  if (abs(first) - 1 >= row) {
+#pragma unroll 4
+    for (int ab = threadIdx.x; ab < npp; ab += 128) {
+      const long z = row + ab;
+      const int fc = D.fmap[z];
+      const double v = D.v_pphh[z];
+      const long f = (long)(fc > 0 ? fc : -fc) - 1;
+      double t = 0.0;
+      if (init == PNM_INIT_MBPT2) t = div_by_eps(v, D.den[z], D.inv_den[z]);
+      else if (init != PNM_INIT_ZERO) t = D.t0[z];
+      if (f < z) continue;
+      if (WRITE && (init == PNM_INIT_MBPT2 || init == PNM_INIT_ZERO)) {
+        D.t0[z] = t;
+        if (f != z) D.t0[f] = fc > 0 ? t : -t;
+      }
+      if (f != z) e2 = fma(v, t, e2);
+      else e1 = fma(v, t, e1);
     }
-    esum += v * t;
+    e1 = block_sum(fma(2.0, e2, e1), sh32);
   }
-  esum = block_sum(esum, sh32);
   if (threadIdx.x == 0) {
-    D.eparts[blockIdx.x] = esum;
-    D.rparts[blockIdx.x] = 0.0;
+    D.eparts[blockIdx.x] = e1;
+    if (WRITE) D.rparts[blockIdx.x] = 0.0;
   }
 }
 
-// MBPT2 with v generated on the fly: sum over restricted pairs of v^2 / eps_ij^ab.
-__global__ void __launch_bounds__(128) k_mbpt2(DevState D, const int* __restrict__ row_lut_off) {
-  __shared__ double sh32[32];
-  int2 it = D.row_item[blockIdx.x];
-  int c = it.x, ij = it.y;
-  int npp = D.ch_npp[c];
-  const double* lut = D.lut + row_lut_off[D.ch_sys[c]];
-  int2 h = D.hh_pair[D.ch_hh_off[c] + ij];
-  char4 si = D.nvec[h.x], sj = D.nvec[h.y];
-  double ei = D.eps[h.x], ej = D.eps[h.y];
-  double s = 0.0;
-  for (int ab = threadIdx.x; ab < npp; ab += blockDim.x) {
-    int2 p = D.pp_pair[D.ch_pp_off[c] + ab];
-    double v = v_minnesota_as(D.nvec[p.x], D.nvec[p.y], si, sj, lut);
-    s += v * v / (ei + ej - D.eps[p.x] - D.eps[p.y]);
-  }
-  s = block_sum(s, sh32);
-  if (threadIdx.x == 0) D.eparts[blockIdx.x] = s;
-}
-
-// Sum of row partials per system (fixed order), into out[sys].
-__global__ void k_reduce_rows(const double* __restrict__ parts, const int* __restrict__ row_lo,
+// Sums of row or CTA partials per system (fixed order): out[plane * nsys + sys], planes of n partials.
+__global__ void k_reduce_rows(const double* __restrict__ parts, long n, const int* __restrict__ row_lo,
                               const int* __restrict__ row_hi, double* __restrict__ out) {
   __shared__ double sh32[32];
-  int s = blockIdx.x;
+  const int s = blockIdx.x;
+  parts += blockIdx.y * n;
   double acc = 0.0;
+#pragma unroll 4
   for (int r = row_lo[s] + threadIdx.x; r < row_hi[s]; r += blockDim.x) acc += parts[r];
   acc = block_sum(acc, sh32);
-  if (threadIdx.x == 0) out[s] = acc;
+  if (threadIdx.x == 0) out[blockIdx.y * gridDim.x + s] = acc;
 }
 
 // Energy of the start amplitudes: history[0] per system, reset of the loop state.
@@ -966,13 +964,40 @@ __global__ void k_start(const double* __restrict__ parts, const int* __restrict_
 
 static void* dmalloc(pnm_ctx* ctx, size_t bytes) { return pnm_ctx_alloc(ctx, bytes); }
 
-// Amplitudes of the update chunks: rows of the channel's run of upd_row one after the other.
-__global__ void k_upd_list(DevState D, const UpdItem* __restrict__ items, long n, int* __restrict__ upd_z) {
-  const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const UpdItem it = items[k >> 5];
-  const int e = it.e0 + (int)(k & 31), r = e / it.npp;
-  upd_z[k] = e < it.ne ? (int)(it.base + (long)D.upd_row[it.uoff + r] * it.npp + (e - r * it.npp)) : -1;
+// The update chunks and their amplitudes: rows of the channel's run of upd_row one after the other, 32
+// amplitudes per chunk; a channel per CTA (its chunks start at first[c]), then a system per CTA for the
+// padding up to whole CTAs of the updates.
+__global__ void __launch_bounds__(128) k_upd_chunks(DevState D, int nch, const int* __restrict__ first,
+                                                    const int2* __restrict__ pad, UpdItem* __restrict__ items,
+                                                    int* __restrict__ upd_z) {
+  UpdItem it{};
+  if ((int)blockIdx.x >= nch) {
+    const int2 p = pad[blockIdx.x - nch];
+    it.npp = 1;
+    it.sys = blockIdx.x - nch;
+    for (int k = p.x * 32 + threadIdx.x; k < p.y * 32; k += blockDim.x) {
+      upd_z[k] = -1;
+      if ((k & 31) == 0) items[k >> 5] = it;
+    }
+    return;
+  }
+  const int c = blockIdx.x;
+  it.npp = D.ch_npp[c];
+  it.nh = D.ch_nhh[c];
+  it.sys = D.ch_sys[c];
+  it.nl = D.ch_vpp[c] ? D.ch_nlad[c] : 0;
+  it.pp_off = D.ch_pp_off[c];
+  it.hh_off = D.ch_hh_off[c];
+  it.base = D.ch_t_off[c];
+  it.vhh_off = D.ch_vhh_off[c];
+  it.s_off = D.ch_s_off[c];
+  const int r0 = D.ch_uoff[c], n = (D.ch_uoff[c + 1] - r0) * it.npp;
+  const long k0 = 32L * first[c];
+  for (int e = threadIdx.x; e < ((n + 31) & ~31); e += blockDim.x) {
+    const int r = e / it.npp;
+    upd_z[k0 + e] = e < n ? (int)(it.base + (long)D.upd_row[r0 + r] * it.npp + (e - r * it.npp)) : -1;
+    if ((e & 31) == 0) items[(k0 + e) >> 5] = it;
+  }
 }
 
 // pp items of nr[c] rows per channel in the order of decreasing work, so that the last CTAs are
@@ -1090,29 +1115,28 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   // Chunks of the updates: 32 amplitudes of one channel each (its last is padded), a CTA's in one
   // system (padded chunks past its end).  A warp takes more than one where the GPU stays full: fewer
   // partial sums for the last CTA to add, and the block sums' FP64 additions count for more amplitudes.
-  std::vector<UpdItem> chunks;
-  std::vector<int> glo(nsys), ghi(nsys);
+  std::vector<int> glo(nsys), ghi(nsys), first(ctx->nch);
+  std::vector<int2> pad(nsys);
   long n_chunks = 0;
   for (int c = 0; c < ctx->nch; c++) n_chunks += ((long)(uoff[c + 1] - uoff[c]) * ctx->h_npp[c] + 31) / 32;
   const int warps = UPD_THREADS / 32;
   ctx->upd_per_warp = 4;
   while (ctx->upd_per_warp > 1 && n_chunks < (long)UPD_FULL * nsm * warps * ctx->upd_per_warp) ctx->upd_per_warp >>= 1;
   const int per_cta = warps * ctx->upd_per_warp;
-  chunks.reserve(n_chunks + (size_t)per_cta * nsys);
+  n_chunks = 0;
   for (int k = 0; k < nsys; k++) {
-    glo[k] = (int)(chunks.size() / per_cta);
+    glo[k] = (int)(n_chunks / per_cta);
     for (int c = ctx->sys[k].ch_begin; c < ctx->sys[k].ch_end; c++) {
-      const int np = ctx->h_npp[c], ne = (uoff[c + 1] - uoff[c]) * np;
-      for (int e0 = 0; e0 < ne; e0 += 32)
-        chunks.push_back(UpdItem{e0, ne, uoff[c], np, ctx->h_nhh[c], k, ctx->h_vpp[c] ? ctx->h_nlad[c] : 0,
-                                 ctx->h_pp_off[c], ctx->h_hh_off[c], 0, ctx->h_t_off[c], ctx->h_vhh_off[c],
-                                 ctx->h_s_off[c]});
+      first[c] = (int)n_chunks;
+      n_chunks += ((long)(uoff[c + 1] - uoff[c]) * ctx->h_npp[c] + 31) / 32;
     }
+    pad[k].x = (int)n_chunks;
     // at least one CTA per system: it closes the system's update
-    while (chunks.size() % per_cta || (int)(chunks.size() / per_cta) == glo[k]) chunks.push_back(UpdItem{0, 0, 0, 1, 0, k, 0, 0, 0, 0, 0, 0, 0});
-    ghi[k] = (int)(chunks.size() / per_cta);
+    n_chunks = std::max<long>(glo[k] + 1, (n_chunks + per_cta - 1) / per_cta) * per_cta;
+    pad[k].y = (int)n_chunks;
+    ghi[k] = (int)(n_chunks / per_cta);
   }
-  ctx->n_upd_ctas = (int)(chunks.size() / per_cta);
+  ctx->n_upd_ctas = (int)(n_chunks / per_cta);
   ctx->max_npp = max_npp;
   ctx->max_nlad = max_nlad;
   std::vector<int> alo(nsys), ahi(nsys);
@@ -1151,14 +1175,14 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   CUDA_TRY(cudaMemcpyAsync(ud + nsys, uhi.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, s));
   ctx->upd_lo_d = ud;
   ctx->upd_hi_d = ud + nsys;
-  ctx->upd_chunks = (UpdItem*)dmalloc(ctx, sizeof(UpdItem) * std::max<size_t>(1, chunks.size()));
-  ctx->upd_z = (int*)dmalloc(ctx, sizeof(int) * 32 * std::max<size_t>(1, chunks.size()));
-  if (!chunks.empty()) {
-    const long n = 32 * (long)chunks.size();
-    CUDA_TRY(cudaMemcpyAsync(ctx->upd_chunks, chunks.data(), sizeof(UpdItem) * chunks.size(), cudaMemcpyHostToDevice, s));
-    k_upd_list<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ctx->d, ctx->upd_chunks, n, ctx->upd_z);
-    CUDA_TRY(cudaGetLastError());
-  }
+  ctx->upd_chunks = (UpdItem*)dmalloc(ctx, sizeof(UpdItem) * std::max<long>(1, n_chunks));
+  ctx->upd_z = (int*)dmalloc(ctx, sizeof(int) * 32 * std::max<long>(1, n_chunks));
+  int* dfirst = (int*)dmalloc(ctx, sizeof(int) * std::max(1, ctx->nch));
+  int2* dpad = (int2*)dmalloc(ctx, sizeof(int2) * nsys);
+  if (ctx->nch) CUDA_TRY(cudaMemcpyAsync(dfirst, first.data(), sizeof(int) * ctx->nch, cudaMemcpyHostToDevice, s));
+  CUDA_TRY(cudaMemcpyAsync(dpad, pad.data(), sizeof(int2) * nsys, cudaMemcpyHostToDevice, s));
+  k_upd_chunks<<<ctx->nch + nsys, 128, 0, s>>>(ctx->d, ctx->nch, dfirst, dpad, ctx->upd_chunks, ctx->upd_z);
+  CUDA_TRY(cudaGetLastError());
   int* gd = (int*)dmalloc(ctx, sizeof(int) * 2 * nsys);
   CUDA_TRY(cudaMemcpyAsync(gd, glo.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(gd + nsys, ghi.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, s));
@@ -1224,9 +1248,8 @@ void pnm_mbpt2_all(pnm_ctx* ctx, double* out) {
   cudaStream_t s = ctx->stream;
   int nsys = (int)ctx->sys.size();
   CUDA_TRY(cudaEventRecord(ctx->ev[0], s));
-  k_mbpt2<<<ctx->nrows, 128, 0, s>>>(ctx->d, ctx->lut_off_d);
-  k_reduce_rows<<<nsys, 256, 0, s>>>(ctx->d.eparts, ctx->row_lo_d, ctx->row_hi_d,
-                                     ctx->d.rparts);
+  k_mbpt2<false><<<ctx->nrows, 128, 0, s>>>(ctx->d, PNM_INIT_MBPT2);
+  k_reduce_rows<<<nsys, 256, 0, s>>>(ctx->d.eparts, 0, ctx->row_lo_d, ctx->row_hi_d, ctx->d.rparts);
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaEventRecord(ctx->ev[1], s));
   CUDA_TRY(cudaMemcpyAsync(out, ctx->d.rparts, sizeof(double) * nsys, cudaMemcpyDeviceToHost, s));
@@ -1238,52 +1261,60 @@ void pnm_mbpt2_all(pnm_ctx* ctx, double* out) {
 
 // Third-order diagrams (Fig. goldstone, Eqs. diag3-diag5) from the MBPT2 amplitudes t0 held in
 // D.t0, the pp ladder of t0 in D.rpp (channels with a V_pppp block) and the linear ph term of t0 in D.xq:
-// per row (channel, ij) the partial sums over ab of
+// the sums over the amplitudes of
 //   (4)  t0_ab^ij sum_{c<d} <ab|v|cd> t0_cd^ij,
 //   (5)  t0_ab^ij sum_{k<l} t0_ab^kl <kl|v|ij>,
 //   (3)  t0_ab^ij [P(ij)P(ab) sum_kc <kb|v|cj> t0_ik^ac],
-// into parts[0..3) x nrows.
-__global__ void __launch_bounds__(128) k_mbpt3_rows(DevState D, double* __restrict__ parts, int nrows) {
-  __shared__ double sh32[32];
-  int2 it = D.row_item[blockIdx.x];
-  int c = it.x, ij = it.y;
-  int npp = D.ch_npp[c], nh = D.ch_nhh[c];
-  long base = D.ch_t_off[c], row = base + (long)ij * npp;
-  const double* __restrict__ vh = D.v_hhhh + D.ch_vhh_off[c];
+// a thread per amplitude of the update chunks (one of each spin-flip pair, counted twice), into
+// parts[0..3) x CTAs.  Bound by the FP64 pipe (the hh sum); a CTA per row, most of whose block sums and
+// threads idled in small channels, took 122 us for three N=66, N_max=36 systems, 87 so.
+__global__ void __launch_bounds__(UPD_THREADS) k_mbpt3(DevState D, const UpdItem* __restrict__ items,
+                                                       const int* __restrict__ upd_z, int per_warp,
+                                                       double* __restrict__ parts) {
+  __shared__ double red[UPD_THREADS / 32][3];
   const double* __restrict__ t = D.t0;
-  bool has_vpp = D.ch_vpp[c] != 0;
   double e4 = 0.0, e5 = 0.0, e3 = 0.0;
-  for (int ab = threadIdx.x; ab < npp; ab += blockDim.x) {
-    long z = row + ab;
-    // one amplitude of each spin-flip pair, counted twice (the ladder is formed on those rows)
+  for (int u = 0; u < per_warp; u++) {
+    const long chunk = ((long)blockIdx.x * per_warp + u) * (UPD_THREADS / 32) + (threadIdx.x >> 5);
+    const UpdItem it = items[chunk];
+    const int zi = upd_z[chunk * 32 + (threadIdx.x & 31)];
+    if (zi < 0) continue;  // padding
+    const long z = zi;
     const int fc = D.fmap[z];
     const long f = (long)(fc > 0 ? fc : -fc) - 1;
     if (f < z) continue;
-    double tz = (f == z ? 1.0 : 2.0) * t[z];
-    if (has_vpp) {
-      int sg;
-      double rl = D.rpp[lad_index(D, c, ij, ab, sg)];
-      e4 += tz * (sg > 0 ? rl : -rl);
+    const int e = (int)(z - it.base), ij = e / it.npp, ab = e - ij * it.npp, nh = it.nh, npp = it.npp;
+    const double tz = (f == z ? 1.0 : 2.0) * t[z];
+    const int4 q = D.qmap[z];
+    double rl = 0.0;
+    if (it.nl) {
+      const int m = D.lad_map[it.pp_off + ab];
+      rl = D.rpp[it.s_off + (long)ij * it.nl + ((m > 0 ? m : -m) - 1)];
+      if (m < 0) rl = -rl;
     }
+    const double q0 = q.x >= 0 ? D.xq[q.x] : 0.0, q1 = q.y >= 0 ? D.xq[q.y] : 0.0;
+    const double q2 = q.z >= 0 ? D.xq[q.z] : 0.0, q3 = q.w >= 0 ? D.xq[q.w] : 0.0;
+    const double* __restrict__ col = t + it.base + ab;
+    const double* __restrict__ vh = D.v_hhhh + it.vhh_off + ij;
     double hh = 0.0;
-    for (int kl = 0; kl < nh; kl++) hh += t[base + (long)kl * npp + ab] * vh[(long)kl * nh + ij];
-    e5 += tz * hh;
-    int4 q = D.qmap[z];
-    double ph = 0.0;
-    if (q.x >= 0) ph += D.xq[q.x];
-    if (q.y >= 0) ph -= D.xq[q.y];
-    if (q.z >= 0) ph -= D.xq[q.z];
-    if (q.w >= 0) ph += D.xq[q.w];
-    e3 += tz * ph;
+#pragma unroll 4
+    for (int kl = 0; kl < nh; kl++) hh = fma(col[(long)kl * npp], vh[(long)kl * nh], hh);
+    e4 = fma(tz, rl, e4);
+    e5 = fma(tz, hh, e5);
+    e3 = fma(tz, ((q0 - q1) - q2) + q3, e3);
   }
-  e4 = block_sum(e4, sh32);
-  e5 = block_sum(e5, sh32);
-  e3 = block_sum(e3, sh32);
-  if (threadIdx.x == 0) {
-    parts[blockIdx.x] = e4;
-    parts[nrows + blockIdx.x] = e5;
-    parts[2 * nrows + blockIdx.x] = e3;
+  e4 = warp_sum(e4);
+  e5 = warp_sum(e5);
+  e3 = warp_sum(e3);
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5][0] = e4;
+    red[threadIdx.x >> 5][1] = e5;
+    red[threadIdx.x >> 5][2] = e3;
   }
+  __syncthreads();
+  if (threadIdx.x < 3)
+    parts[(long)threadIdx.x * gridDim.x + blockIdx.x] =
+        (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
 }
 
 // out[3 s + {0, 1, 2}] = diagrams (4), (5), (3) of system s.  Replaces the context's
@@ -1292,21 +1323,20 @@ void pnm_mbpt3_all(pnm_ctx* ctx, double* out) {
   cudaStream_t s = ctx->stream;
   pnm_need_digits(ctx);
   int nsys = (int)ctx->sys.size();
-  if (!ctx->mbpt3_buf) ctx->mbpt3_buf = (double*)dmalloc(ctx, sizeof(double) * (3 * (size_t)ctx->nrows + 3 * nsys));
+  const int n = ctx->n_upd_ctas;
+  if (!ctx->mbpt3_buf) ctx->mbpt3_buf = (double*)dmalloc(ctx, sizeof(double) * (3 * (size_t)n + 3 * nsys));
   double* parts = ctx->mbpt3_buf;
-  double* res = parts + 3 * (size_t)ctx->nrows;
+  double* res = parts + 3 * (size_t)n;
   CUDA_TRY(cudaEventRecord(ctx->ev[0], s));
   // amplitudes of the start in t0, read by the contraction kernels (iteration parity 0, no
   // system frozen)
   CUDA_TRY(cudaMemsetAsync(&ctx->ctl->iter, 0, sizeof(int), s));
   CUDA_TRY(cudaMemsetAsync(&ctx->ctl->skip_done, 0, sizeof(int), s));
-  k_init<<<ctx->nrows, 128, 0, s>>>(ctx->d, PNM_INIT_MBPT2);
+  k_mbpt2<true><<<ctx->nrows, 128, 0, s>>>(ctx->d, PNM_INIT_MBPT2);
   pnm_launch_pp(ctx, s, true, false);
   if (ctx->nx > 0) launch_ph64(ctx, s, s, true);  // without cross channels no Q is read
-  k_mbpt3_rows<<<ctx->nrows, 128, 0, s>>>(ctx->d, parts, ctx->nrows);
-  for (int k = 0; k < 3; k++)
-    k_reduce_rows<<<nsys, 256, 0, s>>>(parts + (size_t)k * ctx->nrows, ctx->row_lo_d, ctx->row_hi_d,
-                                       res + (size_t)k * nsys);
+  k_mbpt3<<<n, UPD_THREADS, 0, s>>>(ctx->d, ctx->upd_chunks, ctx->upd_z, ctx->upd_per_warp, parts);
+  k_reduce_rows<<<dim3(nsys, 3), 256, 0, s>>>(parts, n, ctx->grp_lo_d, ctx->grp_hi_d, res);
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaEventRecord(ctx->ev[1], s));
   std::vector<double> h(3 * (size_t)nsys);
@@ -1324,9 +1354,8 @@ void pnm_mbpt3_all(pnm_ctx* ctx, double* out) {
 void pnm_launch_mbpt2_into(const pnm_ctx* ctx, double* partials, double* results) {
   DevState d = ctx->d;
   d.eparts = partials;
-  k_mbpt2<<<ctx->nrows, 128, 0, ctx->stream>>>(d, ctx->lut_off_d);
-  k_reduce_rows<<<(int)ctx->sys.size(), 256, 0, ctx->stream>>>(partials, ctx->row_lo_d,
-                                                                ctx->row_hi_d, results);
+  k_mbpt2<false><<<ctx->nrows, 128, 0, ctx->stream>>>(d, PNM_INIT_MBPT2);
+  k_reduce_rows<<<(int)ctx->sys.size(), 256, 0, ctx->stream>>>(partials, 0, ctx->row_lo_d, ctx->row_hi_d, results);
 }
 
 // The body of one update, enqueued on the context stream (FP64 path).
@@ -1656,7 +1685,7 @@ void pnm_start(pnm_ctx* ctx, int init, const std::vector<double>& tol) {
   }
   CUDA_TRY(cudaMemcpyAsync(ctx->sysctl, hs.data(), sizeof(SysCtl) * nsys, cudaMemcpyHostToDevice, s));
   if (init == PNM_INIT_KEEP) pnm_flip_symmetrise(ctx, ctx->d.t0, s);
-  k_init<<<ctx->nrows, 128, 0, s>>>(ctx->d, init);
+  k_mbpt2<true><<<ctx->nrows, 128, 0, s>>>(ctx->d, init);
   k_start<<<1, 256, 0, s>>>(ctx->d.eparts, ctx->row_lo_d, ctx->row_hi_d, nsys, ctx->sysctl,
                             ctx->ctl, ctx->hist, ctx->hist_cap);
   CUDA_TRY(cudaGetLastError());
@@ -1766,7 +1795,7 @@ void pnm_solve_begin(pnm_ctx* ctx) {
 void pnm_start_device(pnm_ctx* ctx, int init) {
   cudaStream_t s = ctx->stream;
   if (init == PNM_INIT_KEEP) pnm_flip_symmetrise(ctx, ctx->d.t0, s);
-  k_init<<<ctx->nrows, 128, 0, s>>>(ctx->d, init);
+  k_mbpt2<true><<<ctx->nrows, 128, 0, s>>>(ctx->d, init);
   k_start<<<1, 256, 0, s>>>(ctx->d.eparts, ctx->row_lo_d, ctx->row_hi_d, (int)ctx->sys.size(), ctx->sysctl,
                             ctx->ctl, ctx->hist, ctx->hist_cap);
   CUDA_TRY(cudaGetLastError());

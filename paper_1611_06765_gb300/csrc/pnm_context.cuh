@@ -83,7 +83,7 @@ struct pnm_ctx {
   int *row_lo_d = nullptr, *row_hi_d = nullptr, *lut_off_d = nullptr;  // per system
   LoopCtl* ctl = nullptr;     // device
   double* small = nullptr;    // device scratch for single-value queries
-  double* mbpt3_buf = nullptr;   // per-row partials and per-system results of pnm_mbpt3
+  double* mbpt3_buf = nullptr;   // per-CTA partials and per-system results of pnm_mbpt3
   double* expand_buf = nullptr;  // the pp ladder or ph term in the amplitude layout (operator calls)
   SysCtl* sysctl = nullptr;   // device, one per system
   int* blocks_done = nullptr; // device, one per system

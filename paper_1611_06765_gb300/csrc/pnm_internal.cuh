@@ -61,9 +61,8 @@ struct SysInfo {
 // 32 amplitudes of a channel's computed rows (a chunk of the update kernels), with what its warp would
 // otherwise look up in the channel tables.
 struct __align__(16) UpdItem {
-  int e0, ne, uoff;            // first element, elements of the channel's run of upd_row, its start
   int npp, nh, sys, nl;        // sizes of the channel, its system, ladder vectors (0: no V_pppp block)
-  int pp_off, hh_off, pad;     // pairs of the channel
+  int pp_off, hh_off;          // pairs of the channel
   long base, vhh_off, s_off;   // amplitudes, chi_hh, ladder layout
 };
 
