@@ -215,31 +215,102 @@ void sgemm(cudaStream_t s, int M, int N, int K, const float* A, int lda, int tA,
 }
 
 // ------------------------------------------------------------ tensor-core training GEMM
-// The k_sgemm contract, C[M][N] (+)= op(A)[M][K] op(B)[K][N], on the tcgen05 tensor cores for the
+// The k_sgemm contract, C[M][N] = op(A)[M][K] op(B)[K][N], on the tcgen05 tensor cores for the
 // BF16 training mode: each operand element is split as it is staged into BF16 hi + lo (exact for
 // the BF16-rounded weights and layer inputs, whose lo part is zero; 2^-18 relative for the FP32
 // error signals of the backward pass), three products per 16-wide k step (hi hi + hi lo +
 // lo hi) accumulate in FP32 in tensor memory.  One CTA (four warps) per 128 x bn tile of C and
-// k-range blockIdx.z (K split into gridDim.z ranges of whole 64-wide stages, results to
-// C + blockIdx.z * cz, summed in order by k_sum_splits); all threads stage a 64-wide k slice of
-// both operands into shared memory in the K-major core-matrix layout, thread 0 issues the MMAs
-// and commits them to an mbarrier (bounded wait: on timeout the CTA stops, writes nothing and
-// sets *err), and each thread drains its TMEM lane (row of C).
+// k-range (K split into kz ranges of whole 64-wide stages, results to C + z * cz, summed in order by
+// k_grad_finish); all threads stage a 64-wide k slice of both operands into shared memory in the
+// K-major core-matrix layout, thread 0 issues the MMAs and commits them to an mbarrier (bounded wait:
+// on timeout the CTA stops, writes nothing and sets *err), and each thread drains its TMEM lane (row
+// of C).  What bounds it at the training sizes is latency, one tile of one or two stages per CTA: a
+// slice's loads are 16 bytes each and all in flight before the first is stored (lanes cover 64
+// contiguous bytes of eight rows, which the stores spread over all banks), and what follows the
+// product element by element is part of the epilogue: the bias and the activation of the forward
+// pass, the derivative of the backward pass.  Up to three products of one launch (the weight
+// gradients) share the grid.  One loss and gradient of 1024 rows: 30 launches of 205 us together,
+// 11 of 138 us so (each timed by itself from a cold cache).
+// M is any, N a multiple of 16, lda, ldb, ldc multiples of 4 and the arrays 16-byte aligned; rows of an
+// operand that is contiguous in k hold zeros from K up to the next multiple of 4.
 constexpr int TG_BM = 128, TG_BN = 128, TG_BK = 64;
 constexpr int TG_PLANE_A = TG_BM * TG_BK, TG_PLANE_B = TG_BN * TG_BK;  // BF16 elements per plane
 constexpr size_t TG_SMEM = 1024 + 2 * (size_t)(TG_PLANE_A + TG_PLANE_B) * sizeof(__nv_bfloat16);
-constexpr int TG_MAX_SPLIT = 16, TG_BATCH = 16;
+constexpr int TG_MAX_SPLIT = 16;
 
-__device__ __forceinline__ void tg_split(float x, __nv_bfloat16* hi, __nv_bfloat16* lo, int o) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  hi[o] = h;
-  lo[o] = __float2bfloat16_rn(x - __bfloat162float(h));
+enum { EPI_NONE, EPI_GELU, EPI_DGELU };
+struct GemmTask {
+  const float *A, *B;
+  float* C;
+  int M, N, K, lda, ldb, ldc;
+  // EPI_GELU: C = product + aux[n], H = bf16(gelu(C)); EPI_DGELU: C = product * gelu'(aux[m][n])
+  const float* aux;
+  float* H;
+};
+struct GemmTasks {
+  GemmTask t[3];
+};
+
+// Four neighbouring elements into the hi and lo planes: along k (8 contiguous bytes) or across rows.
+__device__ __forceinline__ void tg_split(const float (&x)[4], __nv_bfloat16 (&h)[4], __nv_bfloat16 (&l)[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    h[j] = __float2bfloat16_rn(x[j]);
+    l[j] = __float2bfloat16_rn(x[j] - __bfloat162float(h[j]));
+  }
+}
+// Stage rows x TG_BK elements of an operand whose contiguous index is k (KC) or the row: element
+// (r, k) at P[r * ld + k] or P[k * ld + r]; zeros past the rows and past ke.  ROWS / 8 float4 per thread.
+template <int ROWS, bool KC>
+__device__ __forceinline__ void tg_stage(const float* __restrict__ P, int ld, int row0, int rows, int k0, int ke,
+                                         __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+  constexpr int NV = ROWS * TG_BK / 4 / 128;  // float4 per thread
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float4 x[NV];
+  // blocks of 8 (uncontiguous) x 16 (contiguous) elements, one per warp and step
+  auto place = [&](int v, int& r, int& k) {
+    const int blk = v * 4 + w;
+    if (KC) {
+      r = (blk >> 2) * 8 + (lane >> 2);
+      k = (blk & 3) * 16 + (lane & 3) * 4;
+    } else {
+      k = (blk & 7) * 8 + (lane >> 2);
+      r = (blk >> 3) * 16 + (lane & 3) * 4;
+    }
+  };
+#pragma unroll
+  for (int v = 0; v < NV; v++) {
+    int r, k;
+    place(v, r, k);
+    const bool in = row0 + r < rows && k0 + k < ke;
+    x[v] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (in) x[v] = *reinterpret_cast<const float4*>(KC ? P + (long)(row0 + r) * ld + k0 + k : P + (long)(k0 + k) * ld + row0 + r);
+  }
+#pragma unroll
+  for (int v = 0; v < NV; v++) {
+    int r, k;
+    place(v, r, k);
+    const float f[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
+    __align__(8) __nv_bfloat16 h[4], l[4];
+    tg_split(f, h, l);
+    if (KC) {
+      const int o = tc::core_off(r, k, TG_BK / 8);
+      *reinterpret_cast<uint2*>(hi + o) = *reinterpret_cast<const uint2*>(h);
+      *reinterpret_cast<uint2*>(lo + o) = *reinterpret_cast<const uint2*>(l);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int o = tc::core_off(r + j, k, TG_BK / 8);
+        hi[o] = h[j];
+        lo[o] = l[j];
+      }
+    }
+  }
 }
 
-__global__ void __launch_bounds__(128) k_gemm_tc(int M, int N, int K, const float* __restrict__ A, int lda, int tA,
-                                                 const float* __restrict__ B, int ldb, int tB,
-                                                 float* __restrict__ C, int ldc, long cz, int acc, int bn,
-                                                 int* __restrict__ err_flag) {
+// tA, tB as in k_sgemm; BN columns per CTA; task blockIdx.z / kz, k-range blockIdx.z % kz.
+template <int BN, bool TA, bool TB, int EPI>
+__global__ void __launch_bounds__(128) k_gemm_tc(GemmTasks tasks, int kz, long cz, int* __restrict__ err_flag) {
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + 8);
@@ -248,21 +319,22 @@ __global__ void __launch_bounds__(128) k_gemm_tc(int M, int N, int K, const floa
   __nv_bfloat16* Bh = Al + TG_PLANE_A;
   __nv_bfloat16* Bl = Bh + TG_PLANE_B;
   __shared__ int bad;
-  const int m0 = blockIdx.y * TG_BM, n0 = blockIdx.x * bn;  // bn: 32, 64 or TG_BN columns per CTA
-  const int nt = min(bn, N - n0);
-  const int np = (nt + 15) & ~15;  // the MMA's N: a multiple of 16
+  constexpr uint32_t TMEM = EPI == EPI_NONE ? BN : 2 * BN;  // columns
+  const GemmTask& t = tasks.t[blockIdx.z / kz];
+  const int z = blockIdx.z % kz, K = t.K;
+  const int m0 = blockIdx.y * TG_BM, n0 = blockIdx.x * BN;
+  if (n0 >= t.N || m0 >= t.M) return;  // a smaller task of the launch
+  const int np = min(BN, t.N - n0);    // a multiple of 16
   // this CTA's k-range: whole stages
-  const int nstage = (K + TG_BK - 1) / TG_BK;
-  const int per = (nstage + gridDim.z - 1) / gridDim.z;
-  const int kb = blockIdx.z * per * TG_BK, ke = min(K, (int)(blockIdx.z + 1) * per * TG_BK);
-  float* __restrict__ Cz = C + blockIdx.z * cz;
+  const int nstage = (K + TG_BK - 1) / TG_BK, per = (nstage + kz - 1) / kz;
+  const int kb = z * per * TG_BK, ke = min(K, (z + 1) * per * TG_BK);
   if (threadIdx.x == 0) {
     bad = 0;
     tc::mbar_init(bar, 1);
     tc::mbar_fence_init();
   }
   if (threadIdx.x < 32) {
-    tc::tmem_alloc(tslot, 128);
+    tc::tmem_alloc(tslot, TMEM);
     tc::tmem_relinquish();
   }
   tc::fence_before();
@@ -272,63 +344,31 @@ __global__ void __launch_bounds__(128) k_gemm_tc(int M, int N, int K, const floa
   const uint32_t idesc = tc::idesc_bf16(TG_BM, np);
   const uint32_t sbo = (TG_BK / 8) * 128;
   uint32_t phase = 0, fail_parity = 0;
-  bool issued = false;
+  bool issued = false, two = false;
   for (int k0 = kb; k0 < ke; k0 += TG_BK) {
     __syncthreads();
     const int stop = bad;
     __syncthreads();
     if (stop) break;
-    // coalesced along each operand's contiguous index; TG_BATCH independent loads in flight
-    // per thread before their splits are stored
-    for (int e0 = 0; e0 < TG_BM * TG_BK; e0 += TG_BATCH * 128) {
-      float x[TG_BATCH];
-#pragma unroll
-      for (int j = 0; j < TG_BATCH; j++) {
-        const int e = e0 + j * 128 + threadIdx.x;
-        const int r = tA ? e % TG_BM : e / TG_BK, k = tA ? e / TG_BM : e % TG_BK;
-        const int m = m0 + r, kk = k0 + k;
-        x[j] = (m < M && kk < ke) ? (tA ? A[(long)kk * lda + m] : A[(long)m * lda + kk]) : 0.0f;
-      }
-#pragma unroll
-      for (int j = 0; j < TG_BATCH; j++) {
-        const int e = e0 + j * 128 + threadIdx.x;
-        const int r = tA ? e % TG_BM : e / TG_BK, k = tA ? e / TG_BM : e % TG_BK;
-        tg_split(x[j], Ah, Al, tc::core_off(r, k, TG_BK / 8));
-      }
-    }
-    for (int e0 = 0; e0 < np * TG_BK; e0 += TG_BATCH * 128) {
-      float x[TG_BATCH];
-#pragma unroll
-      for (int j = 0; j < TG_BATCH; j++) {
-        const int e = e0 + j * 128 + threadIdx.x;
-        const int r = tB ? e / TG_BK : e % np, k = tB ? e % TG_BK : e / np;
-        const int kk = k0 + k;
-        x[j] = (e < np * TG_BK && r < nt && kk < ke)
-                   ? (tB ? B[(long)(n0 + r) * ldb + kk] : B[(long)kk * ldb + n0 + r])
-                   : 0.0f;
-      }
-#pragma unroll
-      for (int j = 0; j < TG_BATCH; j++) {
-        const int e = e0 + j * 128 + threadIdx.x;
-        if (e < np * TG_BK) {
-          const int r = tB ? e / TG_BK : e % np, k = tB ? e % TG_BK : e / np;
-          tg_split(x[j], Bh, Bl, tc::core_off(r, k, TG_BK / 8));
-        }
-      }
-    }
+    tg_stage<BN, TB>(t.B, t.ldb, n0, t.N, k0, ke, Bh, Bl);
+    tg_stage<TG_BM, !TA>(t.A, t.lda, m0, t.M, k0, ke, Ah, Al);
     tc::fence_async_smem();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
+    // with an epilogue (K of one or two stages) each stage has an accumulator of its own, added there
+    const bool second = EPI != EPI_NONE && issued, started = EPI == EPI_NONE && issued;
+    const uint32_t tacc = tbase + (second ? BN : 0);
+    two = two || second;
     if (threadIdx.x == 0) {
       for (int ks = 0; ks < TG_BK / 16; ks++) {
         const uint64_t ah = tc::smem_desc(reinterpret_cast<const unsigned char*>(Ah) + ks * 256, 128, sbo);
         const uint64_t al = tc::smem_desc(reinterpret_cast<const unsigned char*>(Al) + ks * 256, 128, sbo);
         const uint64_t bh = tc::smem_desc(reinterpret_cast<const unsigned char*>(Bh) + ks * 256, 128, sbo);
         const uint64_t bl = tc::smem_desc(reinterpret_cast<const unsigned char*>(Bl) + ks * 256, 128, sbo);
-        tc::mma_bf16(tbase, ah, bh, idesc, (issued || ks > 0) ? 1u : 0u);
-        tc::mma_bf16(tbase, ah, bl, idesc, 1u);
-        tc::mma_bf16(tbase, al, bh, idesc, 1u);
+        tc::mma_bf16(tacc, ah, bh, idesc, (started || ks > 0) ? 1u : 0u);
+        tc::mma_bf16(tacc, ah, bl, idesc, 1u);
+        tc::mma_bf16(tacc, al, bh, idesc, 1u);
       }
       tc::commit(bar);
     }
@@ -347,52 +387,45 @@ __global__ void __launch_bounds__(128) k_gemm_tc(int M, int N, int K, const floa
   // after a wait that ran out, give the MMAs still in flight one more bounded wait before the
   // tensor memory they write is freed
   if (!ok && threadIdx.x == 0) tc::mbar_wait(bar, fail_parity);
-  // epilogue through shared memory (the operand planes are free once the last wait passed), 64
-  // columns at a time: thread = TMEM lane = row of the tile into Cs, then rows of C written with
-  // consecutive threads on consecutive columns (an empty k-range leaves zeros)
-  constexpr int CS_LD = 65;
-  float* Cs = reinterpret_cast<float*>(smem + 1024);  // 128 x CS_LD floats
-  const int r = threadIdx.x;
+  // epilogue: thread = TMEM lane = row of the tile, 16 columns (64 bytes of its row) at a time (an
+  // empty k-range leaves zeros)
+  const int m = m0 + threadIdx.x;
   const uint32_t lane_addr = tbase + ((uint32_t)((threadIdx.x >> 5) * 32) << 16);
-  for (int c0 = 0; c0 < np; c0 += 64) {
-    const int cw = min(64, np - c0);
-    __syncthreads();
-    if (ok) {
-      for (int cc = 0; cc < cw; cc += 16) {
-        uint32_t v[16];
-        tc::tmem_ld16(lane_addr + c0 + cc, v);
+  for (int c0 = 0; c0 < np && ok; c0 += 16) {
+    __syncwarp();
+    uint32_t v[16];
+    tc::tmem_ld16(lane_addr + c0, v);
+    if (two) {
+      uint32_t v2[16];
+      tc::tmem_ld16(lane_addr + BN + c0, v2);
 #pragma unroll
-        for (int j = 0; j < 16; j++) Cs[r * CS_LD + cc + j] = issued ? __uint_as_float(v[j]) : 0.0f;
-      }
+      for (int j = 0; j < 16; j++) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(v2[j]));
     }
-    __syncthreads();
-    if (ok) {
-      for (int e = threadIdx.x; e < TG_BM * cw; e += blockDim.x) {
-        const int rr = e / cw, c = e % cw;
-        const int m = m0 + rr, n = c0 + c;
-        if (m < M && n < nt) {
-          float* dst = Cz + (long)m * ldc + n0 + n;
-          const float y = Cs[rr * CS_LD + c];
-          *dst = acc ? *dst + y : y;
-        }
+    if (m >= t.M) continue;
+    const int n = n0 + c0;
+    float* dst = t.C + z * cz + (long)m * t.ldc + n;
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) {
+      float y[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) y[q] = issued ? __uint_as_float(v[j + q]) : 0.0f;
+      if constexpr (EPI == EPI_GELU) {
+        const float4 b = *reinterpret_cast<const float4*>(t.aux + n + j);
+        y[0] += b.x; y[1] += b.y; y[2] += b.z; y[3] += b.w;
+        *reinterpret_cast<float4*>(t.H + (long)m * t.ldc + n + j) =
+            make_float4(bf16r(gelu_f(y[0])), bf16r(gelu_f(y[1])), bf16r(gelu_f(y[2])), bf16r(gelu_f(y[3])));
       }
+      if constexpr (EPI == EPI_DGELU) {
+        const float4 a = *reinterpret_cast<const float4*>(t.aux + (long)m * t.ldc + n + j);
+        y[0] *= gelu_prime_f(a.x); y[1] *= gelu_prime_f(a.y); y[2] *= gelu_prime_f(a.z); y[3] *= gelu_prime_f(a.w);
+      }
+      *reinterpret_cast<float4*>(dst + j) = make_float4(y[0], y[1], y[2], y[3]);
     }
   }
   tc::fence_before();
   __syncthreads();
-  if (threadIdx.x < 32) tc::tmem_dealloc(tbase, 128);
+  if (threadIdx.x < 32) tc::tmem_dealloc(tbase, TMEM);
   if (threadIdx.x == 0 && !ok) atomicExch(err_flag, 1);
-}
-
-// C (+)= sum over z of W[z] (M x N, row stride N), in the order z = 0, 1, ...
-__global__ void k_sum_splits(const float* __restrict__ W, int nz, int M, int N, float* __restrict__ C, int ldc,
-                             int acc) {
-  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long)M * N) return;
-  const int m = (int)(e / N), n = (int)(e % N);
-  float s = acc ? C[(long)m * ldc + n] : 0.0f;
-  for (int z = 0; z < nz; z++) s += W[(long)z * M * N + e];
-  C[(long)m * ldc + n] = s;
 }
 
 // h0 = bf16((x - mu) * inv_std) for the rows idx[0..B) of X (rnd = 0: FP32 debug mode, no
@@ -418,25 +451,39 @@ __global__ void k_bias_gelu(float* __restrict__ Z, const float* __restrict__ b, 
   Hn[e] = rnd ? bf16r(h) : h;
 }
 
-// y = h3 . w4 + b4, residual, loss partial and dy = 2 (y - t) / B.  One warp per row.
-__global__ void k_out(const float* __restrict__ H3, const float* __restrict__ w4q, const float* __restrict__ b4,
-                      const float* __restrict__ T, const int* __restrict__ idx, int B, float* __restrict__ Y,
-                      float* __restrict__ dY, double* __restrict__ loss_acc) {
-  int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (r >= B) return;
-  float s = 0.0f;
-  for (int q = lane; q < MH; q += 32) s += H3[(long)r * MH + q] * w4q[q];
+// y = h3 . w4 + b4, residual, loss partial and dy = 2 (y - t) / B (and, as the first operand of the
+// tensor-core product dy w4, in rows of four).  One warp per row.
+__global__ void __launch_bounds__(256) k_out(const float* __restrict__ H3, const float* __restrict__ w4q,
+                                             const float* __restrict__ b4, const float* __restrict__ T,
+                                             const int* __restrict__ idx, int B, float* __restrict__ Y,
+                                             float* __restrict__ dY, double* __restrict__ loss_acc,
+                                             float* __restrict__ dY4 = nullptr) {
+  __shared__ double sq[8];
+  const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) sq[threadIdx.x >> 5] = 0.0;
+  if (r < B) {
+    float s = 0.0f;
+    for (int q = lane; q < MH; q += 32) s += H3[(long)r * MH + q] * w4q[q];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) {
-    float y = s + b4[0];
-    if (Y) Y[r] = y;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float y = s + b4[0];
+    if (lane == 0 && Y) Y[r] = y;
     if (T) {
-      float t = T[idx ? idx[r] : r];
-      float d = y - t;
-      dY[r] = 2.0f * d / (float)B;
-      atomicAdd(loss_acc, (double)d * d);
+      const float d = y - T[idx ? idx[r] : r], dy = 2.0f * d / (float)B;
+      if (lane == 0) {
+        dY[r] = dy;
+        if (dY4) reinterpret_cast<float4*>(dY4)[r] = make_float4(dy, 0.0f, 0.0f, 0.0f);
+        sq[threadIdx.x >> 5] = (double)d * d;
+      }
     }
+  }
+  if (!T) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double l = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) l += sq[k];
+    atomicAdd(loss_acc, l);
   }
 }
 
@@ -446,11 +493,10 @@ __global__ void k_dz(const float* __restrict__ dH, const float* __restrict__ Z, 
 }
 
 // Column sums of a (B x ncol) matrix into g (fixed order per column).
-// g[col] = sum_r w[r] A[r][col] (w == nullptr: w = 1), one block per column.
-__global__ void k_colsum(const float* __restrict__ A, int B, int ncol, float* __restrict__ g,
-                         const float* __restrict__ w = nullptr) {
+// g[col] = sum_r w[r] A[r][col] (w == nullptr: w = 1), one block of 256 per column.
+__device__ __forceinline__ void column_sum(const float* __restrict__ A, int B, int ncol, int col, float* __restrict__ g,
+                                           const float* __restrict__ w) {
   __shared__ float sh[256];
-  int col = blockIdx.x;
   float s = 0.0f;
   if (w)
     for (int r = threadIdx.x; r < B; r += blockDim.x) s = fmaf(w[r], A[(long)r * ncol + col], s);
@@ -463,6 +509,45 @@ __global__ void k_colsum(const float* __restrict__ A, int B, int ncol, float* __
     __syncthreads();
   }
   if (threadIdx.x == 0) g[col] = sh[0];
+}
+__global__ void __launch_bounds__(256) k_colsum(const float* __restrict__ A, int B, int ncol, float* __restrict__ g,
+                                                const float* __restrict__ w = nullptr) {
+  column_sum(A, B, ncol, blockIdx.x, g, w);
+}
+
+// The end of the tensor-core backward pass in one launch: the k-split partial tiles of the three weight
+// gradients summed in order (256 elements per block), then the column sums: biases of the three hidden
+// layers, the output layer's weights and bias (a block per column); the header of g is zero.
+struct GradFinish {
+  const float* ws[3];   // partial tiles [z][MH][N]
+  int N[3], ow[3], ob[3];
+  const float* dZ[3];
+  const float *H3, *dY;
+};
+__global__ void __launch_bounds__(256) k_grad_finish(GradFinish f, int kz, long cz, int B, float* __restrict__ g) {
+  int b = blockIdx.x;
+#pragma unroll
+  for (int l = 0; l < 3; l++) {
+    const int nb = MH * f.N[l] / 256;
+    if (b < nb) {
+      const int e = b * 256 + threadIdx.x;
+      float s = 0.0f;
+#pragma unroll 4
+      for (int z = 0; z < kz; z++) s += f.ws[l][z * cz + e];
+      g[f.ow[l] + e] = s;
+      return;
+    }
+    b -= nb;
+  }
+  if (b < 3 * MH) {
+    const int l = b / MH;
+    column_sum(l == 0 ? f.dZ[0] : l == 1 ? f.dZ[1] : f.dZ[2], B, MH, b % MH, g + (l == 0 ? f.ob[0] : l == 1 ? f.ob[1] : f.ob[2]), nullptr);
+  } else if (b < 4 * MH) {
+    column_sum(f.H3, B, MH, b - 3 * MH, g + O_W4, f.dY);
+  } else {
+    column_sum(f.dY, B, 1, 0, g + O_B4, nullptr);
+    if (threadIdx.x < MHEADER) g[threadIdx.x] = 0.0f;
+  }
 }
 
 // Adam on the parameters (header entries are constants); q = BF16-rounded copy of weights.
@@ -762,117 +847,153 @@ __global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_tc(const float* __restri
   if (threadIdx.x == 0 && bad) atomicExch(err_flag, 1);
 }
 
+// Device memory of one call, from the library's pool on the call's stream (a dozen cudaMalloc and
+// cudaFree took more than half of a gradient of 1024 rows); what is too large to keep in the pool is
+// allocated and freed by itself.
+constexpr size_t SCRATCH_POOLED = (size_t)64 << 20;
+struct Scratch {
+  cudaStream_t stream;
+  std::vector<void*> pooled, plain;
+  explicit Scratch(cudaStream_t s) : stream(s) {}
+  Scratch(const Scratch&) = delete;
+  ~Scratch() {
+    for (void* p : pooled) pnm_pool_free(stream, p);
+    for (void* p : plain) cudaFree(p);
+  }
+};
+
 template <typename T>
-T* xalloc(size_t n, std::vector<void*>& owned) {
+T* xalloc(size_t n, Scratch& sc) {
+  const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
+  if (bytes <= SCRATCH_POOLED) {
+    sc.pooled.push_back(pnm_pool_alloc(sc.stream, bytes));
+    return (T*)sc.pooled.back();
+  }
   void* p = nullptr;
-  if (cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)) != cudaSuccess) {
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
     throw PnmError{PNM_ENOMEM, "cudaMalloc (warm-start network) failed"};
   }
-  owned.push_back(p);
+  sc.plain.push_back(p);
   return (T*)p;
 }
-
-struct Scratch {
-  std::vector<void*> owned;
-  ~Scratch() {
-    for (void* p : owned) cudaFree(p);
-  }
-};
 
 // Training/inference buffers for a batch of B rows.
 struct Net {
   float *w, *q, *g, *m, *v;  // parameters, BF16-rounded copy, gradient, Adam moments
-  float *H0, *Z1, *H1, *Z2, *H2, *Z3, *H3, *Y, *dY, *dA, *dB;
+  float *H0, *Z1, *H1, *Z2, *H2, *Z3, *H3, *Y, *dY, *dY4, *dA, *dB, *dC;
   int B;
   // tc = 1: the matrix products on the tensor cores (k_gemm_tc; BF16 mode only); ws holds the
-  // partial tiles of a k-split product, err the kernel's timeout flag
+  // partial tiles of the k-split weight gradients, err the kernel's timeout flag
   int tc = 0;
   float* ws = nullptr;
-  long ws_cap = 0;
   int* err = nullptr;
-  void alloc(int b, Scratch& s, int use_tc = 0, cudaStream_t st = nullptr) {
+  void alloc(int b, Scratch& s, int use_tc = 0) {
     B = b;
     tc = use_tc;
-    if (tc) {
-      ws_cap = (long)TG_MAX_SPLIT * std::max(b, MH) * MH;
-      ws = xalloc<float>(ws_cap, s.owned);
-      err = xalloc<int>(1, s.owned);
-      CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
-      smem_at_least(k_gemm_tc, TG_SMEM);
+    // one block; every array starts on a 16-byte boundary
+    const size_t r = b, sizes[] = {NPARAM, NPARAM, NPARAM, NPARAM, NPARAM, r * MF, r * MH, r * MH, r * MH,
+                                   r * MH, r * MH, r * MH, r, r, 4 * r, r * MH, r * MH, r * MH,
+                                   tc ? (size_t)3 * TG_MAX_SPLIT * MH * MH : 0, tc ? 1 : 0};
+    float** at[] = {&w, &q, &g, &m, &v, &H0, &Z1, &H1, &Z2, &H2, &Z3, &H3, &Y, &dY, &dY4, &dA, &dB, &dC, &ws, (float**)nullptr};
+    constexpr int n = sizeof(sizes) / sizeof(sizes[0]);
+    size_t total = 0;
+    for (size_t x : sizes) total += (x + 3) & ~(size_t)3;
+    float* p = xalloc<float>(total, s);
+    for (int k = 0; k < n; k++) {
+      if (at[k]) *at[k] = p;
+      else if (tc) err = reinterpret_cast<int*>(p);
+      p += (sizes[k] + 3) & ~(size_t)3;
     }
-    w = xalloc<float>(NPARAM, s.owned);
-    q = xalloc<float>(NPARAM, s.owned);
-    g = xalloc<float>(NPARAM, s.owned);
-    m = xalloc<float>(NPARAM, s.owned);
-    v = xalloc<float>(NPARAM, s.owned);
-    H0 = xalloc<float>((size_t)b * MF, s.owned);
-    Z1 = xalloc<float>((size_t)b * MH, s.owned);
-    H1 = xalloc<float>((size_t)b * MH, s.owned);
-    Z2 = xalloc<float>((size_t)b * MH, s.owned);
-    H2 = xalloc<float>((size_t)b * MH, s.owned);
-    Z3 = xalloc<float>((size_t)b * MH, s.owned);
-    H3 = xalloc<float>((size_t)b * MH, s.owned);
-    Y = xalloc<float>(b, s.owned);
-    dY = xalloc<float>(b, s.owned);
-    dA = xalloc<float>((size_t)b * MH, s.owned);
-    dB = xalloc<float>((size_t)b * MH, s.owned);
+    if (tc) {
+      CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s.stream));
+      smem_at_least(k_gemm_tc<32, false, true, EPI_GELU>, TG_SMEM);
+      smem_at_least(k_gemm_tc<128, false, true, EPI_GELU>, TG_SMEM);
+      smem_at_least(k_gemm_tc<32, false, false, EPI_DGELU>, TG_SMEM);
+      smem_at_least(k_gemm_tc<128, false, false, EPI_DGELU>, TG_SMEM);
+      smem_at_least(k_gemm_tc<32, true, false, EPI_NONE>, TG_SMEM);
+    }
   }
 };
 
-// A matrix product of the training passes: on the tensor cores when nt.tc is set and both output
-// dimensions are at least 16 (the output layer's vector products stay on k_sgemm), with the k
-// range split over up to TG_MAX_SPLIT CTAs when the output has few tiles.
-void gemm(cudaStream_t s, const Net& nt, int M, int N, int K, const float* A, int lda, int tA, const float* B,
-          int ldb, int tB, float* C, int ldc, int acc) {
-  if (!nt.tc || M < 16 || N < 16) {
-    sgemm(s, M, N, K, A, lda, tA, B, ldb, tB, C, ldc, acc);
-    return;
-  }
-  // about 64 CTAs: narrower column tiles first (the row tiles are fixed at 128), then the k split
-  const int gy = (M + TG_BM - 1) / TG_BM;
-  int bn = TG_BN;
-  while (bn > 32 && ((N + bn - 1) / bn) * gy < 64) bn >>= 1;
-  const int gx = (N + bn - 1) / bn;
-  const int nstage = (K + TG_BK - 1) / TG_BK;
-  int kz = 1;
-  if (gx * gy < 64) kz = std::max(1, std::min(std::min(TG_MAX_SPLIT, nstage), 64 / (gx * gy)));
-  while (kz > 1 && (long)kz * M * N > nt.ws_cap) kz--;
-  if (kz == 1) {
-    k_gemm_tc<<<dim3(gx, gy, 1), 128, TG_SMEM, s>>>(M, N, K, A, lda, tA, B, ldb, tB, C, ldc, 0, acc, bn, nt.err);
-  } else {
-    k_gemm_tc<<<dim3(gx, gy, kz), 128, TG_SMEM, s>>>(M, N, K, A, lda, tA, B, ldb, tB, nt.ws, N, (long)M * N, 0,
-                                                     bn, nt.err);
-    k_sum_splits<<<(unsigned)(((long)M * N + 255) / 256), 256, 0, s>>>(nt.ws, kz, M, N, C, ldc, acc);
-  }
+// The products of the passes on the CUDA cores (the SIMT and FP32 modes, and batches below 16 rows).
+bool on_tensor_cores(const Net& nt, int B) { return nt.tc && B >= 16; }
+
+// A B x MH product of the tensor-core passes with its epilogue: 32 columns per CTA while that leaves
+// fewer than 64 row tiles' worth of CTAs, else the whole row.
+template <bool TB, int EPI>
+void gemm_rows(cudaStream_t s, const Net& nt, int B, int K, const float* A, int lda, const float* W, int ldw, float* C,
+               const float* aux, float* H) {
+  GemmTasks t{};
+  t.t[0] = GemmTask{A, W, C, B, MH, K, lda, ldw, MH, aux, H};
+  const int gy = (B + TG_BM - 1) / TG_BM;
+  if (gy < 64) k_gemm_tc<32, false, TB, EPI><<<dim3(MH / 32, gy, 1), 128, TG_SMEM, s>>>(t, 1, 0, nt.err);
+  else k_gemm_tc<128, false, TB, EPI><<<dim3(1, gy, 1), 128, TG_SMEM, s>>>(t, 1, 0, nt.err);
 }
 
 // rnd = 0: the FP32 debug mode (no BF16 rounding of the layer inputs).
 void net_forward(cudaStream_t s, Net& nt, const float* X, const int* idx, int B, int rnd = 1) {
   k_prep<<<(B * MF + 255) / 256, 256, 0, s>>>(X, idx, B, nt.q, nt.H0, rnd);
-  gemm(s, nt, B, MH, MF, nt.H0, MF, 0, nt.q + O_W1, MF, 1, nt.Z1, MH, 0);
-  k_bias_gelu<<<(B * MH + 255) / 256, 256, 0, s>>>(nt.Z1, nt.q + O_B1, nt.H1, B, rnd);
-  gemm(s, nt, B, MH, MH, nt.H1, MH, 0, nt.q + O_W2, MH, 1, nt.Z2, MH, 0);
-  k_bias_gelu<<<(B * MH + 255) / 256, 256, 0, s>>>(nt.Z2, nt.q + O_B2, nt.H2, B, rnd);
-  gemm(s, nt, B, MH, MH, nt.H2, MH, 0, nt.q + O_W3, MH, 1, nt.Z3, MH, 0);
-  k_bias_gelu<<<(B * MH + 255) / 256, 256, 0, s>>>(nt.Z3, nt.q + O_B3, nt.H3, B, rnd);
+  const float* Hin[3] = {nt.H0, nt.H1, nt.H2};
+  float *Zs[3] = {nt.Z1, nt.Z2, nt.Z3}, *Hs[3] = {nt.H1, nt.H2, nt.H3};
+  const int Ow[3] = {O_W1, O_W2, O_W3}, Ob[3] = {O_B1, O_B2, O_B3}, Kin[3] = {MF, MH, MH};
+  for (int l = 0; l < 3; l++) {
+    if (on_tensor_cores(nt, B)) {
+      gemm_rows<true, EPI_GELU>(s, nt, B, Kin[l], Hin[l], Kin[l], nt.q + Ow[l], Kin[l], Zs[l], nt.q + Ob[l], Hs[l]);
+    } else {
+      sgemm(s, B, MH, Kin[l], Hin[l], Kin[l], 0, nt.q + Ow[l], Kin[l], 1, Zs[l], MH, 0);
+      k_bias_gelu<<<(B * MH + 255) / 256, 256, 0, s>>>(Zs[l], nt.q + Ob[l], Hs[l], B, rnd);
+    }
+  }
 }
 
-// Backward pass from dY; writes the gradient blob nt.g (header entries zero).
+// The output layer, the loss and its error signal dY.
+void net_loss(cudaStream_t s, Net& nt, const float* T, const int* idx, int B, double* lacc) {
+  const bool fused = on_tensor_cores(nt, B);
+  k_out<<<(B * 32 + 255) / 256, 256, 0, s>>>(nt.H3, nt.q + O_W4, nt.q + O_B4, T, idx, B, nt.Y, nt.dY, lacc,
+                                             fused ? nt.dY4 : nullptr);
+}
+
+// Backward pass from the error signals; writes the gradient blob nt.g (header entries zero).
 void net_backward(cudaStream_t s, Net& nt, int B) {
+  const float* Zs[3] = {nt.Z1, nt.Z2, nt.Z3};
+  const float* Hin[3] = {nt.H0, nt.H1, nt.H2};
+  const int Ow[3] = {O_W1, O_W2, O_W3}, Ob[3] = {O_B1, O_B2, O_B3}, Kin[3] = {MF, MH, MH};
+  if (on_tensor_cores(nt, B)) {
+    // dZ3, dZ2, dZ1 in turn, then the three weight gradients dZ^T H in one launch, k-split over the batch
+    gemm_rows<false, EPI_DGELU>(s, nt, B, 1, nt.dY4, 4, nt.q + O_W4, MH, nt.dC, nt.Z3, nullptr);
+    gemm_rows<false, EPI_DGELU>(s, nt, B, MH, nt.dC, MH, nt.q + O_W3, MH, nt.dB, nt.Z2, nullptr);
+    gemm_rows<false, EPI_DGELU>(s, nt, B, MH, nt.dB, MH, nt.q + O_W2, MH, nt.dA, nt.Z1, nullptr);
+    const float* dZ[3] = {nt.dA, nt.dB, nt.dC};
+    const int kz = std::min(TG_MAX_SPLIT, (B + TG_BK - 1) / TG_BK);
+    const long cz = (long)MH * MH;
+    GemmTasks t{};
+    GradFinish f{};
+    for (int l = 0; l < 3; l++) {
+      float* ws = nt.ws + l * TG_MAX_SPLIT * cz;
+      t.t[l] = GemmTask{dZ[l], Hin[l], ws, MH, Kin[l], B, MH, Kin[l], Kin[l], nullptr, nullptr};
+      f.ws[l] = ws;
+      f.N[l] = Kin[l];
+      f.ow[l] = Ow[l];
+      f.ob[l] = Ob[l];
+      f.dZ[l] = dZ[l];
+    }
+    f.H3 = nt.H3;
+    f.dY = nt.dY;
+    k_gemm_tc<32, true, false, EPI_NONE><<<dim3(MH / 32, 1, 3 * kz), 128, TG_SMEM, s>>>(t, kz, cz, nt.err);
+    k_grad_finish<<<MH * (MF + 2 * MH) / 256 + 4 * MH + 1, 256, 0, s>>>(f, kz, cz, B, nt.g);
+    return;
+  }
   CUDA_TRY(cudaMemsetAsync(nt.g, 0, sizeof(float) * NPARAM, s));
   // output layer: dw4 = dY^T H3 (a weighted column sum), db4 = sum dY, dH3 = dY w4
   k_colsum<<<MH, 256, 0, s>>>(nt.H3, B, MH, nt.g + O_W4, nt.dY);
   k_colsum<<<1, 256, 0, s>>>(nt.dY, B, 1, nt.g + O_B4);
-  gemm(s, nt, B, MH, 1, nt.dY, 1, 0, nt.q + O_W4, MH, 0, nt.dA, MH, 0);
-  const float* Zs[3] = {nt.Z1, nt.Z2, nt.Z3};
-  const float* Hin[3] = {nt.H0, nt.H1, nt.H2};
-  const int Ow[3] = {O_W1, O_W2, O_W3}, Ob[3] = {O_B1, O_B2, O_B3}, Kin[3] = {MF, MH, MH};
+  sgemm(s, B, MH, 1, nt.dY, 1, 0, nt.q + O_W4, MH, 0, nt.dA, MH, 0);
   for (int l = 2; l >= 0; l--) {
     k_dz<<<(B * MH + 255) / 256, 256, 0, s>>>(nt.dA, Zs[l], nt.dB, B * MH);
-    gemm(s, nt, MH, Kin[l], B, nt.dB, MH, 1, Hin[l], Kin[l], 0, nt.g + Ow[l], Kin[l], 0);
+    sgemm(s, MH, Kin[l], B, nt.dB, MH, 1, Hin[l], Kin[l], 0, nt.g + Ow[l], Kin[l], 0);
     k_colsum<<<MH, 256, 0, s>>>(nt.dB, B, MH, nt.g + Ob[l]);
-    if (l > 0) gemm(s, nt, B, MH, MH, nt.dB, MH, 0, nt.q + Ow[l], MH, 0, nt.dA, MH, 0);
+    if (l > 0) sgemm(s, B, MH, MH, nt.dB, MH, 0, nt.q + Ow[l], MH, 0, nt.dA, MH, 0);
   }
 }
 
@@ -1148,17 +1269,17 @@ int pnm_mlp_forward(const float* blob, const float* X, long n, float* Y, int mod
     const int rnd = mode == PNM_MLP_SIMT_FP32 ? 0 : 1;
     check_blob_header(blob);
     cudaStream_t s = (cudaStream_t)stream;
-    Scratch sc;
-    float* w = xalloc<float>(NPARAM, sc.owned);
-    float* q = xalloc<float>(NPARAM, sc.owned);
-    float* dX = xalloc<float>((size_t)n * MF, sc.owned);
-    float* dY = xalloc<float>(n, sc.owned);
+    Scratch sc(s);
+    float* w = xalloc<float>(NPARAM, sc);
+    float* q = xalloc<float>(NPARAM, sc);
+    float* dX = xalloc<float>((size_t)n * MF, sc);
+    float* dY = xalloc<float>(n, sc);
     CUDA_TRY(cudaMemcpyAsync(w, blob, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(dX, X, sizeof(float) * n * MF, cudaMemcpyHostToDevice, s));
     k_quantize<<<(NPARAM + 255) / 256, 256, 0, s>>>(w, q, rnd);
     if (use_tensor_cores) {
-      __nv_bfloat16* pw = xalloc<__nv_bfloat16>(PW_TOTAL, sc.owned);
-      int* err = xalloc<int>(1, sc.owned);
+      __nv_bfloat16* pw = xalloc<__nv_bfloat16>(PW_TOTAL, sc);
+      int* err = xalloc<int>(1, sc);
       CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
       mlp_tc_attributes();
       k_pack_weights<<<(PW_TOTAL + 255) / 256, 256, 0, s>>>(q, pw);
@@ -1196,12 +1317,12 @@ int pnm_mlp_loss_grad(const float* blob, const float* X, const float* T, int n, 
     check_blob_header(blob);
     cudaStream_t s = (cudaStream_t)stream;
     if (fp32 < 0 || fp32 > 2) throw PnmError{PNM_EINVAL, "unknown gradient mode"};
-    Scratch sc;
+    Scratch sc(s);
     Net nt;
-    nt.alloc(n, sc, fp32 == 0 ? 1 : 0, s);  // 0: BF16 on the tensor cores, 2: BF16 on k_sgemm
-    float* dX = xalloc<float>((size_t)n * MF, sc.owned);
-    float* dT = xalloc<float>(n, sc.owned);
-    double* lacc = xalloc<double>(1, sc.owned);
+    nt.alloc(n, sc, fp32 == 0 ? 1 : 0);  // 0: BF16 on the tensor cores, 2: BF16 on k_sgemm
+    float* dX = xalloc<float>((size_t)n * MF, sc);
+    float* dT = xalloc<float>(n, sc);
+    double* lacc = xalloc<double>(1, sc);
     CUDA_TRY(cudaMemcpyAsync(nt.w, blob, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(dX, X, sizeof(float) * (size_t)n * MF, cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(dT, T, sizeof(float) * n, cudaMemcpyHostToDevice, s));
@@ -1209,7 +1330,7 @@ int pnm_mlp_loss_grad(const float* blob, const float* X, const float* T, int n, 
     const int rnd = fp32 == 1 ? 0 : 1;
     k_quantize<<<(NPARAM + 255) / 256, 256, 0, s>>>(nt.w, nt.q, rnd);
     net_forward(s, nt, dX, nullptr, n, rnd);
-    k_out<<<(n * 32 + 255) / 256, 256, 0, s>>>(nt.H3, nt.q + O_W4, nt.q + O_B4, dT, nullptr, n, nt.Y, nt.dY, lacc);
+    net_loss(s, nt, dT, nullptr, n, lacc);
     net_backward(s, nt, n);
     CUDA_TRY(cudaGetLastError());
     double l = 0;
@@ -1239,9 +1360,10 @@ int pnm_mlp_train(pnm_ctx* const* ctxs, int nctx, const pnm_mlp_opts* o, float* 
       if (!ctxs[k]) throw PnmError{PNM_EINVAL, "null context"};
       ntot += ctxs[k]->nt;
     }
-    Scratch sc;
-    float* X = xalloc<float>((size_t)ntot * MF, sc.owned);
-    float* T = xalloc<float>(ntot, sc.owned);
+    Scratch sc(s);
+    float* X = xalloc<float>((size_t)ntot * MF, sc);
+    float* T = xalloc<float>(ntot, sc);
+    CUDA_TRY(cudaStreamSynchronize(s));  // the contexts fill both on their own streams
     long off = 0;
     for (int k = 0; k < nctx; k++) {
       pnm_ctx* c = ctxs[k];
@@ -1254,7 +1376,7 @@ int pnm_mlp_train(pnm_ctx* const* ctxs, int nctx, const pnm_mlp_opts* o, float* 
       off += c->nt;
     }
     // normalisation from the training data
-    double* st = xalloc<double>(2 * MF + 2, sc.owned);
+    double* st = xalloc<double>(2 * MF + 2, sc);
     k_featstats<<<MF, 256, 0, s>>>(X, ntot, st);
     std::vector<double> hs(2 * MF + 2);
     CUDA_TRY(cudaMemcpyAsync(hs.data(), st, sizeof(double) * 2 * MF, cudaMemcpyDeviceToHost, s));
@@ -1280,9 +1402,9 @@ int pnm_mlp_train(pnm_ctx* const* ctxs, int nctx, const pnm_mlp_opts* o, float* 
     }
     int B = (int)std::min<long>(o->batch, ntot);
     Net nt;
-    nt.alloc(B, sc, 1, s);  // BF16 training: the matrix products on the tensor cores
-    int* idx = xalloc<int>(ntot, sc.owned);
-    double* lacc = xalloc<double>(1, sc.owned);
+    nt.alloc(B, sc, 1);  // BF16 training: the matrix products on the tensor cores
+    int* idx = xalloc<int>(ntot, sc);
+    double* lacc = xalloc<double>(1, sc);
     CUDA_TRY(cudaMemcpyAsync(nt.w, blob, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemsetAsync(nt.m, 0, sizeof(float) * NPARAM, s));
     CUDA_TRY(cudaMemsetAsync(nt.v, 0, sizeof(float) * NPARAM, s));
@@ -1302,8 +1424,7 @@ int pnm_mlp_train(pnm_ctx* const* ctxs, int nctx, const pnm_mlp_opts* o, float* 
       long nb = 0;
       for (long r0 = 0; r0 + B <= ntot; r0 += B, nb++) {
         net_forward(s, nt, X, idx + r0, B);
-        k_out<<<(B * 32 + 255) / 256, 256, 0, s>>>(nt.H3, nt.q + O_W4, nt.q + O_B4, T, idx + r0, B, nt.Y, nt.dY,
-                                                   lacc);
+        net_loss(s, nt, T, idx + r0, B, lacc);
         net_backward(s, nt, B);
         // half-cosine decay from lr to lr_final over the steps (constant when they are equal)
         const double frac = nsteps > 1 ? (double)step / (double)(nsteps - 1) : 0.0;
