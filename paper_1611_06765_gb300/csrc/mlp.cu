@@ -46,10 +46,6 @@ __device__ __forceinline__ float tanh_fast(float x) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ float gelu_fast(float z) {
-  float hz = 0.5f * z;
-  return fmaf(hz, tanh_fast(z * fmaf(GELU_C1, z * z, GELU_C0)), hz);
-}
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
 // ------------------------------------------------------------------------ features
@@ -633,9 +629,36 @@ __global__ void k_pack_weights(const float* __restrict__ q, __nv_bfloat16* __res
   }
 }
 
-constexpr int MLP_THREADS = 256;
+// Inference CTA: MLP_GROUPS groups of 256 threads, a 128-sample tile each, share one copy of the weights.
+constexpr int MLP_GROUPS = 4, MLP_THREADS = MLP_GROUPS * 256;
 constexpr int MLP_PAR = 3 * MH + 1 + 2 * MF;  // b1, b2, b3, b4, mu, inv_std
-constexpr uint32_t MLP_SMEM = 1024 + PW_TOTAL * 2 + MH * MH * 2 + ((MLP_PAR * 4 + 1023) / 1024) * 1024;
+constexpr uint32_t MLP_SMEM =
+    1024 + PW_TOTAL * 2 + MLP_GROUPS * MH * MH * 2 + ((MLP_PAR * 4 + 1023) / 1024) * 1024;
+
+// Two FP32 lanes per instruction (each rounded as the scalar one).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 x, y, z, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\tfma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 gelu_fast2(float2 z) {
+  const float2 h = mul2(make_float2(0.5f, 0.5f), z);
+  const float2 w = mul2(z, fma2(make_float2(GELU_C1, GELU_C1), mul2(z, z), make_float2(GELU_C0, GELU_C0)));
+  return fma2(h, make_float2(tanh_fast(w.x), tanh_fast(w.y)), h);
+}
 
 // Where the inference writes: raw outputs Y, and/or the learned start amplitudes
 // t0 = t_MBPT2 + sigma_sys * y_scale * y of every system (t_begin: first amplitude of each
@@ -661,37 +684,40 @@ struct MlpFused {
   const double* inv_sigma;
 };
 
-// One CTA (8 warps) loops over 128-sample tiles; two CTAs share an SM, so one CTA's
-// epilogue overlaps the other's MMAs.  Warp w reads TMEM lanes 32 (w % 4) ... + 31 (its
-// row quarter) and columns 64 (w / 4) ... + 63 (its column half); thread (w, lane) owns
-// sample row 32 (w % 4) + lane of the tile.
+// One CTA per SM; each of its groups of eight warps loops over 128-sample tiles by itself (named
+// barrier, mbarrier, A operand and 128 columns of tensor memory of its own), so that one group's
+// products and waits overlap the others' epilogues.  Warp w of a group reads TMEM lanes 32 (w % 4) ... + 31
+// (its row quarter) and columns 64 (w / 4) ... + 63 (its column half).
+// Bound by the latencies of the epilogue (49,152 GELUs per tile, the arithmetic around the tanh done on
+// pairs) at 32 warps per SM.  Two CTAs of eight warps per SM, each with its own weights and alternating
+// between product and epilogue, took 366 us for three N=66, N_max=36 systems (1.56 M samples), four
+// groups of four warps 286, this 258 us.
 // FUSED: the samples' features are formed from the context (MlpFused) instead of read from X.
 template <bool FUSED>
-__global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_tc(const float* __restrict__ X, long n,
+__global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp_tc(const float* __restrict__ X, long n,
                                                            const float* __restrict__ q,
                                                            const __nv_bfloat16* __restrict__ pw, MlpOut out,
                                                            MlpFused fin, int* __restrict__ err_flag) {
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bar_w = reinterpret_cast<uint64_t*>(smem);
-  uint64_t* bar_mma = bar_w + 1;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar_w + 2);
+  uint64_t* bars = bar_w + 1;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar_w + 1 + MLP_GROUPS);
+  const int group = threadIdx.x >> 8, half = (threadIdx.x >> 7) & 1, row = threadIdx.x & 127, warp = threadIdx.x >> 5;
+  uint64_t* bar_mma = bars + group;
   __nv_bfloat16* W = reinterpret_cast<__nv_bfloat16*>(smem + 1024);
-  __nv_bfloat16* A = W + PW_TOTAL;
-  float* par = reinterpret_cast<float*>(A + MH * MH);  // b1 b2 b3 | b4 | mu | inv_std
-  const float* mu = par + 3 * MH + 1;
+  __nv_bfloat16* A = W + PW_TOTAL + group * MH * MH;
+  float* par = reinterpret_cast<float*>(W + PW_TOTAL + MLP_GROUPS * MH * MH);  // b1 b2 b3 | mu | inv_std | b4
+  const float* mu = par + 3 * MH;
   const float* istd = mu + MF;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int quarter = warp & 3, half = warp >> 2;
-  const int row = quarter * 32 + lane;
-  __shared__ int bad;
-  if (threadIdx.x == 0) {
-    bad = 0;
-    tc::mbar_init(bar_w, 1);
+  __shared__ int bad[MLP_GROUPS];
+  if ((threadIdx.x & 255) == 0) {
+    bad[group] = 0;
     tc::mbar_init(bar_mma, 1);
+    if (group == 0) tc::mbar_init(bar_w, 1);
     tc::mbar_fence_init();
   }
   if (warp == 2) {
-    tc::tmem_alloc(tslot, MH);
+    tc::tmem_alloc(tslot, MLP_GROUPS * MH);
     tc::tmem_relinquish();
   }
   for (int k = threadIdx.x; k < MH; k += blockDim.x) {
@@ -700,27 +726,28 @@ __global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_tc(const float* __restri
     par[2 * MH + k] = q[O_B3 + k];
   }
   for (int k = threadIdx.x; k < MF; k += blockDim.x) {
-    par[3 * MH + 1 + k] = q[O_MU + k];
-    par[3 * MH + 1 + MF + k] = q[O_IS + k];
+    par[3 * MH + k] = q[O_MU + k];
+    par[3 * MH + MF + k] = q[O_IS + k];
   }
-  if (threadIdx.x == 0) par[3 * MH] = q[O_B4];
+  const float b4 = q[O_B4];
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  const uint32_t tbase = *tslot;
+  const uint32_t tbase = *tslot + group * MH;
   if (threadIdx.x == 0) {
     tc::mbar_expect_tx(bar_w, PW_TOTAL * 2);
     tc::bulk_g2s(W, pw, PW_TOTAL * 2, bar_w);
   }
-  if (!tc::mbar_wait(bar_w, 0)) bad = 1;
+  if (!tc::mbar_wait(bar_w, 0)) bad[group] = 1;
+  auto group_sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(group + 1) : "memory"); };
   uint32_t phase = 0;
-  const long ntiles = (n + MH - 1) / MH;
-  const uint32_t lane_addr = tbase + ((uint32_t)(quarter * 32) << 16);
-  // features [16 half, 16 half + 16) of this thread's row of a tile (zeros past n); the next
-  // tile's are loaded while the current one runs through the layers
+  const long ntiles = (n + MH - 1) / MH, step = (long)gridDim.x * MLP_GROUPS;
+  const uint32_t lane_addr = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+  // features [16 half, 16 half + 16) of this thread's row of a tile (zeros past n); the next tile's are
+  // loaded beside the current one's last product (earlier they would take registers from the epilogues)
   const int k0 = 16 * half;
-  auto load_x = [&](long tile, float4 (&xr)[4]) {
-    long rg = tile * MH + row;
+  auto load_x = [&](long tile, float (&x)[16]) {
+    const long rg = tile * MH + row;
     if (tile < ntiles && rg < n) {
       if constexpr (FUSED) {
         const int2 zc = fin.rep[rg];
@@ -728,57 +755,52 @@ __global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_tc(const float* __restri
         const int rel = (int)(zc.x - fin.D.ch_t_off[zc.y]);
         const int ij = rel / npp, ab = rel - ij * npp;
         const int sy = fin.D.ch_sys[zc.y];
-        float xh[16];
-        feature_half(fin.D, fin.fs[sy], fin.inv_sigma[sy], zc.y, ij, ab, zc.x, half, xh);
-#pragma unroll
-        for (int j = 0; j < 4; j++) xr[j] = make_float4(xh[4 * j], xh[4 * j + 1], xh[4 * j + 2], xh[4 * j + 3]);
+        feature_half(fin.D, fin.fs[sy], fin.inv_sigma[sy], zc.y, ij, ab, zc.x, half, x);
       } else {
         const long zg = out.idx ? (long)out.idx[rg] : rg;
         const float4* xp = reinterpret_cast<const float4*>(X + zg * MF + k0);
 #pragma unroll
-        for (int j = 0; j < 4; j++) xr[j] = __ldg(xp + j);
+        for (int k = 0; k < 16; k += 4) {
+          const float4 v = __ldg(xp + k / 4);
+          x[k] = v.x; x[k + 1] = v.y; x[k + 2] = v.z; x[k + 3] = v.w;
+        }
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < 4; j++) xr[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int k = 0; k < 16; k++) x[k] = 0.0f;
     }
   };
-  float4 xnext[4];
-  load_x(blockIdx.x, xnext);
-  for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    // every thread leaves together after a failed wait (no thread may skip a barrier)
-    __syncthreads();
-    const int stop = bad;
-    __syncthreads();
+  float xnext[16];
+  long tile = (long)group * gridDim.x + blockIdx.x;  // few tiles: one per SM before a second one
+  load_x(tile, xnext);
+  for (; tile < ntiles; tile += step) {
+    // every thread of a group leaves together after a failed wait (no thread may skip a barrier)
+    group_sync();
+    const int stop = bad[group];
+    group_sync();
     if (stop) break;
     const long r_glob = tile * MH + row;
     const bool ok = r_glob < n;
-    float xv[16];
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      xv[4 * j] = xnext[j].x; xv[4 * j + 1] = xnext[j].y; xv[4 * j + 2] = xnext[j].z; xv[4 * j + 3] = xnext[j].w;
-    }
-    load_x(tile + gridDim.x, xnext);
     // layer-1 input: normalised, BF16
-    {
 #pragma unroll
-      for (int k = 0; k < 16; k++) xv[k] = ok ? (xv[k] - mu[k0 + k]) * istd[k0 + k] : 0.0f;
+    for (int h = 0; h < 16; h += 8) {
+      __align__(16) __nv_bfloat162 v4[4];
 #pragma unroll
-      for (int h = 0; h < 16; h += 8) {
-        __align__(16) __nv_bfloat162 v4[4];
-#pragma unroll
-        for (int j = 0; j < 4; j++) v4[j] = __floats2bfloat162_rn(xv[h + 2 * j], xv[h + 2 * j + 1]);
-        *reinterpret_cast<uint4*>(A + tc::core_off(row, k0 + h, MF / 8)) = *reinterpret_cast<uint4*>(v4);
+      for (int j = 0; j < 4; j++) {
+        const int k = h + 2 * j;
+        v4[j] = ok ? __floats2bfloat162_rn((xnext[k] - mu[k0 + k]) * istd[k0 + k], (xnext[k + 1] - mu[k0 + k + 1]) * istd[k0 + k + 1])
+                   : __floats2bfloat162_rn(0.0f, 0.0f);
       }
+      *reinterpret_cast<uint4*>(A + tc::core_off(row, k0 + h, MF / 8)) = *reinterpret_cast<uint4*>(v4);
     }
     for (int layer = 0; layer < 4; layer++) {
       tc::fence_async_smem();
       tc::fence_before();
-      __syncthreads();
+      group_sync();
       tc::fence_after();
       const int K = layer == 0 ? MF : MH;
       const int N = layer == 3 ? 16 : MH;
-      if (threadIdx.x == 0) {
+      if ((threadIdx.x & 255) == 0) {
         const __nv_bfloat16* Wl = W + (layer == 0 ? 0 : layer == 1 ? PW1 : layer == 2 ? PW1 + PW2 : PW1 + 2 * PW2);
         const uint32_t sbo = (K / 8) * 128;
         const uint32_t idesc = tc::idesc_bf16(MH, N);
@@ -790,35 +812,36 @@ __global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_tc(const float* __restri
         tc::commit(bar_mma);
       }
       __syncwarp();
-      if (!tc::mbar_wait(bar_mma, phase & 1)) bad = 1;
+      if (layer == 3) load_x(tile + step, xnext);
+      if (!tc::mbar_wait(bar_mma, phase & 1)) bad[group] = 1;
       phase++;
+      __syncwarp();
       tc::fence_after();
       if (layer < 3) {
-        // bias + GELU of this thread's 64 columns, BF16, into the next layer's A operand
+        // bias + GELU of this thread's row, BF16, into the next layer's A operand
         const float* b = par + layer * MH;
-        const int cbase = 64 * half;
-        uint32_t r[64];
-        tc::tmem_ld16_nowait(lane_addr + cbase, *reinterpret_cast<uint32_t(*)[16]>(r));
-        tc::tmem_ld16_nowait(lane_addr + cbase + 16, *reinterpret_cast<uint32_t(*)[16]>(r + 16));
-        tc::tmem_ld16_nowait(lane_addr + cbase + 32, *reinterpret_cast<uint32_t(*)[16]>(r + 32));
-        tc::tmem_ld16_nowait(lane_addr + cbase + 48, *reinterpret_cast<uint32_t(*)[16]>(r + 48));
-        tc::tmem_wait_ld();
+#pragma unroll 1
+        for (int c0 = 64 * half; c0 < 64 * half + 64; c0 += 16) {
+          uint32_t r[16];
+          tc::tmem_ld16(lane_addr + c0, r);
 #pragma unroll
-        for (int h = 0; h < 64; h += 8) {
-          __align__(16) __nv_bfloat162 v4[4];
+          for (int h = 0; h < 16; h += 8) {
+            __align__(16) __nv_bfloat162 v4[4];
 #pragma unroll
-          for (int j = 0; j < 4; j++) {
-            float z0 = __uint_as_float(r[h + 2 * j]) + b[cbase + h + 2 * j];
-            float z1 = __uint_as_float(r[h + 2 * j + 1]) + b[cbase + h + 2 * j + 1];
-            v4[j] = __floats2bfloat162_rn(gelu_fast(z0), gelu_fast(z1));
+            for (int j = 0; j < 4; j++) {
+              const float2 bb = *reinterpret_cast<const float2*>(b + c0 + h + 2 * j);
+              const float2 g = gelu_fast2(
+                  add2(make_float2(__uint_as_float(r[h + 2 * j]), __uint_as_float(r[h + 2 * j + 1])), bb));
+              v4[j] = __floats2bfloat162_rn(g.x, g.y);
+            }
+            *reinterpret_cast<uint4*>(A + tc::core_off(row, c0 + h, MH / 8)) = *reinterpret_cast<uint4*>(v4);
           }
-          *reinterpret_cast<uint4*>(A + tc::core_off(row, cbase + h, MH / 8)) = *reinterpret_cast<uint4*>(v4);
         }
       } else if (half == 0) {
         uint32_t r[16];
         tc::tmem_ld16(lane_addr, r);
         if (ok) {
-          float y = __uint_as_float(r[0]) + par[3 * MH];
+          float y = __uint_as_float(r[0]) + b4;
           if (out.Y) out.Y[r_glob] = y;
           if (out.t0) {
             long z;
@@ -843,8 +866,8 @@ __global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_tc(const float* __restri
   }
   tc::fence_before();
   __syncthreads();
-  if (warp == 2) tc::tmem_dealloc(tbase, MH);
-  if (threadIdx.x == 0 && bad) atomicExch(err_flag, 1);
+  if (warp == 2) tc::tmem_dealloc(*tslot, MLP_GROUPS * MH);
+  if ((threadIdx.x & 255) == 0 && bad[group]) atomicExch(err_flag, 1);
 }
 
 // Device memory of one call, from the library's pool on the call's stream (a dozen cudaMalloc and
@@ -892,9 +915,9 @@ struct Net {
     B = b;
     tc = use_tc;
     // one block; every array starts on a 16-byte boundary
-    const size_t r = b, sizes[] = {NPARAM, NPARAM, NPARAM, NPARAM, NPARAM, r * MF, r * MH, r * MH, r * MH,
+    const size_t r = b, one = tc ? 1 : 0, sizes[] = {NPARAM, NPARAM, NPARAM, NPARAM, NPARAM, r * MF, r * MH, r * MH, r * MH,
                                    r * MH, r * MH, r * MH, r, r, 4 * r, r * MH, r * MH, r * MH,
-                                   tc ? (size_t)3 * TG_MAX_SPLIT * MH * MH : 0, tc ? 1 : 0};
+                                   one * 3 * TG_MAX_SPLIT * MH * MH, one};
     float** at[] = {&w, &q, &g, &m, &v, &H0, &Z1, &H1, &Z2, &H2, &Z3, &H3, &Y, &dY, &dY4, &dA, &dB, &dC, &ws, (float**)nullptr};
     constexpr int n = sizeof(sizes) / sizeof(sizes[0]);
     size_t total = 0;
@@ -1116,14 +1139,14 @@ static void set_model(pnm_ctx* ctx, const float* blob) {
   pnm_drop_solve_graphs(ctx);  // the learned start's kernels hold y_scale as an argument
 }
 
-// One CTA pair per SM over the 128-sample tiles (fin.rep set: features formed in the kernel).
+// One CTA per SM over the 128-sample tiles (fin.rep set: features formed in the kernel).
 static void tc_infer(cudaStream_t s, const float* X, long n, const float* q, const __nv_bfloat16* pw,
                      const MlpOut& out, int* err, const MlpFused* fin = nullptr) {
   long ntiles = (n + MH - 1) / MH;
   int dev = 0, nsm = 148;
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  int grid = (int)std::min<long>(ntiles, 2L * nsm);
+  int grid = (int)std::min<long>(ntiles, nsm);
   if (grid <= 0) return;
   if (fin) k_mlp_tc<true><<<grid, MLP_THREADS, MLP_SMEM, s>>>(X, n, q, pw, out, *fin, err);
   else k_mlp_tc<false><<<grid, MLP_THREADS, MLP_SMEM, s>>>(X, n, q, pw, out, MlpFused{}, err);
