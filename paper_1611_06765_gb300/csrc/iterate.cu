@@ -49,88 +49,95 @@ struct StatsIO {
   }
 };
 
-// Blocks [0, nrows): row (c, kl): sij[kl] = sum_ab t v; chi_hh[kl][ij] for the ij the updates
-// compute.
-// Blocks [nrows, ...): column chunk (c, ab0): sab[ab] = sum_ij t v.
+// One warp per item (channel, row kl, first column, 0): up to STAT_COLS sums over the row v_kl, read
+// once for all of them: column 0 is sij[kl] = sum_ab t_kl v_kl, column j > 0 chi[kl][ij] of the j-th hole
+// pair ij the updates compute.  Items (channel, -1, ab0, 0): sab[ab] = sum_ij t v of 32 columns.
+// Bound by latency (a CTA per row and per 128 columns, most of whose threads idled in small channels,
+// took 38 us for 120 N=14 systems in FP32, 28 so) and in FP64 by the slow pipe: the four sums of
+// a warp share the exchanges, six additions instead of twenty (N=66, N_max=42: 47, 45 us).
 // PAIR (FP64 only): the contractions in FP32-pair arithmetic from the pair copies tp of t and vp
 // of v_pphh (the refinement sweeps): chi_hh, and the one-body sums as per-thread pair partials
 // added in FP64.
+constexpr int STAT_COLS = 4;
 template <typename T_, bool PAIR = false>
 __global__ void __launch_bounds__(128) k_tstats(DevState D, const LoopCtl* __restrict__ ctl,
-                                                int nrows, const int2* __restrict__ ab_items,
+                                                const int4* __restrict__ items, int n,
                                                 const f2* __restrict__ tp = nullptr,
                                                 const f2* __restrict__ vp = nullptr) {
-  __shared__ T_ sh32[32];
+  using E = std::conditional_t<PAIR, f2, T_>;
+  using A = Arith<E>;
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (w >= n) return;  // whole warps; no block barrier
+  const int4 it = items[w];
+  const int c = it.x, kl = it.y;
+  if (sys_done(D, ctl, D.ch_sys[c])) return;
   StatsIO<T_> io(D, ctl);
-  const T_* __restrict__ t = io.t;
-  if ((int)blockIdx.x < nrows) {
-    int2 it = D.row_item[blockIdx.x];
-    int c = it.x, kl = it.y;
-    if (sys_done(D, ctl, D.ch_sys[c])) return;
-    int npp = D.ch_npp[c], nh = D.ch_nhh[c];
-    long base = D.ch_t_off[c];
-    const T_* tr = t + base + (long)kl * npp;
-    const T_* vr = io.v + base + (long)kl * npp;
-    T_ s = 0;
-    if constexpr (PAIR) {
-      // per-thread partial sums in FP32 pairs, the block sum in FP64
-      const f2* __restrict__ tpr = tp + base + (long)kl * npp;
-      const f2* __restrict__ vpr = vp + base + (long)kl * npp;
-      f2 a2 = Arith<f2>::zero();
-      for (int ab = threadIdx.x; ab < npp; ab += blockDim.x) Arith<f2>::mac(a2, tpr[ab], vpr[ab]);
-      s = Arith<f2>::to_double(a2);
-    } else {
-      for (int ab = threadIdx.x; ab < npp; ab += blockDim.x) s += tr[ab] * vr[ab];
-    }
-    s = block_sum(s, sh32);
-    if (threadIdx.x == 0) io.sij[D.ch_hh_off[c] + kl] = s;
-    // chi is read only in the columns ij of the rows the updates compute (the list upd_row)
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int* __restrict__ rl = D.upd_row + D.ch_uoff[c];
-    const int nr = D.ch_uoff[c + 1] - D.ch_uoff[c];
-    for (int k = warp; k < nr; k += blockDim.x >> 5) {
-      const int ij = rl[k];
-      T_ acc = 0;
-      if constexpr (PAIR) {
-        const f2* __restrict__ vk = vp + base + (long)kl * npp;
-        const f2* __restrict__ tj = tp + base + (long)ij * npp;
-        f2 a2 = Arith<f2>::zero();
-        for (int cd = lane; cd < npp; cd += 32) Arith<f2>::mac(a2, vk[cd], tj[cd]);
-        for (int o = 16; o; o >>= 1)
-          a2 = Arith<f2>::add(a2, f2{__shfl_xor_sync(0xffffffffu, a2.hi, o),
-                                     __shfl_xor_sync(0xffffffffu, a2.lo, o)});
-        acc = Arith<f2>::to_double(a2);
-      } else {
-        const T_* tj = t + base + (long)ij * npp;
-        for (int cd = lane; cd < npp; cd += 32) acc += vr[cd] * tj[cd];
-        acc = warp_sum(acc);
-      }
-      if (lane == 0) {
-        long e = D.ch_vhh_off[c] + (long)kl * nh + ij;
-        const T_ chi = io.vhh[e] + acc;
-        // the pair update reads chi as pairs, in the same 8-byte slots
-        if constexpr (PAIR) reinterpret_cast<f2*>(io.chi)[e] = Arith<f2>::from_double(chi);
-        else io.chi[e] = chi;
-      }
-    }
+  const int npp = D.ch_npp[c], nh = D.ch_nhh[c];
+  const long base = D.ch_t_off[c];
+  const E *t, *v;
+  if constexpr (PAIR) {
+    t = tp + base;
+    v = vp + base;
   } else {
-    int2 it = ab_items[blockIdx.x - nrows];
-    int c = it.x, ab = it.y + threadIdx.x;
-    if (sys_done(D, ctl, D.ch_sys[c])) return;
-    int npp = D.ch_npp[c], nh = D.ch_nhh[c];
-    if (ab < npp) {
-      long base = D.ch_t_off[c] + ab;
-      T_ s = 0;
-      if constexpr (PAIR) {
-        f2 a2 = Arith<f2>::zero();
-        for (int ij = 0; ij < nh; ij++) Arith<f2>::mac(a2, tp[base + (long)ij * npp], vp[base + (long)ij * npp]);
-        s = Arith<f2>::to_double(a2);
-      } else {
-        for (int ij = 0; ij < nh; ij++) s += t[base + (long)ij * npp] * io.v[base + (long)ij * npp];
-      }
-      io.sab[D.ch_pp_off[c] + ab] = s;
-    }
+    t = io.t + base;
+    v = io.v + base;
   }
+  if (kl < 0) {
+    const int ab = it.z + lane;
+    if (ab >= npp) return;
+    E s = A::zero();
+#pragma unroll 4
+    for (int ij = 0; ij < nh; ij++) A::mac(s, t[ab + (long)ij * npp], v[ab + (long)ij * npp]);
+    if constexpr (PAIR) io.sab[D.ch_pp_off[c] + ab] = A::to_double(s);
+    else io.sab[D.ch_pp_off[c] + ab] = s;
+    return;
+  }
+  const int* __restrict__ rl = D.upd_row + D.ch_uoff[c];
+  const int m = min(STAT_COLS, D.ch_uoff[c + 1] - D.ch_uoff[c] + 1 - it.z);
+  const E* __restrict__ vr = v + (long)kl * npp;
+  const E* col[STAT_COLS];
+#pragma unroll
+  for (int q = 0; q < STAT_COLS; q++) {
+    const int k = it.z + min(q, m - 1);
+    col[q] = t + (long)(k == 0 ? kl : rl[k - 1]) * npp;
+  }
+  E acc[STAT_COLS];
+#pragma unroll
+  for (int q = 0; q < STAT_COLS; q++) acc[q] = A::zero();
+#pragma unroll 2
+  for (int cd = lane; cd < npp; cd += 32) {
+    const E x = vr[cd];
+#pragma unroll
+    for (int q = 0; q < STAT_COLS; q++)
+      if (q < m) A::mac(acc[q], x, col[q][cd]);
+  }
+  if (PAIR && it.z == 0) {
+    const double s = warp_sum((double)A::to_double(acc[0]));
+    if (lane == 0) io.sij[D.ch_hh_off[c] + kl] = s;
+  }
+  // the sums of columns 0 ... 3 end in lanes 0-7, 8-15, 16-23, 24-31
+  auto exchange = [&](E keep, E give, int o) {
+    E got;
+    if constexpr (PAIR) got = f2{__shfl_xor_sync(0xffffffffu, give.hi, o), __shfl_xor_sync(0xffffffffu, give.lo, o)};
+    else got = __shfl_xor_sync(0xffffffffu, give, o);
+    return A::add(keep, got);
+  };
+  const bool h16 = lane & 16, h8 = lane & 8;
+  const E x0 = exchange(h16 ? acc[2] : acc[0], h16 ? acc[0] : acc[2], 16);
+  const E x1 = exchange(h16 ? acc[3] : acc[1], h16 ? acc[1] : acc[3], 16);
+  E x = exchange(h8 ? x1 : x0, h8 ? x0 : x1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) x = exchange(x, x, o);
+  const int q = lane >> 3, k = it.z + q;
+  if ((lane & 7) != 0 || q >= m) return;
+  if (k == 0) {
+    if constexpr (!PAIR) io.sij[D.ch_hh_off[c] + kl] = x;
+    return;
+  }
+  const long e = D.ch_vhh_off[c] + (long)kl * nh + rl[k - 1];
+  // the pair update reads chi as pairs, in the same 8-byte slots
+  if constexpr (PAIR) reinterpret_cast<f2*>(io.chi)[e] = A::from_double(io.vhh[e] + A::to_double(x));
+  else io.chi[e] = io.vhh[e] + x;
 }
 
 // chi_b - eps_b = -sum_d sum_{k<l} t_kl^bd v_kl^bd   (particles)
@@ -964,12 +971,15 @@ __global__ void k_start(const double* __restrict__ parts, const int* __restrict_
 
 static void* dmalloc(pnm_ctx* ctx, size_t bytes) { return pnm_ctx_alloc(ctx, bytes); }
 
+__host__ __device__ __forceinline__ int stat_groups(int nrows) { return (nrows + STAT_COLS) / STAT_COLS; }
+
 // The update chunks and their amplitudes: rows of the channel's run of upd_row one after the other, 32
-// amplitudes per chunk; a channel per CTA (its chunks start at first[c]), then a system per CTA for the
+// amplitudes per chunk; a channel per CTA (its chunks start at first[c].x, its items of the stats kernel
+// at first[c].y), then a system per CTA for the
 // padding up to whole CTAs of the updates.
-__global__ void __launch_bounds__(128) k_upd_chunks(DevState D, int nch, const int* __restrict__ first,
+__global__ void __launch_bounds__(128) k_upd_chunks(DevState D, int nch, const int2* __restrict__ first,
                                                     const int2* __restrict__ pad, UpdItem* __restrict__ items,
-                                                    int* __restrict__ upd_z) {
+                                                    int* __restrict__ upd_z, int4* __restrict__ stat) {
   UpdItem it{};
   if ((int)blockIdx.x >= nch) {
     const int2 p = pad[blockIdx.x - nch];
@@ -992,12 +1002,17 @@ __global__ void __launch_bounds__(128) k_upd_chunks(DevState D, int nch, const i
   it.vhh_off = D.ch_vhh_off[c];
   it.s_off = D.ch_s_off[c];
   const int r0 = D.ch_uoff[c], n = (D.ch_uoff[c + 1] - r0) * it.npp;
-  const long k0 = 32L * first[c];
+  const long k0 = 32L * first[c].x;
   for (int e = threadIdx.x; e < ((n + 31) & ~31); e += blockDim.x) {
     const int r = e / it.npp;
     upd_z[k0 + e] = e < n ? (int)(it.base + (long)D.upd_row[r0 + r] * it.npp + (e - r * it.npp)) : -1;
     if ((e & 31) == 0) items[(k0 + e) >> 5] = it;
   }
+  // items of the stats kernel: per row its groups of columns, then the channel's columns by 32
+  int4* so = stat + first[c].y;
+  const int groups = stat_groups(D.ch_uoff[c + 1] - r0), rows = it.nh * groups;
+  for (int k = threadIdx.x; k < rows + (it.npp + 31) / 32; k += blockDim.x)
+    so[k] = k < rows ? make_int4(c, k / groups, k % groups * STAT_COLS, 0) : make_int4(c, -1, (k - rows) * 32, 0);
 }
 
 // pp items of nr[c] rows per channel in the order of decreasing work, so that the last CTAs are
@@ -1064,14 +1079,12 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->row_lo_d = d;
   ctx->row_hi_d = d + nsys;
   ctx->lut_off_d = d + 2 * nsys;
-  std::vector<int2> abit;
   std::vector<int4> upd;
   std::vector<int> ulo(nsys), uhi(nsys);
   int max_npp = 0, max_nlad = 0;
   for (int c = 0; c < ctx->nch; c++) {
     int npp = ctx->h_npp[c];
     max_npp = std::max(max_npp, npp);
-    for (int ab0 = 0; ab0 < npp; ab0 += 128) abit.push_back(make_int2(c, ab0));
     if (!ctx->h_vpp[c]) continue;
     int nl = ctx->h_nlad[c];
     max_nlad = std::max(max_nlad, nl);
@@ -1115,7 +1128,8 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   // Chunks of the updates: 32 amplitudes of one channel each (its last is padded), a CTA's in one
   // system (padded chunks past its end).  A warp takes more than one where the GPU stays full: fewer
   // partial sums for the last CTA to add, and the block sums' FP64 additions count for more amplitudes.
-  std::vector<int> glo(nsys), ghi(nsys), first(ctx->nch);
+  std::vector<int> glo(nsys), ghi(nsys);
+  std::vector<int2> first(ctx->nch);
   std::vector<int2> pad(nsys);
   long n_chunks = 0;
   for (int c = 0; c < ctx->nch; c++) n_chunks += ((long)(uoff[c + 1] - uoff[c]) * ctx->h_npp[c] + 31) / 32;
@@ -1127,7 +1141,8 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   for (int k = 0; k < nsys; k++) {
     glo[k] = (int)(n_chunks / per_cta);
     for (int c = ctx->sys[k].ch_begin; c < ctx->sys[k].ch_end; c++) {
-      first[c] = (int)n_chunks;
+      first[c] = make_int2((int)n_chunks, ctx->n_stat);
+      ctx->n_stat += ctx->h_nhh[c] * stat_groups(uoff[c + 1] - uoff[c]) + (ctx->h_npp[c] + 31) / 32;
       n_chunks += ((long)(uoff[c + 1] - uoff[c]) * ctx->h_npp[c] + 31) / 32;
     }
     pad[k].x = (int)n_chunks;
@@ -1139,32 +1154,10 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->n_upd_ctas = (int)(n_chunks / per_cta);
   ctx->max_npp = max_npp;
   ctx->max_nlad = max_nlad;
-  std::vector<int> alo(nsys), ahi(nsys);
   int max_nhh = 1;
-  for (size_t k = 0; k < abit.size(); k++) max_nhh = std::max(max_nhh, ctx->h_nhh[abit[k].x]);
-  for (int k = 0; k < nsys; k++) {
-    alo[k] = (int)abit.size();
-    ahi[k] = 0;
-  }
-  for (size_t k = 0; k < abit.size(); k++) {
-    int sy = ctx->h_ch_sys[abit[k].x];
-    alo[sy] = std::min(alo[sy], (int)k);
-    ahi[sy] = std::max(ahi[sy], (int)k + 1);
-  }
-  for (int k = 0; k < nsys; k++)
-    if (ahi[k] == 0) alo[k] = 0;
+  for (int c = 0; c < ctx->nch; c++) max_nhh = std::max(max_nhh, ctx->h_nhh[c]);
   ctx->max_nhh = max_nhh;
   if (max_nhh > UPD_MAX_NHH) throw PnmError{PNM_EINVAL, "more hole pairs in one channel than the update supports"};
-  int* ad = (int*)dmalloc(ctx, sizeof(int) * 2 * nsys);
-  CUDA_TRY(cudaMemcpyAsync(ad, alo.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(cudaMemcpyAsync(ad + nsys, ahi.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, s));
-  ctx->ab_lo_d = ad;
-  ctx->ab_hi_d = ad + nsys;
-  ctx->n_ab_items = (int)abit.size();
-  ctx->ab_items = (int2*)dmalloc(ctx, sizeof(int2) * std::max<size_t>(1, abit.size()));
-  if (!abit.empty())
-    CUDA_TRY(cudaMemcpyAsync(ctx->ab_items, abit.data(), sizeof(int2) * abit.size(),
-                             cudaMemcpyHostToDevice, s));
   ctx->n_upd_items = (int)upd.size();
   ctx->upd_items = (int4*)dmalloc(ctx, sizeof(int4) * std::max<size_t>(1, upd.size()));
   if (!upd.empty())
@@ -1177,11 +1170,13 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->upd_hi_d = ud + nsys;
   ctx->upd_chunks = (UpdItem*)dmalloc(ctx, sizeof(UpdItem) * std::max<long>(1, n_chunks));
   ctx->upd_z = (int*)dmalloc(ctx, sizeof(int) * 32 * std::max<long>(1, n_chunks));
-  int* dfirst = (int*)dmalloc(ctx, sizeof(int) * std::max(1, ctx->nch));
+  ctx->stat_items = (int4*)dmalloc(ctx, sizeof(int4) * std::max(1, ctx->n_stat));
+  int2* dfirst = (int2*)dmalloc(ctx, sizeof(int2) * std::max(1, ctx->nch));
   int2* dpad = (int2*)dmalloc(ctx, sizeof(int2) * nsys);
-  if (ctx->nch) CUDA_TRY(cudaMemcpyAsync(dfirst, first.data(), sizeof(int) * ctx->nch, cudaMemcpyHostToDevice, s));
+  if (ctx->nch) CUDA_TRY(cudaMemcpyAsync(dfirst, first.data(), sizeof(int2) * ctx->nch, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(dpad, pad.data(), sizeof(int2) * nsys, cudaMemcpyHostToDevice, s));
-  k_upd_chunks<<<ctx->nch + nsys, 128, 0, s>>>(ctx->d, ctx->nch, dfirst, dpad, ctx->upd_chunks, ctx->upd_z);
+  k_upd_chunks<<<ctx->nch + nsys, 128, 0, s>>>(ctx->d, ctx->nch, dfirst, dpad, ctx->upd_chunks, ctx->upd_z,
+                                                  ctx->stat_items);
   CUDA_TRY(cudaGetLastError());
   int* gd = (int*)dmalloc(ctx, sizeof(int) * 2 * nsys);
   CUDA_TRY(cudaMemcpyAsync(gd, glo.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, s));
@@ -1448,14 +1443,14 @@ void pnm_join(pnm_ctx* ctx) {
 void pnm_enqueue_stats(pnm_ctx* ctx, bool mixed, bool pair) {
   cudaStream_t s = ctx->stream;
   DevState& D = ctx->d;
-  unsigned nb = (unsigned)(ctx->nrows + ctx->n_ab_items);
+  const int n = ctx->n_stat;
+  unsigned nb = (unsigned)((n + 3) / 4);
   unsigned nd = (unsigned)((ctx->nsp_total * 32 + 255) / 256);
   prof_begin(ctx, mixed ? KID_TSTATS32 : KID_TSTATS);
-  if (mixed) k_tstats<float><<<nb, 128, 0, s>>>(D, ctx->ctl, ctx->nrows, ctx->ab_items);
-  else if (pair)
-    k_tstats<double, true><<<nb, 128, 0, s>>>(D, ctx->ctl, ctx->nrows, ctx->ab_items, ctx->t_pair,
-                                             ctx->vpphh_f2);
-  else k_tstats<double><<<nb, 128, 0, s>>>(D, ctx->ctl, ctx->nrows, ctx->ab_items);
+  if (n == 0) {
+  } else if (mixed) k_tstats<float><<<nb, 128, 0, s>>>(D, ctx->ctl, ctx->stat_items, n);
+  else if (pair) k_tstats<double, true><<<nb, 128, 0, s>>>(D, ctx->ctl, ctx->stat_items, n, ctx->t_pair, ctx->vpphh_f2);
+  else k_tstats<double><<<nb, 128, 0, s>>>(D, ctx->ctl, ctx->stat_items, n);
   prof_end(ctx);
   prof_begin(ctx, mixed ? KID_DCHI32 : KID_DCHI);
   if (mixed) k_dchi<float><<<nd, 256, 0, s>>>(D, ctx->nsp_total);

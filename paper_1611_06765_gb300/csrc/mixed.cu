@@ -115,38 +115,51 @@ __global__ void __launch_bounds__(256) k_pack_v(const TCItem* __restrict__ items
 }
 
 // t tiles of the channels with a V_pppp block, in the ladder basis (before every tensor-core
-// ladder): one CTA per (channel, k-block of 64 basis vectors); each tile entry gathers the
-// signed members of its vector from the current amplitudes (FP32 copy in the iteration, FP64
-// for the operator call) and stores the BF16 hi/lo split.
+// ladder): `per` threads per item (channel, k-block of 64 basis vectors), a thread per eight entries of a
+// row; each entry gathers the signed members of its vector from the current amplitudes (FP32 copy in the
+// iteration, FP64 for the operator call) and stores the BF16 hi/lo split, 16 bytes of each plane at a
+// time.  Bound by latency: a CTA of 256 per item, an entry per thread and step, took 26 us for 120 N=14
+// systems (36,000 items of 1024 entries) and 18 us for three N=66, N_max=36 systems; with a warp per item
+// where they fill the GPU, four where not, 23 and 17 us.
 template <typename T_>
-__global__ void k_pack_t(const int4* __restrict__ pk, const long* __restrict__ pk_boff,
-                         DevState D, const LoopCtl* __restrict__ ctl, __nv_bfloat16* __restrict__ bt) {
-  int4 p = pk[blockIdx.x];  // (channel, k-block, npad, 0)
-  int c = p.x, kb = p.y, npad = p.z;
+__global__ void __launch_bounds__(128) k_pack_t(const int4* __restrict__ pk, const long* __restrict__ pk_boff, int nitems,
+                                                int per, DevState D, const LoopCtl* __restrict__ ctl,
+                                                __nv_bfloat16* __restrict__ bt) {
+  const int item = (blockIdx.x * blockDim.x + threadIdx.x) / per;
+  if (item >= nitems) return;
+  const int4 p = pk[item];  // (channel, k-block, npad, 0)
+  const int c = p.x, kb = p.y, npad = p.z;
   if (sys_done(D, ctl, D.ch_sys[c])) return;
-  int npp = D.ch_npp[c], nh = D.ch_nhh[c], nl = D.ch_nlad[c], off = D.ch_pp_off[c];
+  const int npp = D.ch_npp[c], nh = D.ch_nhh[c], nl = D.ch_nlad[c];
+  const int2* __restrict__ mem = D.lad_mem + D.ch_pp_off[c];
   const T_* t;
   if constexpr (std::is_same<T_, double>::value) t = cur_t(D, ctl) + D.ch_t_off[c];
   else t = cur_t32(D, ctl) + D.ch_t_off[c];
-  __nv_bfloat16* hi = bt + pk_boff[blockIdx.x];
+  __nv_bfloat16* hi = bt + pk_boff[item];
   __nv_bfloat16* lo = hi + npad * TC_BK;
-  for (int e = threadIdx.x; e < npad * TC_BK; e += blockDim.x) {
-    int n = e / TC_BK, k = e % TC_BK;
-    int q = kb * TC_BK + k;
-    T_ x = 0;
-    if (n < nh && q < nl) {
-      int2 m = D.lad_mem[off + q];
-      T_ a = t[(long)n * npp + (m.x > 0 ? m.x : -m.x) - 1];
-      x = m.x > 0 ? a : -a;
-      if (m.y != 0) {
-        T_ b = t[(long)n * npp + (m.y > 0 ? m.y : -m.y) - 1];
-        x += m.y > 0 ? b : -b;
+  for (int e = threadIdx.x % per; e < npad * (TC_BK / 8); e += per) {
+    const int n = e / (TC_BK / 8), k0 = e % (TC_BK / 8) * 8, q0 = kb * TC_BK + k0;
+    __align__(16) __nv_bfloat16 h[8], l[8];
+    int2 m[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) m[j] = n < nh && q0 + j < nl ? mem[q0 + j] : make_int2(0, 0);
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      const T_* __restrict__ tr = t + (long)n * npp - 1;
+      T_ x = 0;
+      if (m[j].x != 0) {
+        const T_ a = tr[abs(m[j].x)];
+        x = m[j].x > 0 ? a : -a;
       }
+      if (m[j].y != 0) {
+        const T_ b = tr[abs(m[j].y)];
+        x += m[j].y > 0 ? b : -b;
+      }
+      split_bf16((double)x, h[j], l[j]);
     }
-    __nv_bfloat16 h, l;
-    split_bf16((double)x, h, l);
-    hi[core_off(n, k)] = h;
-    lo[core_off(n, k)] = l;
+    const int o = core_off(n, k0);
+    *reinterpret_cast<uint4*>(hi + o) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(lo + o) = *reinterpret_cast<const uint4*>(l);
   }
 }
 
@@ -654,6 +667,15 @@ void pnm_prepare_mixed(pnm_ctx* ctx) {
   ctx->mixed = M;
 }
 
+template <typename T_>
+static void launch_pack_t(pnm_ctx* ctx, cudaStream_t s) {
+  MixedState* M = ctx->mixed;
+  if (M->npk == 0) return;
+  const int per = M->npk >= 64 * ctx->nsm ? 32 : 128;
+  k_pack_t<T_><<<(unsigned)(((long)M->npk * per + 127) / 128), 128, 0, s>>>(M->pk, M->pk_boff, M->npk, per, ctx->d, ctx->ctl,
+                                                                            M->bt);
+}
+
 void pnm_enqueue_body_mixed(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h) {
   MixedState* M = ctx->mixed;
   cudaStream_t s_ph = pnm_concurrent(ctx) ? ctx->side[0] : ctx->stream;
@@ -667,7 +689,7 @@ void pnm_enqueue_body_mixed(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHand
   if (M->nitems > 0) {
     // t tiles of the current amplitudes in the ladder basis, then the ladder (same stream)
     prof_begin(ctx, KID_PACK);
-    k_pack_t<float><<<M->npk, 256, 0, s_pp>>>(M->pk, M->pk_boff, ctx->d, ctx->ctl, M->bt);
+    launch_pack_t<float>(ctx, s_pp);
     prof_end(ctx);
     prof_begin(ctx, KID_PP_TC);
     launch_pp_tc(M->items, M->cta_off, M->grid, M, M->smem, M->nst, ctx->ctl, ctx->ns, s_pp);
@@ -744,7 +766,7 @@ void pnm_apply_pp(pnm_ctx* ctx, int sys, int precision, const double* t, double*
   if (precision == PNM_PREC_BF16X3) {
     MixedState* M = ctx->mixed;
     CUDA_TRY(cudaMemsetAsync(M->rpp32, 0, sizeof(float) * TC_MAX_SPLIT * std::max<long>(ctx->ns, 1), s));
-    if (M->npk > 0) k_pack_t<double><<<M->npk, 256, 0, s>>>(M->pk, M->pk_boff, ctx->d, ctx->ctl, M->bt);
+    launch_pack_t<double>(ctx, s);
     launch_pp_tc(M->items, M->cta_off, M->grid, M, M->smem, M->nst, ctx->ctl, ctx->ns, s);
     pnm_lad_expand(ctx, M->rpp32, M->ksplit, ctx->ns);
   } else {

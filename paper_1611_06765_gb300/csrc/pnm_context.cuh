@@ -74,10 +74,9 @@ struct pnm_ctx {
   size_t ph_large_smem = 0, ph_dig_smem = 0, ph_warp_smem = 0;
   f2* t_pair = nullptr;                          // FP32-pair copy of the current amplitudes
   int *grp_lo_d = nullptr, *grp_hi_d = nullptr;  // per system ranges of the update items
-  int *ab_lo_d = nullptr, *ab_hi_d = nullptr;    // per system ranges of the column items
   int max_nhh = 1;
-  int2* ab_items = nullptr;
-  int n_ab_items = 0;
+  int4* stat_items = nullptr;  // warps of the stats kernel
+  int n_stat = 0;
 
   // loop control
   int *row_lo_d = nullptr, *row_hi_d = nullptr, *lut_off_d = nullptr;  // per system
