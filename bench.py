@@ -91,7 +91,7 @@ TOL_PER_N = 1e-6
 # DRAM bytes (read + write) per launch of the default workload from one ncu capture, with the
 # first 16 hex digits of the SHA-256 of the kernel's source file at the time of the capture:
 # reported only while that file is unchanged, else null.
-TRAFFIC = {"k_update_mix": (154537728.0, "19db074b78c7acf1"), "k_pp_tc": (257623040.0, "53dafb1834d94e42")}
+TRAFFIC = {"k_update_mix": (174492928.0, "51dbde8a79547b23"), "k_pp_tc": (258304512.0, "72960f5b445f6ef9")}
 ALPHA = 0.5
 
 
@@ -220,14 +220,14 @@ def algorithmic_cost(ctx, kernel):
     # the updates compute one amplitude of each spin-flip pair and write both
     ncomp = 0.5 * nt
     if kernel == "k_pp_f2":
-        kernel = "k_pp64"  # same arrays (V as FP32 pairs, 8 bytes) and the same flops
+        kernel = "k_pp64"  # the same arrays (digit words of V, 8 bytes) and products
     if kernel in ("k_pp64", "k_pp_tc"):
         # the ladder in its basis (pnm_ladder_sizes): V block n_lad x n_lad, operand and result
         # rows x n_lad per channel; k_pp64 takes the rows the update computes, (n_hh + self
         # pairs) / 2 (exact for S_z = 0 channels, right in total over a channel and its flip),
         # k_pp_tc every row
         rows = 0.5 * (nhh + nself) if kernel == "k_pp64" else nhh
-        vb = 8.0 if kernel == "k_pp64" else 4.0          # FP64 V, or BF16 hi + lo
+        vb = 8.0 if kernel == "k_pp64" else 4.0          # digit words of V, or BF16 hi + lo
         tb = 8.0 if kernel == "k_pp64" else 4.0          # t operand in the ladder basis
         rb = 8.0 if kernel == "k_pp64" else 4.0          # result
         byts = float((nlad ** 2).sum()) * vb + float((rows * nlad).sum()) * (tb + rb)
@@ -260,7 +260,7 @@ def kernel_source(kernel):
     """Source file (in the package's csrc/) that defines a kernel."""
     if kernel in ("k_pp_tc", "k_pack"):
         return "mixed.cu"
-    return "iterate.cu"
+    return "ph.cu" if kernel.startswith("k_ph") else "iterate.cu"
 
 
 def measured_traffic(kernel, workload):
@@ -279,6 +279,10 @@ def measured_traffic(kernel, workload):
     return ent[0] if digest == ent[1] else None
 
 
+DIGIT_KERNELS = ("k_pp64", "k_ph64", "k_pp_f2", "k_ph_f2")
+# kernels behind one entry of the profiler, where more than one: the digits of the amplitudes and the
+# ladder; exponents, digits, larger and smallest channels of the ph term
+LAUNCHES = {"k_pp64": 2, "k_pp_f2": 2, "k_ph64": 4, "k_ph_f2": 4, "k_ph32": 2}
 MIXED_KERNELS = ("k_update_mix", "k_ph32", "k_pp_tc", "k_tstats32", "k_pack", "k_dchi32")
 
 
@@ -305,14 +309,13 @@ def implementation_bytes(ctx, kernel):
     nhh, npp, nlad, nph, nhp, xsz, nself = chan_sizes(ctx)
     ncomp = 0.5 * float((nhh * npp).sum())
     if kernel == "k_update":
-        # per computed amplitude: t, v, eps, 1/eps, qmap, flip map, ladder map, rpp, four Q
-        # values read; t_next written for it and its flip
-        return ncomp * (8 + 8 + 8 + 8 + 16 + 4 + 4 + 8 + 4 * 8 + 2 * 8)
+        # per computed amplitude: its index, t, v, eps, 1/eps, qmap, flip map, ladder map, rpp, four
+        # Q values read; t_next written for it and its flip
+        return ncomp * (4 + 8 + 8 + 8 + 8 + 16 + 4 + 4 + 8 + 4 * 8 + 2 * 8)
     if kernel == "k_update_mix":
-        # per computed amplitude: t, alpha/eps, qmap, flip map, t32, ladder map, pp ladder, hh
-        # ladder (v is formed from the interaction table), four Q values read; t written for
-        # it, t32 for it and its flip, four T entries
-        return ncomp * (8 + 8 + 16 + 4 + 4 + 4 + 4 + 4 + 4 * 4 + 8 + 2 * 4 + 4 * 4)
+        # per computed amplitude: its index, t, v, eps, alpha/eps, qmap, flip map, t32, ladder map,
+        # pp ladder, four Q values read; t written for it, t32 for it and its flip, four T entries
+        return ncomp * (4 + 8 + 8 + 8 + 8 + 16 + 4 + 4 + 4 + 4 + 4 * 4 + 8 + 2 * 4 + 4 * 4)
     return None
 
 
@@ -762,14 +765,10 @@ def run_ours(a):
     hbm, bf16, src = read_peaks()
     fp64_peak = P.measure_fma_peak(True, stream.cuda_stream)
     fp32_peak = P.measure_fma_peak(False, stream.cuda_stream)
-    if kname in ("k_pp64", "k_ph64"):
-        roof = {"bound": "alu", "achieved": flops / kavg_s / 1e12, "peak": fp64_peak,
-                "unit": "TFLOP/s", "peak_source": "measured FP64 FMA rate (pnm_measure_fma_peak)"}
-    elif kname in ("k_pp_f2", "k_ph_f2"):
-        # FP64-equivalent flops against the FP32 pipe's rate per FP32-pair multiply-add (12 FP32
-        # instructions, i.e. the measured FP32 FMA rate / 12)
-        roof = {"bound": "alu", "achieved": flops / kavg_s / 1e12, "peak": fp32_peak / 12,
-                "unit": "TFLOP/s", "peak_source": "measured FP32 FMA rate / 12 (FP32-pair multiply-add)"}
+    if kname in DIGIT_KERNELS:
+        # FP64-equivalent flops: each multiply-add is 36 FP16 ones of the tensor cores (digit products)
+        roof = {"bound": "tensor", "achieved": flops / kavg_s / 1e12, "peak": bf16 / 36,
+                "unit": "TFLOP/s", "peak_source": "%s bf16_tflops / 36 (digit products per product)" % src}
     else:
         roof = {"bound": "hbm", "achieved": byts / kavg_s / 1e9, "peak": hbm, "unit": "GB/s",
                 "peak_source": "%s hbm_gbs" % src}
@@ -783,15 +782,16 @@ def run_ours(a):
     if ib is not None:
         roof["implementation_bytes"] = ib * wfrac
         roof["implementation_gbs"] = ib * wfrac / kavg_s / 1e9
-    # the FP64 refinement contractions against the measured FP64 FMA rate
-    for k in ("k_pp64", "k_ph64", "k_ph32", "k_pp_f2", "k_ph_f2"):
+    # the contractions of FP64 accuracy against the tensor cores' rate per digit product, the FP32 ph
+    # term against the measured FP32 FMA rate
+    for k in DIGIT_KERNELS + ("k_ph32",):
         if k in stats and k != kname:
             tk = stats[k][0] / stats[k][1] / 1e3
             bk, fk = algorithmic_cost(ctx, k)
             fk *= work_fraction(ctx, k, [int(x) for x in it_h], stats[k][1], prec_name != "fp64",
                                 solve_kw.get("refine_sweeps", 0))
-            pk = {"k_ph32": fp32_peak, "k_pp_f2": fp32_peak / 12, "k_ph_f2": fp32_peak / 12}.get(k, fp64_peak)
-            roof[k] = {"bound": "alu", "achieved": fk / tk / 1e12, "peak": pk, "unit": "TFLOP/s",
+            pk = fp32_peak if k == "k_ph32" else bf16 / 36
+            roof[k] = {"bound": "alu" if k == "k_ph32" else "tensor", "achieved": fk / tk / 1e12, "peak": pk, "unit": "TFLOP/s",
                        "frac": fk / tk / 1e12 / pk, "kernel_avg_us": tk * 1e6}
     if "k_pp_tc" in stats and kname != "k_pp_tc":
         t_tc = stats["k_pp_tc"][0] / stats["k_pp_tc"][1] / 1e3
@@ -806,7 +806,8 @@ def run_ours(a):
     # kernels of one solve: the loop bodies and refinement sweeps counted by the profiler, plus
     # the start (MBPT2: init + energy; learned: inference, copy to the spin flips, symmetrise,
     # init + energy, FP32 copies)
-    launches_per_solve = sum(n for _, n in stats.values()) + (6 if start == "mlp" else 2)
+    launches_per_solve = (sum(n * LAUNCHES.get(k, 1) for k, (_, n) in stats.items())
+                          + (6 if start == "mlp" else 2))
 
     comparison = None
     if rank == 0 and not a.no_extra:

@@ -12,8 +12,8 @@
 // Twelve FP32 instructions per multiply-add.  The error-free steps use __fmul_rn / __fadd_rn /
 // __fsub_rn, which the compiler never contracts into a fused multiply-add (a contraction of
 // acc.hi + a.hi b.hi would break the two-sum).  For sums of K products the result stays within
-// a few K 2^-48 of the sum of absolute values; the contractions of the ph term (K <= 66, two
-// chained products) come out within about 1e-13 of their largest element.
+// a few K 2^-48 of the sum of absolute values.  The hh ladder, the one-body sums and the smallest
+// channels of the ph term are summed in pairs; the larger contractions are digit products (dig.cuh).
 #pragma once
 #include <cuda_runtime.h>
 

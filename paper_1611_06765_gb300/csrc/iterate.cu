@@ -9,12 +9,13 @@
 //   k_tstats   row and column sums of t o v (one-body intermediates) and
 //              <kl|chi|ij> = <kl|v|ij> + 1/2 <kl|v|cd> t_ij^cd per direct channel
 //   k_dchi     chi_p - eps_p per state, gathered over the pairs holding p
-//   k_ph       T_x = remap(t); C_x = V1_x + 1/2 W_x T_x; Q_x = T_x C_x per cross channel
-//   k_pp       1/2 sum_cd <ab|v|cd> t_cd^ij, grouped over all channels with a V_pppp block (FP64
+//   k_tdig, k_pp   1/2 sum_cd <ab|v|cd> t_cd^ij, grouped over all channels with a V_pppp block (FP64
 //              accuracy from digit products on the tensor cores)
-//   k_update   Jacobi step t_new = (v + rest) / eps_ij^ab, mixing, energy/residual partials
-//   finalize   (last block of k_update) Eq. (ccdcorr) energy per system, |dE| test,
-//              device-side loop condition
+//   k_update, k_update_mix   Jacobi step t_new = (v + rest) / eps_ij^ab, mixing, energy/residual
+//              partials, and by the last block of each system its end (Eq. ccdcorr energy, |dE| test)
+//              and the device-side loop condition
+//   k_mbpt2, k_mbpt3   start amplitudes and MBPT2 energy, third-order sums
+// The ph term is in ph.cu, the tensor-core ladder and the FP32 copies of the mixed iteration in mixed.cu.
 #include <cmath>
 #include <cstdio>
 #include <map>

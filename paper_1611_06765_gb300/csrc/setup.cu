@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(128) k_xflip(const SetupSys* __restrict__ SS, 
   const SetupSys& S = SS[x_sys[x]];
   const unsigned lt = (1u << lane) - 1u;
   const int nph = x_nph[x], nhp = x_nhp[x], po = x_ph_off[x], ho = x_hp_off[x];
-  const int N = S.N, np = S.nsp - N, species = S.species, sp_off = S.sp_off;
+  const int N = S.N, np = S.nsp - N, species = S.species;
   bool bad = nph <= 0 || nhp <= 0;
   int sz = 0, mir = -1, nr = 0, nc = 0;
   if (!bad) {

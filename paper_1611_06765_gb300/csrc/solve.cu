@@ -202,8 +202,8 @@ int pnm_solve(pnm_ctx* ctx, const pnm_solve_opts& o, double* dE, int* iters, dou
   }
   const bool pair_refine = mixed && o.refine_sweeps > 0 && o.refine_kernels == PNM_PREC_F32PAIR;
   if (pair_refine) pnm_prepare_f2(ctx);
-  // the FP64 ladder V and schedule only where an FP64 pp ladder runs (the FP64 iteration, or
-  // refinement sweeps on the FP64 pipe); FP32-pair refinement has its own schedule slot
+  // the digit operands and the FP64 schedule where FP64 contractions run (the FP64 iteration, or FP64
+  // refinement sweeps); FP32-pair refinement has its own schedule slot
   const bool fp64_ladder = !mixed || (o.refine_sweeps > 0 && !pair_refine);
   if (fp64_ladder) {
     pnm_need_digits(ctx);
