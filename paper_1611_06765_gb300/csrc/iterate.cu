@@ -463,8 +463,18 @@ void pnm_split_f2(const double* a, f2* b, long n, cudaStream_t s) {
 // round trips, not bandwidth, that adds to every update, so the systems of a batch go side by side
 // (one CTA closing all 120 systems of 22 partials each, a warp per system, left the GPU idle for half
 // of the update: 141 us, 79 us so).  FIN_UNROLL partial pairs are requested before the first
-// is added.
+// is added; up to 32 times as many take one warp without barriers.
 constexpr int FIN_UNROLL = 8;
+
+// Sums of a and b over a warp, in lanes 0 and 16: the first exchange leaves the a in one half of the
+// warp and the b in the other, so that both take five additions of the slow FP64 pipe instead of ten.
+__device__ __forceinline__ double warp_sum_two(double a, double b) {
+  const bool low = (threadIdx.x & 16) == 0;
+  double x = (low ? a : b) + __shfl_xor_sync(0xffffffffu, low ? b : a, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
 
 __device__ __forceinline__ void sum_partials(const FinArgs& f, int s, int first, int step, double& e, double& r) {
   const int hi = f.hi[s];
@@ -514,13 +524,12 @@ __device__ __forceinline__ bool finalize_one(const FinArgs& f, SysCtl& S, const 
   return bad;
 }
 
-// The last CTA of system s to finish closes it, and the last system the update (no waiting: CTAs and
+// The last of system s's CTAs to finish closes it, and the last system the update (no waiting: CTAs and
 // systems count themselves out with atomics after a fence, as in the CUDA threadfence reduction).
 // Every counter is left at zero for the next update.
-__device__ void finalize_system(const FinArgs& f, LoopCtl* ctl, int s) {
+__device__ void finalize_system(const FinArgs& f, LoopCtl* ctl, int s, int ctas) {
   __shared__ int is_last;
   __shared__ double sh32f[32];
-  const int ctas = f.hi[s] - f.lo[s];
   __syncthreads();
   if (threadIdx.x == 0) {
     // only thread 0 wrote the block's partials: its fence orders them before the count
@@ -534,8 +543,30 @@ __device__ void finalize_system(const FinArgs& f, LoopCtl* ctl, int s) {
   SysCtl S;
   if (threadIdx.x == 0) S = f.sc[s];
   double e, r;
-  sum_partials(f, s, threadIdx.x, blockDim.x, e, r);
-  block_sum2(e, r, sh32f);
+  if (ctas <= 32 * FIN_UNROLL) {  // one warp, without barriers
+    if (threadIdx.x >= 32) return;
+    const int k0 = f.lo[s] + threadIdx.x, hi = f.hi[s];
+    double a[FIN_UNROLL], b[FIN_UNROLL];
+#pragma unroll
+    for (int j = 0; j < FIN_UNROLL; j++) {
+      a[j] = k0 + 32 * j < hi ? __ldcg(f.eparts + k0 + 32 * j) : 0.0;
+      b[j] = k0 + 32 * j < hi ? __ldcg(f.rparts + k0 + 32 * j) : 0.0;
+    }
+    e = a[0];
+    r = b[0];
+#pragma unroll
+    for (int j = 1; j < FIN_UNROLL; j++) {
+      if (32 * j >= ctas) break;
+      e += a[j];
+      r += b[j];
+    }
+    const double x = warp_sum_two(e, r);
+    e = x;
+    r = __shfl_sync(0xffffffffu, x, 16);
+  } else {
+    sum_partials(f, s, threadIdx.x, blockDim.x, e, r);
+    block_sum2(e, r, sh32f);
+  }
   if (threadIdx.x != 0) return;
   f.blocks_done[s] = 0;
   bool bad = finalize_one(f, S, c, s, e, r), all_done = S.done;
@@ -580,7 +611,9 @@ __device__ void finalize_system(const FinArgs& f, LoopCtl* ctl, int s) {
 // ladder and one-body values behind them.  A thread per column that goes through eight rows of a
 // channel, as before, has the hh ladder's t column once for eight rows, but idles where a channel has
 // less than 128 columns and walks the chain once for every row or two; the column is a coalesced load
-// that L1 and L2 serve.
+// that L1 and L2 serve.  A warp's first chunk is requested before the loop control and the system's
+// state are looked at, which takes two round trips off an update of a small system (39 updates of
+// N=14, N_max=4: 0.77 -> 0.70 ms).
 struct UpdSums {  // energy and residual norm, amplitudes with and without a flip of their own
   double e2 = 0.0, e1 = 0.0, r2 = 0.0, r1 = 0.0;
   __device__ __forceinline__ void add(bool flip, double v, double out, double R) {
@@ -594,17 +627,11 @@ struct UpdSums {  // energy and residual norm, amplitudes with and without a fli
   }
 };
 
-// Block sums of the energy and the residual norm into the CTA's partials.  The first exchange leaves
-// the energies in one half of the warp and the residuals in the other, so that both are reduced by
-// five additions of the slow FP64 pipe instead of ten.
+// Block sums of the energy and the residual norm into the CTA's partials.
 __device__ __forceinline__ void upd_partials(const DevState& D, const UpdSums& S) {
   __shared__ double red[UPD_THREADS / 32][2];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const bool low = lane < 16;
-  const double e = fma(2.0, S.e2, S.e1), r = fma(2.0, S.r2, S.r1);
-  double x = (low ? e : r) + __shfl_xor_sync(0xffffffffu, low ? r : e, 16);
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  const double x = warp_sum_two(fma(2.0, S.e2, S.e1), fma(2.0, S.r2, S.r1));
   if ((lane & 15) == 0) red[w][lane >> 4] = x;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -619,6 +646,7 @@ __device__ __forceinline__ void upd_partials(const DevState& D, const UpdSums& S
 // residual, step (alpha / eps_ij^ab prepared per solve, aw) and energy stay FP64.
 // One FP64 update with the thread-per-column layout and here: N=66, N_max=42 93, 69 us (the FP64 pipe
 // busy for 72% of the time the SMs are); 28 nucleons, N_max=20 27.8, 18.4; N=14, N_max=4 16.4, 12.3.
+// Pair sweeps of three N=66, N_max=36 systems: 117, 105.
 template <typename T_, int U>
 __global__ void __launch_bounds__(UPD_THREADS) k_update(DevState D, LoopCtl* __restrict__ ctl,
                                                         const UpdItem* __restrict__ items,
@@ -626,16 +654,47 @@ __global__ void __launch_bounds__(UPD_THREADS) k_update(DevState D, LoopCtl* __r
                                                         const T_* __restrict__ tpair, const double* __restrict__ aw) {
   constexpr bool PAIR = std::is_same<T_, f2>::value;
   using A = Arith<T_>;
+  struct Amp {
+    UpdItem it;
+    long z;
+    double tz, v, den, step;
+    int4 q;
+    int2 p, h;
+    int fc, ij, ab, m;
+  };
+  const double* __restrict__ t = cur_t(D, ctl);
+  const long chunk0 = (long)blockIdx.x * (U * UPD_THREADS / 32) + (threadIdx.x >> 5);
+  // the amplitude's streams and pair data: its place in the channel, then everything indexed by it
+  auto load = [&](int u) {
+    Amp a;
+    const long chunk = chunk0 + u * (UPD_THREADS / 32);
+    a.it = items[chunk];
+    a.z = upd_z[chunk * 32 + (threadIdx.x & 31)];
+    if (a.z < 0) return a;  // padding
+    const int e = (int)(a.z - a.it.base);
+    a.ij = e / a.it.npp;
+    a.ab = e - a.ij * a.it.npp;
+    a.fc = D.fmap[a.z];
+    a.tz = t[a.z];
+    a.v = D.v_pphh[a.z];
+    a.q = D.qmap[a.z];
+    a.den = D.den[a.z];
+    a.step = PAIR ? aw[a.z] : D.inv_den[a.z];
+    a.p = D.pp_pair[a.it.pp_off + a.ab];
+    a.h = D.hh_pair[a.it.hh_off + a.ij];
+    a.m = a.it.nl ? D.lad_map[a.it.pp_off + a.ab] : 0;
+    return a;
+  };
+  // the first chunk is requested before the loop control and the system's state are looked at
+  Amp a = load(0);
   if (ctl->status != 0) return;  // the loop has ended within its body (see pnm_enqueue_loop_body)
-  const long chunk0 = (long)blockIdx.x * (U * UPD_THREADS / 32);
-  const int sys = items[chunk0].sys;
+  const int sys = a.it.sys, ctas = fa.hi[sys] - fa.lo[sys];
   UpdSums S;
   // converged at least two steps ago: both amplitude buffers already hold its values, and its sums
   // are not read any more
   if (!sys_settled(fa.sc[sys], ctl)) {
     const bool frozen = fa.sc[sys].done != 0;
     const double alpha = ctl->alpha;
-    const double* __restrict__ t = cur_t(D, ctl);
     double* __restrict__ tn = next_t(D, ctl);
     const T_* __restrict__ tc;
     if constexpr (PAIR) tc = tpair;
@@ -644,56 +703,50 @@ __global__ void __launch_bounds__(UPD_THREADS) k_update(DevState D, LoopCtl* __r
     const T_* __restrict__ xq = reinterpret_cast<const T_*>(D.xq);
 #pragma unroll
     for (int u = 0; u < U; u++) {
-      const long chunk = chunk0 + u * (UPD_THREADS / 32) + (threadIdx.x >> 5);
-      const UpdItem it = items[chunk];
-      const int zi = upd_z[chunk * 32 + (threadIdx.x & 31)];
-      if (zi < 0) continue;  // padding
-      const long z = zi;
-      const int fc = D.fmap[z];
-      const long f = (long)(fc > 0 ? fc : -fc) - 1;
+      if (u > 0) a = load(u);
+      const long z = a.z;
+      if (z < 0) continue;
+      const long f = (long)(a.fc > 0 ? a.fc : -a.fc) - 1;
       if (f < z) continue;
-      const int e = (int)(z - it.base), ij = e / it.npp, ab = e - ij * it.npp, nh = it.nh, npp = it.npp;
-      const double tz = t[z], v = D.v_pphh[z];
+      const double tz = a.tz, v = a.v;
       double out = tz, R = 0.0;
       if (!frozen) {
-        const int4 q = D.qmap[z];
-        const int2 p = D.pp_pair[it.pp_off + ab], h = D.hh_pair[it.hh_off + ij];
-        const double den = D.den[z], step = PAIR ? aw[z] : D.inv_den[z];
+        const int4 q = a.q;
         T_ rl = A::zero();
-        if (it.nl) {
-          const int m = D.lad_map[it.pp_off + ab];
-          rl = rp[it.s_off + (long)ij * it.nl + ((m > 0 ? m : -m) - 1)];
-          if (m < 0) rl = A::neg(rl);
+        if (a.m != 0) {
+          rl = rp[a.it.s_off + (long)a.ij * a.it.nl + ((a.m > 0 ? a.m : -a.m) - 1)];
+          if (a.m < 0) rl = A::neg(rl);
         }
         const T_ q0 = q.x >= 0 ? xq[q.x] : A::zero(), q1 = q.y >= 0 ? xq[q.y] : A::zero();
         const T_ q2 = q.z >= 0 ? xq[q.z] : A::zero(), q3 = q.w >= 0 ? xq[q.w] : A::zero();
         // one-body part of the bracket: (d_a + d_b - d_i - d_j) t with d_p = chi_p - eps_p
-        const double d = (D.dchi[p.x] + D.dchi[p.y]) - (D.dchi[h.x] + D.dchi[h.y]);
+        const double d = (D.dchi[a.p.x] + D.dchi[a.p.y]) - (D.dchi[a.h.x] + D.dchi[a.h.y]);
         // hh ladder sum_kl t_ab^kl chi_kl^ij
         T_ hs = A::zero();
-        const T_* __restrict__ col = tc + it.base + ab;
-        const T_* __restrict__ chi = reinterpret_cast<const T_*>(D.chi_hh) + it.vhh_off + ij;
+        const int nh = a.it.nh, npp = a.it.npp;
+        const T_* __restrict__ col = tc + a.it.base + a.ab;
+        const T_* __restrict__ chi = reinterpret_cast<const T_*>(D.chi_hh) + a.it.vhh_off + a.ij;
 #pragma unroll 4
         for (int kl = 0; kl < nh; kl++) A::mac(hs, col[(long)kl * npp], chi[(long)kl * nh]);
         if constexpr (PAIR) {
           // pp ladder + hh ladder + P(ij)P(ab) Q in FP32 pairs, converted once
           const f2 corr = A::add(A::sub(A::sub(A::add(A::add(hs, rl), q0), q1), q2), q3);
           const double num = fma(d, tz, v) + A::to_double(corr);
-          R = fma(-den, tz, num);  // bracket - eps_ij^ab t
-          out = fma(R, step, tz);  // t + alpha R / eps_ij^ab
+          R = fma(-a.den, tz, num);  // bracket - eps_ij^ab t
+          out = fma(R, a.step, tz);  // t + alpha R / eps_ij^ab
         } else {
           const double num = ((fma(d, tz, v) + rl) + hs) + (((q0 - q1) - q2) + q3);
-          R = fma(-den, tz, num);
-          out = fma(alpha, num * step, (1.0 - alpha) * tz);
+          R = fma(-a.den, tz, num);
+          out = fma(alpha, num * a.step, (1.0 - alpha) * tz);
         }
       }
       tn[z] = out;
-      if (f != z) tn[f] = fc > 0 ? out : -out;
+      if (f != z) tn[f] = a.fc > 0 ? out : -out;
       S.add(f != z, v, out, R);
     }
     upd_partials(D, S);
   }
-  finalize_system(fa, ctl, sys);
+  finalize_system(fa, ctl, sys, ctas);
 }
 
 template <typename T_>
@@ -739,63 +792,89 @@ __global__ void __launch_bounds__(UPD_THREADS, UPD_MIN_BLOCKS) k_update_mix(
     DevState D, LoopCtl* __restrict__ ctl, const UpdItem* __restrict__ items, const int* __restrict__ upd_z, FinArgs fa,
     const float* __restrict__ rpp, const float* __restrict__ xq, const double* __restrict__ aw, float* __restrict__ xt,
     int nplanes, long pstride) {
+  struct Amp {
+    UpdItem it;
+    long z;
+    double tz, wz, v, den;
+    int4 qm;
+    int2 p, h;
+    float t32z;
+    int fc, ij, ab, m;
+  };
+  const double* __restrict__ t = cur_t(D, ctl);
+  const float* __restrict__ t32 = cur_t32(D, ctl);
+  const long chunk0 = (long)blockIdx.x * (U * UPD_THREADS / 32) + (threadIdx.x >> 5);
+  // the amplitude's streams and pair data: its place in the channel, then everything indexed by it
+  auto load = [&](int u) {
+    Amp a;
+    const long chunk = chunk0 + u * (UPD_THREADS / 32);
+    a.it = items[chunk];
+    a.z = upd_z[chunk * 32 + (threadIdx.x & 31)];
+    if (a.z < 0) return a;  // padding
+    const int e = (int)(a.z - a.it.base);
+    a.ij = e / a.it.npp;
+    a.ab = e - a.ij * a.it.npp;
+    a.tz = __ldcs(t + a.z);
+    a.wz = __ldcs(aw + a.z);
+    a.v = __ldcs(D.v_pphh + a.z);
+    a.den = __ldcs(D.den + a.z);
+    a.fc = __ldcs(D.fmap + a.z);
+    a.qm = __ldcs(D.qmap + a.z);
+    a.t32z = t32[a.z];
+    a.p = D.pp_pair[a.it.pp_off + a.ab];
+    a.h = D.hh_pair[a.it.hh_off + a.ij];
+    a.m = a.it.nl ? D.lad_map[a.it.pp_off + a.ab] : 0;
+    return a;
+  };
+  // the first chunk is requested before the loop control and the system's state are looked at
+  Amp a = load(0);
   if (ctl->status != 0) return;  // the loop has ended within its body (see pnm_enqueue_loop_body)
-  const long chunk0 = (long)blockIdx.x * (U * UPD_THREADS / 32);
-  const int sys = items[chunk0].sys;
+  const int sys = a.it.sys, ctas = fa.hi[sys] - fa.lo[sys];
   UpdSums S;
   // converged at least two steps ago: both amplitude buffers already hold its values, and its sums
   // are not read any more
   if (!sys_settled(fa.sc[sys], ctl)) {
     const bool frozen = fa.sc[sys].done != 0;
-    const double* __restrict__ t = cur_t(D, ctl);
-    const float* __restrict__ t32 = cur_t32(D, ctl);
     double* __restrict__ tn = next_t(D, ctl);
     float* __restrict__ t32n = next_t32(D, ctl);
 #pragma unroll (U < UPD_MIX_UNROLL ? U : UPD_MIX_UNROLL)
     for (int u = 0; u < U; u++) {
-      const long chunk = chunk0 + u * (UPD_THREADS / 32) + (threadIdx.x >> 5);
-      const UpdItem it = items[chunk];
-      const int zi = upd_z[chunk * 32 + (threadIdx.x & 31)];
-      if (zi < 0) continue;  // padding
-      const long z = zi;
-      const int e = (int)(z - it.base), ij = e / it.npp, ab = e - ij * it.npp, nh = it.nh, npp = it.npp;
-      const double tz = __ldcs(t + z), wz = __ldcs(aw + z), v = __ldcs(D.v_pphh + z), den = __ldcs(D.den + z);
-      const int fc = __ldcs(D.fmap + z);
-      const int4 qm = __ldcs(D.qmap + z);
-      const float t32z = t32[z];
-      const int2 p = D.pp_pair[it.pp_off + ab], h = D.hh_pair[it.hh_off + ij];
+      if (u > 0) a = load(u);
+      const long z = a.z;
+      if (z < 0) continue;
+      const int4 qm = a.qm;
       float rl = 0.0f;
-      if (it.nl) {
-        const int m = D.lad_map[it.pp_off + ab];
-        const long zl = it.s_off + (long)ij * it.nl + ((m > 0 ? m : -m) - 1);
+      if (a.m != 0) {
+        const long zl = a.it.s_off + (long)a.ij * a.it.nl + ((a.m > 0 ? a.m : -a.m) - 1);
         for (int pl = 0; pl < nplanes; pl++) rl += rpp[pl * pstride + zl];
-        if (m < 0) rl = -rl;
+        if (a.m < 0) rl = -rl;
       }
       // P(ij)P(ab) Q: Q_ij^ab - Q_ji^ab - Q_ij^ba + Q_ji^ba from the cross-channel layout
       const float a0 = qm.x >= 0 ? xq[qm.x] : 0.0f, a1 = qm.y >= 0 ? xq[qm.y] : 0.0f;
       const float a2 = qm.z >= 0 ? xq[qm.z] : 0.0f, a3 = qm.w >= 0 ? xq[qm.w] : 0.0f;
-      const float d = (D.dchi32[p.x] + D.dchi32[p.y]) - (D.dchi32[h.x] + D.dchi32[h.y]);
+      const float d = (D.dchi32[a.p.x] + D.dchi32[a.p.y]) - (D.dchi32[a.h.x] + D.dchi32[a.h.y]);
       float hh = 0.0f;
       if (!frozen) {
-        const float* __restrict__ col = t32 + it.base + ab;
-        const float* __restrict__ chi = D.chi32 + it.vhh_off + ij;
+        const int nh = a.it.nh, npp = a.it.npp;
+        const float* __restrict__ col = t32 + a.it.base + a.ab;
+        const float* __restrict__ chi = D.chi32 + a.it.vhh_off + a.ij;
 #pragma unroll UPD_HH_UNROLL
         for (int kl = 0; kl < nh; kl++) hh = fmaf(col[(long)kl * npp], chi[(long)kl * nh], hh);
       }
       // one amplitude of each spin-flip pair is computed (the smaller index) and written to both
-      const long f = (long)(fc > 0 ? fc : -fc) - 1;
+      const long f = (long)(a.fc > 0 ? a.fc : -a.fc) - 1;
       if (f < z) continue;
-      double out = tz, R = 0.0;
+      double out = a.tz, R = 0.0;
       if (!frozen) {
-        const float corr = d * t32z + (rl + hh) + ((a0 - a1) - (a2 - a3));
-        R = fma(-den, tz, v) + (double)corr;  // bracket - eps_ij^ab t
-        out = fma(R, wz, tz);
+        const float corr = d * a.t32z + (rl + hh) + ((a0 - a1) - (a2 - a3));
+        R = fma(-a.den, a.tz, a.v) + (double)corr;  // bracket - eps_ij^ab t
+        out = fma(R, a.wz, a.tz);
       }
       const float o32 = (float)out;
       __stcs(tn + z, out);
       t32n[z] = o32;
-      if (f != z) t32n[f] = fc < 0 ? -o32 : o32;
-      S.add(f != z, v, out, R);
+      if (f != z) t32n[f] = a.fc < 0 ? -o32 : o32;
+      S.add(f != z, a.v, out, R);
       if (!frozen) {
         // the T positions of t_ij^ab, t_ji^ab, t_ij^ba, t_ji^ba (the Q positions of the same
         // amplitude; stores only, nothing waits on them)
@@ -807,7 +886,7 @@ __global__ void __launch_bounds__(UPD_THREADS, UPD_MIN_BLOCKS) k_update_mix(
     }
     upd_partials(D, S);
   }
-  finalize_system(fa, ctl, sys);
+  finalize_system(fa, ctl, sys, ctas);
 }
 
 void launch_update_mix(pnm_ctx* ctx, const float* rpp, const float* xq, const double* aw, float* xt, int use_cond,
