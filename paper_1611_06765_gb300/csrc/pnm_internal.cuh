@@ -171,10 +171,13 @@ constexpr int PNM_DIVERGE_STEPS = 6;
 // from the second step on (the first one copies the amplitudes into the other buffer, after
 // which both buffers hold them).
 __device__ __forceinline__ bool sys_done(const DevState& D, const LoopCtl* ctl, int sys) {
-  return ctl->skip_done != 0 && (ctl->status != 0 || (D.sysctl != nullptr && D.sysctl[sys].done != 0));
+  // all three requested together: one round trip, not a chain of them, ahead of every small kernel
+  const int skip = ctl->skip_done, status = ctl->status, done = D.sysctl != nullptr ? D.sysctl[sys].done : 0;
+  return (skip != 0) & ((status != 0) | (done != 0));
 }
 __device__ __forceinline__ bool sys_settled(const SysCtl& S, const LoopCtl* ctl) {
-  return ctl->skip_done != 0 && S.done != 0 && ctl->iter >= S.frozen_at + 2;
+  const int skip = ctl->skip_done, iter = ctl->iter, done = S.done, at = S.frozen_at;
+  return (skip != 0) & (done != 0) & (iter >= at + 2);
 }
 
 // Arguments of the end-of-update step (energy, convergence test, loop condition).
