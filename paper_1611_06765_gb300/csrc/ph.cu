@@ -807,23 +807,23 @@ constexpr size_t PH_DIG_SMEM = 72 * 1024;
 void pnm_need_ph_items(pnm_ctx* ctx) {
   if (ctx->ph_items) return;
   cudaStream_t s = ctx->stream;
-  struct Channel {
-    long cost;
-    int x;
-    bool large;
-  };
-  std::vector<Channel> cta;
-  std::vector<int> by_dim[PH_WARP_DIM + 1];
+  // by cost in quarter octaves (a sort by the exact cost of 2500 channels took longer than the launch)
+  constexpr int COSTS = 4 * 64;
+  std::vector<int> by_dim[PH_WARP_DIM + 1], by_cost[2][COSTS];  // large channels first
   auto problems = [&](int x) { return ctx->h_x_cls[x] == 0 ? 2 : 1; };
+  bool larger = false;  // than the tiny kernels take
   for (int x = 0; x < ctx->nx; x++) {
     if (ctx->h_x_cls[x] < 0) continue;
-    const int nm = problems(x), R = ctx->h_x_nph[x] / nm, H = ctx->h_x_nhp[x] / nm;
-    if (std::max(R, H) <= PH_WARP_DIM) by_dim[std::max(R, H)].push_back(x);
-    else cta.push_back({(long)nm * R * H * H, x, ph_dig_smem(R, H, nm) > PH_DIG_SMEM});
+    const int nm = problems(x), R = ctx->h_x_nph[x] / nm, H = ctx->h_x_nhp[x] / nm, dim = std::max(R, H);
+    larger = larger || dim > PH_TINY_DIM;
+    if (dim <= PH_WARP_DIM) {
+      by_dim[dim].push_back(x);
+    } else {
+      const unsigned long cost = 4UL * nm * R * H * H;  // at least 4: two bits below the leading one
+      const int top = 63 - __builtin_clzl(cost);
+      by_cost[ph_dig_smem(R, H, nm) > PH_DIG_SMEM ? 0 : 1][4 * top + (int)((cost >> (top - 2)) & 3)].push_back(x);
+    }
   }
-  std::sort(cta.begin(), cta.end(), [](const Channel& a, const Channel& b) {
-    return a.large != b.large ? a.large : (a.cost != b.cost ? a.cost > b.cost : a.x < b.x);
-  });
   std::vector<PhItem> items;
   items.reserve(ctx->nx);
   unsigned long wf = 0, v1 = 0, src = 0, fixed = 0;
@@ -852,19 +852,20 @@ void pnm_need_ph_items(pnm_ctx* ctx) {
   };
   ctx->n_ph_large = ctx->n_ph_cta = ctx->n_ph_warp = ctx->n_ph_tiny = ctx->n_ph_tiny64 = 0;
   ctx->ph_large_smem = ctx->ph_dig_smem = ctx->ph_warp_smem = ctx->ph32_smem = ctx->ph32_warp_smem = 0;
-  for (const Channel& c : cta) {
-    add(c.x);
-    (c.large ? ctx->n_ph_large : ctx->n_ph_cta)++;
-    size_t& most = c.large ? ctx->ph_large_smem : ctx->ph_dig_smem;
-    most = std::max(most, dig);
-    ctx->ph32_smem = std::max(ctx->ph32_smem, f32);
+  for (int small = 0; small < 2; small++) {
+    size_t& most = small ? ctx->ph_dig_smem : ctx->ph_large_smem;
+    for (int k = COSTS - 1; k >= 0; k--)
+      for (int x : by_cost[small][k]) {
+        add(x);
+        (small ? ctx->n_ph_cta : ctx->n_ph_large)++;
+        most = std::max(most, dig);
+        ctx->ph32_smem = std::max(ctx->ph32_smem, f32);
+      }
   }
   // FP64 results: where no channel is larger than PH_TINY_DIM all take the tiny kernel, which saves
   // the passes that make the digits (N = 14: the operator call 96 -> 73 us, a solve of one
   // n^2 <= 24 system 955 -> 852 us, of sixteen 4.82 -> 4.22 ms); beside larger channels the digit
   // kernel is the faster one from PH_TINY_FP64 + 1 on.
-  bool larger = !cta.empty();
-  for (int d = PH_TINY_DIM + 1; d <= PH_WARP_DIM; d++) larger = larger || !by_dim[d].empty();
   const int tiny64 = larger ? PH_TINY_FP64 : PH_TINY_DIM;
   for (int d = PH_WARP_DIM; d >= 0; d--) {
     const int n = (int)by_dim[d].size();
