@@ -1909,9 +1909,47 @@ void pnm_flip_copy_device(pnm_ctx* ctx) {
 
 // Schedule tuning: time a few updates with the ph term and the pp ladder on side streams
 // (concurrent with the one-body kernels) and a few with everything on one stream; keep the
-// faster for this precision mode.  The held amplitudes are saved and restored.
+// faster for this precision mode.  Where concurrent mixed updates take SCHED_ORDER_US or more, the
+// orders of pnm_enqueue_body_mixed are timed too, as a graph with the priorities of the solve's (shorter
+// updates gain nothing, and launches from the host would blur the difference).  The held amplitudes
+// are saved and restored.
+constexpr float SCHED_ORDER_US = 150.0f;
 static std::mutex g_sched_mu;
-static std::map<std::string, bool> g_sched_cache;  // (shape key, mode) -> one stream
+static std::map<std::string, int> g_sched_cache;  // (shape key, mode) -> one stream (-1), or the order
+
+// Milliseconds of four mixed updates as one graph.
+static float time_body_graph(pnm_ctx* ctx, int mode, cudaEvent_t e0, cudaEvent_t e1) {
+  cudaStream_t s = ctx->stream;
+  cudaGraph_t g;
+  CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+  try {
+    for (int k = 0; k < 4; k++) pnm_enqueue_body(ctx, mode, 0, 0);
+  } catch (...) {
+    cudaGraph_t dummy;
+    cudaStreamEndCapture(s, &dummy);
+    throw;
+  }
+  CUDA_TRY(cudaStreamEndCapture(s, &g));
+  cudaGraphExec_t ge = nullptr;
+  float ms = 0;
+  try {
+    pnm_set_node_priorities(g);
+    CUDA_TRY(cudaGraphInstantiate(&ge, g, cudaGraphInstantiateFlagUseNodePriority));
+    CUDA_TRY(cudaGraphLaunch(ge, s));
+    CUDA_TRY(cudaEventRecord(e0, s));
+    CUDA_TRY(cudaGraphLaunch(ge, s));
+    CUDA_TRY(cudaEventRecord(e1, s));
+    CUDA_TRY(cudaEventSynchronize(e1));
+    CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
+  } catch (...) {
+    if (ge) cudaGraphExecDestroy(ge);
+    cudaGraphDestroy(g);
+    throw;
+  }
+  cudaGraphExecDestroy(ge);
+  cudaGraphDestroy(g);
+  return ms;
+}
 
 void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
   const bool pair = ((mode >> 8) & 1) != 0;
@@ -1923,7 +1961,8 @@ void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
     std::lock_guard<std::mutex> lock(g_sched_mu);
     auto f = g_sched_cache.find(key);
     if (f != g_sched_cache.end()) {
-      ctx->serial_sched[m] = f->second;
+      ctx->serial_sched[m] = f->second < 0;
+      if (m == 1) ctx->mixed_order = std::max(0, f->second);
       ctx->sched_tuned[m] = true;
       return;
     }
@@ -1956,13 +1995,29 @@ void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
       best_serial = serial;
     }
   }
+  ctx->serial_sched[m] = best_serial != 0;
+  if (m == 1 && !best_serial && best * 1e3f >= 4 * SCHED_ORDER_US) {
+    float fastest = 1e30f;
+    int order = 0;
+    for (int k = 0; k < 3; k++) {
+      ctx->mixed_order = k;
+      CUDA_TRY(cudaMemcpyAsync(ctx->d.t0, save, sizeof(double) * ctx->nt, cudaMemcpyDeviceToDevice, s));
+      pnm_start(ctx, PNM_INIT_KEEP, never);
+      pnm_mixed_pack_initial(ctx, alpha);
+      const float ms = time_body_graph(ctx, mode, e0, e1);
+      if (ms < 0.98f * fastest) {
+        fastest = ms;
+        order = k;
+      }
+    }
+    ctx->mixed_order = order;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  ctx->serial_sched[m] = best_serial != 0;
   ctx->sched_tuned[m] = true;
   {
     std::lock_guard<std::mutex> lock(g_sched_mu);
-    g_sched_cache[key] = ctx->serial_sched[m];
+    g_sched_cache[key] = ctx->serial_sched[m] ? -1 : (m == 1 ? ctx->mixed_order : 0);
   }
   CUDA_TRY(cudaMemcpyAsync(ctx->d.t0, save, sizeof(double) * ctx->nt, cudaMemcpyDeviceToDevice, s));
   CUDA_TRY(cudaGetLastError());

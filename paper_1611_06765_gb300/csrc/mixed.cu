@@ -676,25 +676,40 @@ static void launch_pack_t(pnm_ctx* ctx, cudaStream_t s) {
                                                                             M->bt);
 }
 
+// The ladder streams V and needs an SM's shared memory per CTA; kernels of many small CTAs that start
+// with the update hold the SMs when its t tiles are ready.  Order (measured per shape for long updates,
+// pnm_tune_schedule): 0 ph term, ladder and one-body kernels from the start; 1 the ph term behind the t
+// tiles; 2 the one-body kernels too.  Per update: three N=66, N_max=36 systems 222, 212, 236 us; 120
+// twisted N=14, N_max=20 systems 228, 228, 213; one N=66, N_max=36 system 88, 90, 105.
 void pnm_enqueue_body_mixed(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHandle h) {
   MixedState* M = ctx->mixed;
-  cudaStream_t s_ph = pnm_concurrent(ctx) ? ctx->side[0] : ctx->stream;
-  cudaStream_t s_pp = pnm_concurrent(ctx) ? ctx->side[1] : ctx->stream;
+  const bool side = pnm_concurrent(ctx);
+  const int order = side && M->nitems > 0 ? ctx->mixed_order : 0;
+  cudaStream_t s_ph = side ? ctx->side[0] : ctx->stream;
+  cudaStream_t s_pp = side ? ctx->side[1] : ctx->stream;
   pnm_fork(ctx);
-  if (ctx->nx > 0) {
+  auto ph = [&] {
+    if (ctx->nx == 0) return;
     prof_begin(ctx, KID_PH32);
     launch_ph_mix(ctx, M->xt32, M->xw32, M->xv132, M->xq32, s_ph, ctx->stream);
     prof_end(ctx);
-  }
+  };
+  if (order == 0) ph();
   if (M->nitems > 0) {
     // t tiles of the current amplitudes in the ladder basis, then the ladder (same stream)
     prof_begin(ctx, KID_PACK);
     launch_pack_t<float>(ctx, s_pp);
     prof_end(ctx);
+    if (order > 0) {
+      CUDA_TRY(cudaEventRecord(ctx->ev_join[1], s_pp));
+      CUDA_TRY(cudaStreamWaitEvent(s_ph, ctx->ev_join[1], 0));
+      if (order > 1) CUDA_TRY(cudaStreamWaitEvent(ctx->stream, ctx->ev_join[1], 0));
+    }
     prof_begin(ctx, KID_PP_TC);
     launch_pp_tc(M->items, M->cta_off, M->grid, M, M->smem, M->nst, ctx->ctl, ctx->ns, s_pp);
     prof_end(ctx);
   }
+  if (order > 0) ph();
   pnm_enqueue_stats(ctx, true);
   pnm_join(ctx);
   prof_begin(ctx, KID_UPDATE_MIX);
