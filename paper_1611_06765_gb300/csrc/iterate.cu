@@ -1552,9 +1552,12 @@ static void enqueue_body_fp64(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHa
   bool ph_on = terms == PNM_TERMS_FULL || terms == PNM_TERMS_LINEAR;
   if (pair) pnm_split_cur(ctx, ctx->stream);  // before the fork: both branches read it
   pnm_fork(ctx);
-  // the one-body kernels first: of the branches that start together they are the shortest, and behind
-  // the others they ended last (per update: N=66, N_max=42 303 -> 299 us, 28 nucleons 83 -> 80)
-  if (terms == PNM_TERMS_FULL) pnm_enqueue_stats(ctx, false, pair);
+  // the one-body kernels first beside the digit kernels: they are the shortest branch, and behind the
+  // others they ended last (per update: N=66, N_max=42 303 -> 299 us, 28 nucleons 83 -> 80); last where
+  // the tiny kernel takes every channel, whose FP64 work is then the longest branch (N=14, N_max=20: 32
+  // us, first 39)
+  const bool digits = ctx->n_ph_large + ctx->n_ph_cta + ctx->n_ph_warp > (pair ? ctx->n_ph_tiny : ctx->n_ph_tiny64);
+  if (terms == PNM_TERMS_FULL && digits) pnm_enqueue_stats(ctx, false, pair);
   if (ctx->nx > 0 && ph_on) {
     prof_begin(ctx, pair ? KID_PH_F2 : KID_PH64);
     if (pair) launch_ph_f2(ctx, s_ph, ctx->stream);
@@ -1566,6 +1569,7 @@ static void enqueue_body_fp64(pnm_ctx* ctx, int use_cond, cudaGraphConditionalHa
     pnm_launch_pp(ctx, s_pp, true, pair);
     prof_end(ctx);
   }
+  if (terms == PNM_TERMS_FULL && !digits) pnm_enqueue_stats(ctx, false, pair);
   pnm_join(ctx);
   prof_begin(ctx, KID_UPDATE);
   launch_update64(ctx, use_cond, h, pair);
