@@ -214,11 +214,6 @@ __device__ __forceinline__ Out dig_result(DigSum x, int p) {
 // levels are counted from 256^7 256^7 = 2^112 down to 2^56.
 __device__ __forceinline__ int dig_power(int ea, int eb) { return 56 - 122 + (ea + eb - 2044); }
 
-// The word of -x from the word of x, and of x + y, x - y.
-__device__ __forceinline__ dig_t dig_neg(dig_t w) { return DIG_BIAS + DIG_BIAS - w; }
-__device__ __forceinline__ dig_t dig_sum(dig_t a, dig_t b) { return a + b - DIG_BIAS; }
-__device__ __forceinline__ dig_t dig_diff(dig_t a, dig_t b) { return a - b + DIG_BIAS; }
-
 // The antisymmetrized Minnesota element of v_minnesota_as as an integer, from the table of the
 // Gaussians as integers of one scale (interleaved R, T, S with protons, as the FP64 table): sums
 // of table entries with small integer weights, exact.  The states conserve momentum.

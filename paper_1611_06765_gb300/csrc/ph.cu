@@ -336,25 +336,28 @@ void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* 
 // the matrices are small (N = 66: 17 to 33 rows and columns): per problem (a S_z > 0 channel, or
 // the sum and the difference problem of an S_z = 0 channel)
 //   C[(k,c)][(j,b)] = <kb|v|cj> + 1/2 sum_(e,l) <kl|v|ce> t_lj^eb,   Q[(a,i)][(j,b)] = T C.
-// Operands are integers and their digits from end to end:
-//   - the amplitudes as digit words of one exponent per system (k_tmax, k_twords: two passes over
-//     them per update, where converting at the gather repeated the work for each of the three or
-//     four places of an amplitude and cost two more passes over shared memory);
+// Operands are integers and their digits from end to end, each with an exponent of its own per channel:
 //   - W as digits in fragment order, <kb|v|cj> as integers, and the signed amplitude index of every
 //     staged element, fixed per context (k_ph_pack; sums and differences of S_z = 0 formed there);
-//   - T staged as words (sums and differences of S_z = 0 as exact integer sums), two neighbouring
-//     columns interleaved: the k index of the second product; the first reads its k pairs across
-//     rows;
+//   - T gathered as FP64 and converted in place to words of the channel's exponent (sums and
+//     differences of S_z = 0 as exact integer sums), two neighbouring columns interleaved: the k index
+//     of the second product; the first reads its k pairs across rows;
 //   - C as integers, the two terms aligned to the coarser of their units (2^-60 of their bounds or
 //     finer), its digits stored interleaved by row pairs straight from the first product's registers.
+// An integer holds an element within PH_SPAN octaves of its operand's largest one to its last bit, and a
+// smaller one to 2^-61 of that largest.  FP64 sums round at 2^-53 of the products they add, so the digits
+// stand in for them only where no row or column of T, W or <kb|v|cj> lies wholly further down: a channel
+// with such a row or column (one amplitude far above the others, say) is summed in FP64 (ph_values).
+// MBPT2 amplitudes and the Minnesota interaction stay within it (N = 14 to 66, densities 0.02 to 0.3:
+// rows of T within 6 octaves of their channel's largest, rows of W within 5, of <kb|v|cj> 0).
 // Only the results leave as floating point.  A group of 32 threads (channels of at most PH_WARP_DIM
 // rows and columns) or of 128 (the others) takes a channel; a warp forms 16 x 8 blocks.
 // What bounds it: instruction issue and its latencies around the products (operand expansion,
-// drains, staging) at twelve warps per SM; without the MMAs it takes 6% less time.  Per launch with
-// the two passes over the amplitudes: N = 66, n^2 <= 42, FP64 149 us against 405 us on the FP64
-// pipe; three densities of N = 66, n^2 <= 36, pairs, 290 against 356 us on the FP32 pipe; symmetric
-// matter, 28 nucleons, n^2 <= 20, FP64 50 against 52 us launched one by one, and shorter beside the
-// ladder in a captured update (no FP64 pipe work to share).
+// drains, staging) at twelve warps per SM; without the MMAs it takes 6% less time.  One exponent for
+// all amplitudes of a system, their words made in two passes ahead of this kernel, took 13 us less of an
+// update of 330 (N = 66, n^2 <= 42; third-order sums of three densities of n^2 <= 36: 485, 515 us) but left
+// a channel far below the system's largest amplitude as few bits (relative errors of 5e-6 beside one
+// amplitude 2^20 above the others).
 __host__ __device__ __forceinline__ int ph_h8(int H) { return (H + 7) & ~7; }
 // Row strides in 16-byte pairs: T's odd, C's 2 modulo 8, so that the fragment loads of the first
 // product (two rows per thread) and of the second spread over the banks.
@@ -364,8 +367,50 @@ __host__ __device__ __forceinline__ size_t ph_dig_smem(int R, int H, int nm) {
   return sizeof(uint4) * nm * ((size_t)ph_h8(R) * ph_ts(H) + (size_t)(ph_h8(H) / 2) * ph_cs(H));
 }
 
-// The term of one channel in FP64 arithmetic (infinities, NaN, or values so large that intermediate
-// results might overflow): the sums of the same expressions in order.
+constexpr int PH_SPAN = 8;
+constexpr int PH_MAX_DIM = 128;  // rows or columns of a problem (PhMarks)
+
+// Which rows and columns of a matrix hold an element within PH_SPAN octaves of the largest (big), which a
+// smaller one other than zero (some): bytes that any thread may set, rows [0, n), columns [n, 2 n).
+struct PhMarks {
+  unsigned char* at;
+  int n;
+  __device__ void set(int k, int size, int least) const {
+    if (size > 0) at[size >= least ? k : 2 * n + k] = 1;
+  }
+  // whether one of four rows or columns holds small elements only
+  __device__ bool low(int k4) const {
+    const unsigned* m = reinterpret_cast<const unsigned*>(at);
+    return (m[n / 2 + k4] & ~m[k4]) != 0;
+  }
+};
+// The size of an element in integers (no comparison on the FP64 pipe): its bits above the fraction's
+// low word, 0 for zero alone; and the least size within PH_SPAN octaves of exponent e.
+__device__ __forceinline__ int size_of(double x) {
+  return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0);
+}
+__device__ __forceinline__ int least_size(int e) { return e > PH_SPAN + 1 ? (e - PH_SPAN) << 20 : 1; }
+
+template <int GT>
+__device__ __forceinline__ int group_max(int v, int* sh) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  if constexpr (GT > 32) {
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < GT / 32; w++) v = max(v, sh[w]);
+  }
+  return v;
+}
+template <int GT>
+__device__ __forceinline__ bool group_any(bool b) {
+  if constexpr (GT == 32) return __any_sync(0xffffffffu, b);
+  else return __syncthreads_or(b);
+}
+
+// The term of one channel in FP64 arithmetic (infinities, NaN, values so large that intermediate
+// results might overflow, rows or columns far below the largest element): the sums of the same
+// expressions in order.
 template <typename Out, int GT>
 __device__ __noinline__ void ph_values(const DevState& D, const PhItem& it, int tid, uint4* Ts, uint4* Cs,
                                        const double* __restrict__ t, bool quad, Out* __restrict__ xq) {
@@ -416,12 +461,12 @@ __device__ __noinline__ void ph_values(const DevState& D, const PhItem& it, int 
 // finite below.
 constexpr int PH_MAX_EXP = 2900;
 
-// ex: exponents of W and of <kb|v|cj>.
+// ex: exponents of W and of <kb|v|cj>; marks: 4 PH_MAX_DIM bytes for a CTA's channel, 64 for a warp's.
 template <typename Out, int GT, int NM>
 __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2 ex, unsigned char* smraw,
                                        const double* __restrict__ t, const int* __restrict__ src,
                                        const uint4* __restrict__ wf, const long long* __restrict__ v1, bool quad,
-                                       Out* __restrict__ xq) {
+                                       Out* __restrict__ xq, unsigned char* marks, int* sh_max) {
   const int tid = GT == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, wid = tid >> 5;
   constexpr int NW = GT / 32;
@@ -429,42 +474,76 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
   const int TP = R8 * TS, CP = (H8 / 2) * CS;
   uint4* Ts = reinterpret_cast<uint4*>(smraw);  // [problem][row][column pair]
   uint4* Cs = Ts + NM * TP;                     // [problem][row pair][column]
-  const int et = D.sys_texp[it.sys];
+  const PhMarks mark{marks, GT == 32 ? PH_WARP_DIM : PH_MAX_DIM};  // of T: of both blocks of S_z = 0
+  for (int k = tid; k < mark.n; k += GT) reinterpret_cast<int*>(marks)[k] = 0;
+  // T: two neighbouring columns per step (index rows are padded to H8, rows past R read none), the
+  // amplitudes and their largest exponent first, then their words, each thread its own elements
+  const int wide = H8 / 2, total = R8 * wide, live = R * wide, du = GT / wide, ds = GT % wide;
+  auto amp = [&](int c) { return c == 0 ? 0.0 : (c > 0 ? t[c - 1] : -t[-c - 1]); };
+  int et = 1;
+  {
+    int u = tid / wide, s = tid % wide;
+#pragma unroll 4
+    for (int f = tid; f < total; f += GT) {
+      double2* pa = reinterpret_cast<double2*>(Ts + u * TS + s);
+      if constexpr (NM == 1) {
+        const int2 c = f < live ? reinterpret_cast<const int2*>(src + it.src)[f] : make_int2(0, 0);
+        const double2 a = make_double2(amp(c.x), amp(c.y));
+        et = max(et, max(dig_exp(a.x), dig_exp(a.y)));
+        *pa = a;
+      } else {
+        const int4 c = f < live ? reinterpret_cast<const int4*>(src + it.src)[f] : make_int4(0, 0, 0, 0);
+        const double2 a = make_double2(amp(c.x), amp(c.z)), b = make_double2(amp(c.y), amp(c.w));
+        et = max(et, max(max(dig_exp(a.x), dig_exp(a.y)), max(dig_exp(b.x), dig_exp(b.y))));
+        *pa = a;
+        pa[TP] = b;
+      }
+      u += du;
+      s += ds;
+      if (s >= wide) {
+        s -= wide;
+        u++;
+      }
+    }
+  }
+  et = group_max<GT>(et, sh_max);
+  if constexpr (GT == 32) __syncwarp();  // the marks are clear
   if (et >= DIG_NONFINITE || ex.x >= DIG_NONFINITE || ex.y >= DIG_NONFINITE || et + ex.x > PH_MAX_EXP) {
     ph_values<Out, GT>(D, it, tid, Ts, Cs, t, quad, xq);  // group-uniform branch
     return;
   }
-  // T: two neighbouring columns per step (index rows are padded to H8, rows past R read none)
   {
-    const dig_t* __restrict__ tw = D.twords;
-    auto word = [&](int c) {
-      if (c == 0) return DIG_BIAS;
-      const dig_t w = tw[c > 0 ? c - 1 : -c - 1];
-      return c < 0 ? dig_neg(w) : w;
-    };
-    const int half = H8 / 2, total = R8 * half, live = R * half, du = GT / half, ds = GT % half;
-    int u = tid / half, s = tid % half;
-#pragma unroll 4
+    const int least = least_size(et);
+    int u = tid / wide, s = tid % wide;
+#pragma unroll 2
     for (int f = tid; f < total; f += GT) {
       uint4* pa = Ts + u * TS + s;
+      const double2 a = *reinterpret_cast<const double2*>(pa);
+      int m0 = size_of(a.x), m1 = size_of(a.y);
+      const long long a0 = dig_fixed(a.x, et), a1 = dig_fixed(a.y, et);
       if constexpr (NM == 1) {
-        const int2 c = f < live ? reinterpret_cast<const int2*>(src + it.src)[f] : make_int2(0, 0);
-        *pa = dig_interleave(word(c.x), word(c.y));
+        *pa = dig_interleave(dig_word(a0), dig_word(a1));
       } else {
-        const int4 c = f < live ? reinterpret_cast<const int4*>(src + it.src)[f] : make_int4(0, 0, 0, 0);
-        const dig_t a0 = word(c.x), b0 = word(c.y), a1 = word(c.z), b1 = word(c.w);
-        *pa = dig_interleave(dig_sum(a0, b0), dig_sum(a1, b1));
-        pa[TP] = dig_interleave(dig_diff(a0, b0), dig_diff(a1, b1));
+        const double2 b = *reinterpret_cast<const double2*>(pa + TP);
+        m0 = max(m0, size_of(b.x));
+        m1 = max(m1, size_of(b.y));
+        const long long b0 = dig_fixed(b.x, et), b1 = dig_fixed(b.y, et);
+        *pa = dig_interleave(dig_word(a0 + b0), dig_word(a1 + b1));
+        pa[TP] = dig_interleave(dig_word(a0 - b0), dig_word(a1 - b1));
       }
+      mark.set(u, max(m0, m1), least);
+      mark.set(mark.n + 2 * s, m0, least);
+      mark.set(mark.n + 2 * s + 1, m1, least);
       u += du;
       s += ds;
-      if (s >= half) {
-        s -= half;
+      if (s >= wide) {
+        s -= wide;
         u++;
       }
     }
   }
   group_sync<GT>();
+  const bool low = tid < mark.n / 2 && mark.low(tid);  // known to the group after the first product
   // C: 16 x 8 blocks of every problem; the fragments of W are requested one step ahead, across
   // blocks too
   const int nt = H8 / 8, sc = (H + 15) >> 4, kr = (R + 15) >> 4, blocks = NM * sc * nt;
@@ -516,7 +595,11 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
     if (strip * 16 + g + 8 < H8)
       pc0[4 * CS] = dig_interleave(DIG_BIAS + (odd ? r1 : o1), DIG_BIAS + (odd ? o1 : r1));
   }
-  group_sync<GT>();
+  if constexpr (GT == 32) __syncwarp();
+  if (group_any<GT>(low)) {
+    ph_values<Out, GT>(D, it, tid, Ts, Cs, t, quad, xq);
+    return;
+  }
   // Q
   const int sr = (R + 15) >> 4, kh = (H + 15) >> 4;
   const int p2 = 56 + (et - 1022 - 61) + pc - (NM == 2 ? 1 : 0);  // the half of sum and difference
@@ -572,46 +655,6 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
       }
     }
   }
-}
-
-// Digit words of the current amplitudes of every system, of one exponent per system.  TW_PARTS CTAs
-// per system find the largest exponents of their parts (k_tmax); k_twords reduces them (again in
-// every CTA) and converts; part 0 publishes the system's exponent.
-constexpr int TW_THREADS = 256, TW_PARTS = 512;
-__global__ void __launch_bounds__(TW_THREADS) k_tmax(DevState D, const LoopCtl* __restrict__ ctl,
-                                                     const long* __restrict__ t_lo, int* __restrict__ parts) {
-  const int sys = blockIdx.x;
-  if (sys_done(D, ctl, sys)) return;
-  const double* __restrict__ t = cur_t(D, ctl);
-  const long hi = t_lo[sys + 1];
-  int e = 1;
-#pragma unroll 4
-  for (long z = t_lo[sys] + blockIdx.y * TW_THREADS + threadIdx.x; z < hi; z += gridDim.y * TW_THREADS)
-    e = max(e, dig_exp(t[z]));
-  e = __reduce_max_sync(0xffffffffu, e);
-  __shared__ int top;
-  if (threadIdx.x == 0) top = 1;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) atomicMax(&top, e);
-  __syncthreads();
-  if (threadIdx.x == 0) parts[sys * TW_PARTS + blockIdx.y] = top;
-}
-
-__global__ void __launch_bounds__(TW_THREADS) k_twords(DevState D, const LoopCtl* __restrict__ ctl,
-                                                       const long* __restrict__ t_lo, const int* __restrict__ parts,
-                                                       int nparts) {
-  const int sys = blockIdx.x;
-  if (sys_done(D, ctl, sys)) return;
-  int e = 1;
-  for (int k = threadIdx.x & 31; k < nparts; k += 32) e = max(e, parts[sys * TW_PARTS + k]);
-  e = __reduce_max_sync(0xffffffffu, e);
-  if (blockIdx.y == 0 && threadIdx.x == 0) D.sys_texp[sys] = e;
-  if (e >= DIG_NONFINITE) return;  // the term is then formed from the FP64 values
-  const double* __restrict__ t = cur_t(D, ctl);
-  const long hi = t_lo[sys + 1];
-#pragma unroll 4
-  for (long z = t_lo[sys] + blockIdx.y * TW_THREADS + threadIdx.x; z < hi; z += gridDim.y * TW_THREADS)
-    D.twords[z] = dig_word(dig_fixed(t[z], e));
 }
 
 // Channels of at most PH_TINY_DIM (FP32-pair results) or PH_TINY_FP64 (FP64 results) rows and
@@ -684,13 +727,15 @@ __global__ void __launch_bounds__(PH_THREADS, 3) k_ph_dig(DevState D, const Loop
                                                           const uint4* __restrict__ wf, const long long* __restrict__ v1,
                                                           int quad, Out* __restrict__ xq) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ __align__(4) unsigned char marks[4 * PH_MAX_DIM];
+  __shared__ int sh_max[PH_WARPS];
   const double* __restrict__ t = cur_t(D, ctl);
   if ((int)blockIdx.x < nblk) {
     const PhItem it = items[blockIdx.x];
     if (sys_done(D, ctl, it.sys)) return;  // CTA-uniform
     const int2 ex = exps[blockIdx.x];
-    if (it.nm == 2) ph_dig<Out, PH_THREADS, 2>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq);
-    else ph_dig<Out, PH_THREADS, 1>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq);
+    if (it.nm == 2) ph_dig<Out, PH_THREADS, 2>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq, marks, sh_max);
+    else ph_dig<Out, PH_THREADS, 1>(D, it, ex, smraw, t, src, wf, v1, quad != 0, xq, marks, sh_max);
     return;
   }
   const int w = threadIdx.x >> 5, idx = ((int)blockIdx.x - nblk) * PH_WARPS + w;
@@ -699,8 +744,9 @@ __global__ void __launch_bounds__(PH_THREADS, 3) k_ph_dig(DevState D, const Loop
   if (sys_done(D, ctl, it.sys)) return;
   const int2 ex = exps[nblk + idx];
   unsigned char* sm = smraw + (size_t)w * warp_smem;
-  if (it.nm == 2) ph_dig<Out, 32, 2>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq);
-  else ph_dig<Out, 32, 1>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq);
+  unsigned char* mk = marks + w * 4 * PH_WARP_DIM;
+  if (it.nm == 2) ph_dig<Out, 32, 2>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq, mk, sh_max);
+  else ph_dig<Out, 32, 1>(D, it, ex, sm, t, src, wf, v1, quad != 0, xq, mk, sh_max);
 }
 
 // The smallest channels, one warp each, in a kernel of their own: it needs a third of the registers.
@@ -721,11 +767,13 @@ __global__ void __launch_bounds__(PH_THREADS) k_ph_tiny(DevState D, const LoopCt
 }
 
 // The fixed operands of the items (one CTA each): source indices (rows padded to H8), <kb|v|cj> of
-// the problems as integers (padded to whole blocks) and the digits of W, with their exponents.
+// the problems as integers (padded to whole blocks) and the digits of W, with their exponents
+// (DIG_NONFINITE where a row or column lies too far below the largest element).
 __global__ void __launch_bounds__(128) k_ph_pack(DevState D, const PhItem* __restrict__ items, int2* __restrict__ exps,
                                                  int* __restrict__ src, uint4* __restrict__ wf, long long* __restrict__ v1,
                                                  double* __restrict__ fixed64, f2* __restrict__ fixed_f2) {
   __shared__ int top[2];
+  __shared__ __align__(4) unsigned char marks[2][4 * PH_MAX_DIM];
   const PhItem it = items[blockIdx.x];
   const int R = it.R, H = it.H, H8 = ph_h8(H), H4 = formed_width(H), RW = R * H4, HW = H * H4;
   const double* __restrict__ W = D.x_w + it.to;
@@ -737,6 +785,8 @@ __global__ void __launch_bounds__(128) k_ph_pack(DevState D, const PhItem* __res
     fixed64[it.fx + o] = v;
     fixed_f2[it.fx + o] = Arith<f2>::from_double(v);
   };
+  const PhMarks mw{marks[0], PH_MAX_DIM}, mv{marks[1], PH_MAX_DIM};
+  for (int k = threadIdx.x; k < 8 * PH_MAX_DIM; k += blockDim.x) marks[0][k] = 0;
   if (threadIdx.x < 2) top[threadIdx.x] = 1;
   __syncthreads();
   int e = 1;
@@ -769,8 +819,19 @@ __global__ void __launch_bounds__(128) k_ph_pack(DevState D, const PhItem* __res
   if ((threadIdx.x & 31) == 0) atomicMax(&top[1], e);
   __syncthreads();
   const int ew = top[0], ev = top[1];
-  if (threadIdx.x == 0) exps[blockIdx.x] = make_int2(ew, ev);
-  if (ew >= DIG_NONFINITE || ev >= DIG_NONFINITE) return;
+  auto span = [&](const PhMarks& m, const double* __restrict__ M, int rows, int n, int least) {
+    for (int f = threadIdx.x; f < rows * H; f += blockDim.x) {
+      const int u = f / H, s = f % H, o = u * H4 + s, x = max(size_of(M[o]), two ? size_of(M[n + o]) : 0);
+      m.set(u, x, least);
+      m.set(m.n + s, x, least);
+    }
+  };
+  span(mw, W, R, RW, least_size(ew));
+  span(mv, V, H, HW, least_size(ev));
+  __syncthreads();
+  const bool low = __syncthreads_or((int)threadIdx.x < PH_MAX_DIM / 2 && (mw.low(threadIdx.x) || mv.low(threadIdx.x)));
+  if (threadIdx.x == 0) exps[blockIdx.x] = low ? make_int2(DIG_NONFINITE, DIG_NONFINITE) : make_int2(ew, ev);
+  if (low || ew >= DIG_NONFINITE || ev >= DIG_NONFINITE) return;
   const int sc = (H + 15) >> 4, kr = (R + 15) >> 4;
   for (int f = threadIdx.x; f < sc * 16 * H8; f += blockDim.x) {
     const int r = f / H8, c = f % H8;
@@ -908,20 +969,6 @@ void pnm_need_phdig(pnm_ctx* ctx) {
     k_ph_pack<<<ctx->n_ph_items, 128, 0, s>>>(ctx->d, ctx->ph_items, exps, ctx->ph_src, ctx->ph_wf, ctx->ph_v1,
                                               ctx->ph_fixed64, ctx->ph_fixed_f2);
   CUDA_TRY(cudaGetLastError());
-  const int nsys = (int)ctx->sys.size();
-  std::vector<long> lo(nsys + 1, ctx->nt);
-  long longest = 0;
-  for (int k = 0; k < nsys; k++) {
-    lo[k] = ctx->sys[k].t_begin;
-    longest = std::max(longest, ctx->sys[k].t_end - ctx->sys[k].t_begin);
-  }
-  // parts of about a thousand amplitudes
-  ctx->n_tw_parts = (int)std::max<long>(1, std::min<long>(TW_PARTS, longest / (4 * TW_THREADS)));
-  ctx->tw_lo = ctx_alloc<long>(ctx, nsys + 1);
-  ctx->tw_parts = ctx_alloc<int>(ctx, (size_t)nsys * TW_PARTS);
-  ctx->d.sys_texp = ctx_alloc<int>(ctx, nsys);
-  ctx->d.twords = ctx_alloc<unsigned long long>(ctx, ctx->nt);
-  CUDA_TRY(cudaMemcpyAsync(ctx->tw_lo, lo.data(), sizeof(long) * (nsys + 1), cudaMemcpyHostToDevice, s));
   const size_t most = std::max(ctx->ph_large_smem, ctx->ph_dig_smem);
   smem_at_least(k_ph_dig<double>, most);
   smem_at_least(k_ph_dig<f2>, most);
@@ -938,11 +985,6 @@ static void launch_ph_dig(pnm_ctx* ctx, bool linear, cudaStream_t s, cudaStream_
   Out* xq = reinterpret_cast<Out*>(ctx->d.xq);
   const PhItem* items = ctx->ph_items;
   if (nl + n + nw == 0) s_tiny = s;
-  if (nl + n + nw > 0) {
-    const dim3 grid((unsigned)ctx->sys.size(), ctx->n_tw_parts);
-    k_tmax<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts);
-    k_twords<<<grid, TW_THREADS, 0, s>>>(ctx->d, ctx->ctl, ctx->tw_lo, ctx->tw_parts, ctx->n_tw_parts);
-  }
   if (nl > 0)
     k_ph_dig<Out><<<nl, PH_THREADS, ctx->ph_large_smem, s>>>(ctx->d, ctx->ctl, items, ctx->ph_exps, nl, 0, 0, ctx->ph_src,
                                                              ctx->ph_wf, ctx->ph_v1, quad, xq);
@@ -961,8 +1003,8 @@ static void launch_ph_dig(pnm_ctx* ctx, bool linear, cudaStream_t s, cudaStream_
 
 // FP64 ph term (linear: without the quadratic part), and the same with its results as FP32 pairs
 // in the 8-byte slots of the FP64 Q (the refinement sweeps with FP32-pair contractions).
-// s_tiny: the stream of the smallest channels, which wait for no digits (a captured update runs them
-// beside the two passes over the amplitudes; in a context without larger channels they keep s).
+// s_tiny: the stream of the smallest channels (beside larger ones a stream of their own; in a context
+// without larger channels they keep s).
 void launch_ph64(pnm_ctx* ctx, cudaStream_t s, cudaStream_t s_tiny, bool linear) {
   launch_ph_dig<double>(ctx, linear, s, s_tiny);
 }

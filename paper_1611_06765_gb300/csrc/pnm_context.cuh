@@ -68,9 +68,6 @@ struct pnm_ctx {
   long long* ph_v1 = nullptr;
   double* ph_fixed64 = nullptr;
   f2* ph_fixed_f2 = nullptr;  // the fixed operands of the smallest channels as element values
-  long* tw_lo = nullptr;                         // first amplitude of each system
-  int* tw_parts = nullptr;
-  int n_tw_parts = 1;
   size_t ph_large_smem = 0, ph_dig_smem = 0, ph_warp_smem = 0;
   f2* t_pair = nullptr;                          // FP32-pair copy of the current amplitudes
   int *grp_lo_d = nullptr, *grp_hi_d = nullptr;  // per system ranges of the update items

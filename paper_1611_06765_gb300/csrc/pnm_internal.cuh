@@ -105,9 +105,6 @@ struct DevState {
   unsigned long long *vdig, *tdig;
   long *ch_vd_off, *ch_td_off;
   int *ch_vexp, *texp;
-  // digit words of the current amplitudes and their exponent per system (digit ph term)
-  unsigned long long* twords;
-  int* sys_texp;
   double *den, *inv_den;  // eps_i + eps_j - eps_a - eps_b per amplitude, and its reciprocal
   // iteration state
   double *t0, *t1;       // double buffer, parity = iteration & 1

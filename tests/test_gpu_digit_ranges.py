@@ -1,0 +1,86 @@
+"""The ph term of FP64 accuracy on amplitudes of very different size: every cross channel has its own
+scale, so that what lies in one channel costs the others no accuracy, and a channel whose rows or
+columns lie too far apart for one scale is summed in FP64."""
+import numpy as np
+import pytest
+
+import spinflip
+from conftest import minnesota_params
+from inputs import random_amplitudes
+from oracle import channel
+
+pytestmark = pytest.mark.gpu
+
+# (neutrons, protons, density, n2max) with channels of more than eight rows, S_z = 0 and S_z > 0
+SYSTEMS = [(38, 0, 0.12, 10), (66, 0, 0.16, 14), (14, 14, 0.16, 6)]
+# two chained sums of at most 33 products and the four terms of an amplitude: 70 roundings of 2^-53, and of
+# 2^-47 where pairs of 48 bits are summed
+TOL, TOL_PAIR = 1e-14, 5e-13
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    from paper_1611_06765_gb300 import build
+    build.build()
+    import paper_1611_06765_gb300 as P
+    return P
+
+
+class Case:
+    """A system, random flip-symmetric amplitudes with one of them scaled by `factor`, and which cross
+    channels that one is in."""
+
+    def __init__(self, pkg, N, Z, rho, n2, factor):
+        P = minnesota_params()
+        self.g = pkg.Context(N, rho, n2, params=P, Z=Z) if Z else pkg.Context(N, rho, n2, params=P)
+        self.o = channel.OracleSystem(N, rho, n2, P, Z=Z)
+        lab, st = self.g.amplitude_labels(), self.o.states()
+        perm = spinflip.flip_permutation(lab, st)
+        self.even = spinflip.symmetrise(random_amplitudes(len(lab), seed=9), perm)
+        # one amplitude between states of the two channels every pair of states has: in the middle
+        big = len(lab) // 3
+        both = np.unique([big, perm[0][big]])
+        self.t = self.even.copy()
+        self.t[both] *= factor
+        # keys of the four cross channels that each amplitude is an element of and reads from
+        a, b, i, j = lab.T
+        diff = np.stack([st[p] - st[h] for p, h in ((a, i), (a, j), (b, i), (b, j))], axis=1)
+        self.sz0 = diff[:, :, 3] == 0
+        self.key = np.ravel_multi_index(tuple((diff + 32).reshape(-1, diff.shape[2]).T), (65,) * diff.shape[2])
+        _, self.key = np.unique(self.key, return_inverse=True)
+        self.key = self.key.reshape(len(lab), 4)
+        self.far = ~np.isin(self.key, np.unique(self.key[both]))  # channels without the scaled amplitude
+
+    def tolerance(self, bound):
+        """Per amplitude, in units of the relative error: its own sum of absolute products, of channels
+        without the scaled amplitude the largest such sum in them (the scale of their digits), and of
+        S_z = 0 channels with it the largest of all (they are formed from sums and differences of two
+        blocks)."""
+        apart = self.far.all(axis=1)
+        top = np.zeros(self.key.max() + 1)
+        np.maximum.at(top, self.key[apart].ravel(), np.repeat(bound[apart], 4))
+        return bound + np.where(self.far, top[self.key], np.where(self.sz0, bound.max(), 0.0)).sum(axis=1)
+
+
+@pytest.mark.parametrize("N,Z,rho,n2", SYSTEMS)
+@pytest.mark.parametrize("factor", [2.0 ** 10, 2.0 ** 20, 2.0 ** 53])
+def test_one_dominant_amplitude(pkg, N, Z, rho, n2, factor):
+    c = Case(pkg, N, Z, rho, n2, factor)
+    ref, bound = c.o.ph_apply(c.t), c.o.ph_apply(c.t, absval=True)
+    tol = c.tolerance(bound)
+    assert np.count_nonzero(c.far.all(axis=1)) > len(ref) // 2
+    assert np.all(np.abs(c.g.apply_ph_term(c.t) - ref) <= TOL * tol)
+    assert np.all(np.abs(c.g.apply_ph_term(c.t, precision=pkg.PNM_PREC_F32PAIR) - ref) <= TOL_PAIR * tol)
+    c.g.close()
+
+
+@pytest.mark.parametrize("N,Z,rho,n2", SYSTEMS)
+def test_infinite_amplitude_stays_in_its_channels(pkg, N, Z, rho, n2):
+    """The channels without it give the same bits whatever its value."""
+    c = Case(pkg, N, Z, rho, n2, np.inf)
+    apart = c.far.all(axis=1)
+    for prec in (pkg.PNM_PREC_FP64, pkg.PNM_PREC_F32PAIR):
+        r, plain = c.g.apply_ph_term(c.t, precision=prec), c.g.apply_ph_term(c.even, precision=prec)
+        assert np.array_equal(r[apart], plain[apart])
+        assert not np.all(np.isfinite(r[~apart])) and np.all(np.isfinite(plain))
+    c.g.close()
