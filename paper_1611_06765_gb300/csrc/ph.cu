@@ -342,12 +342,15 @@ void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* 
 //   - T gathered as FP64 and converted in place to words of the channel's exponent (sums and
 //     differences of S_z = 0 as exact integer sums), two neighbouring columns interleaved: the k index
 //     of the second product; the first reads its k pairs across rows;
-//   - C as integers, the two terms aligned to the coarser of their units (2^-60 of their bounds or
-//     finer), its digits stored interleaved by row pairs straight from the first product's registers.
+//   - C as integers, the two terms rounded to the coarser of their units: <kb|v|cj> 2^-61 of its largest,
+//     the product 2^-60 of what its sum of R products can reach.  Its digits are stored interleaved by row
+//     pairs straight from the first product's registers.
 // An integer holds an element within PH_SPAN octaves of its operand's largest one to its last bit, and a
 // smaller one to 2^-61 of that largest.  FP64 sums round at 2^-53 of the products they add, so the digits
 // stand in for them only where no row or column of T, W or <kb|v|cj> lies wholly further down: a channel
-// with such a row or column (one amplitude far above the others, say) is summed in FP64 (ph_values).
+// with such a row or column (one amplitude far above the others, say) is summed in FP64 (ph_values), and
+// so is one whose product's unit is more than PH_SPAN octaves above that of <kb|v|cj> (amplitudes above
+// about 10) while T has an empty column, where <kb|v|cj> stands alone.
 // MBPT2 amplitudes and the Minnesota interaction stay within it (N = 14 to 66, densities 0.02 to 0.3:
 // rows of T within 6 octaves of their channel's largest, rows of W within 5, of <kb|v|cj> 0).
 // Only the results leave as floating point.  A group of 32 threads (channels of at most PH_WARP_DIM
@@ -378,6 +381,7 @@ struct PhMarks {
   __device__ void set(int k, int size, int least) const {
     if (size > 0) at[size >= least ? k : 2 * n + k] = 1;
   }
+  __device__ bool empty(int k) const { return !at[k] && !at[2 * n + k]; }
   // whether one of four rows or columns holds small elements only
   __device__ bool low(int k4) const {
     const unsigned* m = reinterpret_cast<const unsigned*>(at);
@@ -542,13 +546,21 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
       }
     }
   }
+  // units of C's terms (p1 with the factor 1/2), head bits finer than the product's digits allow for any R:
+  // sums of R products of 61-bit (62 bits each for sums and differences) integers within 2^60, <kb|v|cj>
+  // within 2^62, so that the leading digit of C stays within 82
+  const int head = max(0, __clz(R - 1) - 24 - 2 * (NM - 1));
+  const int p1 = dig_power(ex.x, et) + 14 - head - 1, pv = ex.y - 1022 - 61;
+  const int pc = quad ? max(p1, pv) : pv, sx = min(pc - p1, 63), sv = min(pc - pv, 63);
+  const long long rx = (1ll << sx) >> 1, rv = (1ll << sv) >> 1;  // half a unit
+  const int rl = (1 << (14 - head)) >> 1;
   group_sync<GT>();
-  const bool low = tid < mark.n / 2 && mark.low(tid);  // known to the group after the first product
+  bool low = tid < mark.n / 2 && mark.low(tid);  // known to the group after the first product
+  if (sv > PH_SPAN)
+    for (int k = tid; k < H; k += GT) low = low || mark.empty(mark.n + k);
   // C: 16 x 8 blocks of every problem; the fragments of W are requested one step ahead, across
   // blocks too
   const int nt = H8 / 8, sc = (H + 15) >> 4, kr = (R + 15) >> 4, blocks = NM * sc * nt;
-  const int p1 = dig_power(ex.x, et) + 14 - 1, pv = ex.y - 1022 - 61;  // units of the two terms (factor 1/2)
-  const int pc = quad ? max(p1, pv) : pv, sx = min(pc - p1, 63), sv = min(pc - pv, 63);
   const bool small_r = R <= DIG_SMALL_K, small_h = H <= DIG_SMALL_K;
   uint4 w[4];
   auto load_w = [&](int b, int ks) {  // block b is strip b / nt of the problems' strips in turn
@@ -562,7 +574,8 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
     const longlong2* __restrict__ vp =
         reinterpret_cast<const longlong2*>(v1 + it.v1) + (((long)ms * 16 + g) * H8 + n0) / 2 + q;
     const longlong2 va = __ldg(vp), vb = __ldg(vp + 4 * H8);
-    dig_t c[4] = {(dig_t)(va.x >> sv), (dig_t)(va.y >> sv), (dig_t)(vb.x >> sv), (dig_t)(vb.y >> sv)};
+    dig_t c[4] = {(dig_t)((va.x + rv) >> sv), (dig_t)((va.y + rv) >> sv), (dig_t)((vb.x + rv) >> sv),
+                  (dig_t)((vb.y + rv) >> sv)};
     if (quad) {
       float acc[DIG_LEVELS][4] = {};
       const uint4* tb = Ts + m * TP + (2 * q) * TS + ((n0 + g) >> 1);
@@ -581,7 +594,7 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
 #pragma unroll
       for (int k = 0; k < 4; k++) {
         const DigSum x = small_r ? dig_drain_small(acc, k) : dig_drain(acc, k);
-        c[k] += (dig_t)(((x.hi << 18) + (x.lo >> 14)) >> sx);  // 2^-54 of the maxima's product or finer
+        c[k] += (dig_t)(((x.hi << (18 + head)) + ((x.lo + rl) >> (14 - head)) + rx) >> sx);
       }
     }
     // digits of the row pairs (g, g ^ 1): the lanes of even g take the block's even columns

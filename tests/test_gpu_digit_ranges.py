@@ -84,3 +84,21 @@ def test_infinite_amplitude_stays_in_its_channels(pkg, N, Z, rho, n2):
         assert np.array_equal(r[apart], plain[apart])
         assert not np.all(np.isfinite(r[~apart])) and np.all(np.isfinite(plain))
     c.g.close()
+
+
+@pytest.mark.parametrize("N,Z,rho,n2", SYSTEMS)
+@pytest.mark.parametrize("alone", [False, True])
+def test_large_amplitudes(pkg, N, Z, rho, n2, alone):
+    """Amplitudes of a million, where the quadratic part is far above <kb|v|cj>, and one of 1e10 with zeros
+    for the others, which meets <kb|v|cj> by itself."""
+    c = Case(pkg, N, Z, rho, n2, 1.0)
+    one, k = np.zeros_like(c.even), len(c.even) // 3
+    idx, sign = spinflip.flip_permutation(c.g.amplitude_labels(), c.o.states())
+    one[k] = 1e10
+    one[idx[k]] = sign[k] * 1e10
+    t = one if alone else 1e6 * c.even
+    ref, bound = c.o.ph_apply(t), c.o.ph_apply(t, absval=True)
+    tol = bound + (np.where(~c.far & c.sz0, bound.max(), 0.0).sum(axis=1) if alone else 0.0)
+    assert np.all(np.abs(c.g.apply_ph_term(t) - ref) <= TOL * tol)
+    assert np.all(np.abs(c.g.apply_ph_term(t, precision=pkg.PNM_PREC_F32PAIR) - ref) <= TOL_PAIR * tol)
+    c.g.close()
