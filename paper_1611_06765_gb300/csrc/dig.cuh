@@ -66,16 +66,18 @@ __device__ __forceinline__ double dig_to_double(long long s, int p) {
   return __longlong_as_double((long long)((((dig_t)(e - 1)) << 52) + m) | (s & (long long)0x8000000000000000ull));
 }
 
-// s 2^p as an FP32 pair: the 48 leading bits.
+// s 2^p as an FP32 pair: rounded to 24 bits, and the rest to 24 more.
 __device__ __forceinline__ f2 dig_to_f2(long long s, int p) {
   if (s == 0) return f2{0.0f, 0.0f};
   const dig_t a = s < 0 ? (dig_t)0 - (dig_t)s : (dig_t)s;
   const int z = __clzll((long long)a);
   const dig_t m = a << z;
-  auto scaled = [](unsigned v, int e) {  // v 2^e, v < 2^24
-    return e < -126 ? 0.0f : __uint2float_rn(v) * __int_as_float((min(e, 127) + 127) << 23);
+  auto scaled = [](float v, int e) {  // v 2^e
+    return e < -126 ? 0.0f : v * __int_as_float((min(e, 127) + 127) << 23);
   };
-  const float h = scaled((unsigned)(m >> 40), p - z + 40), l = scaled((unsigned)(m >> 16) & 0xffffffu, p - z + 16);
+  const unsigned top = (unsigned)(m >> 40) + (unsigned)((m >> 39) & 1);
+  const long long rest = (long long)(m - ((dig_t)top << 40));  // within 2^39; top 2^24 wraps around
+  const float h = scaled(__uint2float_rn(top), p - z + 40), l = scaled(__int2float_rn((int)(rest >> 8)), p - z + 8);
   return s < 0 ? f2{-h, -l} : f2{h, l};
 }
 

@@ -102,3 +102,15 @@ def test_large_amplitudes(pkg, N, Z, rho, n2, alone):
     assert np.all(np.abs(c.g.apply_ph_term(t) - ref) <= TOL * tol)
     assert np.all(np.abs(c.g.apply_ph_term(t, precision=pkg.PNM_PREC_F32PAIR) - ref) <= TOL_PAIR * tol)
     c.g.close()
+
+
+@pytest.mark.parametrize("N,Z,rho,n2", SYSTEMS)
+def test_pair_results_are_rounded(pkg, N, Z, rho, n2):
+    """The ladder's sums are the same integers for both result types: a pair of FP32 numbers, rounded to 24
+    bits and the rest to 24 more, is within 2^-49 of them, an FP64 number within 2^-53."""
+    P = minnesota_params()
+    g = pkg.Context(N, rho, n2, params=P, Z=Z) if Z else pkg.Context(N, rho, n2, params=P)
+    t = random_amplitudes(len(g.amplitude_labels()), seed=13)
+    r, pair = g.apply_pp_ladder(t), g.apply_pp_ladder(t, precision=pkg.PNM_PREC_F32PAIR)
+    assert np.any(r) and np.all(np.abs(pair - r) <= 2.0 ** -48 * np.abs(r))
+    g.close()
