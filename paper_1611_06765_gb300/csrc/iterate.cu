@@ -571,13 +571,17 @@ __device__ void finalize_system(const FinArgs& f, LoopCtl* ctl, int s, int ctas)
   f.blocks_done[s] = 0;
   bool bad = finalize_one(f, S, c, s, e, r), all_done = S.done;
   if (f.nsys > 1) {
-    // systems closed, converged and diverged, counted in 21 bits each
-    const unsigned long long one = 1ull | (unsigned long long)(S.done != 0) << 21 | (unsigned long long)bad << 42;
-    const unsigned long long now = atomicAdd(&ctl->closed, one) + one;
-    if ((now & 0x1fffff) != (unsigned)f.nsys) return;
+    if (bad) {  // before this system is counted
+      atomicExch(&ctl->bad, 1);
+      __threadfence();
+    }
+    const unsigned long long one = UpdCount::one(S.done != 0);
+    const UpdCount now{atomicAdd(&ctl->closed, one) + one};
+    if (now.finished() != (unsigned)f.nsys) return;
     ctl->closed = 0;
-    all_done = (now >> 21 & 0x1fffff) == (unsigned)f.nsys;
-    bad = now >> 42 != 0;
+    all_done = now.converged() == (unsigned)f.nsys;
+    __threadfence();
+    bad = atomicExch(&ctl->bad, 0) != 0;
   }
   ctl->iter = c.iter + 1;
   int cont = 1;

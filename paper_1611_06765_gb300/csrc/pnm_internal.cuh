@@ -139,7 +139,17 @@ struct LoopCtl {
   int min_iter;      // no system counts as converged before this many updates
   int skip_done;     // 1 inside the solve loop: kernels skip the work of converged systems
   double alpha;
-  unsigned long long closed;  // systems whose last CTA of the current update has finished (finalize_system)
+  unsigned long long closed;  // systems whose last CTA of the current update has finished (UpdCount)
+  int bad;                    // one of them has diverged
+};
+
+// Systems of a batch that have finished the current update and, of these, those that have converged: 32
+// bits each, counted together by atomic additions of one().
+struct UpdCount {
+  unsigned long long v;
+  __host__ __device__ static unsigned long long one(bool done) { return 1ull | (unsigned long long)done << 32; }
+  __host__ __device__ unsigned finished() const { return (unsigned)v; }
+  __host__ __device__ unsigned converged() const { return (unsigned)(v >> 32); }
 };
 
 // Run-time parameters of a whole-solve graph, copied from pinned host memory by its first node.

@@ -1,0 +1,47 @@
+"""Host-side rules of the library's headers, compiled into a small program and run here (no GPU)."""
+import os
+import subprocess
+
+import pytest
+
+from conftest import ROOT
+from paper_1611_06765_gb300 import build
+
+PROGRAM = r"""
+#include <cstdio>
+#include "pnm_internal.cuh"
+
+static int failed = 0;
+#define CHECK(x) do { if (!(x)) { std::printf("line %d: %s\n", __LINE__, #x); failed = 1; } } while (0)
+
+// n systems finish an update, c of them converged: the count is complete after the last one only
+static void counts(unsigned long long n, unsigned long long c) {
+  const UpdCount all{(n - c) * UpdCount::one(false) + c * UpdCount::one(true)};
+  CHECK(all.finished() == n && all.converged() == c);
+  const UpdCount before{all.v - UpdCount::one(c == n)};
+  CHECK(before.finished() == n - 1);
+}
+
+int main() {
+  for (unsigned long long n : {2ull, 3ull, (1ull << 21) - 1, 1ull << 21, (1ull << 21) + 5, (1ull << 31) - 1})
+    for (unsigned long long c : {0ull, 1ull, n - 1, n}) counts(n, c);
+  return failed;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    src, exe = str(d / "rules.cu"), str(d / "rules")
+    open(src, "w").write(PROGRAM)
+    cmd = [build.nvcc()] + build.ARCH + ["-std=c++17", "--expt-relaxed-constexpr", "-cudart", "static", "-I" + build.CSRC,
+                                         "-I" + os.path.join(ROOT, "include"), src, "-o", exe]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return exe
+
+
+def test_rules(program):
+    r = subprocess.run([program], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
