@@ -1393,7 +1393,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
     }
     S.x_end = x;
   }
-  if (t_acc >= (1L << 31) - 2 || xt_full >= (1L << 31) - 2)
+  if (!fits_maps(t_acc, xt_full, xt_acc, xc_acc))
     throw PnmError{PNM_EINVAL, "problem too large for 32-bit element maps"};
   const int nrows = (int)h_rows.size();
   ctx->nch = C;

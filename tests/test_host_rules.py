@@ -22,7 +22,19 @@ static void counts(unsigned long long n, unsigned long long c) {
   CHECK(before.finished() == n - 1);
 }
 
+// no size that a 32-bit map indexes may pass it
+static void maps() {
+  const long ok = (1L << 31) - 3, over = (1L << 31) - 2;
+  CHECK(fits_maps(ok, ok, ok, ok) && fits_maps(0, 0, 0, 0));
+  CHECK(!fits_maps(over, 1, 1, 1) && !fits_maps(1, over, 1, 1) && !fits_maps(1, 1, over, 1) && !fits_maps(1, 1, 1, over));
+  // S_z > 0 channels of one row and one column (two states of a shell): one element each, a row of
+  // formed_width(1) as laid out; 2^30 of them have 2^30 elements and 2^32 as laid out
+  const long channels = 1L << 30;
+  CHECK(fits_maps(1, channels, 1, 1) && !fits_maps(1, channels, channels * formed_width(1), channels * formed_width(1)));
+}
+
 int main() {
+  maps();
   for (unsigned long long n : {2ull, 3ull, (1ull << 21) - 1, 1ull << 21, (1ull << 21) + 5, (1ull << 31) - 1})
     for (unsigned long long c : {0ull, 1ull, n - 1, n}) counts(n, c);
   return failed;
