@@ -122,11 +122,11 @@ struct DevState {
 __host__ __device__ __forceinline__ int formed_width(int H) { return (H + 3) & ~3; }
 
 // Whether 32-bit maps reach every element of a context: its amplitudes, and the cross-channel matrices in
-// full and as they are laid out (formed T and <kb|v|cj>, whose padding can be the larger part where
-// channels have one or two columns).
+// full and as they are laid out, whose padding can be the larger part where channels have one or two
+// columns (signed positions in T, unsigned offsets of <kb|v|cj>).
 inline bool fits_maps(long nt, long full, long formed_t, long formed_v1) {
   const long most = (1L << 31) - 2;
-  return nt < most && full < most && formed_t < most && formed_v1 < most;
+  return nt < most && full < most && formed_t < most && formed_v1 < 2 * most;
 }
 
 // Work item of the pp ladder in digits: a strip of 16 ladder vectors and a pass over up to 8 hole

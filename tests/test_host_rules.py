@@ -26,7 +26,7 @@ static void counts(unsigned long long n, unsigned long long c) {
 static void maps() {
   const long ok = (1L << 31) - 3, over = (1L << 31) - 2;
   CHECK(fits_maps(ok, ok, ok, ok) && fits_maps(0, 0, 0, 0));
-  CHECK(!fits_maps(over, 1, 1, 1) && !fits_maps(1, over, 1, 1) && !fits_maps(1, 1, over, 1) && !fits_maps(1, 1, 1, over));
+  CHECK(!fits_maps(over, 1, 1, 1) && !fits_maps(1, over, 1, 1) && !fits_maps(1, 1, over, 1) && !fits_maps(1, 1, 1, 2 * over) && fits_maps(1, 1, 1, over));
   // S_z > 0 channels of one row and one column (two states of a shell): one element each, a row of
   // formed_width(1) as laid out; 2^30 of them have 2^30 elements and 2^32 as laid out
   const long channels = 1L << 30;
