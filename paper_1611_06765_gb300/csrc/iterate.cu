@@ -1282,15 +1282,9 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   ctx->sysctl = (SysCtl*)dmalloc(ctx, sizeof(SysCtl) * nsys);
   CUDA_TRY(cudaMemsetAsync(ctx->sysctl, 0, sizeof(SysCtl) * nsys, s));
   ctx->d.sysctl = ctx->sysctl;
-  // three 8-byte matrices of the largest cross channel (of its half-size problems for S_z = 0) and
-  // index tables, in tiles of four: the size limit of a context
-  size_t ph_staged = 0;
-  for (int x = 0; x < ctx->nx; x++) {
-    const int nm = ctx->h_x_cls[x] == 0 ? 2 : 1, d = std::max(ctx->h_x_nph[x], ctx->h_x_nhp[x]) / nm;
-    const size_t m4 = (d + 3) & ~3;
-    if (ctx->h_x_cls[x] >= 0 && d > 16) ph_staged = std::max(ph_staged, 4 * m4 * sizeof(int) + sizeof(double) * 3 * nm * m4 * m4);
-  }
-  if (ph_staged > 227 * 1024 || max_nlad > PP_MAX_NLAD)
+  bool fits = max_nlad <= PP_MAX_NLAD;
+  for (int x = 0; x < ctx->nx; x++) fits = fits && ph_fits(ctx->h_x_nph[x], ctx->h_x_nhp[x], ctx->h_x_cls[x]);
+  if (!fits)
     throw PnmError{PNM_EINVAL, "channel too large for the shared-memory tiles"};
   for (int k = 0; k < 2; k++) {
     CUDA_TRY(cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking));

@@ -47,7 +47,7 @@ __device__ __forceinline__ void copy16(void* dst, const void* src) {
 
 // ------------------------------------------------------------------------------ FP32
 // Shared memory of a group: T, W and C of every problem, rows padded to the 4 x 4 register tiles.
-__host__ __device__ __forceinline__ size_t ph32_smem(int R, int H, int nm) {
+__host__ __device__ __forceinline__ constexpr size_t ph32_smem(int R, int H, int nm) {
   const int R4 = (R + 3) & ~3, H4 = formed_width(H);
   return sizeof(float) * nm * ((size_t)2 * R4 * H4 + (size_t)H4 * H4);
 }
@@ -361,17 +361,23 @@ void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* 
 // update of 330 (N = 66, n^2 <= 42; third-order sums of three densities of n^2 <= 36: 485, 515 us) but left
 // a channel far below the system's largest amplitude as few bits (relative errors of 5e-6 beside one
 // amplitude 2^20 above the others).
-__host__ __device__ __forceinline__ int ph_h8(int H) { return (H + 7) & ~7; }
+__host__ __device__ __forceinline__ constexpr int ph_h8(int H) { return (H + 7) & ~7; }
 // Row strides in 16-byte pairs: T's odd, C's 2 modulo 8, so that the fragment loads of the first
 // product (two rows per thread) and of the second spread over the banks.
-__host__ __device__ __forceinline__ int ph_ts(int H) { return ph_h8(H) / 2 + 1; }
-__host__ __device__ __forceinline__ int ph_cs(int H) { return ph_h8(H) + 2; }
-__host__ __device__ __forceinline__ size_t ph_dig_smem(int R, int H, int nm) {
+__host__ __device__ __forceinline__ constexpr int ph_ts(int H) { return ph_h8(H) / 2 + 1; }
+__host__ __device__ __forceinline__ constexpr int ph_cs(int H) { return ph_h8(H) + 2; }
+__host__ __device__ __forceinline__ constexpr size_t ph_dig_smem(int R, int H, int nm) {
   return sizeof(uint4) * nm * ((size_t)ph_h8(R) * ph_ts(H) + (size_t)(ph_h8(H) / 2) * ph_cs(H));
 }
+// beside the static shared memory of the kernels
+constexpr size_t PH_SMEM = 227 * 1024 - 2048;
+static_assert(ph_dig_smem(PH_LIMIT_ONE, PH_LIMIT_ONE, 1) <= PH_SMEM && ph_dig_smem(PH_LIMIT_TWO, PH_LIMIT_TWO, 2) <= PH_SMEM &&
+                  ph32_smem(PH_LIMIT_ONE, PH_LIMIT_ONE, 1) <= PH_SMEM && ph32_smem(PH_LIMIT_TWO, PH_LIMIT_TWO, 2) <= PH_SMEM,
+              "a channel's tiles would not fit an SM");
 
 constexpr int PH_SPAN = 8;
-constexpr int PH_MAX_DIM = 128;  // rows or columns of a problem (PhMarks)
+constexpr int PH_MAX_DIM = DIG_FLUSH;  // rows or columns of a problem: the products drain once, at their end
+static_assert(PH_LIMIT_ONE <= PH_MAX_DIM && PH_LIMIT_TWO <= PH_MAX_DIM, "digit sums would not be exact");
 
 // Which rows and columns of a matrix hold an element within PH_SPAN octaves of the largest (big), which a
 // smaller one other than zero (some): bytes that any thread may set, rows [0, n), columns [n, 2 n).

@@ -119,7 +119,7 @@ struct DevState {
 };
 
 // Row stride of the formed matrices of a cross channel: 16-byte groups of FP32.
-__host__ __device__ __forceinline__ int formed_width(int H) { return (H + 3) & ~3; }
+__host__ __device__ __forceinline__ constexpr int formed_width(int H) { return (H + 3) & ~3; }
 
 // Whether 32-bit maps reach every element of a context: its amplitudes, and the cross-channel matrices in
 // full and as they are laid out, whose padding can be the larger part where channels have one or two
@@ -211,7 +211,8 @@ struct FinArgs {
 };
 
 // The update kernels: threads of a CTA, CTAs of the mixed update per SM at least, CTAs per SM above
-// which a warp takes more than one chunk; channels may hold at most UPD_MAX_NHH hole pairs.  The
+// which a warp takes more than one chunk.  Contexts with more than UPD_MAX_NHH hole pairs in a channel are
+// refused: no kernel relies on it, but none has been run beyond it.  The
 // PNM_UPD_* macros override the tuning constants at build time.
 #ifndef PNM_UPD_MIN_BLOCKS
 #define PNM_UPD_MIN_BLOCKS 7
@@ -223,6 +224,16 @@ constexpr int UPD_THREADS = 128, UPD_MAX_NHH = 128;
 constexpr int UPD_MIN_BLOCKS = PNM_UPD_MIN_BLOCKS, UPD_FULL = PNM_UPD_FULL;
 
 constexpr int PH_THREADS = 128;  // threads of a ph-term CTA
+
+// Largest dimension of a problem of the ph term: of an S_z > 0 channel, and of the half-size problems of an
+// S_z = 0 one.  Contexts with larger channels are refused at creation.  The kernels rely on it: sums of
+// digit products are exact up to 128 rows or columns, and a channel's tiles have to fit the shared memory
+// of an SM (asserted in ph.cu).
+constexpr int PH_LIMIT_ONE = 96, PH_LIMIT_TWO = 68;
+__host__ __device__ constexpr bool ph_fits(int nph, int nhp, int cls) {
+  const int d = nph > nhp ? nph : nhp;
+  return cls < 0 || (cls == 0 ? d / 2 <= PH_LIMIT_TWO : d <= PH_LIMIT_ONE);
+}
 
 // pp ladder of amplitude (ij, ab) of channel c from its ladder-layout value (planes summed by
 // the caller where there are several).

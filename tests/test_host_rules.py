@@ -33,7 +33,20 @@ static void maps() {
   CHECK(fits_maps(1, channels, 1, 1) && !fits_maps(1, channels, channels * formed_width(1), channels * formed_width(1)));
 }
 
+// the channels that have always been refused: three 8-byte matrices per problem, in tiles of four, and
+// index tables past 227 KB
+static void channels() {
+  for (int cls = -1; cls <= 1; cls++)
+    for (int d = 1; d <= 300; d++) {
+      const int nm = cls == 0 ? 2 : 1, h = d / nm;
+      const size_t m4 = (h + 3) & ~3, staged = 4 * m4 * sizeof(int) + sizeof(double) * 3 * nm * m4 * m4;
+      const bool refused = cls >= 0 && h > 16 && staged > 227 * 1024;
+      CHECK(ph_fits(d, 1, cls) == !refused && ph_fits(1, d, cls) == !refused);
+    }
+}
+
 int main() {
+  channels();
   maps();
   for (unsigned long long n : {2ull, 3ull, (1ull << 21) - 1, 1ull << 21, (1ull << 21) + 5, (1ull << 31) - 1})
     for (unsigned long long c : {0ull, 1ull, n - 1, n}) counts(n, c);
