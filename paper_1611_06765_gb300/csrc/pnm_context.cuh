@@ -138,13 +138,17 @@ struct pnm_ctx {
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 };
 
-// Autotuner cache key: device and the (N, n2max) of every system, which fix all channel
-// sizes (the density only rescales values).
+// Autotuner cache key: device and, of every system, what fixes its channels (the density only rescales
+// values): neutrons, protons, n2max, and whether it is twisted.  Twists move channels about but leave
+// their sizes alike, so the systems of a twist average share an entry.
 inline std::string pnm_shape_key(const pnm_ctx* ctx) {
   int dev = 0;
   cudaGetDevice(&dev);
   std::string k = "dev" + std::to_string(dev);
-  for (const SysInfo& S : ctx->sys) k += ";" + std::to_string(S.N) + "," + std::to_string(S.n2max);
+  for (const SysInfo& S : ctx->sys) {
+    k += ";" + std::to_string(S.N - S.Z) + "," + std::to_string(S.Z) + "," + std::to_string(S.n2max);
+    if (S.phi[0] != 0.0 || S.phi[1] != 0.0 || S.phi[2] != 0.0) k += "t";
+  }
   return k;
 }
 

@@ -9,7 +9,7 @@ from paper_1611_06765_gb300 import build
 
 PROGRAM = r"""
 #include <cstdio>
-#include "pnm_internal.cuh"
+#include "pnm_context.cuh"
 
 static int failed = 0;
 #define CHECK(x) do { if (!(x)) { std::printf("line %d: %s\n", __LINE__, #x); failed = 1; } } while (0)
@@ -45,7 +45,27 @@ static void channels() {
     }
 }
 
+// contexts whose channels differ do not share what the autotuners measured; densities and twists do
+static std::string key(int n, int z, int n2max, double rho, double phi) {
+  pnm_ctx c;
+  c.sys.resize(1);
+  c.sys[0].N = n + z;
+  c.sys[0].Z = z;
+  c.sys[0].n2max = n2max;
+  c.sys[0].rho = rho;
+  for (double& p : c.sys[0].phi) p = 0.0;
+  c.sys[0].phi[1] = phi;
+  return pnm_shape_key(&c);
+}
+static void keys() {
+  const std::string k = key(14, 0, 20, 0.08, 0.0);
+  CHECK(k == key(14, 0, 20, 0.16, 0.0) && key(14, 0, 20, 0.08, 0.1) == key(14, 0, 20, 0.08, 0.3));
+  CHECK(k != key(14, 0, 20, 0.08, 0.1) && k != key(0, 14, 20, 0.08, 0.0) && k != key(7, 7, 20, 0.08, 0.0));
+  CHECK(k != key(14, 0, 21, 0.08, 0.0) && k != key(38, 0, 20, 0.08, 0.0));
+}
+
 int main() {
+  keys();
   channels();
   maps();
   for (unsigned long long n : {2ull, 3ull, (1ull << 21) - 1, 1ull << 21, (1ull << 21) + 5, (1ull << 31) - 1})
