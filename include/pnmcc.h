@@ -396,7 +396,8 @@ int pnm_kernel_stats(const pnm_ctx *ctx, int id, const char **name, double *tota
  * measured microseconds per launch.  Schedule autotuner (run at the first solve of each
  * precision): serial_mask bit 0 / bit 1 / bit 4 set when the FP64 update / the mixed update /
  * the refinement update with FP32-pair contractions runs on one stream instead of three
- * concurrent ones; bit 2 / bit 3 / bit 5 set while that mode is not tuned yet.
+ * concurrent ones; bit 2 / bit 3 / bit 5 set while that mode is not tuned (before its first solve, or
+ * where the updates to be timed diverge from the MBPT2 start).
  * Any output may be NULL; PNM_EINVAL (after writing serial_mask) before the first
  * mixed-precision solve. */
 int pnm_get_tuning(const pnm_ctx *ctx, int *ksplit, int *stages, float *us, int *serial_mask);

@@ -1915,8 +1915,10 @@ void pnm_flip_copy_device(pnm_ctx* ctx) {
 // (concurrent with the one-body kernels) and a few with everything on one stream; keep the
 // faster for this precision mode.  Where concurrent mixed updates take SCHED_ORDER_US or more, the
 // orders of pnm_enqueue_body_mixed are timed too, as a graph with the priorities of the solve's (shorter
-// updates gain nothing, and launches from the host would blur the difference).  The held amplitudes
-// are saved and restored.
+// updates gain nothing, and launches from the host would blur the difference).  The updates start from
+// MBPT2, whatever is held (saved and restored): kernels skip their work once an iteration has ended, so the
+// times of updates that diverge at once say nothing.  Where they do so from MBPT2 too (an interaction
+// without a solution) the context keeps the concurrent schedule, untuned, and nothing is kept for the shape.
 constexpr float SCHED_ORDER_US = 150.0f;
 static std::mutex g_sched_mu;
 static std::map<std::string, int> g_sched_cache;  // (shape key, mode) -> one stream (-1), or the order
@@ -1958,7 +1960,7 @@ static float time_body_graph(pnm_ctx* ctx, int mode, cudaEvent_t e0, cudaEvent_t
 void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
   const bool pair = ((mode >> 8) & 1) != 0;
   int m = (mode & 15) == PNM_PREC_FP64 ? (pair ? 2 : 0) : 1;
-  if (ctx->sched_tuned[m]) return;
+  if (ctx->sched_tuned[m] || ctx->sched_ended[m]) return;
   if (m == 0) pnm_need_digits(ctx);
   const std::string key = pnm_shape_key(ctx) + (m == 1 ? "|mixed" : m == 2 ? "|pair" : "|fp64");
   {
@@ -1982,11 +1984,20 @@ void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
   CUDA_TRY(cudaEventCreate(&e1));
   float best = 1e30f;
   int best_serial = 0;
+  bool ended = false;
+  auto start = [&] {
+    pnm_start(ctx, PNM_INIT_MBPT2, never);
+    if (m == 1) pnm_mixed_pack_initial(ctx, alpha);
+  };
+  auto check = [&] {  // after a measurement
+    int status = 0;
+    CUDA_TRY(cudaMemcpyAsync(&status, &ctx->ctl->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+    ended = ended || status != 0;
+  };
   for (int serial = 0; serial < 2; serial++) {
     ctx->serial_sched[m] = serial != 0;
-    CUDA_TRY(cudaMemcpyAsync(ctx->d.t0, save, sizeof(double) * ctx->nt, cudaMemcpyDeviceToDevice, s));
-    pnm_start(ctx, PNM_INIT_KEEP, never);
-    if (m == 1) pnm_mixed_pack_initial(ctx, alpha);
+    start();
     pnm_enqueue_body(ctx, mode, 0, 0);
     CUDA_TRY(cudaEventRecord(e0, s));
     for (int k = 0; k < 4; k++) pnm_enqueue_body(ctx, mode, 0, 0);
@@ -1994,6 +2005,7 @@ void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
     CUDA_TRY(cudaEventSynchronize(e1));
     float ms = 0;
     CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
+    check();
     if (ms < best) {
       best = ms;
       best_serial = serial;
@@ -2005,10 +2017,9 @@ void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
     int order = 0;
     for (int k = 0; k < 3; k++) {
       ctx->mixed_order = k;
-      CUDA_TRY(cudaMemcpyAsync(ctx->d.t0, save, sizeof(double) * ctx->nt, cudaMemcpyDeviceToDevice, s));
-      pnm_start(ctx, PNM_INIT_KEEP, never);
-      pnm_mixed_pack_initial(ctx, alpha);
+      start();
       const float ms = time_body_graph(ctx, mode, e0, e1);
+      check();
       if (ms < 0.98f * fastest) {
         fastest = ms;
         order = k;
@@ -2018,8 +2029,12 @@ void pnm_tune_schedule(pnm_ctx* ctx, int mode, double alpha) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  ctx->sched_tuned[m] = true;
-  {
+  ctx->sched_ended[m] = ended;
+  if (ended) {
+    ctx->serial_sched[m] = false;
+    if (m == 1) ctx->mixed_order = 0;
+  } else {
+    ctx->sched_tuned[m] = true;
     std::lock_guard<std::mutex> lock(g_sched_mu);
     g_sched_cache[key] = ctx->serial_sched[m] ? -1 : (m == 1 ? ctx->mixed_order : 0);
   }

@@ -120,6 +120,7 @@ struct pnm_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
   bool serial_sched[3] = {false, false, false};  // per mode (0 FP64, 1 mixed, 2 FP32-pair refinement): one stream only
   bool sched_tuned[3] = {false, false, false};
+  bool sched_ended[3] = {false, false, false};  // the timed updates diverged: left untuned
   int mixed_order = 0;  // of a concurrent mixed update: what waits for the t tiles of the ladder (pnm_enqueue_body_mixed)
   int cur_mode = 0;
 
