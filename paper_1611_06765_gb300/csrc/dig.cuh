@@ -15,10 +15,12 @@
 //   - the levels are added in two 64-bit integers (every DIG_FLUSH products) and the result is
 //     rounded once, to its own leading bits (a sum cut at a fixed 2^-52 of the product of the maxima
 //     was further off than FP64 where the largest values do not meet).
-// Eight levels (36 digit products) drop terms below 2^-62 of the product of the two maxima; an
-// FP64 sum of K products rounds K times at 2^-53 of its partial sums.  Measured against 80- and
-// 128-bit sums: ladder N = 2, n^2 <= 9, largest error 7.0e-16 against 2.1e-15 in FP64 (scale 12.5);
-// ph term N = 38, n^2 <= 8, 5.8e-17 of the norm before the result's rounding against 1.6e-16.
+// Operands are cut (toward zero) at their last bit, and eight levels (36 of the 64 digit products) leave out
+// up to 2^-57 of the product of the two maxima per term, 2^-60 on average and of either sign; an FP64 sum of
+// K products rounds K times at 2^-53 of its partial sums.  These errors are relative to the operands' largest
+// elements: where all products of a sum are many octaves smaller, the kernels sum in FP64 (ph.cu PH_SPAN,
+// iterate.cu PP_FAR).  Measured from MBPT2 amplitudes, largest error of an element's own sum of absolute
+// products: ladder N = 66, n^2 <= 14, 2.8e-15 against 3.2e-15 in FP64; ph term 6.0e-16 against 1.1e-15.
 // Seven levels (28 products) drop terms below 2^-54, which left the FP32-pair results, whose 48 bits
 // would allow it, further from the exact ladder than FP32-pair arithmetic (1.8e-14 against 1.4e-14 of
 // the norm: the interaction spans many orders of magnitude, its maximum is far above its mean).
@@ -51,6 +53,9 @@ __device__ __forceinline__ long long dig_fixed(double x, int e) {
   const long long a = (m << 8) >> min(e - max(ex, 1), 63);
   return hi < 0 ? -a : a;
 }
+
+// The leading 16 bits of a magnitude among those an integer of its scale can have.
+__device__ __forceinline__ unsigned dig_top(long long x) { return (unsigned)((x < 0 ? -x : x) >> 46); }
 
 __device__ __forceinline__ dig_t dig_word(long long x) { return (dig_t)x + DIG_BIAS; }
 
@@ -94,15 +99,6 @@ __device__ __forceinline__ uint4 dig_interleave(dig_t w0, dig_t w1) {
   return make_uint4(__byte_perm(h0, h1, 0x6273), __byte_perm(h0, h1, 0x4051), __byte_perm(l0, l1, 0x6273),
                     __byte_perm(l0, l1, 0x4051));
 }
-// Element k (0, 1) of an interleaved pair.
-__device__ __forceinline__ dig_t dig_pick(uint4 v, int k) {
-  const uint32_t p[4] = {v.x, v.y, v.z, v.w};
-  dig_t w = 0;
-#pragma unroll
-  for (int j = 0; j < 8; j++) w = (w << 8) | ((p[j >> 1] >> (16 * (j & 1) + 8 * k)) & 0xffu);
-  return w;
-}
-
 // FP16 digits (two elements: low and high half) of an interleaved pair: out[j] is digit j from the
 // most significant.
 template <int COUNT>

@@ -167,13 +167,14 @@ __global__ void k_dchi(DevState D, int nsp_total) {
 // s(ij, q) = sum over the (one or two) pairs of vector q of sign * t(ij, pair) from the current
 // FP64 amplitudes, as digit words of the row's common exponent (dig.cuh), zero words in the
 // padding.  One CTA per (channel, ij) row of a channel with V_pppp.  A row that holds an infinity
-// or a NaN keeps its FP64 values instead of digits (exponent DIG_NONFINITE; the ladder kernel
-// then sums it in FP64).
+// or a NaN has the exponent DIG_NONFINITE (the ladder kernel then sums it in FP64).  s64: s itself too,
+// in the ladder layout, where the ladder checks its results (else null).
 constexpr int TDIG_THREADS = 128;
 __global__ void __launch_bounds__(TDIG_THREADS) k_tdig(DevState D, const LoopCtl* __restrict__ ctl,
-                                                       const int2* __restrict__ rows) {
+                                                       const int2* __restrict__ rows, double* __restrict__ s64) {
   extern __shared__ double ssum[];
   __shared__ int warp_max[TDIG_THREADS / 32];
+  __shared__ unsigned sh_top;
   const int2 it = rows[blockIdx.x];
   const int c = it.x, ij = it.y;
   if (sys_done(D, ctl, D.ch_sys[c])) return;
@@ -189,13 +190,16 @@ __global__ void __launch_bounds__(TDIG_THREADS) k_tdig(DevState D, const LoopCtl
       v += m.y > 0 ? b : -b;
     }
     ssum[q] = v;
+    if (s64) s64[D.ch_s_off[c] + (long)ij * nl + q] = v;
     e = max(e, dig_exp(v));
   }
   e = __reduce_max_sync(0xffffffffu, e);
   if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = e;
+  if (threadIdx.x == 0) sh_top = 0;
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < TDIG_THREADS / 32; w++) e = max(e, warp_max[w]);
+  unsigned top = 0;
   const int steps = (nl + 15) >> 4;
   uint4* o = reinterpret_cast<uint4*>(D.tdig + D.ch_td_off[c]) + (long)ij * steps * 16;
   if (threadIdx.x == 0) D.texp[D.ch_hh_off[c] + ij] = e;
@@ -209,18 +213,22 @@ __global__ void __launch_bounds__(TDIG_THREADS) k_tdig(DevState D, const LoopCtl
       const int q = k0 + (u & 1) + (u >> 1) * 8;
       v[u] = q < nl ? ssum[q] : 0.0;
     }
-    if (e < DIG_NONFINITE) {
-      uint32_t b0[8], b1[8];
-      dig_expand<8>(dig_interleave(dig_word(dig_fixed(v[0], e)), dig_word(dig_fixed(v[1], e))), b0);
-      dig_expand<8>(dig_interleave(dig_word(dig_fixed(v[2], e)), dig_word(dig_fixed(v[3], e))), b1);
+    long long x[4];
 #pragma unroll
-      for (int u = 0; u < 4; u++) o[f * 4 + u] = make_uint4(b0[2 * u], b1[2 * u], b0[2 * u + 1], b1[2 * u + 1]);
-    } else {
-      double* raw = reinterpret_cast<double*>(o + f * 4);
-#pragma unroll
-      for (int u = 0; u < 4; u++) raw[u] = v[u];
+    for (int u = 0; u < 4; u++) {
+      x[u] = dig_fixed(v[u], e);
+      top = max(top, dig_top(x[u]));
     }
+    uint32_t b0[8], b1[8];
+    dig_expand<8>(dig_interleave(dig_word(x[0]), dig_word(x[1])), b0);
+    dig_expand<8>(dig_interleave(dig_word(x[2]), dig_word(x[3])), b1);
+#pragma unroll
+    for (int u = 0; u < 4; u++) o[f * 4 + u] = make_uint4(b0[2 * u], b1[2 * u], b0[2 * u + 1], b1[2 * u + 1]);
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((threadIdx.x & 31) == 0) atomicMax(&sh_top, top);
+  __syncthreads();
+  if (threadIdx.x == 0) D.ttop[D.ch_hh_off[c] + ij] = sh_top;
 }
 
 // FP32-pair copy of the current amplitudes (the start of a sweep with FP32-pair contractions).
@@ -282,14 +290,48 @@ constexpr int PP_WARPS = 4, PP_CTAS = 3, PP_DEPTH = 4;  // warps per CTA, CTAs p
 constexpr size_t PP_SMEM = sizeof(uint4) * 256 * PP_DEPTH * PP_WARPS;  // 64 KB: three CTAs per SM
 constexpr int PP_MAX_NLAD = 3376;  // ladder basis of a channel (the amplitudes of a row in shared memory)
 
-// sum_cd t(ij, cd) V(cd, ab) in FP64 for a row ij kept as FP64 values (infinities, NaN).
-__device__ __noinline__ double pp_nonfinite(const uint4* __restrict__ vstrip, const double* __restrict__ trow, int row,
-                                            int nl, int vexp) {
+// The digits leave an error of 2^-59 or so of the product of V's and the row's largest values in every term,
+// mostly of the digit products left out, which add up rather than average in channels of high symmetry (P = 0,
+// N = 14: to 2^-52).  In ordinary rows that is less than FP64 sums leave, but V and t fall off
+// exponentially, and a result all of whose products are small keeps little of them (two neutrons at density
+// 0.3, n^2 <= 36, where V spans more than 60 octaves: results off by 1e-3 of themselves).  So results PP_FAR
+// octaves below the product of the strip's and the row's largest values are summed in FP64 for amplitudes
+// given by the caller, and PP_FAR_STEEP below it where the interaction falls by more than PP_STEEP octaves
+// over the model space, with V held in FP64 for them (CHECK).  Elsewhere the errors from MBPT2 amplitudes
+// are those of FP64 sums (N = 2 to 66, densities 0.02 to 0.3: at most 8e-15 of the sum of absolute products,
+// FP64 sums 7e-15), and looking at every result would cost 3% of an update.  Rows or interactions with
+// infinities or NaN are summed in FP64 always.  N = 14, density 0.3, n^2 <= 24, FP64: 0.66 ms a solve without
+// the check, 0.68 at 8 octaves and 1.1 at 4 (1.4 on the FP64 pipe), errors 1.6e-14, 1.6e-14 and 6.8e-15
+// (4.5e-15).
+constexpr int PP_FAR = 12, PP_FAR_STEEP = 4;
+
+// sum_cd t(ij, cd) V(cd, ab) of one result in FP64 over every step-th cd from first, V from the states as
+// every FP64 kernel forms it; the row from the ladder basis (sr) or else from its amplitudes (tr).  Where
+// the interaction is steep and many results are taken so (two neutrons, density 0.3, n^2 <= 36: most of them)
+// V is stored too and four results share a pass of contiguous, independent loads (k_pp): 6 us a result here.
+__device__ __noinline__ double pp_direct(const DevState& D, const double* __restrict__ lut,
+                                         const double* __restrict__ tr, const double* __restrict__ sr,
+                                         int off, int nl, int ab, int first, int step) {
   double s = 0.0;
-  for (int k = 0; k < nl; k++) {
-    const int q = (k & 7) >> 1, half = (k >> 3) & 1;
-    const dig_t w = dig_pick(vstrip[((long)(k >> 4) * 4 + (row >> 3) + 2 * half) * 32 + (row & 7) * 4 + q], k & 1);
-    s += trow[((k >> 4) * 4 + q) * 8 + half * 2 + (k & 1)] * dig_to_double((long long)(w - DIG_BIAS), vexp - 1022 - 61);
+  const int2* __restrict__ mem = D.lad_mem + off;
+  const int2* __restrict__ pair = D.pp_pair + off;
+  const int mr = mem[ab].x;
+  const int2 pr = pair[abs(mr) - 1];
+  const char4 ra = D.nvec[pr.x], rb = D.nvec[pr.y];
+#pragma unroll 4
+  for (int q = first; q < nl; q += step) {
+    const int2 m = mem[q];
+    const int2 p = pair[abs(m.x) - 1];
+    const double y = v_minnesota_as(D.nvec[p.x], D.nvec[p.y], ra, rb, lut);
+    double x;
+    if (sr) {
+      x = sr[q];
+    } else {
+      x = tr[abs(m.x) - 1];
+      if (m.x < 0) x = -x;
+      if (m.y != 0) x += m.y > 0 ? tr[m.y - 1] : -tr[-m.y - 1];
+    }
+    s = fma(x, (m.x > 0) == (mr > 0) ? y : -y, s);
   }
   return s;
 }
@@ -314,16 +356,18 @@ __device__ __forceinline__ void pp_copy(uint4* __restrict__ slot, const uint4* _
 }
 
 // part: this warp's place among the wk warps of the item; ring: this warp's steps; red: the sums
-// of the item's warps (4 per lane and warp).
-template <int SLOTS, typename Out>
-__device__ __forceinline__ void pp_pass(const DevState& D, const PPItem& it, const int* __restrict__ rows, int part,
-                                        int wk, uint4* __restrict__ ring, DigSum* __restrict__ red) {
+// of the item's warps (4 per lane and warp).  t: the channel's amplitudes.  CHECK: returns in the warp of
+// part 0 the number of results left to FP64 sums, listed in far (8 row + column).
+template <int SLOTS, typename Out, bool CHECK>
+__device__ __forceinline__ int pp_pass(const DevState& D, const PPItem& it, const int* __restrict__ rows, int part,
+                                       int wk, uint4* __restrict__ ring, DigSum* __restrict__ red,
+                                       const double* __restrict__ lut, const double* __restrict__ t0,
+                                       unsigned char* __restrict__ far) {
   constexpr int Q = 8 / SLOTS;  // rows ij of this pass, and digits per slot
   const int c = it.c, strip = it.strip, nl = it.nl, n0 = it.n0, nr = it.nr;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int steps = (nl + 15) >> 4;
-  const uint4* __restrict__ vstrip = reinterpret_cast<const uint4*>(D.vdig + it.voff);
-  const uint4* __restrict__ vp = vstrip + lane;
+  const uint4* __restrict__ vp = reinterpret_cast<const uint4*>(D.vdig + it.voff) + lane;
   const int rg = min(n0 + g % Q, nr - 1), ijg = rows ? rows[rg] : rg;
   const uint4* __restrict__ tch = reinterpret_cast<const uint4*>(D.tdig + D.ch_td_off[c]);
   const uint4* __restrict__ tp = tch + ((long)ijg * steps * 4 + t) * 4 + (g / Q) * (Q / 2);
@@ -377,7 +421,7 @@ __device__ __forceinline__ void pp_pass(const DevState& D, const PPItem& it, con
     for (int e = 0; e < 4; e++) red[(part * 4 + e) * 32 + lane] = sum[e];
   }
   __syncthreads();
-  if (part != 0) return;
+  if (part != 0) return 0;
   for (int p = 1; p < wk; p++)
 #pragma unroll
     for (int e = 0; e < 4; e++) {
@@ -386,6 +430,8 @@ __device__ __forceinline__ void pp_pass(const DevState& D, const PPItem& it, con
     }
   // accumulator columns 2t, 2t + 1: slot s counts 256^(-Q s); the slots of a row added up
   const int vexp = D.ch_vexp[c];
+  const unsigned vtop = CHECK ? D.vtop[it.voff / 256] : 0;
+  int nfar = 0;
 #pragma unroll
   for (int e = 0; e < 4; e++) {
     const int s = (2 * t + (e & 1)) / Q;
@@ -403,46 +449,104 @@ __device__ __forceinline__ void pp_pass(const DevState& D, const PPItem& it, con
       x.lo += __shfl_xor_sync(0xffffffffu, x.lo, 1);
     }
     const int col = 2 * t + (e & 1), row = g + 8 * (e >> 1), ab = strip * 16 + row;
+    bool direct = false;
     if (col < Q && n0 + col < nr && ab < nl) {
       const int ij = rows ? rows[n0 + col] : n0 + col;
       const int te = D.texp[D.ch_hh_off[c] + ij];
-      Out v;
-      if (te < DIG_NONFINITE && vexp < DIG_NONFINITE) v = dig_result<Out>(x, dig_power(vexp, te));
-      else
-        v = Arith<Out>::from_double(
-            vexp < DIG_NONFINITE
-                ? pp_nonfinite(vstrip, reinterpret_cast<const double*>(tch + (long)ij * steps * 16), row, nl, vexp)
-                : __longlong_as_double(0x7ff8000000000000ll));
-      reinterpret_cast<Out*>(D.rpp)[D.ch_s_off[c] + (long)ij * nl + ab] = v;
+      direct = te >= DIG_NONFINITE || vexp >= DIG_NONFINITE;
+      if constexpr (CHECK) {
+        // the largest V of the strip times the largest amplitude of the row: 2^92 vtop ttop, the sum counts
+        // in 2^56 and its part top in 2^88
+        const long long top = x.hi + (x.lo >> 32);
+        const long long least = (long long)vtop * D.ttop[D.ch_hh_off[c] + ij] >> ((D.v64 ? PP_FAR_STEEP : PP_FAR) - 4);
+        direct = direct || (top < least && top >= -least);
+      }
+      Out* o = reinterpret_cast<Out*>(D.rpp) + D.ch_s_off[c] + (long)ij * nl + ab;
+      if (!direct) *o = dig_result<Out>(x, dig_power(vexp, te));
+      else if (!CHECK)
+        *o = Arith<Out>::from_double(pp_direct(D, lut, t0 + (long)ij * D.ch_npp[c], nullptr, D.ch_pp_off[c], nl, ab, 0, 1));
+    }
+    if constexpr (CHECK) {
+      const unsigned b = __ballot_sync(0xffffffffu, direct);
+      if (direct) far[nfar + __popc(b & ((1u << lane) - 1u))] = (unsigned char)(8 * row + col);
+      nfar += __popc(b);
     }
   }
+  return nfar;
 }
 
 // rep_only: the rows ij of the items count the list upd_row of the channel, else every hole pair.
 // wk (2 or 4) divides PP_WARPS: PP_WARPS / wk items per CTA.  slots: ring steps per warp, PP_DEPTH or
-// as many as a warp has.
-template <typename Out>
+// as many as a warp has.  lut_off: interaction table of every system.  s64: the rows in the
+// ladder basis (CHECK).
+template <typename Out, bool CHECK>
 __global__ void __launch_bounds__(PP_WARPS * 32, PP_CTAS) k_pp(DevState D, const LoopCtl* __restrict__ ctl,
                                                                const PPItem* __restrict__ items, int nitems, int rep_only,
-                                                               int wk, int slots) {
+                                                               int wk, int slots, const int* __restrict__ lut_off,
+                                                               const double* __restrict__ s64) {
   extern __shared__ __align__(16) uint4 pp_ring[];
   __shared__ DigSum red[PP_WARPS * 128];
-  const int warp = threadIdx.x >> 5, part = warp % wk;
+  __shared__ unsigned char far[CHECK ? PP_WARPS : 1][128];
+  __shared__ int nfar[CHECK ? PP_WARPS : 1];
+  const int warp = threadIdx.x >> 5, part = warp % wk, first = warp - part;
   const int item = blockIdx.x * (PP_WARPS / wk) + warp / wk;
   PPItem it;
   if (item < nitems) it = items[item];
-  // the barrier of pp_pass is the block's only one: warps without work join it here
+  // warps without work join the barriers of pp_pass and after it here
   if (item >= nitems || sys_done(D, ctl, it.sys)) {
     __syncthreads();
+    if (CHECK) __syncthreads();
     return;
   }
   const int* __restrict__ rows = rep_only ? D.upd_row + D.ch_uoff[it.c] : nullptr;
-  DigSum* mine = red + (warp / wk) * wk * 128;
+  DigSum* mine = red + first * 128;
   uint4* ring = pp_ring + warp * slots * 256;
   const int n = it.nr - it.n0;
-  if (n > 4) pp_pass<1, Out>(D, it, rows, part, wk, ring, mine);
-  else if (n > 2) pp_pass<2, Out>(D, it, rows, part, wk, ring, mine);
-  else pp_pass<4, Out>(D, it, rows, part, wk, ring, mine);
+  const int c = it.c;
+  const double* __restrict__ lut = D.lut + lut_off[it.sys];
+  const double* __restrict__ t = cur_t(D, ctl) + D.ch_t_off[c];
+  unsigned char* list = far[CHECK ? first : 0];
+  int left;
+  if (n > 4) left = pp_pass<1, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, list);
+  else if (n > 2) left = pp_pass<2, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, list);
+  else left = pp_pass<4, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, list);
+  if (!CHECK) return;
+  if (part == 0 && (threadIdx.x & 31) == 0) nfar[CHECK ? first : 0] = left;
+  __syncthreads();
+  left = nfar[CHECK ? first : 0];
+  if (left == 0) return;
+  // the item's warps take the results left in turn, four at a time
+  const int lane = threadIdx.x & 31, nl = it.nl;
+  for (int k0 = 4 * part; k0 < left; k0 += 4 * wk) {
+    const int n4 = min(4, left - k0);
+    int ab[4], ij[4];
+    double v[4] = {};
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const int f = list[k0 + min(u, n4 - 1)], r = it.n0 + f % 8;
+      ab[u] = it.strip * 16 + f / 8;
+      ij[u] = rows ? rows[r] : r;
+    }
+    const double* __restrict__ sc = s64 + D.ch_s_off[c];
+    if (D.v64) {
+      const double* __restrict__ vc = D.v64 + D.ch_vd_off[c];
+      const int wide = (nl + 15) & ~15;
+#pragma unroll 2
+      for (int q = lane; q < nl; q += 32)
+#pragma unroll
+        for (int u = 0; u < 4; u++) v[u] = fma(sc[(long)ij[u] * nl + q], vc[(long)ab[u] * wide + q], v[u]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        if (u < n4) v[u] = pp_direct(D, lut, nullptr, sc + (long)ij[u] * nl, D.ch_pp_off[c], nl, ab[u], lane, 32);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const double y = warp_sum(v[u]);
+      if (lane == u && u < n4)
+        reinterpret_cast<Out*>(D.rpp)[D.ch_s_off[c] + (long)ij[u] * nl + ab[u]] = Arith<Out>::from_double(y);
+    }
+  }
 }
 
 // FP32-pair copy of an FP64 array.
@@ -1292,8 +1396,10 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   }
   CUDA_TRY(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
   smem_at_least(k_tdig, sizeof(double) * max_nlad);
-  smem_at_least(k_pp<double>, PP_SMEM);
-  smem_at_least(k_pp<f2>, PP_SMEM);
+  smem_at_least(k_pp<double, false>, PP_SMEM);
+  smem_at_least(k_pp<double, true>, PP_SMEM);
+  smem_at_least(k_pp<f2, false>, PP_SMEM);
+  smem_at_least(k_pp<f2, true>, PP_SMEM);
   CUDA_TRY(cudaStreamSynchronize(s));
 }
 
@@ -1482,7 +1588,10 @@ void pnm_launch_pp(pnm_ctx* ctx, cudaStream_t s, bool rep_only, bool pair) {
   if (!ctx->d.vdig) throw PnmError{PNM_EINVAL, "the ladder V has not been built"};
   if (ctx->n_lad_rows == 0) return;
   const int nrow = rep_only ? ctx->n_lad_rep : ctx->n_lad_rows;
-  k_tdig<<<nrow, TDIG_THREADS, sizeof(double) * ctx->max_nlad, s>>>(ctx->d, ctx->ctl, ctx->lad_rows);
+  // the operator takes any amplitudes (it is not captured); in a solve the interaction decides
+  const bool check = !rep_only || ctx->d.v64;
+  if (check && !ctx->s64) ctx->s64 = (double*)dmalloc(ctx, sizeof(double) * std::max<long>(ctx->ns, 1));
+  k_tdig<<<nrow, TDIG_THREADS, sizeof(double) * ctx->max_nlad, s>>>(ctx->d, ctx->ctl, ctx->lad_rows, check ? ctx->s64 : nullptr);
   if (!rep_only && !ctx->pp_items_all) ctx->n_pp_all = pp_work_list(ctx, ctx->h_nhh, &ctx->pp_items_all);
   const PPItem* items = rep_only ? ctx->pp_items : ctx->pp_items_all;
   const int n = rep_only ? ctx->n_pp_items : ctx->n_pp_all;
@@ -1494,8 +1603,16 @@ void pnm_launch_pp(pnm_ctx* ctx, cudaStream_t s, bool rep_only, bool pair) {
   const int steps = (ctx->max_nlad + 15) / 16;
   const int slots = std::min(PP_DEPTH, std::max(1, (steps + wk - 1) / wk));
   const size_t smem = PP_SMEM / PP_DEPTH * slots;
-  if (pair) k_pp<f2><<<nb, PP_WARPS * 32, smem, s>>>(ctx->d, ctx->ctl, items, n, rep_only ? 1 : 0, wk, slots);
-  else k_pp<double><<<nb, PP_WARPS * 32, smem, s>>>(ctx->d, ctx->ctl, items, n, rep_only ? 1 : 0, wk, slots);
+  auto go = [&](auto k) {
+    k<<<nb, PP_WARPS * 32, smem, s>>>(ctx->d, ctx->ctl, items, n, rep_only ? 1 : 0, wk, slots, ctx->lut_off_d, ctx->s64);
+  };
+  if (check) {
+    if (pair) go(k_pp<f2, true>);
+    else go(k_pp<double, true>);
+  } else {
+    if (pair) go(k_pp<f2, false>);
+    else go(k_pp<double, false>);
+  }
 }
 
 // The ph term and the pp ladder do not depend on each other nor on the one-body sums: in a

@@ -16,6 +16,11 @@ enum {
 };
 extern const char* const pnm_kernel_names[PNM_NKERNELS];
 
+// Octaves of the interaction's fall above which the FP64 ladder checks its results (iterate.cu); with
+// protons, whose channels lie up to three octaves below the scale of their digits and mix three Gaussians,
+// errors of 2^-48 are reached at 47 octaves already.
+constexpr double PP_STEEP = 60.0, PP_STEEP_PROTONS = 40.0;
+
 struct pnm_ctx {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -80,6 +85,7 @@ struct pnm_ctx {
   LoopCtl* ctl = nullptr;     // device
   double* small = nullptr;    // device scratch for single-value queries
   double* mbpt3_buf = nullptr;   // per-CTA partials and per-system results of pnm_mbpt3
+  double* s64 = nullptr;         // the amplitudes in the ladder layout (FP64 ladders that check their results)
   double* expand_buf = nullptr;  // the pp ladder or ph term in the amplitude layout (operator calls)
   SysCtl* sysctl = nullptr;   // device, one per system
   int* blocks_done = nullptr; // device, one per system
@@ -113,6 +119,7 @@ struct pnm_ctx {
   int n_vl_items = 0;
   size_t vl_smem = 0;
   double hbar2_2m = 0.0;
+  bool steep = false;  // the interaction of a system falls by more than PP_STEEP octaves over its model space
   int mlp_fallback = 0;  // 1 when the last learned start was replaced by the MBPT2 start
 
   // side streams for the independent parts of an update (ph term, pp ladder), joined by events

@@ -101,10 +101,13 @@ struct DevState {
   double *v_pphh, *v_hhhh, *x_v1, *x_w;
   // pp ladder in digit words (dig.cuh): per channel with a V_pppp block the ladder-basis V at
   // ch_vd_off in fragment order (16-row strips of 16-column steps) with its exponent, and the
-  // ladder-basis amplitudes at ch_td_off, n_hh rows of the padded width, an exponent per hole pair
+  // ladder-basis amplitudes at ch_td_off, n_hh rows of the padded width, an exponent per hole pair.
+  // vtop, ttop: dig_top of the largest element of a strip (at its first word / 256) and of a row
   unsigned long long *vdig, *tdig;
   long *ch_vd_off, *ch_td_off;
   int *ch_vexp, *texp;
+  unsigned *vtop, *ttop;
+  double* v64;  // the ladder-basis V in FP64, rows of the padded width at ch_vd_off (steep interactions only, else null)
   double *den, *inv_den;  // eps_i + eps_j - eps_a - eps_b per amplitude, and its reciprocal
   // iteration state
   double *t0, *t1;       // double buffer, parity = iteration & 1

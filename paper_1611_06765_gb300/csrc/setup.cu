@@ -1008,10 +1008,11 @@ __global__ void __launch_bounds__(256) k_v_dig(const int4* __restrict__ items, c
                                                const int* __restrict__ ch_nlad, const long* __restrict__ ch_vd_off,
                                                const int2* __restrict__ lad_mem, const int2* __restrict__ pp_pair,
                                                const char4* __restrict__ nvec, const double* __restrict__ lut,
-                                               int* __restrict__ ch_vexp,
+                                               int* __restrict__ ch_vexp, unsigned* __restrict__ vtop, double* __restrict__ v64,
                                                dig_t* __restrict__ vdig) {
   extern __shared__ __align__(16) unsigned char vsm[];
   __shared__ int sh_max;
+  __shared__ unsigned sh_top;
   long long* xlut = reinterpret_cast<long long*>(vsm);
   const int4 it = items[blockIdx.x];  // channel, first row, interaction table and its size (< 0: with protons)
   const int c = it.x, r0 = it.y, lut_elems = abs(it.w);
@@ -1028,10 +1029,14 @@ __global__ void __launch_bounds__(256) k_v_dig(const int4* __restrict__ items, c
     sb[q] = nvec[pr.y];
     sg[q] = m > 0 ? 1 : -1;
   }
-  if (threadIdx.x == 0) ch_vexp[c] = e;
+  if (threadIdx.x == 0) {
+    ch_vexp[c] = e;
+    sh_top = 0;
+  }
   __syncthreads();
   const int steps = (nl + 15) >> 4;
   uint4* out = reinterpret_cast<uint4*>(vdig + ch_vd_off[c]) + (long)(r0 >> 4) * steps * 128;
+  unsigned top = 0;
   for (int f = threadIdx.x; f < steps * 128; f += blockDim.x) {
     const int lane = f & 31, g = (f >> 5) & 3, ks = f >> 7;
     const int row = r0 + (lane >> 2) + (g & 1) * 8, col = ks * 16 + (lane & 3) * 2 + (g >> 1) * 8;
@@ -1043,11 +1048,20 @@ __global__ void __launch_bounds__(256) k_v_dig(const int4* __restrict__ items, c
       if (row < nl && q < nl) {
         v = v_minnesota_fixed(sa[q], sb[q], sa[row], sb[row], xlut);
         v = sg[row] * sg[q] > 0 ? v : -v;
+        if (v64) {
+          const double y = v_minnesota_as(sa[q], sb[q], sa[row], sb[row], lut + it.z);
+          v64[ch_vd_off[c] + (long)row * steps * 16 + q] = sg[row] * sg[q] > 0 ? y : -y;
+        }
       }
+      top = max(top, dig_top(v));
       w[k] = dig_word(v);
     }
     out[f] = dig_interleave(w[0], w[1]);
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((threadIdx.x & 31) == 0) atomicMax(&sh_top, top);
+  __syncthreads();
+  if (threadIdx.x == 0) vtop[ch_vd_off[c] / 256 + (r0 >> 4) * steps] = sh_top;
 }
 
 __global__ void k_v_hhhh(const SetupSys* __restrict__ SS, const int* __restrict__ ch_sys,
@@ -1153,11 +1167,17 @@ void pnm_need_vdig(pnm_ctx* ctx) {
   pnm_need_pp_lists(ctx);
   D.tdig = ctx_alloc<dig_t>(ctx, ctx->ntdig);
   D.texp = ctx_alloc<int>(ctx, ctx->n_hh_pairs);
+  D.ttop = ctx_alloc<unsigned>(ctx, ctx->n_hh_pairs);
+  D.vtop = ctx_alloc<unsigned>(ctx, ctx->nvdig / 256);
+  if (ctx->steep) {  // before any capture of the ladder
+    D.v64 = ctx_alloc<double>(ctx, ctx->nvdig);
+    ctx->s64 = ctx_alloc<double>(ctx, std::max<long>(ctx->ns, 1));
+  }
   D.vdig = ctx_alloc<dig_t>(ctx, std::max<long>(ctx->nvdig, 1));
   smem_at_least(k_v_dig, ctx->vl_smem);
   if (ctx->n_vl_items > 0)
     k_v_dig<<<ctx->n_vl_items, 256, ctx->vl_smem, s>>>(ctx->vl_items, D.ch_pp_off, D.ch_nlad, D.ch_vd_off, D.lad_mem,
-                                                       D.pp_pair, D.nvec, D.lut, D.ch_vexp, D.vdig);
+                                                       D.pp_pair, D.nvec, D.lut, D.ch_vexp, D.vtop, D.v64, D.vdig);
   CUDA_TRY(cudaGetLastError());
 }
 
@@ -1204,6 +1224,12 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
     if (S.N >= S.nsp) throw PnmError{PNM_EINVAL, "no particle states: n2max too small for N"};
     S.sp_off = nsp_total;
     nsp_total += S.nsp;
+    // exp(-q^2 / 4 kappa) of the widest Gaussian at q = (2 pi / L) 2 sqrt(n2max)
+    const double q1 = 2.0 * PNM_PI / S.L;
+    double kappa = std::max(P.VR != 0.0 ? P.kR : 0.0, P.VS != 0.0 ? P.kS : 0.0);
+    if (S.species != 1 && P.VT != 0.0) kappa = std::max(kappa, P.kT);
+    const double octaves = kappa > 0.0 ? q1 * q1 * S.n2max / kappa / std::log(2.0) : 0.0;
+    ctx->steep = ctx->steep || octaves > (S.species == 1 ? PP_STEEP : PP_STEEP_PROTONS);
     S.lut_off = lut_total;
     S.lut_len = 4 * S.n2max + 1;
     lut_total += S.lut_len * (S.species == 1 ? 1 : 3);  // interleaved R, T, S halves with protons
@@ -1534,6 +1560,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   D.occ_idx = dalloc<int>(h_occ_off[nsp_total], ctx->owned, s);
   k_occ<<<nsp_total, OCC_THREADS, 0, s>>>(1, SS, D.sp_sys, D.nvec, D.ch_pp_off, nullptr, D.occ_off, D.occ_idx);
   D.vdig = nullptr;  // the ladder V is built on first use
+  D.v64 = nullptr;
   D.rpp = dalloc<double>(s_acc, ctx->owned, s);
   ctx->ntdig = td_acc;
   ctx->n_vl_items = (int)vl_items.size();

@@ -114,3 +114,47 @@ def test_pair_results_are_rounded(pkg, N, Z, rho, n2):
     r, pair = g.apply_pp_ladder(t), g.apply_pp_ladder(t, precision=pkg.PNM_PREC_F32PAIR)
     assert np.any(r) and np.all(np.abs(pair - r) <= 2.0 ** -48 * np.abs(r))
     g.close()
+
+
+def _ladder(o, t):
+    """(reference, sum of absolute products) of the pp ladder in the library's order."""
+    tab = o.channel_tables()
+    ref, bound, off = np.zeros(len(t)), np.zeros(len(t)), 0
+    for c, (nh, npp) in enumerate(zip(tab["nhh"], tab["npp"])):
+        s = slice(off, off + int(nh) * int(npp))
+        off = s.stop
+        V, tb = o.vpp_block(c), t[s].reshape(int(nh), int(npp))
+        ref[s], bound[s] = (tb @ V).ravel(), (np.abs(tb) @ np.abs(V)).ravel()
+    return ref, bound
+
+
+@pytest.mark.parametrize("N,Z,rho,n2", [(2, 0, 0.3, 36), (14, 0, 0.3, 24), (38, 0, 0.12, 10), (2, 2, 0.2, 9),
+                                           (14, 14, 0.2, 8)])
+@pytest.mark.parametrize("kind", ["mbpt2", "random", "dominant", "single"])
+def test_ladder_of_an_interaction_of_wide_range(pkg, N, Z, rho, n2, kind):
+    """Every result against its own sum of absolute products.  The Gaussians exp(-x) of both sides carry an
+    argument of three roundings, 4 x units of the last place with the function, x up to q^2 / 4 kappa_S at the
+    largest momentum transfer 2 sqrt(n2max); sums of at most 900 products carry 900 more.  FP32 pairs, where the
+    result is far from their smallest number, 2^-48."""
+    P = minnesota_params()
+    g = pkg.Context(N, rho, n2, params=P, Z=Z) if Z else pkg.Context(N, rho, n2, params=P)
+    o = channel.OracleSystem(N, rho, n2, P, Z=Z)
+    x = (2 * np.pi / o.L) ** 2 * 4 * n2 / (4 * P[5])
+    tol = (4 * x + 900) * 2.0 ** -53
+    t = random_amplitudes(len(g.amplitude_labels()), seed=31)
+    k = np.flatnonzero(_ladder(o, t)[1])
+    k = k[len(k) // 3]
+    if kind == "mbpt2":
+        g.mbpt3()
+        t = g.get_amplitudes()
+    elif kind == "dominant":
+        t[k] = 2.0 ** 53
+    elif kind == "single":
+        t = np.zeros_like(t)
+        t[k] = 1.0
+    ref, bound = _ladder(o, t)
+    assert np.all(np.abs(g.apply_pp_ladder(t) - ref) <= tol * bound)
+    pair = g.apply_pp_ladder(t, precision=pkg.PNM_PREC_F32PAIR)
+    seen = np.abs(ref) > 1e-20
+    assert np.all(np.abs(pair - ref)[seen] <= ((tol + 2.0 ** -48) * bound)[seen])
+    g.close()
