@@ -56,13 +56,17 @@ static_assert(TC_BK == 64, "tile_core_off assumes 64-element k-blocks");
 __device__ __forceinline__ int core_off(int r, int k) { return tile_core_off(r, k); }
 
 // ------------------------------------------------------------------------ kernels
+constexpr double PACK_OCTAVES = 36.0;
+
 // V tiles of the channels with a V_pppp block (setup): one CTA per (item, k-block), the elements
 // straight from the interaction table as integers (dig.cuh), rounded to FP32 and split into BF16
 // hi + lo: neither an FP64 operation nor a stored V (forming them from a stored FP32-pair copy
-// took a write and a read of 8 bytes per element and four FP64-pipe instructions).
+// took a write and a read of 8 bytes per element and four FP64-pipe instructions).  An integer holds the 24
+// bits of an FP32 number down to 2^-36 of the table's largest entry; where the interaction falls further
+// over the model space (wide) the elements are formed in FP64.
 __global__ void __launch_bounds__(256) k_pack_v(const TCItem* __restrict__ items, DevState D,
                                                 const int* __restrict__ lut_off, const int2* __restrict__ lut_info,
-                                                __nv_bfloat16* __restrict__ vt) {
+                                                bool wide, __nv_bfloat16* __restrict__ vt) {
   extern __shared__ __align__(16) unsigned char psm[];
   __shared__ int sh_max;
   __shared__ char4 ra[TC_M], rb[TC_M], ca[TC_BK], cb[TC_BK];
@@ -101,7 +105,10 @@ __global__ void __launch_bounds__(256) k_pack_v(const TCItem* __restrict__ items
     for (int j = 0; j < 8; j++) {
       const int sg = rs[r] * cs[k0 + j];
       float x = 0.0f;
-      if (sg != 0) {
+      if (sg != 0 && wide) {
+        x = (float)v_minnesota_as(ca[k0 + j], cb[k0 + j], ra[r], rb[r], D.lut + lut_off[it.sys]);
+        x = sg > 0 ? x : -x;
+      } else if (sg != 0) {
         const long long v = v_minnesota_fixed(ca[k0 + j], cb[k0 + j], ra[r], rb[r], xlut);
         x = e < DIG_NONFINITE ? scalbnf(__ll2float_rn(sg > 0 ? v : -v), e - 1022 - 61) : __int_as_float(0x7fc00000);
       }
@@ -576,7 +583,7 @@ void pnm_prepare_mixed(pnm_ctx* ctx) {
       CUDA_TRY(cudaMemcpyAsync(dli, li.data(), sizeof(int2) * li.size(), cudaMemcpyHostToDevice, s));
       smem_at_least(k_pack_v, sizeof(long long) * max_lut);
       k_pack_v<<<dim3(M->nitems, max_nkb), 256, sizeof(long long) * max_lut, s>>>(M->items, ctx->d, ctx->lut_off_d, dli,
-                                                                                  M->vt);
+                                                                                  ctx->fall > PACK_OCTAVES, M->vt);
     }
     CUDA_TRY(cudaGetLastError());
     M->stage_bytes = (2 * A_PLANE + 2 * (uint32_t)max_npad * TC_BK * 2 + 1023) / 1024 * 1024;

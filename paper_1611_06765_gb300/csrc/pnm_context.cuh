@@ -119,6 +119,7 @@ struct pnm_ctx {
   int n_vl_items = 0;
   size_t vl_smem = 0;
   double hbar2_2m = 0.0;
+  double fall = 0.0;   // octaves by which a system's interaction falls over its model space, at most
   bool steep = false;  // the interaction of a system falls by more than PP_STEEP octaves over its model space
   int mlp_fallback = 0;  // 1 when the last learned start was replaced by the MBPT2 start
 

@@ -1229,6 +1229,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
     double kappa = std::max(P.VR != 0.0 ? P.kR : 0.0, P.VS != 0.0 ? P.kS : 0.0);
     if (S.species != 1 && P.VT != 0.0) kappa = std::max(kappa, P.kT);
     const double octaves = kappa > 0.0 ? q1 * q1 * S.n2max / kappa / std::log(2.0) : 0.0;
+    ctx->fall = std::max(ctx->fall, octaves);
     ctx->steep = ctx->steep || octaves > (S.species == 1 ? PP_STEEP : PP_STEEP_PROTONS);
     S.lut_off = lut_total;
     S.lut_len = 4 * S.n2max + 1;

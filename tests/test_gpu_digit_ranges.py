@@ -158,3 +158,24 @@ def test_ladder_of_an_interaction_of_wide_range(pkg, N, Z, rho, n2, kind):
     seen = np.abs(ref) > 1e-20
     assert np.all(np.abs(pair - ref)[seen] <= ((tol + 2.0 ** -48) * bound)[seen])
     g.close()
+
+
+@pytest.mark.parametrize("N,Z,rho,n2", [(2, 0, 0.3, 36), (14, 0, 0.3, 24), (38, 0, 0.3, 20), (2, 2, 0.2, 9)])
+@pytest.mark.parametrize("single", [False, True])
+def test_mixed_ladder_of_an_interaction_of_wide_range(pkg, N, Z, rho, n2, single):
+    """V and t as BF16 hi + lo of their FP32 values, three products: 3 * 2^-18 of every product and the FP32
+    sums of at most 500 terms, 2^-24 each; where the sum of absolute products is an ordinary FP32 number."""
+    P = minnesota_params()
+    g = pkg.Context(N, rho, n2, params=P, Z=Z) if Z else pkg.Context(N, rho, n2, params=P)
+    o = channel.OracleSystem(N, rho, n2, P, Z=Z)
+    g.mbpt3()
+    t = g.get_amplitudes()
+    if single:
+        k = np.flatnonzero(_ladder(o, t)[1])
+        t = np.zeros_like(t)
+        t[k[len(k) // 3]] = 1.0
+    ref, bound = _ladder(o, t)
+    r = g.apply_pp_ladder(t, precision=pkg.PNM_PREC_BF16X3)
+    seen = bound > 1e-30
+    assert np.all(np.abs(r - ref)[seen] <= ((3 * 2.0 ** -18 + 500 * 2.0 ** -24) * bound)[seen])
+    g.close()
