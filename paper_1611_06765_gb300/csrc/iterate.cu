@@ -1375,9 +1375,6 @@ void pnm_prepare_iteration(pnm_ctx* ctx) {
   size_t nparts = std::max<size_t>(std::max<size_t>(upd.size(), ctx->n_upd_ctas), (size_t)ctx->nrows);
   ctx->d.eparts = (double*)dmalloc(ctx, sizeof(double) * nparts);
   ctx->d.rparts = (double*)dmalloc(ctx, sizeof(double) * nparts);
-  int mx = 0;
-  for (int x = 0; x < ctx->nx; x++) mx = std::max(mx, std::max(ctx->h_x_nph[x], ctx->h_x_nhp[x]));
-  ctx->max_x_dim = mx;
   ctx->ctl = (LoopCtl*)dmalloc(ctx, sizeof(LoopCtl));
   CUDA_TRY(cudaMemsetAsync(ctx->ctl, 0, sizeof(LoopCtl), s));
   ctx->blocks_done = (int*)dmalloc(ctx, sizeof(int) * nsys);

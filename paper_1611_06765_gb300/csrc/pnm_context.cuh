@@ -32,7 +32,7 @@ struct pnm_ctx {
   int nsp_total = 0, nch = 0, nx = 0, nrows = 0, n_hh_pairs = 0, n_pp_pairs = 0;
   long nt = 0, nvhh = 0, nxt = 0, nxc = 0;
   long ns = 0;  // elements of the ladder layout (n_hh x n_lad over the channels with V_pppp)
-  int max_x_dim = 0, max_npp = 0, max_nlad = 0;
+  int max_npp = 0, max_nlad = 0;
   // (channel, ij) rows of the channels with V_pppp (digits of the ladder amplitudes): first those
   // the updates compute, then the others
   int2* lad_rows = nullptr;
@@ -54,9 +54,9 @@ struct pnm_ctx {
   // pp ladder: items for the rows the updates compute, and (made on first use) for every row
   PPItem *pp_items = nullptr, *pp_items_all = nullptr;
   int n_pp_items = 0, n_pp_all = 0, nsm = 148;
-  int4* upd_items = nullptr;  // (channel, ij, first pp column) of the update
+  int4* upd_items = nullptr;  // (channel, ij, first pp column), 128 columns each (the learned start)
   int n_upd_items = 0;
-  int *upd_lo_d = nullptr, *upd_hi_d = nullptr;  // per system ranges of the (row, column) items
+  int *upd_lo_d = nullptr, *upd_hi_d = nullptr;  // per system ranges of these items
   UpdItem* upd_chunks = nullptr;  // of the updates: chunks of 32 amplitudes, and the amplitudes
   int* upd_z = nullptr;
   int n_upd_ctas = 0, upd_per_warp = 1;
@@ -108,7 +108,6 @@ struct pnm_ctx {
   SolveParams* d_par = nullptr;
   double* d_tol = nullptr;       // per-system tolerance of the energy test
   std::vector<double> tol_host;  // the values d_tol holds
-  unsigned long long cond_handle_for_mode[4] = {0, 0, 0, 0};
 
   MixedState* mixed = nullptr;
   MlpState* mlp = nullptr;

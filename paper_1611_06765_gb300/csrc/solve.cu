@@ -19,7 +19,7 @@ static float elapsed(cudaEvent_t a, cudaEvent_t b) {
 
 // ------------------------------------------------------------------ whole-solve graphs
 // A solve that is not host-driven runs as one graph: the start (learned-start inference, control
-// blocks, initial energy, FP32 copies), the first iteration loop (a WHILE node over one update),
+// blocks, initial energy, FP32 copies), the first iteration loop (a WHILE node over several updates),
 // the spin flips of the FP64 amplitudes, the refinement gate and loop, settling and the copy of
 // the control blocks to pinned host memory.  One launch and one synchronisation per solve: no
 // host round trip between the phases leaves the device idle.
@@ -54,7 +54,7 @@ static void solve_buffers(pnm_ctx* ctx) {
 }
 
 // Graph under construction: stream segments captured after the current frontier `deps`, and
-// WHILE nodes whose body is one update.
+// WHILE nodes whose body is a few updates (pnm_enqueue_loop_body).
 struct SolveGraphBuilder {
   pnm_ctx* ctx;
   cudaGraph_t g = nullptr;
