@@ -305,35 +305,86 @@ constexpr int PP_MAX_NLAD = 3376;  // ladder basis of a channel (the amplitudes 
 // (4.5e-15).
 constexpr int PP_FAR = 12, PP_FAR_STEEP = 4;
 
-// sum_cd t(ij, cd) V(cd, ab) of one result in FP64 over every step-th cd from first, V from the states as
-// every FP64 kernel forms it; the row from the ladder basis (sr) or else from its amplitudes (tr).  Where
-// the interaction is steep and many results are taken so (two neutrons, density 0.3, n^2 <= 36: most of them)
-// V is stored too and four results share a pass of contiguous, independent loads (k_pp): 6 us a result here.
+// Element q of row ab of the ladder-basis V, from the states as every FP64 kernel forms it: mr, ra, rb are
+// the row's representative and its states.
+__device__ __forceinline__ double lad_v(const DevState& D, const double* __restrict__ lut, int2 pair, int m, int mr,
+                                        char4 ra, char4 rb) {
+  const double y = v_minnesota_as(D.nvec[pair.x], D.nvec[pair.y], ra, rb, lut);
+  return (m > 0) == (mr > 0) ? y : -y;
+}
+
+// sum_cd t(ij, cd) V(cd, ab) of one result in FP64, by one thread (rows with infinities or NaN in a solve,
+// which ends with them); tr: the row's amplitudes.
 __device__ __noinline__ double pp_direct(const DevState& D, const double* __restrict__ lut,
-                                         const double* __restrict__ tr, const double* __restrict__ sr,
-                                         int off, int nl, int ab, int first, int step) {
-  double s = 0.0;
+                                         const double* __restrict__ tr, int off, int nl, int ab) {
   const int2* __restrict__ mem = D.lad_mem + off;
   const int2* __restrict__ pair = D.pp_pair + off;
   const int mr = mem[ab].x;
   const int2 pr = pair[abs(mr) - 1];
   const char4 ra = D.nvec[pr.x], rb = D.nvec[pr.y];
-#pragma unroll 4
-  for (int q = first; q < nl; q += step) {
+  double s = 0.0;
+  for (int q = 0; q < nl; q++) {
     const int2 m = mem[q];
-    const int2 p = pair[abs(m.x) - 1];
-    const double y = v_minnesota_as(D.nvec[p.x], D.nvec[p.y], ra, rb, lut);
-    double x;
-    if (sr) {
-      x = sr[q];
-    } else {
-      x = tr[abs(m.x) - 1];
-      if (m.x < 0) x = -x;
-      if (m.y != 0) x += m.y > 0 ? tr[m.y - 1] : -tr[-m.y - 1];
-    }
-    s = fma(x, (m.x > 0) == (mr > 0) ? y : -y, s);
+    double x = tr[abs(m.x) - 1];
+    if (m.x < 0) x = -x;
+    if (m.y != 0) x += m.y > 0 ? tr[m.y - 1] : -tr[-m.y - 1];
+    s = fma(x, lad_v(D, lut, pair[abs(m.x) - 1], m.x, mr, ra, rb), s);
   }
   return s;
+}
+
+// Up to four of an item's results, listed in far, by a warp: the rows from the ladder basis (s64), V stored
+// where the interaction is steep and many results are taken so (two neutrons, density 0.3, n^2 <= 36: most of
+// them), else from the states.  Four share the loads, which are a chain of round trips (one at a time took
+// 6 us a result).
+template <typename Out>
+__device__ __forceinline__ void pp_far(const DevState& D, const PPItem& it, const int* __restrict__ rows,
+                                       const double* __restrict__ lut, const double* __restrict__ s64,
+                                       const unsigned char* __restrict__ far, int n) {
+  const int lane = threadIdx.x & 31, nl = it.nl, off = D.ch_pp_off[it.c];
+  const int2* __restrict__ mem = D.lad_mem + off;
+  const int2* __restrict__ pair = D.pp_pair + off;
+  const long base = D.ch_s_off[it.c];
+  int ab[4], ij[4];
+  double v[4] = {};
+#pragma unroll
+  for (int u = 0; u < 4; u++) {
+    const int f = far[min(u, n - 1)], r = it.n0 + f % 8;
+    ab[u] = it.strip * 16 + f / 8;
+    ij[u] = rows ? rows[r] : r;
+  }
+  const double* __restrict__ sc = s64 + base;
+  if (D.v64) {
+    const double* __restrict__ vc = D.v64 + D.ch_vd_off[it.c];
+    const int wide = (nl + 15) & ~15;
+#pragma unroll 2
+    for (int q = lane; q < nl; q += 32)
+#pragma unroll
+      for (int u = 0; u < 4; u++) v[u] = fma(sc[(long)ij[u] * nl + q], vc[(long)ab[u] * wide + q], v[u]);
+  } else {
+    int mr[4];
+    char4 ra[4], rb[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      mr[u] = mem[ab[u]].x;
+      const int2 p = pair[abs(mr[u]) - 1];
+      ra[u] = D.nvec[p.x];
+      rb[u] = D.nvec[p.y];
+    }
+#pragma unroll 2
+    for (int q = lane; q < nl; q += 32) {
+      const int m = mem[q].x;
+      const int2 p = pair[abs(m) - 1];
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        if (u < n) v[u] = fma(sc[(long)ij[u] * nl + q], lad_v(D, lut, p, m, mr[u], ra[u], rb[u]), v[u]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; u++) {
+    const double y = warp_sum(v[u]);
+    if (lane == u && u < n) reinterpret_cast<Out*>(D.rpp)[base + (long)ij[u] * nl + ab[u]] = Arith<Out>::from_double(y);
+  }
 }
 
 // One step of an item's operands into this lane's ring slots: V's four 16-byte groups and the
@@ -464,7 +515,7 @@ __device__ __forceinline__ int pp_pass(const DevState& D, const PPItem& it, cons
       Out* o = reinterpret_cast<Out*>(D.rpp) + D.ch_s_off[c] + (long)ij * nl + ab;
       if (!direct) *o = dig_result<Out>(x, dig_power(vexp, te));
       else if (!CHECK)
-        *o = Arith<Out>::from_double(pp_direct(D, lut, t0 + (long)ij * D.ch_npp[c], nullptr, D.ch_pp_off[c], nl, ab, 0, 1));
+        *o = Arith<Out>::from_double(pp_direct(D, lut, t0 + (long)ij * D.ch_npp[c], D.ch_pp_off[c], nl, ab));
     }
     if constexpr (CHECK) {
       const unsigned b = __ballot_sync(0xffffffffu, direct);
@@ -516,37 +567,7 @@ __global__ void __launch_bounds__(PP_WARPS * 32, PP_CTAS) k_pp(DevState D, const
   left = nfar[CHECK ? first : 0];
   if (left == 0) return;
   // the item's warps take the results left in turn, four at a time
-  const int lane = threadIdx.x & 31, nl = it.nl;
-  for (int k0 = 4 * part; k0 < left; k0 += 4 * wk) {
-    const int n4 = min(4, left - k0);
-    int ab[4], ij[4];
-    double v[4] = {};
-#pragma unroll
-    for (int u = 0; u < 4; u++) {
-      const int f = list[k0 + min(u, n4 - 1)], r = it.n0 + f % 8;
-      ab[u] = it.strip * 16 + f / 8;
-      ij[u] = rows ? rows[r] : r;
-    }
-    const double* __restrict__ sc = s64 + D.ch_s_off[c];
-    if (D.v64) {
-      const double* __restrict__ vc = D.v64 + D.ch_vd_off[c];
-      const int wide = (nl + 15) & ~15;
-#pragma unroll 2
-      for (int q = lane; q < nl; q += 32)
-#pragma unroll
-        for (int u = 0; u < 4; u++) v[u] = fma(sc[(long)ij[u] * nl + q], vc[(long)ab[u] * wide + q], v[u]);
-    } else {
-#pragma unroll
-      for (int u = 0; u < 4; u++)
-        if (u < n4) v[u] = pp_direct(D, lut, nullptr, sc + (long)ij[u] * nl, D.ch_pp_off[c], nl, ab[u], lane, 32);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; u++) {
-      const double y = warp_sum(v[u]);
-      if (lane == u && u < n4)
-        reinterpret_cast<Out*>(D.rpp)[D.ch_s_off[c] + (long)ij[u] * nl + ab[u]] = Arith<Out>::from_double(y);
-    }
-  }
+  for (int k = 4 * part; k < left; k += 4 * wk) pp_far<Out>(D, it, rows, lut, s64, list + k, min(4, left - k));
 }
 
 // FP32-pair copy of an FP64 array.
