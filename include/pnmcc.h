@@ -287,7 +287,14 @@ int pnm_checkpoint_load(pnm_ctx *ctx, const char *path);
  * digit products of FP64 accuracy (FP64 results, or FP32 pairs: PNM_PREC_F32PAIR) or the BF16x3
  * tensor-core kernel (precision).  t and r hold n restricted
  * amplitudes of system `sys` in library order; r is 0 on channels whose V block vanishes
- * (S_z != 0 for neutrons).  Resets the solver's iteration state. */
+ * (S_z != 0 for neutrons).  Resets the solver's iteration state.
+ * Accuracy of the FP64 and pair forms: digits carry 61 bits below the largest element of V and
+ * of the row ij of t, and leave an error of about 2^-59 of the product of these two per term.
+ * Results 2^-12 and more below that product are summed in FP64 instead (2^-4 where the interaction
+ * falls by more than 60 octaves over the model space, 40 with protons), as are rows that hold
+ * infinities or NaN.  The error of a result stays at that of an FP64 sum of its terms (measured:
+ * at most 1e-14 of the sum of their absolute values, for MBPT2, random and sparse amplitudes and
+ * amplitudes up to 2^53 apart); pairs round it to 48 bits. */
 int pnm_apply_pp_ladder(pnm_ctx *ctx, int sys, int precision, const double *t, double *r,
                         size_t n);
 
@@ -298,7 +305,14 @@ int pnm_apply_pp_ladder(pnm_ctx *ctx, int sys, int precision, const double *t, d
  * digit products of FP64 accuracy (FP64 results, or FP32 pairs: PNM_PREC_F32PAIR), or the
  * mixed-precision kernels (FP32 operands and products).  t and r hold n restricted
  * amplitudes of system `sys` in library order; r is the term of the flip-symmetric part
- * (t + F t)/2 of t (see PNM_INIT_KEEP).  Resets the solver's iteration state. */
+ * (t + F t)/2 of t (see PNM_INIT_KEEP).  Resets the solver's iteration state.
+ * Accuracy of the FP64 and pair forms: every cross channel has scales of its own; digits carry 61
+ * bits below the largest element of t, <kl|v|cd> and <kb|v|cj> in it.  A channel in which a row or
+ * column of one of them lies wholly more than 8 octaves below its largest element, or whose quadratic
+ * part is far above <kb|v|cj> where that stands alone, or that holds infinities or NaN, is summed in
+ * FP64, and so are channels of at most 8 rows and columns (pairs: in pair arithmetic).  Amplitudes in
+ * other channels do not enter; the error of a result stays at about 1e-14 of the largest sum of
+ * absolute products in its channels (measured from MBPT2 amplitudes: at most 3e-15 of its own). */
 int pnm_apply_ph_term(pnm_ctx *ctx, int sys, int precision, const double *t, double *r, size_t n);
 
 /* Device time (ms, CUDA events) of the last pnm_create*, pnm_mbpt2 and pnm_ccd_solve:

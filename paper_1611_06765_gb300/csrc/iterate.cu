@@ -283,9 +283,9 @@ __global__ void __launch_bounds__(128) k_lad_expand(DevState D, const T_* __rest
 // column holds the digits from 8 / SLOTS * s on, and one MMA forms SLOTS levels; 36, 26 and 15
 // MMAs per 16 x 16 block of V for up to 8, 4 and 2 rows.
 // What bounds it: the V stream for few rows, the tensor pipe (1024 multiply-adds per clock and SM
-// through mma.sync) for many.  Per launch with k_tdig (N = 66, n^2 <= 42, FP64): 80 us (V 250 MB in
+// through mma.sync) for many.  Per launch with k_tdig (N = 66, n^2 <= 42, FP64): 76 us (V 250 MB in
 // 60 us, 4.2 TB/s) against 291 us on the FP64 pipe; symmetric matter, 28 nucleons, n^2 <= 20: 43
-// against 119 us; three densities of N = 66, n^2 <= 36, pairs: 126 against 190 us on the FP32 pipe.
+// against 119 us; three densities of N = 66, n^2 <= 36, pairs: 125 against 190 us on the FP32 pipe.
 constexpr int PP_WARPS = 4, PP_CTAS = 3, PP_DEPTH = 4;  // warps per CTA, CTAs per SM, ring steps
 constexpr size_t PP_SMEM = sizeof(uint4) * 256 * PP_DEPTH * PP_WARPS;  // 64 KB: three CTAs per SM
 constexpr int PP_MAX_NLAD = 3376;  // ladder basis of a channel (the amplitudes of a row in shared memory)
@@ -294,7 +294,7 @@ constexpr int PP_MAX_NLAD = 3376;  // ladder basis of a channel (the amplitudes 
 // mostly of the digit products left out, which add up rather than average in channels of high symmetry (P = 0,
 // N = 14: to 2^-52).  In ordinary rows that is less than FP64 sums leave, but V and t fall off
 // exponentially, and a result all of whose products are small keeps little of them (two neutrons at density
-// 0.3, n^2 <= 36, where V spans more than 60 octaves: results off by 1e-3 of themselves).  So results PP_FAR
+// 0.3, n^2 <= 36, where V falls by 390 octaves: results off by 1e-3 of themselves).  So results PP_FAR
 // octaves below the product of the strip's and the row's largest values are summed in FP64 for amplitudes
 // given by the caller, and PP_FAR_STEEP below it where the interaction falls by more than PP_STEEP octaves
 // over the model space, with V held in FP64 for them (CHECK).  Elsewhere the errors from MBPT2 amplitudes

@@ -356,11 +356,12 @@ void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* 
 // Only the results leave as floating point.  A group of 32 threads (channels of at most PH_WARP_DIM
 // rows and columns) or of 128 (the others) takes a channel; a warp forms 16 x 8 blocks.
 // What bounds it: instruction issue and its latencies around the products (operand expansion,
-// drains, staging) at twelve warps per SM; without the MMAs it takes 6% less time.  One exponent for
-// all amplitudes of a system, their words made in two passes ahead of this kernel, took 13 us less of an
-// update of 330 (N = 66, n^2 <= 42; third-order sums of three densities of n^2 <= 36: 485, 515 us) but left
-// a channel far below the system's largest amplitude as few bits (relative errors of 5e-6 beside one
-// amplitude 2^20 above the others).
+// drains, staging) at twelve warps per SM; without the MMAs it takes 6% less time.  Per launch: N = 66,
+// n^2 <= 42, FP64 160 us against 405 us on the FP64 pipe; three densities of N = 66, n^2 <= 36, pairs, 337
+// against 356 us on the FP32 pipe; symmetric matter, 28 nucleons, n^2 <= 20, FP64 41 against 52 us.  One
+// exponent for all amplitudes of a system, their words made in two passes ahead of this kernel, took 153, 298
+// and 48 us but left a channel far below the system's largest amplitude few bits (errors of 5e-6 of
+// an element's own sum of products beside one amplitude 2^20 above the others).
 __host__ __device__ __forceinline__ constexpr int ph_h8(int H) { return (H + 7) & ~7; }
 // Row strides in 16-byte pairs: T's odd, C's 2 modulo 8, so that the fragment loads of the first
 // product (two rows per thread) and of the second spread over the banks.
