@@ -281,7 +281,7 @@ def measured_traffic(kernel, workload):
 
 DIGIT_KERNELS = ("k_pp64", "k_ph64", "k_pp_f2", "k_ph_f2")
 # kernels behind one entry of the profiler, where more than one: the digits of the amplitudes and the
-# ladder; exponents, digits, larger and smallest channels of the ph term
+# ladder; larger and smallest channels of the ph term
 LAUNCHES = {"k_pp64": 2, "k_pp_f2": 2, "k_ph64": 2, "k_ph_f2": 2, "k_ph32": 2}
 MIXED_KERNELS = ("k_update_mix", "k_ph32", "k_pp_tc", "k_tstats32", "k_pack", "k_dchi32")
 

@@ -310,7 +310,7 @@ constexpr int PP_FAR = 12, PP_FAR_STEEP = 4;
 __device__ __forceinline__ double lad_v(const DevState& D, const double* __restrict__ lut, int2 pair, int m, int mr,
                                         char4 ra, char4 rb) {
   const double y = v_minnesota_as(D.nvec[pair.x], D.nvec[pair.y], ra, rb, lut);
-  return (m > 0) == (mr > 0) ? y : -y;
+  return __hiloint2double(__double2hiint(y) ^ ((m ^ mr) & (int)0x80000000), __double2loint(y));
 }
 
 // sum_cd t(ij, cd) V(cd, ab) of one result in FP64, by one thread (rows with infinities or NaN in a solve,

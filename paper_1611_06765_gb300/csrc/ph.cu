@@ -357,11 +357,12 @@ void launch_ph_mix(pnm_ctx* ctx, const float* xt, const float* xw, const float* 
 // rows and columns) or of 128 (the others) takes a channel; a warp forms 16 x 8 blocks.
 // What bounds it: instruction issue and its latencies around the products (operand expansion,
 // drains, staging) at twelve warps per SM; without the MMAs it takes 6% less time.  Per launch: N = 66,
-// n^2 <= 42, FP64 160 us against 405 us on the FP64 pipe; three densities of N = 66, n^2 <= 36, pairs, 337
-// against 356 us on the FP32 pipe; symmetric matter, 28 nucleons, n^2 <= 20, FP64 41 against 52 us.  One
+// n^2 <= 42, FP64 149 us against 405 us on the FP64 pipe; three densities of N = 66, n^2 <= 36, pairs, 298
+// against 356 us on the FP32 pipe; symmetric matter, 28 nucleons, n^2 <= 20, FP64 40 against 52 us.  One
 // exponent for all amplitudes of a system, their words made in two passes ahead of this kernel, took 153, 298
-// and 48 us but left a channel far below the system's largest amplitude few bits (errors of 5e-6 of
-// an element's own sum of products beside one amplitude 2^20 above the others).
+// and 48 us and left a channel far below the system's largest amplitude few bits (errors of 5e-6 of
+// an element's own sum of products beside one amplitude 2^20 above the others).  Nothing of the staging may
+// take the FP64 pipe: the signs of the gathered amplitudes as negations made it 160, 337 and 41 us.
 __host__ __device__ __forceinline__ constexpr int ph_h8(int H) { return (H + 7) & ~7; }
 // Row strides in 16-byte pairs: T's odd, C's 2 modulo 8, so that the fragment loads of the first
 // product (two rows per thread) and of the second spread over the banks.
@@ -490,7 +491,11 @@ __device__ __forceinline__ void ph_dig(const DevState& D, const PhItem& it, int2
   // T: two neighbouring columns per step (index rows are padded to H8, rows past R read none), the
   // amplitudes and their largest exponent first, then their words, each thread its own elements
   const int wide = H8 / 2, total = R8 * wide, live = R * wide, du = GT / wide, ds = GT % wide;
-  auto amp = [&](int c) { return c == 0 ? 0.0 : (c > 0 ? t[c - 1] : -t[-c - 1]); };
+  auto amp = [&](int c) {  // the sign on its bit: a negation would take the FP64 pipe
+    if (c == 0) return 0.0;
+    const double v = t[abs(c) - 1];
+    return __hiloint2double(__double2hiint(v) ^ (c & (int)0x80000000), __double2loint(v));
+  };
   int et = 1;
   {
     int u = tid / wide, s = tid % wide;
