@@ -340,7 +340,7 @@ __device__ __noinline__ double pp_direct(const DevState& D, const double* __rest
 // 6 us a result).
 template <typename Out>
 __device__ __forceinline__ void pp_far(const DevState& D, const PPItem& it, const int* __restrict__ rows,
-                                       const double* __restrict__ lut, const double* __restrict__ s64,
+                                       const double* __restrict__ lut, const double* __restrict__ s64, bool steep,
                                        const unsigned char* __restrict__ far, int n) {
   const int lane = threadIdx.x & 31, nl = it.nl, off = D.ch_pp_off[it.c];
   const int2* __restrict__ mem = D.lad_mem + off;
@@ -355,7 +355,7 @@ __device__ __forceinline__ void pp_far(const DevState& D, const PPItem& it, cons
     ij[u] = rows ? rows[r] : r;
   }
   const double* __restrict__ sc = s64 + base;
-  if (D.v64) {
+  if (steep) {
     const double* __restrict__ vc = D.v64 + D.ch_vd_off[it.c];
     const int wide = (nl + 15) & ~15;
 #pragma unroll 2
@@ -414,7 +414,7 @@ template <int SLOTS, typename Out, bool CHECK>
 __device__ __forceinline__ int pp_pass(const DevState& D, const PPItem& it, const int* __restrict__ rows, int part,
                                        int wk, uint4* __restrict__ ring, DigSum* __restrict__ red,
                                        const double* __restrict__ lut, const double* __restrict__ t0,
-                                       const double* __restrict__ s64, unsigned char* __restrict__ far) {
+                                       const double* __restrict__ s64, bool steep, unsigned char* __restrict__ far) {
   constexpr int Q = 8 / SLOTS;  // rows ij of this pass, and digits per slot
   const int c = it.c, strip = it.strip, nl = it.nl, n0 = it.n0, nr = it.nr;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -510,10 +510,13 @@ __device__ __forceinline__ int pp_pass(const DevState& D, const PPItem& it, cons
         // the largest V of the strip times the largest amplitude of the row: 2^92 vtop ttop, the sum counts
         // in 2^56 and its part top in 2^88
         const long long top = x.hi + (x.lo >> 32);
-        const long long least = (long long)vtop * D.ttop[D.ch_hh_off[c] + ij] >> ((D.v64 ? PP_FAR_STEEP : PP_FAR) - 4);
+        // (nothing is less than 0: in a solve the systems beside a steep one)
+        const long long least = steep  ? (long long)vtop * D.ttop[D.ch_hh_off[c] + ij] >> (PP_FAR_STEEP - 4)
+                                : rows ? 0
+                                       : (long long)vtop * D.ttop[D.ch_hh_off[c] + ij] >> (PP_FAR - 4);
         if (!direct && top < least && top >= -least) {
           direct = true;
-          if (!D.v64) {  // small by cancellation only where the diagonal term is not (random amplitudes)
+          if (!steep) {  // small by cancellation only where the diagonal term is not (random amplitudes)
             const int off = D.ch_pp_off[c];
             const int2 p = D.pp_pair[off + abs(D.lad_mem[off + ab].x) - 1];
             const char4 a = D.nvec[p.x], b = D.nvec[p.y];
@@ -536,7 +539,8 @@ __device__ __forceinline__ int pp_pass(const DevState& D, const PPItem& it, cons
   return nfar;
 }
 
-// rep_only: the rows ij of the items count the list upd_row of the channel, else every hole pair.
+// rep_only: the rows ij of the items count the list upd_row of the channel, else every hole pair (the
+// operator: amplitudes given by the caller).
 // wk (2 or 4) divides PP_WARPS: PP_WARPS / wk items per CTA.  slots: ring steps per warp, PP_DEPTH or
 // as many as a warp has.  lut_off: interaction table of every system.  s64: the rows in the
 // ladder basis (CHECK).
@@ -566,18 +570,19 @@ __global__ void __launch_bounds__(PP_WARPS * 32, PP_CTAS) k_pp(DevState D, const
   const int c = it.c;
   const double* __restrict__ lut = D.lut + lut_off[it.sys];
   const double* __restrict__ t = cur_t(D, ctl) + D.ch_t_off[c];
+  const bool steep = CHECK && D.sys_steep && D.sys_steep[it.sys];
   unsigned char* list = far[CHECK ? first : 0];
   int left;
-  if (n > 4) left = pp_pass<1, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, s64, list);
-  else if (n > 2) left = pp_pass<2, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, s64, list);
-  else left = pp_pass<4, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, s64, list);
+  if (n > 4) left = pp_pass<1, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, s64, steep, list);
+  else if (n > 2) left = pp_pass<2, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, s64, steep, list);
+  else left = pp_pass<4, Out, CHECK>(D, it, rows, part, wk, ring, mine, lut, t, s64, steep, list);
   if (!CHECK) return;
   if (part == 0 && (threadIdx.x & 31) == 0) nfar[CHECK ? first : 0] = left;
   __syncthreads();
   left = nfar[CHECK ? first : 0];
   if (left == 0) return;
   // the item's warps take the results left in turn, four at a time
-  for (int k = 4 * part; k < left; k += 4 * wk) pp_far<Out>(D, it, rows, lut, s64, list + k, min(4, left - k));
+  for (int k = 4 * part; k < left; k += 4 * wk) pp_far<Out>(D, it, rows, lut, s64, steep, list + k, min(4, left - k));
 }
 
 // FP32-pair copy of an FP64 array.

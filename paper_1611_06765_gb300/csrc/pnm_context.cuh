@@ -119,7 +119,7 @@ struct pnm_ctx {
   size_t vl_smem = 0;
   double hbar2_2m = 0.0;
   double fall = 0.0;   // octaves by which a system's interaction falls over its model space, at most
-  bool steep = false;  // the interaction of a system falls by more than PP_STEEP octaves over its model space
+  std::vector<int> h_steep;  // per system: its interaction falls by more than PP_STEEP octaves over the model space
   int mlp_fallback = 0;  // 1 when the last learned start was replaced by the MBPT2 start
 
   // side streams for the independent parts of an update (ph term, pp ladder), joined by events

@@ -107,7 +107,10 @@ struct DevState {
   long *ch_vd_off, *ch_td_off;
   int *ch_vexp, *texp;
   unsigned *vtop, *ttop;
-  double* v64;  // the ladder-basis V in FP64, rows of the padded width at ch_vd_off (steep interactions only, else null)
+  // the ladder-basis V in FP64, rows of the padded width at ch_vd_off, of the systems whose interaction is
+  // steep (sys_steep; both null where none is)
+  double* v64;
+  int* sys_steep;
   double *den, *inv_den;  // eps_i + eps_j - eps_a - eps_b per amplitude, and its reciprocal
   // iteration state
   double *t0, *t1;       // double buffer, parity = iteration & 1

@@ -1008,7 +1008,8 @@ __global__ void __launch_bounds__(256) k_v_dig(const int4* __restrict__ items, c
                                                const int* __restrict__ ch_nlad, const long* __restrict__ ch_vd_off,
                                                const int2* __restrict__ lad_mem, const int2* __restrict__ pp_pair,
                                                const char4* __restrict__ nvec, const double* __restrict__ lut,
-                                               int* __restrict__ ch_vexp, unsigned* __restrict__ vtop, double* __restrict__ v64,
+                                               int* __restrict__ ch_vexp, unsigned* __restrict__ vtop, double* __restrict__ v64_all,
+                                               const int* __restrict__ ch_sys, const int* __restrict__ sys_steep,
                                                dig_t* __restrict__ vdig) {
   extern __shared__ __align__(16) unsigned char vsm[];
   __shared__ int sh_max;
@@ -1016,6 +1017,7 @@ __global__ void __launch_bounds__(256) k_v_dig(const int4* __restrict__ items, c
   long long* xlut = reinterpret_cast<long long*>(vsm);
   const int4 it = items[blockIdx.x];  // channel, first row, interaction table and its size (< 0: with protons)
   const int c = it.x, r0 = it.y, lut_elems = abs(it.w);
+  double* __restrict__ v64 = v64_all && sys_steep[ch_sys[c]] ? v64_all : nullptr;
   int nl = ch_nlad[c], off = ch_pp_off[c];
   char4* sa = reinterpret_cast<char4*>(xlut + lut_elems);
   char4* sb = sa + nl;
@@ -1169,7 +1171,9 @@ void pnm_need_vdig(pnm_ctx* ctx) {
   D.texp = ctx_alloc<int>(ctx, ctx->n_hh_pairs);
   D.ttop = ctx_alloc<unsigned>(ctx, ctx->n_hh_pairs);
   D.vtop = ctx_alloc<unsigned>(ctx, ctx->nvdig / 256);
-  if (ctx->steep) {  // before any capture of the ladder
+  if (std::find(ctx->h_steep.begin(), ctx->h_steep.end(), 1) != ctx->h_steep.end()) {  // before any capture
+    D.sys_steep = ctx_alloc<int>(ctx, ctx->h_steep.size());
+    h2d(D.sys_steep, ctx->h_steep, s);
     D.v64 = ctx_alloc<double>(ctx, ctx->nvdig);
     ctx->s64 = ctx_alloc<double>(ctx, std::max<long>(ctx->ns, 1));
   }
@@ -1177,7 +1181,7 @@ void pnm_need_vdig(pnm_ctx* ctx) {
   smem_at_least(k_v_dig, ctx->vl_smem);
   if (ctx->n_vl_items > 0)
     k_v_dig<<<ctx->n_vl_items, 256, ctx->vl_smem, s>>>(ctx->vl_items, D.ch_pp_off, D.ch_nlad, D.ch_vd_off, D.lad_mem,
-                                                       D.pp_pair, D.nvec, D.lut, D.ch_vexp, D.vtop, D.v64, D.vdig);
+                                                       D.pp_pair, D.nvec, D.lut, D.ch_vexp, D.vtop, D.v64, D.ch_sys, D.sys_steep, D.vdig);
   CUDA_TRY(cudaGetLastError());
 }
 
@@ -1230,7 +1234,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
     if (S.species != 1 && P.VT != 0.0) kappa = std::max(kappa, P.kT);
     const double octaves = kappa > 0.0 ? q1 * q1 * S.n2max / kappa / std::log(2.0) : 0.0;
     ctx->fall = std::max(ctx->fall, octaves);
-    ctx->steep = ctx->steep || octaves > (S.species == 1 ? PP_STEEP : PP_STEEP_PROTONS);
+    ctx->h_steep.push_back(octaves > (S.species == 1 ? PP_STEEP : PP_STEEP_PROTONS));
     S.lut_off = lut_total;
     S.lut_len = 4 * S.n2max + 1;
     lut_total += S.lut_len * (S.species == 1 ? 1 : 3);  // interleaved R, T, S halves with protons
@@ -1562,6 +1566,7 @@ void pnm_build(pnm_ctx* ctx, int nsys, const int* Ns, const int* Zs, const doubl
   k_occ<<<nsp_total, OCC_THREADS, 0, s>>>(1, SS, D.sp_sys, D.nvec, D.ch_pp_off, nullptr, D.occ_off, D.occ_idx);
   D.vdig = nullptr;  // the ladder V is built on first use
   D.v64 = nullptr;
+  D.sys_steep = nullptr;
   D.rpp = dalloc<double>(s_acc, ctx->owned, s);
   ctx->ntdig = td_acc;
   ctx->n_vl_items = (int)vl_items.size();

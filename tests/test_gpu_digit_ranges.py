@@ -179,3 +179,22 @@ def test_mixed_ladder_of_an_interaction_of_wide_range(pkg, N, Z, rho, n2, single
     seen = bound > 1e-30
     assert np.all(np.abs(r - ref)[seen] <= ((3 * 2.0 ** -18 + 500 * 2.0 ** -24) * bound)[seen])
     g.close()
+
+
+def test_steep_and_ordinary_systems_in_one_context(pkg):
+    """Only the systems whose interaction is steep have V in FP64 and their results checked in a solve: the
+    same arithmetic per system as in contexts of their own, so the same bits but for the order of the energy
+    sums, which end the iteration; 12 updates for all."""
+    Ns, rhos, n2 = [2, 14, 14], [0.3, 0.08, 0.3], [24, 9, 24]
+    kw = dict(alpha=0.5, tol=1e-300, max_iter=12, allow=(pkg.PNM_ENOTCONV,))
+    g = pkg.Context(Ns, rhos, n2)
+    g.solve(**kw)
+    for k in range(3):
+        one = pkg.Context(Ns[k], rhos[k], n2[k])
+        one.solve(**kw)
+        t, ref = g.get_amplitudes(k), one.get_amplitudes()
+        assert np.all(np.abs(t - ref) <= 1e-13 * np.abs(ref))
+        a = random_amplitudes(len(t), seed=k)
+        assert np.array_equal(g.apply_pp_ladder(a, sys=k), one.apply_pp_ladder(a))
+        one.close()
+    g.close()
